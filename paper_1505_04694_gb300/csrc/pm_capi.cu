@@ -82,8 +82,11 @@ __global__ void k_ingest(Store S, const double* xy, const int* tri, const uint8_
     if (g < nv) {
       int mi = seg_of(pv, n, g);
       int slot = S.tab.vbase[mi] + (g - pv[mi]);
-      S.xy[slot] = make_double2(xy[2 * (size_t)g], xy[2 * (size_t)g + 1]);
-      S.M[slot] = make_double4(1.0, 0.0, 1.0, 0.0);
+      const double2 p = make_double2(xy[2 * (size_t)g], xy[2 * (size_t)g + 1]);
+      const double4 m = make_double4(1.0, 0.0, 1.0, 0.0);
+      S.xy[slot] = p;
+      S.M[slot] = m;
+      store_vf(S, slot, p, m);
       S.vflag[slot] = (uint8_t)(VF_ALIVE | ((corner && corner[g]) ? VF_CORNER : 0));
     }
     if (g < ne) {
@@ -109,7 +112,10 @@ __global__ void k_metric_set(Store S, const double* m, int nv) {
   for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < nv; g += gridDim.x * blockDim.x) {
     int mi = seg_of(S.tab.pre, n, g);
     int slot = S.tab.vbase[mi] + (g - S.tab.pre[mi]);
-    S.M[slot] = make_double4(m[3 * (size_t)g], m[3 * (size_t)g + 1], m[3 * (size_t)g + 2], 0.0);
+    const double4 mv =
+        make_double4(m[3 * (size_t)g], m[3 * (size_t)g + 1], m[3 * (size_t)g + 2], 0.0);
+    S.M[slot] = mv;
+    store_vf(S, slot, S.xy[slot], mv);
   }
 }
 
@@ -429,6 +435,7 @@ pm_status copy_region(MeshSet& dst, int di, MeshSet& src, int si, cudaStream_t s
   cudaError_t e = cudaSuccess;
   if (!e) e = cp(dst.S.xy + vd, src.S.xy + vs, nv * sizeof(double2));
   if (!e) e = cp(dst.S.M + vd, src.S.M + vs, nv * sizeof(double4));
+  if (!e) e = cp(dst.S.F + 2 * vd, src.S.F + 2 * vs, nv * 2 * sizeof(float4));
   if (!e) e = cp(dst.S.vflag + vd, src.S.vflag + vs, nv);
   if (!e) e = cp(dst.S.NNlen + vd, src.S.NNlen + vs, nv * sizeof(int));
   if (!e) e = cp(dst.S.NElen + vd, src.S.NElen + vs, nv * sizeof(int));

@@ -9,6 +9,7 @@
 #include <stdint.h>
 
 #include "../../include/pm.h"
+#include "pm_filter.cuh"
 
 namespace pm {
 
@@ -60,6 +61,7 @@ struct Store {
   int eused;
   double2* xy;
   double4* M;     // (m00, m01, m11, 0)
+  float4* F;      // FP32 record of every vertex slot (VF, two float4): follows xy and M
   uint8_t* vflag;
   int4* EN;       // (v0, v1, v2, alive)
   double* qK;     // quality of every live element (kept current by all operators)
@@ -308,6 +310,19 @@ __device__ __forceinline__ VD load_vd(const Store& S, int slot) {
   double2 p = S.xy[slot];
   double4 m = S.M[slot];
   return VD{p.x, p.y, m.x, m.y, m.z};
+}
+
+// The FP32 record of a slot (pm_filter.cuh): one 32-byte sector.
+__device__ __forceinline__ VF load_vf(const Store& S, int slot) {
+  const float4 p = S.F[2 * (size_t)slot], m = S.F[2 * (size_t)slot + 1];
+  return VF{p.x, p.y, p.z, p.w, m.x, m.y, m.z, m.w};
+}
+
+// Writes a slot's record; every change of xy or M is followed by this.
+__device__ __forceinline__ void store_vf(const Store& S, int slot, double2 p, double4 m) {
+  const VF v = make_vf(p.x, p.y, m.x, m.y, m.z);
+  S.F[2 * (size_t)slot] = make_float4(v.xh, v.xl, v.yh, v.yl);
+  S.F[2 * (size_t)slot + 1] = make_float4(v.m00, v.m01, v.m11, v.e);
 }
 
 // The position alone, read again through L2 (ld.global.cg, never merged

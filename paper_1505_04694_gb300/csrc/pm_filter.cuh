@@ -1,0 +1,183 @@
+// FP32 filters in front of the exact FP64 decisions.
+//
+// GB300 retires 2 FP64 results per SM and cycle and 128 FP32 results, so the
+// evaluation kernels were bound by FP64 arithmetic whose answer is a yes or
+// no (a quality not above a bound, an edge longer than L_up, a point on one
+// side of a line), most of which single precision with a rigorous error bound
+// can give.  Every filter returns "undecided" unless its answer is certain
+// for the value the FP64 code computes; the caller then runs that code.  So
+// no result changes, only the number of FP64 instructions behind it.
+//
+// Input: one 32-byte record per vertex (one DRAM sector; position and metric
+// in double take 48 bytes in two sectors): each coordinate as two floats
+// xh = RN(x), xl = RN(x - xh), the metric rounded to float, and `e`, an
+// absolute error that covers what two floats leave out.
+//
+// Error bounds, u = 2^-24 (half an ulp).  A coordinate is x = xh + xl + d,
+// |d| <= u^2 |x|.  The difference D = (qh - ph) + (ql - pl): the first
+// subtraction is exact when the operands are within a factor of two, else its
+// rounding is relative to D; so
+//   |D - (q - p)| <= 3 u |D| + e_q + e_p,   e = 2^-46 max(|x|, |y|) + 1e-37
+// (twice the bound u |ql - pl| + u^2 (|q| + |p|)).  Everything below bounds the
+// rounding of its own formula on top of that; constants are rounded up.  The
+// FP64 code's own rounding error is that of the same formula with 2^-53 in
+// place of u, far inside the margin.  Overflow and NaN make every test false
+// (undecided); underflow is covered by the absolute terms 1e-36.
+//
+// Plain C++ apart from the markers, so that a host build can check the bounds
+// against exact arithmetic.
+#pragma once
+
+#include <math.h>
+
+#ifdef __CUDACC__
+#define PM_HD __host__ __device__ __forceinline__
+#else
+#define PM_HD inline
+#endif
+
+namespace pm {
+
+struct VF {
+  float xh, xl, yh, yl;
+  float m00, m01, m11, e;
+};
+
+constexpr float kU = 5.9604645e-8f;  // 2^-24
+constexpr float kTiny = 1e-36f;
+
+// sqrt and reciprocal to within 2 u relative on either side (the device's
+// approximate instructions are specified to 2^-23; inputs here are normal or
+// lead to an undecided result)
+PM_HD float f_sqrt(float x) {
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+#else
+  return sqrtf(x);
+#endif
+}
+PM_HD float f_rcp(float x) {
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+#else
+  return 1.0f / x;
+#endif
+}
+
+PM_HD VF make_vf(double x, double y, double m00, double m01, double m11) {
+  VF v;
+  v.xh = (float)x;
+  v.xl = (float)(x - (double)v.xh);
+  v.yh = (float)y;
+  v.yl = (float)(y - (double)v.yh);
+  v.m00 = (float)m00;
+  v.m01 = (float)m01;
+  v.m11 = (float)m11;
+  v.e = 1.4210855e-14f * fmaxf(fabsf(v.xh), fabsf(v.yh)) + 1e-37f;  // 2^-46
+  // a metric that single precision cannot hold with full relative precision:
+  // every test of the vertex is undecided
+  const bool holds = v.m00 > 1e-30f && v.m00 < 1e30f && v.m11 > 1e-30f && v.m11 < 1e30f;
+  if (!holds) v.e = INFINITY;
+  return v;
+}
+
+PM_HD float f_dx(const VF& p, const VF& q) { return (q.xh - p.xh) + (q.xl - p.xl); }
+PM_HD float f_dy(const VF& p, const VF& q) { return (q.yh - p.yh) + (q.yl - p.yl); }
+
+// Twice the signed area of (p, q, r) and a bound of its error.  Products of
+// differences: 2 * 3 u + u each, their difference u: 8 u (|t1| + |t2|), taken
+// as 10 u; the absolute parts E of the differences enter linearly and squared.
+struct FDet {
+  float det, err;
+};
+PM_HD FDet f_det(float ax, float ay, float bx, float by, float E) {
+  const float t1 = ax * by, t2 = ay * bx;
+  FDet d;
+  d.det = t1 - t2;
+  const float sum = (fabsf(ax) + fabsf(ay)) + (fabsf(bx) + fabsf(by));
+  d.err = 10.0f * kU * (fabsf(t1) + fabsf(t2)) + (1.25f * E * (sum + 2.0f * E) + kTiny);
+  return d;
+}
+
+// Sign of the exact orientation of (p, q, r): +1, -1, or 0 when undecided.
+PM_HD int f_orient(const VF& p, const VF& q, const VF& r) {
+  const FDet d = f_det(f_dx(p, q), f_dy(p, q), f_dx(p, r), f_dy(p, r), p.e + (q.e + r.e));
+  return d.det > d.err ? 1 : (d.det < -d.err ? -1 : 0);
+}
+
+// Squared length of (dx, dy) under the metric (k00, k01, k11), relative error
+// `ku` of its entries (of |k01|'s bound sqrt(k00 k11) for k01), and a bound of
+// the error: (ku + 8 u) (t0 + |t1| + t2) for the three terms, 2 u of the same
+// for their sum, and |t1| <= t0 + t2 for a positive definite metric.
+struct FLen {
+  float L2, err;
+};
+PM_HD FLen f_len2(float k00, float k01, float k11, float dx, float dy, float E, float ku) {
+  const float t0 = (k00 * dx) * dx, t2 = (k11 * dy) * dy;
+  FLen l;
+  l.L2 = (t0 + ((2.0f * k01) * dx) * dy) + t2;
+  l.err = (2.0f * ku + 24.0f * kU) * (t0 + t2) +
+          (4.0f * E * (k00 + k11) * ((fabsf(dx) + fabsf(dy)) + E) + kTiny);
+  return l;
+}
+
+// Squared metric length of edge (a, b) under the mean of its ends' metrics.
+PM_HD FLen f_edge2(const VF& a, const VF& b) {
+  return f_len2(0.5f * (a.m00 + b.m00), 0.5f * (a.m01 + b.m01), 0.5f * (a.m11 + b.m11),
+                f_dx(a, b), f_dy(a, b), a.e + b.e, 2.0f * kU);
+}
+
+// The length against a bound t whose square lies between lo2 and hi2 (floats
+// rounded outwards): +1 certainly longer, -1 certainly shorter, 0 undecided.
+PM_HD int f_len_cmp(const FLen& l, float lo2, float hi2) {
+  return l.L2 - l.err > hi2 ? 1 : (l.L2 + l.err < lo2 ? -1 : 0);
+}
+
+// An upper bound of the quality (12 sqrt 3 A / P^2) F(P / 3) of element
+// (a, b, c) in its mean metric, or NaN when the bound would be loose.  The
+// quality grows with the area and the metric's determinant, which are taken at
+// their upper bounds; as a function of P it is h(P) = F(P / 3) / P^2 with
+// |d ln h / d ln P| <= 5 (between -2 and 1 below the ideal perimeter, between
+// -5 and -2 above), so a relative error rP of P changes it by at most 5 rP to
+// first order (rP <= 0.04 is required, the rest of the series is inside the
+// factor 1.15).  `sign` receives the orientation's sign, 0 when undecided.
+PM_HD float f_quality_up(const VF& a, const VF& b, const VF& c, int& sign) {
+  const float E = a.e + (b.e + c.e);
+  const float dx0 = f_dx(a, b), dy0 = f_dy(a, b);
+  const float dx1 = f_dx(b, c), dy1 = f_dy(b, c);
+  const float dx2 = f_dx(a, c), dy2 = f_dy(a, c);
+  const FDet d = f_det(dx0, dy0, dx2, dy2, E);
+  sign = d.det > d.err ? 1 : (d.det < -d.err ? -1 : 0);
+  constexpr float third = 0.33333334f;
+  const float k00 = ((a.m00 + b.m00) + c.m00) * third;
+  const float k01 = ((a.m01 + b.m01) + c.m01) * third;
+  const float k11 = ((a.m11 + b.m11) + c.m11) * third;
+  constexpr float ku = 5.0f * kU;
+  const FLen q0 = f_len2(k00, k01, k11, dx0, dy0, E, ku);
+  const FLen q1 = f_len2(k00, k01, k11, dx1, dy1, E, ku);
+  const FLen q2 = f_len2(k00, k01, k11, dx2, dy2, E, ku);
+  const float l0 = f_sqrt(q0.L2), l1 = f_sqrt(q1.L2), l2 = f_sqrt(q2.L2);
+  const float P = (l0 + l1) + l2;
+  const float rp = f_rcp(P);
+  // sqrt(L2) - sqrt(L2 - err) <= 0.75 err / sqrt(L2) while err <= L2 / 2
+  const float eP = 0.75f * ((q0.err * f_rcp(l0) + q1.err * f_rcp(l1)) + q2.err * f_rcp(l2));
+  const float rP = eP * rp + 6.0f * kU;
+  const float kk = k00 * k11;
+  // (perimeters and metrics whose powers would underflow give no bound)
+  const bool fine = rP < 0.04f && q0.err < 0.4f * q0.L2 && q1.err < 0.4f * q1.L2 &&
+                    q2.err < 0.4f * q2.L2 && P > 1e-6f && P < 1e6f && kk > 1e-30f;
+  const float D = (kk - k01 * k01) + 28.0f * kU * kk;
+  const float up = 0.5f * (d.det + d.err);
+  const float area = up < 0.0f ? 0.0f : up;  // a negative quality is below 0 (a NaN stays)
+  const float x = P * third;
+  const float s = x > 1.0f ? 3.0f * rp : x;
+  const float f = s * (2.0f - s);
+  const float q = ((20.784612f * area) * f_sqrt(D)) * ((rp * rp) * ((f * f) * f));
+  return fine ? q + (q * (5.75f * rP + 40.0f * kU) + 1e-30f) : nanf("");
+}
+
+}  // namespace pm

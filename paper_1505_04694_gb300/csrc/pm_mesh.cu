@@ -132,6 +132,8 @@ __global__ void k_relayout_v(Store A, Store B) {
     int ns = B.tab.vbase[mi] + (s - A.tab.vbase[mi]);
     B.xy[ns] = A.xy[s];
     B.M[ns] = A.M[s];
+    B.F[2 * (size_t)ns] = A.F[2 * (size_t)s];
+    B.F[2 * (size_t)ns + 1] = A.F[2 * (size_t)s + 1];
     B.vflag[ns] = A.vflag[s];
     B.touch[ns] = A.touch[s];
     B.ntouch[ns] = A.ntouch[s];
@@ -406,6 +408,8 @@ __global__ void k_renum_v(Store A, Store B, const int* vscan, const int* escan,
     int ns = vb + (vscan[s] - v0);
     B.xy[ns] = A.xy[s];
     B.M[ns] = A.M[s];
+    B.F[2 * (size_t)ns] = A.F[2 * (size_t)s];
+    B.F[2 * (size_t)ns + 1] = A.F[2 * (size_t)s + 1];
     B.vflag[ns] = A.vflag[s];
     B.touch[ns] = A.touch[s];
     B.ntouch[ns] = A.ntouch[s];
@@ -690,6 +694,7 @@ static void carve_store(Carver& cv, Store& S) {
   size_t V = S.vslots, E = S.eslots, W = S.W;
   cv.add(&S.xy, V);
   cv.add(&S.M, V);
+  cv.add(&S.F, 2 * V);
   cv.add(&S.EN, E);
   cv.add(&S.qK, E);
   cv.add(&S.NN, V * W);
@@ -1069,6 +1074,7 @@ int renumber(MeshSet& m, bool final) {
   }
   std::swap(m.S.xy, m.B.xy);
   std::swap(m.S.M, m.B.M);
+  std::swap(m.S.F, m.B.F);
   std::swap(m.S.vflag, m.B.vflag);
   std::swap(m.S.EN, m.B.EN);
   std::swap(m.S.qK, m.B.qK);

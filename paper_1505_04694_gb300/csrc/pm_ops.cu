@@ -1322,215 +1322,142 @@ __device__ __forceinline__ double flip_gain(const Store& S, MeshCtx c, int lv, c
 // into both vertices' slots (the other's slot of the same element pair is
 // found in its sorted element row); the other item does no arithmetic.
 //
-// A warp pays the FP64 issue cost of an instruction once whatever its active
-// lanes, so the items that need arithmetic are collected in per-warp queues
-// in shared memory and evaluated 32 at a time (full warps).  The tests of a
-// gain end early (a decided negative orientation, a quality not above the
-// old minimum), so each stage has its own queue: orientations, first
-// quality, second quality and gain; an item that passes a stage joins the
-// next stage's queue.  Only the last batch of each queue may be partial.
+// The gain is -1, which the scan has left in its slot, unless both new
+// elements are counter-clockwise and their qualities above the old minimum.
+// Most items fail one of these, and the FP32 filters decide that (an
+// orientation certainly negative, an upper bound of a quality below the old
+// minimum) without an FP64 instruction.  What is left is collected in a
+// per-warp queue in shared memory and evaluated in FP64, 16 flips at a time:
+// two lanes a flip, one new element each, so that a warp's FP64 instructions
+// run with all lanes and the two qualities of a flip side by side instead of
+// one after the other.
 // At most 8 warps per block.
 constexpr int kEdgeQueueWarps = 8;
 
-// Queued item q = (v, k1 | k2 << 8 | both << 16 | open << 17, mesh, slot of
-// w): the flip of edge (v, w) between v's ball elements k1 and k2.
-struct FlipGeom {
-  MeshCtx c;
-  int lv, w, cc, d, K1, K2;
+// A queued flip of edge (v, w) between v's ball elements K1 = (v, w, c) and
+// K2 = (v, d, w): id = (v, k1 | k2 << 8 | both << 16 | open signs << 17,
+// first vertex slot of the mesh, K2), vt = local ids (v, w, c, d).
+struct FlipQueue {
+  int4 *id, *vt;
+  double* qold;
+  int n;  // entries, the same in every lane
 };
 
-__device__ __forceinline__ FlipGeom flip_geom(const Store& S, int4 q) {
-  FlipGeom g;
-  g.c.mi = q.z;
-  g.c.vb = S.tab.vbase[q.z];
-  g.c.eb = S.tab.ebase[q.z];
-  g.lv = q.x - g.c.vb;
-  const int* ne = ne_row(S, q.x);
-  g.K1 = ne[q.y & 0xFF];
-  g.K2 = ne[(q.y >> 8) & 0xFF];
-  const int4 e = S.EN[g.c.eb + g.K1];
-  const int4 f = S.EN[g.c.eb + g.K2];
-  g.w = (e.x == g.lv) ? e.y : (e.y == g.lv) ? e.z : e.x;
-  g.cc = (e.x == g.lv) ? e.z : (e.y == g.lv) ? e.x : e.y;
-  g.d = (f.x == g.lv) ? f.y : (f.y == g.lv) ? f.z : f.x;
-  return g;
-}
-
-__device__ __forceinline__ double flip_qold(const Store& S, const FlipGeom& g) {
-  const double q1 = S.qK[g.c.eb + g.K1], q2 = S.qK[g.c.eb + g.K2];
-  return dlt(q1, q2) ? q1 : q2;
-}
-
-// The tests of flip_gain in the same order, one stage per queue: A the two
-// orientation filters (0: failed, else 1 | the open signs << 1), B the first
-// new quality, C the second, the open signs exactly, the gain.
-__device__ __forceinline__ int flip_stage_a(const Store& S, int4 q, unsigned& ops) {
-  const FlipGeom g = flip_geom(S, q);
-  // the flipped edge (c, d) must not exist already
-  if (row_has(nn_row(S, g.c.vb + g.d), S.NNlen[g.c.vb + g.d], g.cc)) return 0;
-  const VD dv = load_vd(S, g.c.vb + g.lv), dw = load_vd(S, g.c.vb + g.w),
-           dc = load_vd(S, g.c.vb + g.cc), dd = load_vd(S, g.c.vb + g.d);
-  const int s1 = orient_filter(dv, dd, dc);
-  ops += kOpsOrient;
-  if (s1 < 0) return 0;
-  const int s2 = orient_filter(dd, dw, dc);
-  ops += kOpsOrient;
-  if (s2 < 0) return 0;
-  return 1 | (s1 == 0 ? 2 : 0) | (s2 == 0 ? 4 : 0);
-}
-
-__device__ __forceinline__ bool flip_stage_b(const Store& S, int4 q, double& n1, unsigned& ops) {
-  const FlipGeom g = flip_geom(S, q);
-  const VD dv = load_vd(S, g.c.vb + g.lv), dc = load_vd(S, g.c.vb + g.cc),
-           dd = load_vd(S, g.c.vb + g.d);
-  n1 = quality_c(g.lv, g.d, g.cc, dv, dd, dc);
-  ops += kOpsQuality;
-  return dgt(n1, flip_qold(S, g));
-}
-
-__device__ __forceinline__ double flip_stage_c(const Store& S, int4 q, double n1, unsigned& ops) {
-  const FlipGeom g = flip_geom(S, q);
-  const double qold = flip_qold(S, g);
-  const VD dw = load_vd(S, g.c.vb + g.w), dc = load_vd(S, g.c.vb + g.cc),
-           dd = load_vd(S, g.c.vb + g.d);
-  const double n2 = quality_c(g.d, g.w, g.cc, dd, dw, dc);
-  ops += kOpsQuality;
-  if (!dgt(n2, qold)) return -1.0;
-  const int open = (q.y >> 18) & 3;
-  if (open) {
-    const VD pv = load_xy_again(S, g.c.vb + g.lv), pw = load_xy_again(S, g.c.vb + g.w),
-             pc = load_xy_again(S, g.c.vb + g.cc), pd = load_xy_again(S, g.c.vb + g.d);
-    if ((open & 1) && orient_resolve(pv, pd, pc) <= 0) return -1.0;
-    if ((open & 2) && orient_resolve(pd, pw, pc) <= 0) return -1.0;
+// Evaluates the first `cnt` (<= 16) queued flips; all lanes call.
+__device__ __forceinline__ void flip_run(const Store& S, FlipQueue& Q, int cnt, double* gains,
+                                         unsigned& ops) {
+  const int lane = threadIdx.x & 31, j = lane >> 1;
+  const bool second = lane & 1;  // element (d, w, c); else (v, d, c)
+  bool ok = false;
+  double q = 0.0, qold = 0.0;
+  int4 id = make_int4(0, 0, 0, 0), vt = make_int4(0, 0, 0, 0);
+  if (j < cnt) {
+    id = Q.id[j];
+    vt = Q.vt[j];
+    qold = Q.qold[j];
+    const int i0 = second ? vt.w : vt.x, i1 = second ? vt.y : vt.w, i2 = vt.z;
+    const VD a = load_vd(S, id.z + i0), b = load_vd(S, id.z + i1), c = load_vd(S, id.z + i2);
+    q = quality_c(i0, i1, i2, a, b, c);
+    ops += kOpsQuality;
+    ok = dgt(q, qold);
+    if (ok && ((id.y >> (second ? 18 : 17)) & 1)) {
+      ops += kOpsOrient;
+      ok = orient_sign(load_xy_again(S, id.z + i0), load_xy_again(S, id.z + i1),
+                       load_xy_again(S, id.z + i2)) > 0;
+    }
   }
-  ops += 1;
-  return (dlt(n1, n2) ? n1 : n2) - qold;
-}
-
-// The gain of item q into v's slot and, when w evaluates the same edge this
-// round, into w's slot of the same element pair.
-__device__ __forceinline__ void flip_store_gain(const Store& S, int4 q, double g, double* gains) {
-  const int v = q.x;
-  gains[(size_t)v * S.W + (q.y & 0xFF)] = g;
-  if ((q.y >> 16) & 1) {
-    // from w's side the pair is (K2, K1): w's slot of K2
-    const int K2 = ne_row(S, v)[(q.y >> 8) & 0xFF];
-    const int* nw = ne_row(S, q.w);
-    const int nwl = S.NElen[q.w];
-    int kk = 0;
-    while (kk < nwl && nw[kk] < K2) ++kk;
-    if (kk < nwl) gains[(size_t)q.w * S.W + kk] = g;
-  }
-}
-
-// Per-warp stage queues (shared memory), each holding fewer than 32 entries
-// between calls; the counts are the same in every lane.  All lanes call.
-struct FlipQueues {
-  int4 *a, *b, *c;
-  double* n1;
-  int na, nb, nc;
-};
-
-__device__ __forceinline__ void flip_run_c(const Store& S, FlipQueues& Q, int cnt, double* gains,
-                                           unsigned& ops) {
-  const int lane = threadIdx.x & 31;
-  if (lane < cnt) {
-    const int4 q = Q.c[lane];
-    flip_store_gain(S, q, flip_stage_c(S, q, Q.n1[lane], ops), gains);
+  const unsigned okm = __ballot_sync(0xffffffffu, ok);
+  const double q2 = __shfl_xor_sync(0xffffffffu, q, 1);
+  if (!second && ((okm >> lane) & 3u) == 3u) {
+    ++ops;
+    const double g = (dlt(q, q2) ? q : q2) - qold;
+    const int v = id.x;
+    gains[(size_t)v * S.W + (id.y & 0xFF)] = g;
+    if ((id.y >> 16) & 1) {
+      // from w's side the pair is (K2, K1): w's slot of K2
+      const int ws = id.z + vt.y;
+      const int* nw = ne_row(S, ws);
+      const int kk = row_find(nw, S.NElen[ws], id.w);
+      if (kk >= 0) gains[(size_t)ws * S.W + kk] = g;
+    }
   }
   __syncwarp();
-  if (lane < Q.nc - cnt) {
-    Q.c[lane] = Q.c[cnt + lane];
-    Q.n1[lane] = Q.n1[cnt + lane];
-  }
-  Q.nc -= cnt;
-  __syncwarp();
-}
-
-__device__ __forceinline__ void flip_run_b(const Store& S, FlipQueues& Q, int cnt, double* gains,
-                                           unsigned& ops) {
-  const int lane = threadIdx.x & 31;
-  bool pass = false;
-  int4 q = make_int4(0, 0, 0, 0);
-  double n1 = 0.0;
-  if (lane < cnt) {
-    q = Q.b[lane];
-    pass = flip_stage_b(S, q, n1, ops);
-    if (!pass) flip_store_gain(S, q, -1.0, gains);
+  int4 mid = make_int4(0, 0, 0, 0), mvt = mid;
+  double mq = 0.0;
+  const bool move = lane < Q.n - cnt;
+  if (move) {
+    mid = Q.id[cnt + lane];
+    mvt = Q.vt[cnt + lane];
+    mq = Q.qold[cnt + lane];
   }
   __syncwarp();
-  if (lane < Q.nb - cnt) Q.b[lane] = Q.b[cnt + lane];
-  Q.nb -= cnt;
-  const unsigned m = __ballot_sync(0xffffffffu, pass);
-  if (pass) {
-    const int at = Q.nc + __popc(m & ((1u << lane) - 1u));
-    Q.c[at] = q;
-    Q.n1[at] = n1;
+  if (move) {
+    Q.id[lane] = mid;
+    Q.vt[lane] = mvt;
+    Q.qold[lane] = mq;
   }
-  Q.nc += __popc(m);
+  Q.n -= cnt;
   __syncwarp();
-  if (Q.nc >= 32) flip_run_c(S, Q, 32, gains, ops);
-}
-
-__device__ __forceinline__ void flip_run_a(const Store& S, FlipQueues& Q, int cnt, double* gains,
-                                           unsigned& ops) {
-  const int lane = threadIdx.x & 31;
-  bool pass = false;
-  int4 q = make_int4(0, 0, 0, 0);
-  if (lane < cnt) {
-    q = Q.a[lane];
-    const int r = flip_stage_a(S, q, ops);
-    pass = r != 0;
-    if (pass) q.y |= (r >> 1) << 18;
-    else flip_store_gain(S, q, -1.0, gains);
-  }
-  __syncwarp();
-  if (lane < Q.na - cnt) Q.a[lane] = Q.a[cnt + lane];
-  Q.na -= cnt;
-  const unsigned m = __ballot_sync(0xffffffffu, pass);
-  if (pass) Q.b[Q.nb + __popc(m & ((1u << lane) - 1u))] = q;
-  Q.nb += __popc(m);
-  __syncwarp();
-  if (Q.nb >= 32) flip_run_b(S, Q, 32, gains, ops);
 }
 
 __device__ __forceinline__ void swap_edge_phase(Store S, const int2* items, const int* nIp,
                                                 double* gains, int tag, unsigned long long* work,
                                                 bool il = false) {
-  __shared__ int4 sqa[kEdgeQueueWarps][64];
-  __shared__ int4 sqb[kEdgeQueueWarps][64];
-  __shared__ int4 sqc[kEdgeQueueWarps][64];
-  __shared__ double sn1[kEdgeQueueWarps][64];
+  // at most 15 entries stay queued between turns, a turn adds at most 32
+  __shared__ int4 s_id[kEdgeQueueWarps][48];
+  __shared__ int4 s_vt[kEdgeQueueWarps][48];
+  __shared__ double s_q[kEdgeQueueWarps][48];
   const int n = *nIp;
   const int lane = threadIdx.x & 31;
   const int wq = (threadIdx.x >> 5) % kEdgeQueueWarps;
-  FlipQueues Q{sqa[wq], sqb[wq], sqc[wq], sn1[wq], 0, 0, 0};
+  FlipQueue Q{s_id[wq], s_vt[wq], s_q[wq], 0};
   unsigned ops = 0;
   for (int i0 = 0; i0 < n; i0 += gsize()) {
     const int i = i0 + grank(il);
     bool need = false;
-    int4 rec = make_int4(0, 0, 0, 0);
+    int4 id = make_int4(0, 0, 0, 0), vt = make_int4(0, 0, 0, 0);
+    double qold = 0.0;
     if (i < n) {
-      int2 it = items[i];
-      int v = it.x, k1 = it.y & 0xFF, k2 = it.y >> 8;
-      MeshCtx c = ctx_of(S, v);
+      const int2 it = items[i];
+      const int v = it.x, k1 = it.y & 0xFF, k2 = it.y >> 8;
+      const MeshCtx c = ctx_of(S, v);
       const int lv = v - c.vb;
-      const int4 e = S.EN[c.eb + ne_row(S, v)[k1]];
+      const int* ne = ne_row(S, v);
+      const int K1 = ne[k1], K2 = ne[k2];
+      const int4 e = S.EN[c.eb + K1], f = S.EN[c.eb + K2];
+      const double qa = S.qK[c.eb + K1], qb = S.qK[c.eb + K2];
       const int w = (e.x == lv) ? e.y : (e.y == lv) ? e.z : e.x;
-      const int sw = c.vb + w;
-      const bool both = S.evs[sw] == tag;
-      need = !both || lv < w;
-      rec = make_int4(v, k1 | (k2 << 8) | ((both ? 1 : 0) << 16), c.mi, sw);
+      const int cc = (e.x == lv) ? e.z : (e.y == lv) ? e.x : e.y;
+      const int d = (f.x == lv) ? f.y : (f.y == lv) ? f.z : f.x;
+      const bool both = S.evs[c.vb + w] == tag;
+      if (!both || lv < w) {
+        const VF fv = load_vf(S, v), fw = load_vf(S, c.vb + w), fc = load_vf(S, c.vb + cc),
+                 fd = load_vf(S, c.vb + d);
+        // the flipped edge (c, d) must not exist already
+        const bool dup = row_has(nn_row(S, c.vb + d), S.NNlen[c.vb + d], cc);
+        qold = dlt(qa, qb) ? qa : qb;
+        const float floor = __double2float_rd(qold);
+        int s1, s2;
+        const float u1 = f_quality_up(fv, fd, fc, s1), u2 = f_quality_up(fd, fw, fc, s2);
+        need = !dup && s1 >= 0 && s2 >= 0 && !(u1 < floor) && !(u2 < floor);
+        id = make_int4(v, k1 | (k2 << 8) | ((both ? 1 : 0) << 16) | ((s1 == 0 ? 1 : 0) << 17) |
+                              ((s2 == 0 ? 1 : 0) << 18),
+                       c.vb, K2);
+        vt = make_int4(lv, w, cc, d);
+      }
     }
     const unsigned m = __ballot_sync(0xffffffffu, need);
-    if (need) Q.a[Q.na + __popc(m & ((1u << lane) - 1u))] = rec;
-    Q.na += __popc(m);
+    if (need) {
+      const int at = Q.n + __popc(m & ((1u << lane) - 1u));
+      Q.id[at] = id;
+      Q.vt[at] = vt;
+      Q.qold[at] = qold;
+    }
+    Q.n += __popc(m);
     __syncwarp();
-    if (Q.na >= 32) flip_run_a(S, Q, 32, gains, ops);
+    while (Q.n >= 16) flip_run(S, Q, 16, gains, ops);
   }
-  if (Q.na > 0) flip_run_a(S, Q, Q.na, gains, ops);
-  if (Q.nb > 0) flip_run_b(S, Q, Q.nb, gains, ops);
-  if (Q.nc > 0) flip_run_c(S, Q, Q.nc, gains, ops);
+  if (Q.n > 0) flip_run(S, Q, Q.n, gains, ops);
   add_work(work, ops);
 }
 
@@ -2252,10 +2179,12 @@ __device__ __forceinline__ void smooth_apply_one(const Store& S, bool ok, int v,
       MeshCtx c = ctx_of(S, v);
       mi = c.mi;
       vb = c.vb;
-      S.xy[v] = mvxy[v];
+      const double2 p = mvxy[v];
       double4 mv = mvM[v];
       mv.w = 0.0;
+      S.xy[v] = p;
       S.M[v] = mv;
+      store_vf(S, v, p, mv);
       S.touch[v] = stamp;
       const int* ne = ne_row(S, v);
       int nel = S.NElen[v];
@@ -2400,6 +2329,7 @@ __global__ void k_opt_apply(Store S, const int* Sl, const int* nSp, double* qbal
       if (moved && t.tl == 0) {
         S.xy[v] = X;
         S.M[v] = Mv;
+        store_vf(S, v, X, Mv);
         S.touch[v] = stamp;
         const int* ne = ne_row(S, v);
         int nel = S.NElen[v];
@@ -2514,9 +2444,12 @@ __global__ void k_refine_newverts(Store S, const int* vscan, const RowMask* mask
       VD db = load_vd(S, vb + b);
       int slot = vb + base + rank;
       ++rank;
-      S.xy[slot] = make_double2(0.5 * (da.x + db.x), 0.5 * (da.y + db.y));
-      S.M[slot] = make_double4(0.5 * (da.m00 + db.m00), 0.5 * (da.m01 + db.m01),
-                               0.5 * (da.m11 + db.m11), 0.0);
+      const double2 p = make_double2(0.5 * (da.x + db.x), 0.5 * (da.y + db.y));
+      const double4 mid = make_double4(0.5 * (da.m00 + db.m00), 0.5 * (da.m01 + db.m01),
+                                       0.5 * (da.m11 + db.m11), 0.0);
+      S.xy[slot] = p;
+      S.M[slot] = mid;
+      store_vf(S, slot, p, mid);
       bool bedge = count_elems_with(S, ne, nel, eb, b) == 1;
       S.vflag[slot] = (uint8_t)(VF_ALIVE | (bedge ? VF_BND : 0));
       if (S.lid) S.lid[slot] = (slot - vb) - S.voff[mi];
