@@ -38,7 +38,7 @@ struct Work {
   int* target = nullptr;           // collapse target (local id) per vertex
   int4* opA = nullptr;             // flip record (w, c, d, K1) per vertex
   int* opK2 = nullptr;
-  double2* mvxy = nullptr;         // smoothing move per vertex
+  double2* mvxy = nullptr;         // smoothing move per vertex (shares its place with items)
   double4* mvM = nullptr;
   int* dmark = nullptr;            // per-round stamps
   int* amark = nullptr;
@@ -55,7 +55,8 @@ struct Work {
   int* clist = nullptr;            // refine: their children's slots, eslots
   int* E = nullptr;                // vertices evaluated in full this round
   int2* items = nullptr;           // flip candidates (vertex, edge slots) of this round
-  double* gains = nullptr;         // gain of each (vertex, ball-element slot), vslots * W
+  double* gains = nullptr;         // gain of each (vertex, ball-element slot), vslots * W (in the
+                                   // spare rows)
   int2* items2 = nullptr;          // second wave list (vertex, candidate rank)
   int* cand = nullptr;             // collapse candidates of each vertex by (length, id), vslots * W
   int* ncand = nullptr;
@@ -101,6 +102,7 @@ struct MeshSet {
   void* pinned = nullptr;      // slot of the process-wide pinned arena (hst, hcounts)
   bool pinned_own = false;     // slot too small: a private pinned allocation
   void* tabmem = nullptr;      // device block holding MeshTab arrays
+  void* rowmem = nullptr;      // device block holding the adjacency rows of both buffer sets
   int* lidbuf = nullptr;       // S.lid and S.voff when in use (vslots, nmesh)
   int* voffbuf = nullptr;
   int tag = 0;                 // per-round tag (even); the round's change stamp is tag + 1

@@ -53,6 +53,15 @@ void pinned_put(void* p) {
 // Only the arrays that are read before they are first written (stamps,
 // marks, counters, scan state) are cleared: clearing a whole store of many
 // gigabytes at every growth cost more than the growth itself.
+// Sizes are rounded up to a sixteenth of their power of two: meshes of nearly
+// the same size then ask the pool for the same blocks again, where a block a
+// little too small costs a new mapping (about 1 ms per GB).
+size_t pool_size(size_t bytes) {
+  size_t step = 256;
+  while (step * 32 <= bytes) step *= 2;
+  return (bytes + step - 1) / step * step;
+}
+
 struct Carver {
   struct Req {
     void** p;
@@ -69,7 +78,7 @@ struct Carver {
     size_t total = 0;
     for (auto& r : req) total += r.bytes;
     char* base = nullptr;
-    cudaError_t e = cudaMallocAsync((void**)&base, total, m.stream);
+    cudaError_t e = cudaMallocAsync((void**)&base, pool_size(total), m.stream);
     if (e != cudaSuccess) return e;
     m.allocs.push_back(base);
     size_t off = 0, zoff = 0, zlen = 0;  // adjacent cleared arrays share one memset
@@ -89,14 +98,29 @@ struct Carver {
   }
 };
 
-template <class T>
-cudaError_t dalloc(MeshSet& m, T** p, size_t count, bool zero) {
-  size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
-  cudaError_t e = cudaMallocAsync((void**)p, bytes, m.stream);
+// Everything whose size follows the row width W, in one allocation of its own
+// (a change of W replaces it and leaves no hole in the store): the rows of both
+// buffer sets and the collapse candidates.  The spare set's rows are written
+// only by a refinement round and by a compaction, both of which read no flip
+// gain, collapse length or moved ball quality, so those W doubles per vertex
+// (Work::gains) share them.
+cudaError_t rows_alloc(MeshSet& m, int W) {
+  const size_t n = (size_t)m.S.vslots * W;
+  char* base = nullptr;
+  cudaError_t e = cudaMallocAsync((void**)&base, pool_size(std::max<size_t>(5 * n, 1) * sizeof(int)),
+                                  m.stream);
   if (e != cudaSuccess) return e;
-  m.allocs.push_back(*p);
-  if (zero) e = cudaMemsetAsync(*p, 0, bytes, m.stream);
-  return e;
+  m.allocs.push_back(base);
+  m.rowmem = base;
+  int* p = (int*)base;
+  m.S.NN = p;
+  m.S.NE = p + n;
+  m.B.NN = p + 2 * n;
+  m.B.NE = p + 3 * n;
+  m.w.cand = p + 4 * n;
+  m.w.gains = (double*)m.B.NN;
+  m.S.W = m.B.W = W;
+  return cudaSuccess;
 }
 
 __device__ __forceinline__ bool vslot_used(const Store& S, int slot, int& mi) {
@@ -691,14 +715,12 @@ cudaError_t refresh_sizes(MeshSet& m) {
 }
 
 static void carve_store(Carver& cv, Store& S) {
-  size_t V = S.vslots, E = S.eslots, W = S.W;
+  size_t V = S.vslots, E = S.eslots;
   cv.add(&S.xy, V);
   cv.add(&S.M, V);
   cv.add(&S.F, 2 * V);
   cv.add(&S.EN, E);
   cv.add(&S.qK, E);
-  cv.add(&S.NN, V * W);
-  cv.add(&S.NE, V * W);
   // cleared: flags, row lengths and stamps
   cv.add(&S.vflag, V, true);
   cv.add(&S.NNlen, V, true);
@@ -762,8 +784,11 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   cv.add(&w.target, vs);
   cv.add(&w.opA, vs);
   cv.add(&w.opK2, vs);
+  // smoothing moves (16 + 32 bytes a vertex), and in the same place the flip and
+  // collapse work items (each interior edge gives at most two items and a
+  // planar mesh has < 3V edges): no operator uses both
   cv.add(&w.mvxy, vs);
-  cv.add(&w.mvM, vs);
+  cv.add(&w.mvM, (size_t)vs + 16);
   cv.add(&w.dmark, vs, true);
   cv.add(&w.amark, vs, true);
   cv.add(&w.cmark, vs, true);
@@ -778,11 +803,7 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   cv.add(&w.elist, es);
   cv.add(&w.clist, es);
   cv.add(&w.E, vs);
-  // each interior edge gives at most two items and a planar mesh has < 3V edges
-  cv.add(&w.items, (size_t)vs * 6 + 64);
-  cv.add(&w.gains, (size_t)vs * W);
   cv.add(&w.items2, vs);
-  cv.add(&w.cand, (size_t)vs * W);
   cv.add(&w.ncand, vs);
   cv.add(&w.counts, CN_NUM + 2 * n + 8, true);
   cv.add(&w.cprop, vs);
@@ -794,6 +815,8 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   cv.add(&m.scan.ticket, 1, true);
   m.scan.tiles_cap = tiles;
   if ((e = cv.commit(m))) return e;
+  if ((e = rows_alloc(m, W))) return e;
+  w.items = (int2*)w.mvxy;  // 48 bytes a vertex and 512 more: 6 vs + 64 items
   m.tabmem = t;
   MeshTab& T = S.tab;
   // 32-byte, then 8-byte aligned members first
@@ -924,6 +947,7 @@ cudaError_t grow(MeshSet& m, const std::vector<int>& vcap, const std::vector<int
   m.w = n2.w;
   m.scan = n2.scan;
   m.tabmem = n2.tabmem;
+  m.rowmem = n2.rowmem;
   m.lidbuf = n2.lidbuf;
   m.voffbuf = n2.voffbuf;
   m.allocs = n2.allocs;
@@ -936,30 +960,13 @@ cudaError_t grow(MeshSet& m, const std::vector<int>& vcap, const std::vector<int
 
 // Widen the adjacency rows to W (contents are rebuilt by the caller); every
 // other array, worklist and stamp keeps its place.
-// Frees `p` only when it is an allocation of its own (arrays carved from the
-// store's block go with the block).
-static void free_if_own(MeshSet& m, void* p) {
-  auto it = std::find(m.allocs.begin(), m.allocs.end(), p);
-  if (it == m.allocs.end()) return;
-  cudaFreeAsync(p, m.stream);
-  m.allocs.erase(it);
-}
-
 cudaError_t grow_rows(MeshSet& m, int W) {
-  void* ptrs[4] = {m.S.NN, m.S.NE, m.B.NN, m.B.NE};
-  for (void* p : ptrs) free_if_own(m, p);
-  size_t n = (size_t)m.S.vslots * W;
-  cudaError_t e;
-  if ((e = dalloc(m, &m.S.NN, n, false))) return e;
-  if ((e = dalloc(m, &m.S.NE, n, false))) return e;
-  if ((e = dalloc(m, &m.B.NN, n, false))) return e;
-  if ((e = dalloc(m, &m.B.NE, n, false))) return e;
-  m.S.W = W;
-  m.B.W = W;
-  free_if_own(m, m.w.gains);
-  free_if_own(m, m.w.cand);
-  if ((e = dalloc(m, &m.w.cand, n, false))) return e;
-  return dalloc(m, &m.w.gains, n, false);
+  auto it = std::find(m.allocs.begin(), m.allocs.end(), m.rowmem);
+  if (it != m.allocs.end()) {
+    cudaFreeAsync(m.rowmem, m.stream);
+    m.allocs.erase(it);
+  }
+  return rows_alloc(m, W);
 }
 
 int sync_status(MeshSet& m) {
@@ -1059,7 +1066,12 @@ int renumber(MeshSet& m, bool final) {
       vdead += m.nv[i] - m.hcounts[2 * i];
       edead += m.ne[i] - m.hcounts[2 * i + 1];
     }
-    if (8 * vdead <= m.S.vused && 8 * edead <= m.S.eused) {
+    long long vu = 0, eu = 0;
+    for (int i = 0; i < m.nmesh; ++i) {
+      vu += m.nv[i];
+      eu += m.ne[i];
+    }
+    if (8 * vdead <= vu && 8 * edead <= eu) {
       m.S.lid = m.lidbuf;
       m.S.voff = m.voffbuf;
       PM_LAUNCH(k_renum_ids, grid_for(m, m.S.vused), BLOCK, 0, m.stream, m.S, w.vscan, tot,
@@ -1082,6 +1094,7 @@ int renumber(MeshSet& m, bool final) {
   std::swap(m.S.NNlen, m.B.NNlen);
   std::swap(m.S.NE, m.B.NE);
   std::swap(m.S.NElen, m.B.NElen);
+  w.gains = (double*)m.B.NN;  // the scratch goes with the spare rows
   std::swap(m.S.touch, m.B.touch);
   std::swap(m.S.ntouch, m.B.ntouch);
   std::swap(m.S.evc, m.B.evc);
@@ -1149,7 +1162,9 @@ int compact_out_set(MeshSet& m, double* xy, int32_t* tri, double* mt, int* nv_ou
 // holds at most about 2.2 times the larger of its element count and the
 // element count its metric asks for (refinement overshoots before the
 // collapses that follow), so every mesh below 2.5 times the estimate grows
-// now, together, instead of round after round of refinement.
+// now, together, instead of round after round of refinement (and some
+// thousands more: the estimate knows nothing of the boundary, which dominates
+// a coarse mesh of long elements).
 int presize(MeshSet& m) {
   const int n = m.nmesh;
   double* est = m.w.gains;  // scratch: no evaluation is kept across calls
@@ -1170,8 +1185,8 @@ int presize(MeshSet& m) {
     const double ne_est = 4.0 / std::sqrt(3.0) * h[i];
     const double want_e = 2.5 * std::max(ne_est, (double)m.ne[i]);
     if (std::isfinite(want_e) && want_e > ecap[i] && want_e < (double)(1 << 29)) {
-      ecap[i] = (int)want_e + 64;
-      vcap[i] = std::max(vcap[i], (int)(0.6 * want_e) + 64);
+      ecap[i] = (int)want_e + 8192;
+      vcap[i] = std::max(vcap[i], (int)(0.6 * want_e) + 4096);
       need = true;
     }
     vt += vcap[i];

@@ -3254,9 +3254,9 @@ int op_refine(MeshSet& m, int max_rounds) {
       if (err) return err;
     }
     for (int i = 0; i < m.nmesh; ++i) newv[i] = m.hcounts[CN_NUM + i];
-    // A growth moves every mesh of the set, so when one mesh needs room,
-    // every mesh that is splitting gets twice what this round needs (the
-    // next rounds of a refinement pass usually split again).
+    // A growth moves every mesh of the set, so when one mesh needs room, every
+    // mesh that this round leaves with little gets half as much again as it
+    // needs now, and some thousands at least (the next rounds of a refinement pass usually split again).
     long long total = 0;
     bool need_grow = false;
     for (int i = 0; i < m.nmesh; ++i) {
@@ -3267,14 +3267,12 @@ int op_refine(MeshSet& m, int max_rounds) {
     std::vector<int> vcap = m.vcap, ecap = m.ecap;
     for (int i = 0; need_grow && i < m.nmesh; ++i) {
       if (newv[i] == 0) continue;
-      long long vneed = (long long)m.nv[i] + newv[i];
-      long long eneed = (long long)m.ne[i] + 2LL * newv[i];
-      if (2 * vneed > m.vcap[i])
-        vcap[i] = (int)std::min<long long>(std::max<long long>(2LL * m.vcap[i], 2 * vneed),
-                                           (1LL << 30));
-      if (2 * eneed > m.ecap[i])
-        ecap[i] = (int)std::min<long long>(std::max<long long>(2LL * m.ecap[i], 2 * eneed),
-                                           (1LL << 30));
+      const long long vneed = (long long)m.nv[i] + newv[i] + 64;
+      const long long eneed = (long long)m.ne[i] + 2LL * newv[i] + 64;
+      if (vneed + vneed / 8 > m.vcap[i])
+        vcap[i] = (int)std::min<long long>(std::max(vneed + vneed / 2, vneed + 8192), (1LL << 30));
+      if (eneed + eneed / 8 > m.ecap[i])
+        ecap[i] = (int)std::min<long long>(std::max(eneed + eneed / 2, eneed + 16384), (1LL << 30));
     }
     if (total == 0) {
       complete = true;
