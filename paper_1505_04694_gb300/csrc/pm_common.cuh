@@ -39,6 +39,7 @@ struct MeshTab {
   double* L_up;
   double* q_thresh;
   double4* band;                 // (L_low_lo^2, L_low_hi^2, L_up_lo^2, L_up_hi^2)
+  float4* bandf;                 // the same, each float rounded away from its bound
   // 2 * (nmesh + 1) ints: exclusive prefix sums over the meshes of a vertex
   // count and an element count (pre[0..nmesh] vertices, pre[nmesh+1..]
   // elements); the offsets of each mesh in a concatenated input or output.

@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <limits>
 #include <mutex>
 
 #include "pm_internal.cuh"
@@ -21,10 +22,10 @@ namespace {
 // process: page-locking is slow and gets slower after many allocate/free
 // cycles, so slots of one arena are handed out and recycled instead.
 constexpr size_t kPinnedSlot = 16384;
-// staging per mesh of upload_tab: band (double4), L_low/L_up/q_thresh, seven
-// ints, the seed
-constexpr size_t kTabUploadBytes = sizeof(double4) + 3 * sizeof(double) + 7 * sizeof(int) +
-                                   sizeof(uint32_t);
+// staging per mesh of upload_tab: band (double4, float4), L_low/L_up/q_thresh,
+// seven ints, the seed
+constexpr size_t kTabUploadBytes = sizeof(double4) + sizeof(float4) + 3 * sizeof(double) +
+                                   7 * sizeof(int) + sizeof(uint32_t);
 constexpr size_t kPinnedBlock = 64 * kPinnedSlot;
 std::mutex g_pin_mu;
 std::vector<void*> g_pin_free;
@@ -659,7 +660,8 @@ cudaError_t upload_tab(MeshSet& m) {
   // of this set has normally long left it
   if (m.upev) cudaEventSynchronize(m.upev);
   double4* band = (double4*)m.hup;
-  double* dbl = (double*)(band + n);
+  float4* bandf = (float4*)(band + n);
+  double* dbl = (double*)(bandf + n);
   int* ints = (int*)(dbl + 3 * n);
   uint32_t* seed = (uint32_t*)(ints + 7 * n);
   for (int i = 0; i < n; ++i) {
@@ -678,6 +680,12 @@ cudaError_t upload_tab(MeshSet& m) {
     double alo = a * (1.0 - 1e-9), ahi = a * (1.0 + 1e-9);
     double blo = b * (1.0 - 1e-9), bhi = b * (1.0 + 1e-9);
     band[i] = make_double4(alo * alo, ahi * ahi, blo * blo, bhi * bhi);
+    // one float step outwards from the nearest float
+    const float big = std::numeric_limits<float>::infinity();
+    bandf[i] = make_float4(std::nextafterf((float)band[i].x, -big),
+                           std::nextafterf((float)band[i].y, big),
+                           std::nextafterf((float)band[i].z, -big),
+                           std::nextafterf((float)band[i].w, big));
   }
   cudaError_t e = cudaMemcpyAsync(m.S.tab.vbase, ints, 7 * n * sizeof(int), cudaMemcpyHostToDevice,
                                   m.stream);
@@ -685,8 +693,8 @@ cudaError_t upload_tab(MeshSet& m) {
                               m.stream);
   if (!e) e = cudaMemcpyAsync(m.S.tab.L_low, dbl, 3 * n * sizeof(double), cudaMemcpyHostToDevice,
                               m.stream);
-  if (!e) e = cudaMemcpyAsync(m.S.tab.band, band, n * sizeof(double4), cudaMemcpyHostToDevice,
-                              m.stream);
+  if (!e) e = cudaMemcpyAsync(m.S.tab.band, band, n * (sizeof(double4) + sizeof(float4)),
+                              cudaMemcpyHostToDevice, m.stream);
   if (!e && m.upev) e = cudaEventRecord(m.upev, m.stream);
   if (!e && !m.mesh_index_ok) {
     PM_LAUNCH(k_mesh_index, grid_for(m, m.S.vslots), BLOCK, 0, m.stream, n,
@@ -762,7 +770,7 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   carve_store(cv, m.B);
   size_t tab_bytes = (size_t)n * (8 * sizeof(int) + 2 * sizeof(uint32_t) + 3 * sizeof(int) +
                                   2 * sizeof(unsigned long long) + 3 * sizeof(double) +
-                                  sizeof(double4)) +
+                                  sizeof(double4) + sizeof(float4)) +
                      2 * ((size_t)n + 1) * sizeof(int) + 64;
   char* t = nullptr;
   cv.add(&t, tab_bytes, true);
@@ -821,6 +829,7 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   MeshTab& T = S.tab;
   // 32-byte, then 8-byte aligned members first
   T.band = (double4*)t; t += n * sizeof(double4);
+  T.bandf = (float4*)t; t += n * sizeof(float4);
   T.L_low = (double*)t; t += n * sizeof(double);
   T.L_up = (double*)t; t += n * sizeof(double);
   T.q_thresh = (double*)t; t += n * sizeof(double);

@@ -378,9 +378,6 @@ __device__ __forceinline__ int tcount() { return gridDim.x * (blockDim.x / TW); 
 
 // ---- coarsening (Sec. 2.4.1) ---------------------------------------------------
 
-struct CoarsenCtx;
-__device__ __forceinline__ double S_L_up(const CoarsenCtx& x);
-
 struct CoarsenCtx {
   const Store* S;
   MeshCtx c;
@@ -389,44 +386,40 @@ struct CoarsenCtx {
   int nnl;
   const int* ne;
   int nel;
-  VD dv;
   bool bnd;
 };
 
-__device__ __forceinline__ double S_L_up(const CoarsenCtx& x) { return x.S->tab.L_up[x.c.mi]; }
+// Is edge (a, b) certainly longer (+1) or shorter (-1) than a bound, or is
+// that for the exact length to say (0)?
+__device__ __forceinline__ int edge_cmp(const VF& a, const VF& b, float lo2, float hi2) {
+  return f_len_cmp(f_edge2(a, b), lo2, hi2);
+}
 
-// The integer part of the validity of collapsing v onto local neighbour u:
-// the link condition (|NN(v) & NN(u)| = 2 for an interior edge, 1 for a
-// boundary edge; a boundary vertex only along a boundary edge).
-__device__ bool collapse_link(const Store& S, const CoarsenCtx& x, int u) {
-  const bool bedge = count_elems_with(S, x.ne, x.nel, x.c.eb, u) == 1;
-  if (x.bnd && !bedge) return false;
-  const int ws = x.c.vb + u;
-  const int* nnw = nn_row(S, ws);
-  const int nnwl = S.NNlen[ws];
-  int common = 0, a = 0, b = 0;
-  while (a < x.nnl && b < nnwl) {
-    const int p = x.nn[a], q = nnw[b];
-    if (p == q) {
-      ++common;
-      ++a;
-      ++b;
-    } else if (p < q) {
-      ++a;
-    } else {
-      ++b;
-    }
-  }
-  return common == (bedge ? 1 : 2);
+// Edge (va, vb) longer than L_up, shorter than L_low: the FP32 filter first.
+__device__ __forceinline__ bool edge_longer(const Store& S, int mi, const VF& fa, const VF& fb,
+                                            int va, int vb, unsigned& ops) {
+  const float4 bf = S.tab.bandf[mi];
+  const int r = edge_cmp(fa, fb, bf.z, bf.w);
+  if (r != 0) return r > 0;
+  const double4 band = S.tab.band[mi];
+  ops += kOpsLen2;
+  return len_gt(metric_len2(load_vd(S, va), load_vd(S, vb)), band.z, band.w, S.tab.L_up[mi]);
+}
+__device__ __forceinline__ bool edge_shorter(const Store& S, int mi, const VF& fa, const VF& fb,
+                                             int va, int vb, unsigned& ops) {
+  const float4 bf = S.tab.bandf[mi];
+  const int r = edge_cmp(fa, fb, bf.x, bf.y);
+  if (r != 0) return r < 0;
+  const double4 band = S.tab.band[mi];
+  ops += kOpsLen2;
+  return len_lt(metric_len2(load_vd(S, va), load_vd(S, vb)), band.x, band.y, S.tab.L_low[mi]);
 }
 
 // collapse_valid with the lanes of a tile splitting v's ball elements (the
 // element count of the edge and the orientations with v on u) and v's
 // neighbours (the link condition and the new edge lengths): the same
 // conjunction of the same tests.  Every lane returns the tile's answer.
-__device__ bool tile_collapse_valid(const Tile& t, const CoarsenCtx& x, int u, double4 band,
-                                    unsigned& ops) {
-  const double L_up = S_L_up(x);
+__device__ bool tile_collapse_valid(const Tile& t, const CoarsenCtx& x, int u, unsigned& ops) {
   const Store& S = *x.S;
   int cnt = 0;
   for (int k = t.tl; k < x.nel; k += TW) {
@@ -441,23 +434,25 @@ __device__ bool tile_collapse_valid(const Tile& t, const CoarsenCtx& x, int u, d
   int common = 0;
   for (int k = t.tl; k < x.nnl; k += TW) common += row_has(nnw, nnwl, x.nn[k]) ? 1 : 0;
   if (tsum(t, common) != (bedge ? 1 : 2)) return false;
-  const VD dw = load_vd(S, ws);
+  const VF fw = load_vf(S, ws);
   bool ok = true;
   for (int k = t.tl; k < x.nel; k += TW) {
     int4 e = S.EN[x.c.eb + x.ne[k]];
     if (e.x == u || e.y == u || e.z == u) continue;
-    VD d0 = (e.x == x.lv) ? dw : load_vd(S, x.c.vb + e.x);
-    VD d1 = (e.y == x.lv) ? dw : load_vd(S, x.c.vb + e.y);
-    VD d2 = (e.z == x.lv) ? dw : load_vd(S, x.c.vb + e.z);
-    ok &= orient_sign(d0, d1, d2) > 0;
-    ops += kOpsOrient;
+    const int s0 = (e.x == x.lv) ? ws : x.c.vb + e.x, s1 = (e.y == x.lv) ? ws : x.c.vb + e.y,
+              s2 = (e.z == x.lv) ? ws : x.c.vb + e.z;
+    int o = f_orient(load_vf(S, s0), load_vf(S, s1), load_vf(S, s2));
+    if (o == 0) {
+      o = orient_sign(load_vd(S, s0), load_vd(S, s1), load_vd(S, s2)) > 0 ? 1 : -1;
+      ops += kOpsOrient;
+    }
+    ok &= o > 0;
   }
   if (!tall(t, ok)) return false;
   for (int k = t.tl; k < x.nnl; k += TW) {
     int y = x.nn[k];
     if (y == u || row_has(nnw, nnwl, y)) continue;
-    ok &= !len_gt(metric_len2(dw, load_vd(S, x.c.vb + y)), band.z, band.w, L_up);
-    ops += kOpsLen2;
+    ok &= !edge_longer(S, x.c.mi, fw, load_vf(S, x.c.vb + y), ws, x.c.vb + y, ops);
   }
   return tall(t, ok);
 }
@@ -479,9 +474,7 @@ __device__ int tile_coarsen_candidates(const Tile& t, const Store& S, int v, Mes
   const int nnl = S.NNlen[v];
   const int* ne = ne_row(S, v);
   const int nel = S.NElen[v];
-  const VD dv = load_vd(S, v);
-  const double L_low = S.tab.L_low[c.mi];
-  const double4 band = S.tab.band[c.mi];
+  const VF fv = load_vf(S, v);
   constexpr int kPer = MAXW / TW;
   double L[kPer];
   bool is[kPer];
@@ -493,17 +486,25 @@ __device__ int tile_coarsen_candidates(const Tile& t, const Store& S, int v, Mes
     L[j] = 0.0;
     if (k < nnl) {
       const int u = nn[k];
-      const double L2 = metric_len2(dv, load_vd(S, c.vb + u));
-      ops += kOpsLen2;
-      bool cand = len_lt(L2, band.x, band.y, L_low);
+      bool cand = edge_shorter(S, c.mi, fv, load_vf(S, c.vb + u), v, c.vb + u, ops);
       if (cand && bnd) cand = count_elems_with(S, ne, nel, c.eb, u) == 1;
       if (cand) {
-        L[j] = sqrt(L2);
-        ++ops;
         is[j] = true;
         ++mine;
       }
     }
+  }
+  const int total = tsum(t, mine);
+  if (total == 0) return 0;
+  // the exact lengths, for the order of several candidates
+  if (total > 1) {
+    const VD dv = load_vd(S, v);
+#pragma unroll
+    for (int j = 0; j < kPer; ++j)
+      if (is[j]) {
+        L[j] = sqrt(metric_len2(dv, load_vd(S, c.vb + nn[j * TW + t.tl])));
+        ops += kOpsLen2 + 1;
+      }
   }
   const int steps = (nnl + TW - 1) / TW;
   for (int j = 0; j < steps; ++j) {
@@ -519,7 +520,7 @@ __device__ int tile_coarsen_candidates(const Tile& t, const Store& S, int v, Mes
     }
     if (is[j]) out[rank] = nn[j * TW + t.tl];
   }
-  return tsum(t, mine);
+  return total;
 }
 
 __device__ __forceinline__ CoarsenCtx coarsen_ctx(const Store& S, int v, MeshCtx c) {
@@ -532,28 +533,118 @@ __device__ __forceinline__ CoarsenCtx coarsen_ctx(const Store& S, int v, MeshCtx
   x.nnl = S.NNlen[v];
   x.ne = ne_row(S, v);
   x.nel = S.NElen[v];
-  x.dv = load_vd(S, v);
   x.bnd = (S.vflag[v] & VF_BND) != 0;
   return x;
 }
 
 // Collapse evaluation.  The target of v is the first candidate, by (metric
 // length, id), whose collapse is valid.  Pass 1 (per dirty vertex) reuses an
-// unchanged earlier result or lists v's sorted candidates; a dense pass then
-// checks every listed vertex's best candidate (one work item each), and a
-// last pass goes through the remaining candidates of the vertices whose best
-// one failed.  Candidates are listed by an 8-lane tile per vertex (see
-// tile_coarsen_candidates), so the FP64 lengths of the neighbours run side
-// by side.  The tile takes the stamp decision from lane 0 before lane 0
-// overwrites the stamp.
-// Pass 1 of the large rounds, one dirty vertex per thread: reuse an unchanged
-// earlier result, or list v's collapse candidates.  The metric lengths of all
-// the warp's vertices' edges are the FP64 work; they are evaluated 32 at a
-// time from a per-warp queue (full warps on the FP64 pipe, where a tile per
-// vertex kept about 19 of 32 lanes busy), each candidate's length stored in
-// a scratch row and its bit in a per-lane mask; then each thread places its
-// own candidates by rank in the (length, id) order, as tile_coarsen_candidates
-// does in the persistent rounds.
+// unchanged earlier result or finds v's first candidate; a dense pass then
+// checks every listed vertex's first candidate (one work item each), and a
+// last pass puts the candidates of the vertices whose first one failed in
+// order and goes through the rest of them.
+//
+// Pass 1 of the large rounds, one dirty vertex per thread.  Which neighbours
+// are candidates is a length against L_low, and which of them comes first is
+// mostly plain from the FP32 lengths too: only candidates whose error
+// intervals overlap that of the shortest (equal lengths on regular grids) are
+// compared by their exact lengths.  A length that is certainly above another's
+// stays above it after rounding, so the order is the exact one.
+__device__ __forceinline__ void coarsen_scan_phase(Store S, const int* D, const int* nDp,
+                                                   int* target, int* cand, int* ncand, int* C,
+                                                   int* nC, int* cmark, int tag, int pass0,
+                                                   int2* W0, int* nW0) {
+  const int n = *nDp;
+  unsigned ops = 0;
+  for (int i0 = blockIdx.x * blockDim.x; i0 < n; i0 += gridDim.x * blockDim.x) {
+    const int i = i0 + threadIdx.x;
+    int v = 0, nc = 0;
+    bool reuse_cand = false, eval = false;
+    if (i < n) {
+      v = D[i];
+      const MeshCtx c = ctx_of(S, v);
+      if (unchanged(S, v, c.vb, S.evc[v], pass0)) {
+        reuse_cand = target[v] >= 0;
+        if (reuse_cand) {
+          cmark[v] = tag;
+          S.tab.had[c.mi] = 1;
+        }
+      } else {
+        S.evc[v] = tag;
+        eval = true;
+        const uint8_t f = S.vflag[v];
+        // corners and dead vertices have no candidates
+        const int nnl = ((f & VF_ALIVE) && !(f & VF_CORNER)) ? S.NNlen[v] : 0;
+        const int* nn = nn_row(S, v);
+        const VF fv = load_vf(S, v);
+        const float4 bf = S.tab.bandf[c.mi];
+        float lo[MAXW];      // candidates: lower bound of the squared length
+        float first = INFINITY;  // the smallest upper bound
+        RowMask cm;
+#pragma unroll 4
+        for (int k = 0; k < nnl; ++k) {
+          const int us = c.vb + nn[k];
+          const VF fu = load_vf(S, us);
+          const FLen l = f_edge2(fv, fu);
+          const int r = f_len_cmp(l, bf.x, bf.y);
+          bool is = r < 0;
+          if (r == 0) is = edge_shorter(S, c.mi, fv, fu, v, us, ops);
+          // a boundary vertex collapses only along a boundary edge
+          if (is && (f & VF_BND))
+            is = count_elems_with(S, ne_row(S, v), S.NElen[v], c.eb, nn[k]) == 1;
+          if (is) {
+            cm.set(k);
+            lo[k] = l.L2 - l.err;
+            // (a NaN bound leaves `first` as it is and passes the test below)
+            first = l.L2 + l.err < first ? l.L2 + l.err : first;
+          }
+        }
+        nc = cm.count();
+        int best = -1;
+        if (nc > 0) {
+          RowMask near;
+          RowMask a = cm;
+          while (a.any()) {
+            const int k = a.pop();
+            if (!(lo[k] > first)) near.set(k);
+          }
+          best = near.pop();
+          if (near.any()) {
+            const VD dv = load_vd(S, v);
+            double Lb = sqrt(metric_len2(dv, load_vd(S, c.vb + nn[best])));
+            ops += kOpsLen2 + 1;
+            while (near.any()) {  // ascending position, hence id
+              const int k = near.pop();
+              const double L = sqrt(metric_len2(dv, load_vd(S, c.vb + nn[k])));
+              ops += kOpsLen2 + 1;
+              if (dlt(L, Lb)) {
+                Lb = L;
+                best = k;
+              }
+            }
+          }
+          cand[(size_t)v * S.W] = nn[best];
+        }
+        ncand[v] = nc;
+        if (nc == 0) target[v] = -1;
+      }
+    }
+    warp_append(reuse_cand, v, C, nC);
+    warp_append_t(eval && nc > 0, make_int2(v, 0), W0, nW0);
+  }
+}
+
+__global__ void k_coarsen_scan(Store S, const int* D, const int* nDp, int* target, int* cand,
+                               int* ncand, int* C, int* nC, int* cmark, int tag, int pass0,
+                               int2* W0, int* nW0) {
+  coarsen_scan_phase(S, D, nDp, target, cand, ncand, C, nC, cmark, tag, pass0, W0, nW0);
+}
+
+// The candidates of the warp's vertices (one per lane, `eval` lanes) by
+// (exact length, id) into their rows of `cand`.  The exact lengths are
+// evaluated 32 at a time from a per-warp queue, each candidate's length
+// stored in a scratch row and its bit in a per-lane mask; then each thread
+// places its own candidates by rank.
 __device__ __forceinline__ void coarsen_len_chunk(const Store& S, const int2* q, int cnt, int v,
                                                   MeshCtx c, unsigned long long (*cm)[2],
                                                   double* Lbuf) {
@@ -577,104 +668,71 @@ __device__ __forceinline__ void coarsen_len_chunk(const Store& S, const int2* q,
   }
 }
 
-__device__ __forceinline__ void coarsen_scan_phase(Store S, const int* D, const int* nDp,
-                                                   int* target, int* cand, int* ncand, int* C,
-                                                   int* nC, int* cmark, int tag, int pass0,
-                                                   int2* W0, int* nW0, double* Lbuf) {
-  __shared__ int2 sq[kScanWarps][64];
-  __shared__ unsigned long long scm[kScanWarps][32][2];
-  const int lane = threadIdx.x & 31, wq = (threadIdx.x >> 5) % kScanWarps;
+__device__ __forceinline__ void coarsen_rank(const Store& S, bool eval, int v, MeshCtx c, int2* q,
+                                             unsigned long long (*scm)[2], int* cand,
+                                             double* Lbuf) {
+  const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
-  const int n = *nDp;
-  for (int i0 = blockIdx.x * blockDim.x; i0 < n; i0 += gridDim.x * blockDim.x) {
-    const int i = i0 + threadIdx.x;
-    int v = 0, nnl = 0;
-    bool reuse_cand = false, eval = false;
-    MeshCtx c{0, 0, 0};
-    if (i < n) {
-      v = D[i];
-      c = ctx_of(S, v);
-      if (unchanged(S, v, c.vb, S.evc[v], pass0)) {
-        reuse_cand = target[v] >= 0;
-        if (reuse_cand) {
-          cmark[v] = tag;
-          S.tab.had[c.mi] = 1;
-        }
-      } else {
-        S.evc[v] = tag;
-        eval = true;
-        const uint8_t f = S.vflag[v];
-        // corners and dead vertices have no candidates
-        if ((f & VF_ALIVE) && !(f & VF_CORNER)) nnl = S.NNlen[v];
-      }
-    }
-    scm[wq][lane][0] = scm[wq][lane][1] = 0ull;
+  scm[lane][0] = scm[lane][1] = 0ull;
+  __syncwarp();
+  const int nnl = eval ? S.NNlen[v] : 0;
+  const float4 bf = eval ? S.tab.bandf[c.mi] : make_float4(0.f, 0.f, 0.f, 0.f);
+  VF fv{};
+  if (eval) fv = load_vf(S, v);
+  const int tmax = __reduce_max_sync(0xffffffffu, nnl);
+  int qn = 0;  // the same in every lane
+  for (int t = 0; t < tmax; ++t) {
+    const bool p =
+        t < nnl && edge_cmp(fv, load_vf(S, c.vb + nn_row(S, v)[t]), bf.x, bf.y) <= 0;
+    const unsigned m = __ballot_sync(0xffffffffu, p);
+    if (p) q[qn + __popc(m & lt)] = make_int2(lane, t);
+    qn += __popc(m);
     __syncwarp();
-    const int tmax = __reduce_max_sync(0xffffffffu, nnl);
-    int qn = 0;  // the same in every lane
-    for (int t = 0; t < tmax; ++t) {
-      const bool p = t < nnl;
-      const unsigned m = __ballot_sync(0xffffffffu, p);
-      if (p) sq[wq][qn + __popc(m & lt)] = make_int2(lane, t);
-      qn += __popc(m);
+    if (qn >= 32) {
+      coarsen_len_chunk(S, q, 32, v, c, scm, Lbuf);
       __syncwarp();
-      if (qn >= 32) {
-        coarsen_len_chunk(S, sq[wq], 32, v, c, scm[wq], Lbuf);
-        __syncwarp();
-        if (lane < qn - 32) sq[wq][lane] = sq[wq][32 + lane];
-        qn -= 32;
-        __syncwarp();
-      }
+      if (lane < qn - 32) q[lane] = q[32 + lane];
+      qn -= 32;
+      __syncwarp();
     }
-    if (qn > 0) coarsen_len_chunk(S, sq[wq], qn, v, c, scm[wq], Lbuf);
-    __syncwarp();
-    int nc = 0;
-    if (eval) {
-      RowMask cm;
-      cm.lo = scm[wq][lane][0];
-      cm.hi = scm[wq][lane][1];
-      nc = cm.count();
-      const int* nn = nn_row(S, v);
-      const double* L = Lbuf + (size_t)v * S.W;
-      int* out = cand + (size_t)v * S.W;
-      RowMask a = cm;
-      while (a.any()) {
-        const int k = a.pop();
-        const double Lk = L[k];
-        int rank = 0;
-        RowMask b = cm;
-        while (b.any()) {
-          const int k2 = b.pop();
-          const double Lo = L[k2];
-          if (dlt(Lo, Lk) || (dbits(Lo) == dbits(Lk) && k2 < k)) ++rank;
-        }
-        out[rank] = nn[k];
-      }
-      ncand[v] = nc;
-      if (nc == 0) target[v] = -1;
-    }
-    warp_append(reuse_cand, v, C, nC);
-    warp_append_t(eval && nc > 0, make_int2(v, 0), W0, nW0);
   }
-}
-
-__global__ void k_coarsen_scan(Store S, const int* D, const int* nDp, int* target, int* cand,
-                               int* ncand, int* C, int* nC, int* cmark, int tag, int pass0,
-                               int2* W0, int* nW0, double* Lbuf) {
-  coarsen_scan_phase(S, D, nDp, target, cand, ncand, C, nC, cmark, tag, pass0, W0, nW0, Lbuf);
+  if (qn > 0) coarsen_len_chunk(S, q, qn, v, c, scm, Lbuf);
+  __syncwarp();
+  if (eval) {
+    RowMask cm;
+    cm.lo = scm[lane][0];
+    cm.hi = scm[lane][1];
+    const int* nn = nn_row(S, v);
+    const double* L = Lbuf + (size_t)v * S.W;
+    int* out = cand + (size_t)v * S.W;
+    RowMask a = cm;
+    while (a.any()) {
+      const int k = a.pop();
+      const double Lk = L[k];
+      int rank = 0;
+      RowMask b = cm;
+      while (b.any()) {
+        const int k2 = b.pop();
+        const double Lo = L[k2];
+        if (dlt(Lo, Lk) || (dbits(Lo) == dbits(Lk) && k2 < k)) ++rank;
+      }
+      out[rank] = nn[k];
+    }
+  }
+  __syncwarp();
 }
 
 // The check passes, one work item (v, k) per thread: is collapsing v onto
 // its k-th candidate valid (in the last pass: the first valid one from k on)?
-// Validity is the conjunction of the link condition and, for the collapse
-// with v on u, every remaining ball element counter-clockwise and no new edge
-// longer than L_up (collapse_valid below, tile form).  Balls differ in size
-// and most tests need no arithmetic (elements containing u, neighbours
-// shared with u), so the FP64 tests of a warp's items are queued in shared
-// memory per warp, orientations and lengths apart, and evaluated 32 at a
-// time: full warps on the FP64 pipe instead of the lanes whose own loop is
-// still running.  Any failed test clears the owner's flag; the conjunction
-// does not depend on the order of its tests.
+// Validity is the conjunction of the link condition (|NN(v) & NN(u)| = 2 for
+// an interior edge, 1 for a boundary edge; a boundary vertex only along a
+// boundary edge) and, for the collapse with v on u, every remaining ball
+// element counter-clockwise and no new edge longer than L_up (the tile form
+// above).  The FP32 filters decide most tests; what they leave open of an
+// item that has not failed (collinear points of regular grids above all) is
+// queued in shared memory per warp, orientations and lengths apart, and
+// evaluated in FP64 32 at a time.  Any failed test clears the owner's flag;
+// the conjunction does not depend on the order of its tests.
 constexpr int kCheckWarps = 8;
 
 struct CheckQueues {
@@ -718,14 +776,57 @@ __device__ __forceinline__ void check_len_chunk(const Store& S, const CheckQueue
   }
 }
 
+// The integer part and the FP32 filters for collapsing x.v onto u: false when
+// it is certainly invalid; else the tests left open, as bits over the ball's
+// elements and v's neighbours.
+__device__ __forceinline__ bool check_filter(const Store& S, const CoarsenCtx& x, int u,
+                                             RowMask& oo, RowMask& ol) {
+  const bool bedge = count_elems_with(S, x.ne, x.nel, x.c.eb, u) == 1;
+  if (x.bnd && !bedge) return false;
+  const int ws = x.c.vb + u;
+  const int* nnw = nn_row(S, ws);
+  const int nnwl = S.NNlen[ws];
+  RowMask common;
+#pragma unroll 2
+  for (int k = 0; k < x.nnl; ++k)
+    if (row_has(nnw, nnwl, x.nn[k])) common.set(k);
+  if (common.count() != (bedge ? 1 : 2)) return false;
+  const VF fw = load_vf(S, ws);
+  bool ok = true;
+#pragma unroll 2
+  for (int k = 0; k < x.nel; ++k) {
+    const int4 e = S.EN[x.c.eb + x.ne[k]];
+    if (e.x == u || e.y == u || e.z == u) continue;
+    // the element in the order (u in place of v, next, before)
+    const int n1 = (e.x == x.lv) ? e.y : (e.y == x.lv) ? e.z : e.x;
+    const int n2 = (e.x == x.lv) ? e.z : (e.y == x.lv) ? e.x : e.y;
+    const int o = f_orient(fw, load_vf(S, x.c.vb + n1), load_vf(S, x.c.vb + n2));
+    ok &= o >= 0;
+    if (o == 0) oo.set(k);
+  }
+  if (!ok) return false;
+  const float4 bf = S.tab.bandf[x.c.mi];
+#pragma unroll 2
+  for (int k = 0; k < x.nnl; ++k) {
+    const int y = x.nn[k];
+    if (y == u || common.test(k)) continue;
+    const int r = edge_cmp(fw, load_vf(S, x.c.vb + y), bf.z, bf.w);
+    ok &= r <= 0;
+    if (r == 0) ol.set(k);
+  }
+  return ok;
+}
+
+template <bool LAST>
 __device__ __forceinline__ void coarsen_check_phase(Store S, const int2* Win, const int* nWin,
                                                     int2* Wout, int* nWout, int* target,
-                                                    const int* cand, const int* ncand, int* C,
-                                                    int* nC, int* cmark, int tag, int last,
+                                                    int* cand, const int* ncand, int* C,
+                                                    int* nC, int* cmark, int tag, double* Lbuf,
                                                     unsigned long long* work) {
   __shared__ int4 sqo[kCheckWarps][64];
   __shared__ int2 sql[kCheckWarps][64];
   __shared__ int sok[kCheckWarps][32];
+  __shared__ unsigned long long scm[LAST ? kCheckWarps : 1][32][2];
   const int lane = threadIdx.x & 31, wq = (threadIdx.x >> 5) % kCheckWarps;
   CheckQueues Q{sqo[wq], sql[wq], sok[wq]};
   const unsigned lt = (1u << lane) - 1u;
@@ -745,38 +846,27 @@ __device__ __forceinline__ void coarsen_check_phase(Store S, const int2* Win, co
       cv = cand + (size_t)v * S.W;
       nc = ncand[v];
     }
+    if (LAST) coarsen_rank(S, !done, v, x.c, Q.ql, scm[LAST ? wq : 0], cand, Lbuf);
     // one candidate per lane and turn; the last pass moves on to the next
     // candidate of each lane whose candidate failed
     while (__ballot_sync(0xffffffffu, !done)) {
       const int u = done ? 0 : cv[k];
-      const bool link = !done && collapse_link(S, x, u);
+      RowMask oo, ol;
+      const bool may = !done && check_filter(S, x, u, oo, ol);
+      Q.ok[lane] = may ? 1 : 0;
+      if (!may) oo = ol = RowMask();
       const int ws = x.c.vb + u;
-      const int* nnw = link ? nn_row(S, ws) : nullptr;
-      const int nnwl = link ? S.NNlen[ws] : 0;
-      Q.ok[lane] = link ? 1 : 0;
-      const int T = link ? x.nel + x.nnl : 0;
-      const int Tmax = __reduce_max_sync(0xffffffffu, T);
       int no = 0, nl = 0;  // queue lengths, the same in every lane
       __syncwarp();
-      for (int t = 0; t < Tmax; ++t) {
-        bool po = false, pl = false;
-        int4 ro = make_int4(lane, 0, 0, 0);
-        int2 rl = make_int2(lane, 0);
-        if (t < T) {
-          if (t < x.nel) {
-            const int4 e = S.EN[x.c.eb + x.ne[t]];
-            po = e.x != u && e.y != u && e.z != u;
-            ro = make_int4(lane, e.x, e.y, e.z);
-          } else {
-            const int y = x.nn[t - x.nel];
-            pl = y != u && !row_has(nnw, nnwl, y);
-            rl = make_int2(lane, y);
-          }
-        }
+      while (__ballot_sync(0xffffffffu, oo.any() || ol.any())) {
+        const bool po = oo.any(), pl = ol.any();
         const unsigned mo = __ballot_sync(0xffffffffu, po);
         const unsigned ml = __ballot_sync(0xffffffffu, pl);
-        if (po) Q.qo[no + __popc(mo & lt)] = ro;
-        if (pl) Q.ql[nl + __popc(ml & lt)] = rl;
+        if (po) {
+          const int4 e = S.EN[x.c.eb + x.ne[oo.pop()]];
+          Q.qo[no + __popc(mo & lt)] = make_int4(lane, e.x, e.y, e.z);
+        }
+        if (pl) Q.ql[nl + __popc(ml & lt)] = make_int2(lane, x.nn[ol.pop()]);
         no += __popc(mo);
         nl += __popc(ml);
         __syncwarp();
@@ -800,7 +890,7 @@ __device__ __forceinline__ void coarsen_check_phase(Store S, const int2* Win, co
       __syncwarp();
       if (!done) {
         found = Q.ok[lane] != 0;
-        if (found || !last || k + 1 >= nc) done = true;
+        if (found || !LAST || k + 1 >= nc) done = true;
         else ++k;
       }
       __syncwarp();
@@ -811,23 +901,24 @@ __device__ __forceinline__ void coarsen_check_phase(Store S, const int2* Win, co
         target[v] = cv[k];
         cmark[v] = tag;
         S.tab.had[x.c.mi] = 1;
-      } else if (!last && k + 1 < nc) {
+      } else if (!LAST && k + 1 < nc) {
         next = true;
       } else {
         target[v] = -1;
       }
     }
     warp_append(found, v, C, nC);
-    if (!last) warp_append_t(next, make_int2(v, k + 1), Wout, nWout);
+    if (!LAST) warp_append_t(next, make_int2(v, k + 1), Wout, nWout);
   }
   add_work(work, ops);
 }
 
+template <bool LAST>
 __global__ void k_coarsen_check(Store S, const int2* Win, const int* nWin, int2* Wout, int* nWout,
-                                int* target, const int* cand, const int* ncand, int* C, int* nC,
-                                int* cmark, int tag, int last, unsigned long long* work) {
-  coarsen_check_phase(S, Win, nWin, Wout, nWout, target, cand, ncand, C, nC, cmark, tag, last,
-                      work);
+                                int* target, int* cand, const int* ncand, int* C, int* nC,
+                                int* cmark, int tag, double* Lbuf, unsigned long long* work) {
+  coarsen_check_phase<LAST>(S, Win, nWin, Wout, nWout, target, cand, ncand, C, nC, cmark, tag,
+                            Lbuf, work);
 }
 
 // One tile per listed vertex, listing and checking at once (persistent
@@ -858,9 +949,8 @@ __device__ __forceinline__ void coarsen_eval_phase(Store S, const int* D, const 
         __syncwarp(t.mask);  // the candidates written by every lane
         if (nc > 0) {
           CoarsenCtx x = coarsen_ctx(S, v, c);
-          const double4 band = S.tab.band[c.mi];
           for (int k = 0; k < nc && !found; ++k)
-            if (tile_collapse_valid(t, x, cv[k], band, ops)) {
+            if (tile_collapse_valid(t, x, cv[k], ops)) {
               found = true;
               if (t.tl == 0) target[v] = cv[k];
             }
@@ -2377,16 +2467,15 @@ __global__ void k_refine_mark(Store S, int* cnt, RowMask* mask, int tag, int pas
       int la = s - vb;
       const int* nn = nn_row(S, s);
       int nnl = S.NNlen[s];
-      VD da = load_vd(S, s);
-      const double L_up = S.tab.L_up[mi];
-      const double4 band = S.tab.band[mi];
+      const VF fa = load_vf(S, s);
+      unsigned ops = 0;
       // the row is sorted, so the neighbours above la form a suffix; four
       // lengths at a time so that their loads overlap
       int k0 = 0;
       while (k0 < nnl && nn[k0] <= la) ++k0;
 #pragma unroll 4
       for (int k = k0; k < nnl; ++k)
-        if (len_gt(metric_len2(da, load_vd(S, vb + nn[k])), band.z, band.w, L_up)) m.set(k);
+        if (edge_longer(S, mi, fa, load_vf(S, vb + nn[k]), s, vb + nn[k], ops)) m.set(k);
       mask[s] = m;
     } else {
       mask[s] = RowMask();
@@ -3124,15 +3213,15 @@ int op_coarsen(MeshSet& m, int max_rounds) {
     zero_round(m, nxt);
     PM_LAUNCH(k_coarsen_scan, gv, bs, 0, m.stream, m.S, w.D[cur], w.counts + cn_list(cur),
               w.target, w.cand, w.ncand, w.C, w.counts + CN_C, w.cmark, tag, pass0, w.items,
-              w.counts + CN_I, w.gains);
+              w.counts + CN_I);
     // one dense wave checking every vertex's best candidate, then the
     // remaining candidates of the vertices whose best one failed
-    PM_LAUNCH(k_coarsen_check, gv, bs, 0, m.stream, m.S, w.items, w.counts + CN_I, w.items2,
-              w.counts + CN_I2, w.target, w.cand, w.ncand, w.C, w.counts + CN_C, w.cmark, tag, 0,
-              prof_work("k_coarsen_check"));
-    PM_LAUNCH(k_coarsen_check, gv, bs, 0, m.stream, m.S, w.items2, w.counts + CN_I2, w.items,
-              w.counts + CN_I, w.target, w.cand, w.ncand, w.C, w.counts + CN_C, w.cmark, tag, 1,
-              prof_work("k_coarsen_check"));
+    PM_LAUNCH(k_coarsen_check<false>, gv, bs, 0, m.stream, m.S, w.items, w.counts + CN_I, w.items2,
+              w.counts + CN_I2, w.target, w.cand, w.ncand, w.C, w.counts + CN_C, w.cmark, tag,
+              w.gains, prof_work("k_coarsen_check"));
+    PM_LAUNCH(k_coarsen_check<true>, gv, bs, 0, m.stream, m.S, w.items2, w.counts + CN_I2, w.items,
+              w.counts + CN_I, w.target, w.cand, w.ncand, w.C, w.counts + CN_C, w.cmark, tag,
+              w.gains, prof_work("k_coarsen_check"));
     zero_counts(m, CN_CL, 1);
     PM_LAUNCH(k_coarsen_select_apply, gv, bs, 0, m.stream, m.S, w.C, w.counts + CN_C, w.cmark,
               w.smark, tag, w.target, w.A, w.counts + CN_A, w.amark, w.D[nxt],
