@@ -68,16 +68,23 @@ PM_HD float f_rcp(float x) {
 #endif
 }
 
-PM_HD VF make_vf(double x, double y, double m00, double m01, double m11) {
+// The record of a position without a metric (orientations only).
+PM_HD VF make_vf_xy(double x, double y) {
   VF v;
+  v.m00 = v.m01 = v.m11 = 0.0f;
   v.xh = (float)x;
   v.xl = (float)(x - (double)v.xh);
   v.yh = (float)y;
   v.yl = (float)(y - (double)v.yh);
+  v.e = 1.4210855e-14f * fmaxf(fabsf(v.xh), fabsf(v.yh)) + 1e-37f;  // 2^-46
+  return v;
+}
+
+PM_HD VF make_vf(double x, double y, double m00, double m01, double m11) {
+  VF v = make_vf_xy(x, y);
   v.m00 = (float)m00;
   v.m01 = (float)m01;
   v.m11 = (float)m11;
-  v.e = 1.4210855e-14f * fmaxf(fabsf(v.xh), fabsf(v.yh)) + 1e-37f;  // 2^-46
   // a metric that single precision cannot hold with full relative precision:
   // every test of the vertex is undecided
   const bool holds = v.m00 > 1e-30f && v.m00 < 1e30f && v.m11 > 1e-30f && v.m11 < 1e30f;

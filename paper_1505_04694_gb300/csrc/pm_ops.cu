@@ -2007,52 +2007,66 @@ __device__ double tile_ball_quality(const Tile& t, const Store& S, MeshCtx c, co
   return tmin(t, qmin);
 }
 
+// Whether the closed element (a, b, d) contains X = px: the FP32 filters of the
+// three sub-triangles first; a sign they leave open is taken exactly, unless
+// another one is negative.
+__device__ __forceinline__ bool contains(const Store& S, const VF& fx, double X, double Y, int sa,
+                                         int sb, int sd) {
+  const VF fa = load_vf(S, sa), fb = load_vf(S, sb), fd = load_vf(S, sd);
+  const int f0 = f_orient(fx, fb, fd), f1 = f_orient(fa, fx, fd), f2 = f_orient(fa, fb, fx);
+  if ((f0 | f1 | f2) < 0) return false;
+  if (f0 > 0 && f1 > 0 && f2 > 0) return true;
+  const VD px{X, Y, 0.0, 0.0, 0.0}, a = load_vd(S, sa), b = load_vd(S, sb), d = load_vd(S, sd);
+  if (f0 == 0 && orient_sign(px, b, d) < 0) return false;
+  if (f1 == 0 && orient_sign(a, px, d) < 0) return false;
+  return f2 != 0 || orient_sign(a, b, px) >= 0;
+}
+
+// Barycentric interpolation of the metric at X in element e (canonical
+// rotation).
+__device__ __forceinline__ double4 interpolate_in(const Store& S, int vb, int4 e, double X,
+                                                  double Y) {
+  const VD px{X, Y, 0.0, 0.0, 0.0};
+  int i0 = e.x, i1 = e.y, i2 = e.z;
+  VD a = load_vd(S, vb + i0), b = load_vd(S, vb + i1), d = load_vd(S, vb + i2);
+  canon(i0, i1, i2, a, b, d);
+  const double o = orient3(a, b, d);
+  const double l0 = orient3(px, b, d) / o, l1 = orient3(a, px, d) / o, l2 = orient3(a, b, px) / o;
+  return make_double4((l0 * a.m00 + l1 * b.m00) + l2 * d.m00,
+                      (l0 * a.m01 + l1 * b.m01) + l2 * d.m01,
+                      (l0 * a.m11 + l1 * b.m11) + l2 * d.m11, 0.0);
+}
+
+// Element e of v's ball with v moved to the record `fn`: certainly not
+// counter-clockwise, or its quality certainly below `floor`.
+__device__ __forceinline__ bool move_fails(const Store& S, int vb, int lv, int4 e, const VF& fn,
+                                           float floor) {
+  const VF a = e.x == lv ? fn : load_vf(S, vb + e.x), b = e.y == lv ? fn : load_vf(S, vb + e.y),
+           c = e.z == lv ? fn : load_vf(S, vb + e.z);
+  int sign;
+  const float up = f_quality_up(a, b, c, sign);
+  return sign < 0 || up < floor;
+}
+
 // First ball element (ascending id) that contains X, with v at its current
 // place: its barycentric metric interpolation.
 __device__ bool tile_interpolate(const Tile& t, const Store& S, MeshCtx c, const int* ne, int nel,
-                                 double X, double Y, double4& Mout, int* tested = nullptr) {
-  VD px{X, Y, 0.0, 0.0, 0.0};
+                                 double X, double Y, double4& Mout) {
+  const VF fx = make_vf_xy(X, Y);
   for (int base = 0; base < nel; base += TW) {
-    if (tested) *tested += min(TW, nel - base);
     int k = base + t.tl;
+    int4 e = make_int4(0, 0, 0, 0);
     bool inside = false;
-    VD a{}, b{}, d{};
-    double o = 1.0, s0 = 0.0, s1 = 0.0, s2 = 0.0;
     if (k < nel) {
-      int4 e = S.EN[c.eb + ne[k]];
-      int i0 = e.x, i1 = e.y, i2 = e.z;
-      a = load_vd(S, c.vb + i0);
-      b = load_vd(S, c.vb + i1);
-      d = load_vd(S, c.vb + i2);
-      canon(i0, i1, i2, a, b, d);
-      // filters first; a lane with a sign left open (X on or near an edge
-      // line) resolves it exactly below, all such lanes in one pass per sign
-      int f0 = orient_filter(px, b, d), f1 = orient_filter(a, px, d), f2 = orient_filter(a, b, px);
-      while ((f0 | f1 | f2) >= 0 && (f0 == 0 || f1 == 0 || f2 == 0)) {
-        const int j = f0 == 0 ? 0 : (f1 == 0 ? 1 : 2);
-        const int r = orient_resolve(j == 0 ? px : a, j == 1 ? px : b, j == 2 ? px : d);
-        const int fr = r == 0 ? 2 : r;  // decided: an exact zero counts as inside
-        if (j == 0) f0 = fr; else if (j == 1) f1 = fr; else f2 = fr;
-      }
-      inside = f0 > 0 && f1 > 0 && f2 > 0;
-      if (inside) {
-        o = orient3(a, b, d);
-        s0 = orient3(px, b, d);
-        s1 = orient3(a, px, d);
-        s2 = orient3(a, b, px);
-      }
+      e = S.EN[c.eb + ne[k]];
+      inside = contains(S, fx, X, Y, c.vb + e.x, c.vb + e.y, c.vb + e.z);
     }
     unsigned bal = (__ballot_sync(t.mask, inside) >> t.shift) & 0xFFu;
     if (bal) {
       int src = __ffs(bal) - 1;
-      double m0 = 0.0, m1 = 0.0, m2 = 0.0;
-      if (t.tl == src) {
-        double l0 = s0 / o, l1 = s1 / o, l2 = s2 / o;
-        m0 = (l0 * a.m00 + l1 * b.m00) + l2 * d.m00;
-        m1 = (l0 * a.m01 + l1 * b.m01) + l2 * d.m01;
-        m2 = (l0 * a.m11 + l1 * b.m11) + l2 * d.m11;
-      }
-      Mout = make_double4(tshfl(t, m0, src), tshfl(t, m1, src), tshfl(t, m2, src), 0.0);
+      double4 m = make_double4(0.0, 0.0, 0.0, 0.0);
+      if (t.tl == src) m = interpolate_in(S, c.vb, e, X, Y);
+      Mout = make_double4(tshfl(t, m.x, src), tshfl(t, m.y, src), tshfl(t, m.z, src), 0.0);
       return true;
     }
   }
@@ -2062,9 +2076,9 @@ __device__ bool tile_interpolate(const Tile& t, const Store& S, MeshCtx c, const
 // Ball with v moved to (X, Y, Mv): every element counter-clockwise, and every
 // quality above *floor (strict) or at least *floor (non-strict).  Writes each
 // element's new quality to qout[k] and returns the ascending-order sum.
-__device__ bool tile_ball_after_move(const Tile& t, const Store& S, MeshCtx c, int lv,
-                                     const int* ne, int nel, double X, double Y, double4 Mv,
-                                     double floor, bool strict, double* qout, double* qsum) {
+__device__ bool tile_ball_exact(const Tile& t, const Store& S, MeshCtx c, int lv,
+                                const int* ne, int nel, double X, double Y, double4 Mv,
+                                double floor, bool strict, double* qout, double* qsum) {
   VD nvd{X, Y, Mv.x, Mv.y, Mv.z};
   bool ok = true;
   double sum = 0.0;
@@ -2093,13 +2107,25 @@ __device__ bool tile_ball_after_move(const Tile& t, const Store& S, MeshCtx c, i
   return tall(t, ok);
 }
 
+// The same after the FP32 bounds: most moves fail, and they mostly show it.
+__device__ bool tile_ball_after_move(const Tile& t, const Store& S, MeshCtx c, int lv,
+                                     const int* ne, int nel, double X, double Y, double4 Mv,
+                                     double floor, bool strict, double* qout, double* qsum) {
+  const VF fn = make_vf(X, Y, Mv.x, Mv.y, Mv.z);
+  const float ffloor = __double2float_rd(floor);
+  bool fails = false;
+  for (int k = t.tl; k < nel; k += TW)
+    fails |= move_fails(S, c.vb, lv, S.EN[c.eb + ne[k]], fn, ffloor);
+  if (!tall(t, !fails)) return false;
+  return tile_ball_exact(t, S, c, lv, ne, nel, X, Y, Mv, floor, strict, qout, qsum);
+}
+
 // Quality-constrained Laplacian move of v: metric-weighted neighbour mean,
 // metric interpolated at the target, kept when the ball stays valid and its
 // minimum quality strictly increases.
 // `ops` receives the FP64 operations (+ - * / sqrt) of the path taken: 17 per
-// neighbour (Laplacian), 11 (solve), 28 per element tested in the location
-// (four orientations), 18 (barycentrics and metric) and 77 per element of the
-// ball check (orientation 7 + quality 70).
+// neighbour (Laplacian), 11 (solve), 46 (barycentrics and metric) and 85 per
+// element of the ball of an accepted move (orientation and quality).
 __device__ bool tile_smooth_eval(const Tile& t, const Store& S, int v, MeshCtx c, double2& Xo,
                                  double4& Mo, double* qout, int& ops) {
   ops = 0;
@@ -2142,57 +2168,143 @@ __device__ bool tile_smooth_eval(const Tile& t, const Store& S, int v, MeshCtx c
   double y = (a00 * b1 - a01 * b0) / det;
   ops += 8;
   double4 Mn;
-  int tested = 0;
-  bool found = tile_interpolate(t, S, c, ne, nel, x, y, Mn, &tested);
-  ops += 28 * tested;
-  if (!found) return false;
-  ops += 18 + 77 * nel;
+  if (!tile_interpolate(t, S, c, ne, nel, x, y, Mn)) return false;
+  ops += 46;
   if (!tile_ball_after_move(t, S, c, v - c.vb, ne, nel, x, y, Mn, qold, true, qout, nullptr))
     return false;
+  ops += 85 * nel;
   Xo = make_double2(x, y);
   Mo = Mn;
   return true;
 }
 
-// Pass 2 (one 8-lane tile per listed vertex): the full quality-constrained move.
+// Pass 2 of the longer lists, one listed vertex per thread: the Laplacian sums,
+// the 2x2 solve, the location and the interpolation run per thread (a tile of
+// lanes per vertex repeats the ordered sums in every lane: four vertices per
+// warp instruction of FP64 instead of 32), the FP32 bounds of the moved ball
+// drop the moves that certainly fail, and the remaining ones get the exact
+// ball check, four at a time on 8-lane tiles.  Every value is computed by the
+// same operations in the same order as in tile_smooth_eval.
 __device__ __forceinline__ void smooth_eval_phase(Store S, const int* E, const int* nEp,
                                                   double2* mvxy, double4* mvM, double* qball,
                                                   int* C, int* nC, int* cmark, int tag,
                                                   unsigned long long* work, bool il = false) {
   const int n = *nEp;
   const Tile t = tile_of();
-  const int tiles_per_block = blockDim.x / TW;
-  const int tile_rank = il ? (threadIdx.x / TW) * gridDim.x + blockIdx.x
-                          : blockIdx.x * tiles_per_block + threadIdx.x / TW;
-  for (int j0 = 0; j0 < n; j0 += gridDim.x * tiles_per_block) {
-    int j = j0 + tile_rank;
-    int v = 0, ops = 0;
-    bool cand = false;
+  unsigned ops = 0;
+  for (int j0 = 0; j0 < n; j0 += gsize()) {
+    const int j = j0 + grank(il);
+    int v = 0, mi = 0;
+    bool may = false;
+    double x = 0.0, y = 0.0, qold = 0.0;
+    double4 Mn = make_double4(0.0, 0.0, 0.0, 0.0);
     if (j < n) {
       v = E[j];
-      MeshCtx c = ctx_of(S, v);
-      double2 X;
-      double4 Mv;
-      // the new ball qualities of an accepted move are kept for the apply
-      cand = tile_smooth_eval(t, S, v, c, X, Mv, qball + (size_t)v * S.W, ops);
-      if (t.tl == 0) {
-        if (cand) {
-          Mv.w = 1.0;  // marks a stored move
-          mvxy[v] = X;
-          mvM[v] = Mv;
-          cmark[v] = tag;
-          S.tab.had[c.mi] = 1;
-        } else {
-          mvM[v].w = 0.0;
+      const MeshCtx c = ctx_of(S, v);
+      mi = c.mi;
+      const int lv = v - c.vb;
+      const int* ne = ne_row(S, v);
+      const int nel = S.NElen[v];
+      const int* nn = nn_row(S, v);
+      const int nnl = S.NNlen[v];
+      qold = 1e300;
+#pragma unroll 4
+      for (int k = 0; k < nel; ++k) {
+        const double q = S.qK[c.eb + ne[k]];
+        qold = dlt(q, qold) ? q : qold;
+      }
+      const double4 mv = S.M[v];
+      double a00 = 0.0, a01 = 0.0, a11 = 0.0, b0 = 0.0, b1 = 0.0;
+#pragma unroll 2
+      for (int k = 0; k < nnl; ++k) {
+        const int js = c.vb + nn[k];
+        const double2 pj = S.xy[js];
+        const double4 mj = S.M[js];
+        const double w00 = 0.5 * (mv.x + mj.x);
+        const double w01 = 0.5 * (mv.y + mj.y);
+        const double w11 = 0.5 * (mv.z + mj.z);
+        a00 = a00 + w00;
+        a01 = a01 + w01;
+        a11 = a11 + w11;
+        b0 = b0 + (w00 * pj.x + w01 * pj.y);
+        b1 = b1 + (w01 * pj.x + w11 * pj.y);
+      }
+      const double det = a00 * a11 - a01 * a01;
+      ops += 17 * nnl + 3;
+      if (dgt(det, 0.0)) {
+        x = (a11 * b0 - a01 * b1) / det;
+        y = (a00 * b1 - a01 * b0) / det;
+        ops += 8;
+        const VF fx = make_vf_xy(x, y);
+        int4 e = make_int4(0, 0, 0, 0);
+        for (int k = 0; k < nel && !may; ++k) {
+          e = S.EN[c.eb + ne[k]];
+          may = contains(S, fx, x, y, c.vb + e.x, c.vb + e.y, c.vb + e.z);
+        }
+        if (may) {
+          Mn = interpolate_in(S, c.vb, e, x, y);
+          ops += 46;
+          const VF fn = make_vf(x, y, Mn.x, Mn.y, Mn.z);
+          const float ffloor = __double2float_rd(qold);
+#pragma unroll 2
+          for (int k = 0; k < nel; ++k)
+            may = may && !move_fails(S, c.vb, lv, S.EN[c.eb + ne[k]], fn, ffloor);
+        }
+      }
+      if (!may) mvM[v].w = 0.0;
+    }
+    // the exact check of the moves that may succeed: tile i of the warp takes
+    // the i-th of the next four
+    bool cand = false;
+    for (unsigned m = __ballot_sync(0xffffffffu, may); m;) {
+      int src = -1;
+      unsigned rest = m;
+#pragma unroll
+      for (int i = 0; i < 32 / TW; ++i) {
+        const int b = rest ? __ffs(rest) - 1 : -1;
+        if (i == t.shift / TW) src = b;
+        rest &= rest - 1u;
+      }
+      const int from = src >= 0 ? src : 0;
+      const int tv = __shfl_sync(0xffffffffu, v, from);
+      const double tx = __shfl_sync(0xffffffffu, x, from), ty = __shfl_sync(0xffffffffu, y, from);
+      const double tq = __shfl_sync(0xffffffffu, qold, from);
+      const double4 tm = make_double4(__shfl_sync(0xffffffffu, Mn.x, from),
+                                      __shfl_sync(0xffffffffu, Mn.y, from),
+                                      __shfl_sync(0xffffffffu, Mn.z, from), 0.0);
+      bool ok = false;
+      if (src >= 0) {
+        const MeshCtx c = ctx_of(S, tv);
+        const int nel = S.NElen[tv];
+        // the new ball qualities of an accepted move are kept for the apply
+        ok = tile_ball_exact(t, S, c, tv - c.vb, ne_row(S, tv), nel, tx, ty, tm, tq, true,
+                             qball + (size_t)tv * S.W, nullptr);
+        if (t.tl == 0) ops += 85 * nel;
+      }
+      const unsigned okm = __ballot_sync(0xffffffffu, ok && t.tl == 0);  // bit 8 i: tile i
+#pragma unroll
+      for (int i = 0; i < 32 / TW; ++i) {
+        if (m) {
+          const int b = __ffs(m) - 1;
+          m &= m - 1u;
+          if ((threadIdx.x & 31) == b) cand = (okm >> (TW * i)) & 1u;
         }
       }
     }
-    warp_append(cand && t.tl == 0, v, C, nC);
-    if (work) {  // measurement only: one atomic per warp
-      unsigned tot = __reduce_add_sync(0xffffffffu, t.tl == 0 ? (unsigned)ops : 0u);
-      if ((threadIdx.x & 31) == 0 && tot) atomicAdd(work, (unsigned long long)tot);
+    if (may) {
+      if (cand) {
+        mvxy[v] = make_double2(x, y);
+        Mn.w = 1.0;  // marks a stored move
+        mvM[v] = Mn;
+        cmark[v] = tag;
+        S.tab.had[mi] = 1;
+      } else {
+        mvM[v].w = 0.0;
+      }
     }
+    warp_append(cand, v, C, nC);
   }
+  add_work(work, ops);
 }
 
 // Passes 1 and 2 in one (persistent rounds whose list fits one tile per
@@ -3452,8 +3564,7 @@ int op_smooth(MeshSet& m, int max_sweeps, int max_rounds) {
       zero_round(m, nxt);
       PM_LAUNCH(k_smooth_scan, gv, bs, 0, m.stream, m.S, w.D[cur], w.counts + cn_list(cur),
                 w.mvM, w.C, w.counts + CN_C, w.cmark, tag, pass0, w.E, w.counts + CN_E);
-      PM_LAUNCH(k_smooth_eval, grid_tuned(m, (long long)m.S.vused * TW, bs, bps), bs, 0, m.stream, m.S,
-                w.E, w.counts + CN_E, w.mvxy, w.mvM, w.gains, w.C, w.counts + CN_C, w.cmark, tag,
+      PM_LAUNCH(k_smooth_eval, gv, bs, 0, m.stream, m.S, w.E, w.counts + CN_E, w.mvxy, w.mvM, w.gains, w.C, w.counts + CN_C, w.cmark, tag,
                 prof_work("k_smooth_eval"));
       PM_LAUNCH(k_smooth_select_apply, gv, bs, 0, m.stream, m.S, w.C, w.counts + CN_C,
                 w.cmark, w.smark, tag, w.D[nxt], w.counts + cn_list(nxt), w.dmark, w.mvxy, w.mvM,
