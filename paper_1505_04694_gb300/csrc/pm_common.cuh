@@ -208,6 +208,38 @@ __device__ __forceinline__ void write_row_bits(RowMask bits, const int* row, int
   while (bits.any()) list[pos++] = vb + row[bits.pop()];
 }
 
+// Room in three lists at once: the counts of a lane are at most 2^20 / 32, so
+// their sums are packed in one 64-bit scan, and the three atomics are issued
+// by three lanes together (one round trip instead of three).  All 32 lanes of
+// the warp must call it; null counters are skipped.
+struct Room3 {
+  int a, b, c;
+};
+__device__ __forceinline__ Room3 warp_reserve3(int na, int* pa, int nb, int* pb, int nc, int* pc) {
+  const int lane = threadIdx.x & 31;
+  const unsigned long long mine = (unsigned long long)na | ((unsigned long long)nb << 21) |
+                                  ((unsigned long long)nc << 42);
+  unsigned long long incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  const unsigned long long total = __shfl_sync(0xffffffffu, incl, 31);
+  int base = 0;
+  if (lane < 3) {
+    const int n = (int)(total >> (21 * lane)) & 0x1FFFFF;
+    int* p = lane == 0 ? pa : (lane == 1 ? pb : pc);
+    if (n > 0) base = atomicAdd(p, n);
+  }
+  const unsigned long long excl = incl - mine;
+  Room3 r;
+  r.a = __shfl_sync(0xffffffffu, base, 0) + ((int)excl & 0x1FFFFF);
+  r.b = __shfl_sync(0xffffffffu, base, 1) + ((int)(excl >> 21) & 0x1FFFFF);
+  r.c = __shfl_sync(0xffffffffu, base, 2) + (int)(excl >> 42);
+  return r;
+}
+
 template <class T>
 __device__ __forceinline__ void warp_append_t(bool pred, T val, T* list, int* count) {
   unsigned m = __ballot_sync(0xffffffffu, pred);
@@ -298,6 +330,63 @@ __device__ __forceinline__ void sorted_erase(int* buf, int& n, int val) {
     --n;
   }
 }
+
+// A sorted adjacency row of up to 16 entries in registers (every loop is
+// unrolled, so no index into local memory), padded with kRowPad.
+constexpr int kRowReg = 16;
+constexpr int kRowPad = 0x7fffffff;
+
+struct Row16 {
+  int a[kRowReg];
+  __device__ __forceinline__ void load(const int* row, int len) {
+    const int4* r4 = reinterpret_cast<const int4*>(row);
+#pragma unroll
+    for (int q = 0; q < kRowReg / 4; ++q) {
+      int4 x = make_int4(kRowPad, kRowPad, kRowPad, kRowPad);
+      if (4 * q < len) x = r4[q];
+      a[4 * q] = x.x;
+      a[4 * q + 1] = 4 * q + 1 < len ? x.y : kRowPad;
+      a[4 * q + 2] = 4 * q + 2 < len ? x.z : kRowPad;
+      a[4 * q + 3] = 4 * q + 3 < len ? x.w : kRowPad;
+    }
+  }
+  __device__ __forceinline__ bool has(int val) const {
+    bool f = false;
+#pragma unroll
+    for (int j = 0; j < kRowReg; ++j) f |= a[j] == val;
+    return f;
+  }
+  __device__ __forceinline__ void erase(int val) {
+    bool past = false;
+#pragma unroll
+    for (int j = 0; j < kRowReg; ++j) {
+      past |= a[j] == val;
+      if (past) a[j] = j + 1 < kRowReg ? a[j + 1] : kRowPad;
+    }
+  }
+  // false when the row is full (its contents are then not to be used)
+  __device__ __forceinline__ bool insert(int val) {
+    if (has(val)) return true;
+    const bool room = a[kRowReg - 1] == kRowPad;
+#pragma unroll
+    for (int j = kRowReg - 1; j > 0; --j) a[j] = max(a[j - 1], min(a[j], val));
+    a[0] = min(a[0], val);
+    return room;
+  }
+  __device__ __forceinline__ int len() const {
+    int n = 0;
+#pragma unroll
+    for (int j = 0; j < kRowReg; ++j) n += a[j] != kRowPad ? 1 : 0;
+    return n;
+  }
+  // writes the first n entries in whole 16-byte chunks
+  __device__ __forceinline__ void store(int* row, int n) const {
+    int4* r4 = reinterpret_cast<int4*>(row);
+#pragma unroll
+    for (int q = 0; q < kRowReg / 4; ++q)
+      if (4 * q < n) r4[q] = make_int4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]);
+  }
+};
 
 // ---------------------------------------------------------------------------
 // Arithmetic (Sec. 2.2).

@@ -123,7 +123,9 @@ __device__ __forceinline__ void elem_quality_phase(const Store& S, const int* li
                                                    unsigned long long* work, bool il = false) {
   const int n = *np;
   for (int i0 = 0; i0 < n; i0 += gsize()) {
-    int i = i0 + grank(il);
+    // in the persistent rounds from the last warp of every block backwards: the
+    // commit that shares the phase fills the blocks from their first warp
+    int i = i0 + (il ? (blockDim.x - 1 - threadIdx.x) * gridDim.x + blockIdx.x : grank(false));
     unsigned ops = 0;
     if (i < n) {
       int slot = list[i];
@@ -213,7 +215,7 @@ __device__ __forceinline__ bool local_max(const Store& S, int v, const int* cmar
   const int* nn = nn_row(S, v);
   int nnl = S.NNlen[v];
   bool win = true;
-#pragma unroll 4
+#pragma unroll 8
   for (int k = 0; k < nnl; ++k) {
     int u = c.vb + nn[k];
     int cu = cmark[u];
@@ -967,68 +969,15 @@ __device__ __forceinline__ void coarsen_eval_phase(Store S, const int* D, const 
   add_work(work, ops);
 }
 
-// Apply the collapses of S: elements containing edge (v, w) die, the other
-// ball elements take w in v's place (slot and orientation kept), v dies.
+// One round's independent set and its collapses: a winner applies its
+// collapse at once (no other vertex of the round reads what a collapse
+// writes); losers stay dirty for the next round.  Elements containing edge
+// (v, w) die, the other ball elements take w in v's place (slot and
+// orientation kept), v dies.
 // Neighbours of v are affected (rows change) and dirty for the next round.
 // The qualities of the elements that change are not computed here: their
 // slots join list Q and a dense pass computes them (one element per thread
 // instead of a serial chain of qualities per collapse).
-__device__ __forceinline__ void coarsen_apply_one(const Store& S, bool ok, int v,
-                                                  const int* target, int* A, int* nA,
-                                                  int* amark, int* Dn, int* nDn, int* dmark,
-                                                  int tag, int* Q, int* nQ) {
-  {
-    int nnl = 0, mi = 0, vb = 0, eb = 0;
-    const int* nn = nullptr;
-    const int* ne_v = nullptr;
-    RowMask qbits;
-    if (ok) {
-      MeshCtx c = ctx_of(S, v);
-      mi = c.mi;
-      vb = c.vb;
-      int lv = v - c.vb;
-      int w = target[v];
-      const int* ne = ne_row(S, v);
-      int nel = S.NElen[v];
-      for (int k = 0; k < nel; ++k) {
-        int4* pe = S.EN + c.eb + ne[k];
-        int4 e = *pe;
-        if (e.x == w || e.y == w || e.z == w) {
-          e.w = 0;
-        } else {
-          if (e.x == lv) e.x = w;
-          if (e.y == lv) e.y = w;
-          if (e.z == lv) e.z = w;
-          qbits.set(k);
-        }
-        *pe = e;
-      }
-      S.vflag[v] = (uint8_t)(S.vflag[v] & ~VF_ALIVE);
-      nn = nn_row(S, v);
-      nnl = S.NNlen[v];
-      ne_v = ne;
-      eb = c.eb;
-    }
-    count_op(S, ok, mi);
-    int pq = warp_reserve(qbits.count(), nQ);
-    while (qbits.any()) Q[pq++] = eb + ne_v[qbits.pop()];
-    RowMask fa, fd;
-#pragma unroll 4
-    for (int k = 0; k < nnl; ++k) {
-      int s = vb + nn[k];
-      if (stamp_first(amark, s, tag)) fa.set(k);
-      if (stamp_first(dmark, s, tag)) fd.set(k);
-    }
-    int pa = warp_reserve(fa.count(), nA);
-    int pd = warp_reserve(fd.count(), nDn);
-    write_row_bits(fa, nn, vb, A, pa);
-    write_row_bits(fd, nn, vb, Dn, pd);
-  }
-}
-
-// One round's independent set and its collapses: a winner applies its
-// collapse at once (no other vertex of the round reads what a collapse
-// writes); losers stay dirty for the next round.
 __device__ __forceinline__ void coarsen_select_apply_phase(Store S, const int* C, const int* nCp,
                                                            const int* cmark, int* smark, int tag,
                                                            const int* target, int* A, int* nA,
@@ -1040,15 +989,63 @@ __device__ __forceinline__ void coarsen_select_apply_phase(Store S, const int* C
   for (int i0 = 0; i0 < n; i0 += gsize()) {
     int i = i0 + grank(il);
     bool win = false, lose = false;
-    int v = 0;
+    int v = 0, nnl = 0, mi = 0, vb = 0, eb = 0;
+    const int* nn = nullptr;
+    const int* ne = nullptr;
+    RowMask qbits, fa, fd;
     if (i < n) {
       v = C[i];
       win = local_max(S, v, cmark, tag);
       if (win) smark[v] = tag;
       else lose = stamp_first(dmark, v, tag);
     }
-    warp_append(lose, v, Dn, nDn);
-    coarsen_apply_one(S, win, v, target, A, nA, amark, Dn, nDn, dmark, tag, Q, nQ);
+    if (win) {
+      const MeshCtx c = ctx_of(S, v);
+      mi = c.mi;
+      vb = c.vb;
+      eb = c.eb;
+      const int lv = v - c.vb;
+      const int w = target[v];
+      ne = ne_row(S, v);
+      nn = nn_row(S, v);
+      nnl = S.NNlen[v];
+      const int nel = S.NElen[v];
+      // the ball is read first (all loads in flight), then only the words that
+      // change are written: v's slot takes w, or the alive word is cleared in
+      // the elements that hold w.  Two bits per element: the word to write.
+      for (int k0 = 0; k0 < nel; k0 += 32) {
+        unsigned long long word = 0ull;
+        const int m = min(32, nel - k0);
+#pragma unroll 8
+        for (int k = 0; k < m; ++k) {
+          const int4 e = S.EN[c.eb + ne[k0 + k]];
+          const bool dies = e.x == w || e.y == w || e.z == w;
+          const unsigned f = dies ? 3u : (e.x == lv ? 0u : (e.y == lv ? 1u : 2u));
+          word |= (unsigned long long)f << (2 * k);
+          if (!dies) qbits.set(k0 + k);
+        }
+#pragma unroll 8
+        for (int k = 0; k < m; ++k) {
+          const int f = (int)(word >> (2 * k)) & 3;
+          reinterpret_cast<int*>(S.EN + c.eb + ne[k0 + k])[f] = f == 3 ? 0 : w;
+        }
+      }
+      S.vflag[v] = (uint8_t)(S.vflag[v] & ~VF_ALIVE);
+#pragma unroll 8
+      for (int k = 0; k < nnl; ++k) {
+        const int s = vb + nn[k];
+        if (stamp_first(amark, s, tag)) fa.set(k);
+        if (stamp_first(dmark, s, tag)) fd.set(k);
+      }
+    }
+    count_op(S, win, mi);
+    // a loser's one entry of the next list is itself
+    const Room3 at = warp_reserve3(fa.count(), nA, lose ? 1 : fd.count(), nDn, qbits.count(), nQ);
+    int pq = at.c;
+    while (qbits.any()) Q[pq++] = eb + ne[qbits.pop()];
+    write_row_bits(fa, nn, vb, A, at.a);
+    if (lose) Dn[at.b] = v;
+    else write_row_bits(fd, nn, vb, Dn, at.b);
   }
 }
 
@@ -1059,6 +1056,59 @@ __global__ void k_coarsen_select_apply(Store S, const int* C, const int* nCp, co
   coarsen_select_apply_phase(S, C, nCp, cmark, smark, tag, target, A, nA, amark, Dn, nDn, dmark,
                              Q, nQ);
   round_done(S, done);
+}
+
+// The commit below for rows of at most 16 entries that stay so: both rows in
+// registers, edited in place (a row of dependent local-memory accesses per
+// edit otherwise).  False, with nothing written, when a row grows past 16.
+__device__ __forceinline__ bool coarsen_commit_short(const Store& S, int u, MeshCtx c, int lu,
+                                                     int nnl, int nel, const int* target,
+                                                     const int* smark, int tag) {
+  int* nn = S.NN + (size_t)u * S.W;
+  int* ne = S.NE + (size_t)u * S.W;
+  Row16 R, Q;
+  R.load(nn, nnl);
+  Q.load(ne, nel);
+  unsigned dead = 0, sel = 0;
+#pragma unroll
+  for (int k = 0; k < kRowReg; ++k)
+    if (k < nel && S.EN[c.eb + Q.a[k]].w == 0) dead |= 1u << k;
+#pragma unroll
+  for (int k = 0; k < kRowReg; ++k)
+    if (k < nnl && smark[c.vb + R.a[k]] == tag) sel |= 1u << k;
+  for (; dead; dead &= dead - 1u) Q.erase(ne[__ffs(dead) - 1]);
+  bool ok = true;
+  for (; sel && ok; sel &= sel - 1u) {
+    const int x = nn[__ffs(sel) - 1], xs = c.vb + x;
+    const int t = target[xs];
+    R.erase(x);
+    if (t != lu) {
+      ok = R.insert(t);
+      continue;
+    }
+    // the collapsed neighbour's rows join u's
+    const int* nx = nn_row(S, xs);
+    const int nxl = S.NNlen[xs];
+    for (int j = 0; j < nxl && ok; ++j)
+      if (nx[j] != lu) ok = R.insert(nx[j]);
+    const int* ex = ne_row(S, xs);
+    const int exl = S.NElen[xs];
+    RowMask live;
+#pragma unroll 4
+    for (int j = 0; j < exl; ++j)
+      if (S.EN[c.eb + ex[j]].w) live.set(j);
+    while (live.any() && ok) ok = Q.insert(ex[live.pop()]);
+  }
+  if (!ok) return false;
+  const int nn2 = R.len(), ne2 = Q.len();
+  R.store(nn, nn2);
+  Q.store(ne, ne2);
+  S.NNlen[u] = nn2;
+  S.NElen[u] = ne2;
+#pragma unroll
+  for (int k = 0; k < kRowReg; ++k)
+    if (k < nn2) S.ntouch[c.vb + R.a[k]] = tag + 1;
+  return true;
 }
 
 // Deferred-update commit of a coarsening round for affected vertex u:
@@ -1077,6 +1127,9 @@ __device__ __forceinline__ void coarsen_commit_phase(Store S, const int* A, cons
     const int* nn = nn_row(S, u);
     const int* ne = ne_row(S, u);
     int nnl = S.NNlen[u], nel = S.NElen[u];
+    if (nnl <= kRowReg && nel <= kRowReg &&
+        coarsen_commit_short(S, u, c, lu, nnl, nel, target, smark, tag))
+      continue;
     int nb[MAXW], eb[MAXW];
     int nn2 = 0, ne2 = 0;
     bool ok = true;
@@ -1779,61 +1832,9 @@ __device__ __forceinline__ void swap_scan_eval_phase(Store S, const int* D, cons
   add_work(work, ops);
 }
 
+// One round's independent set and its flips (see k_coarsen_select_apply).
 // The two new elements' qualities are left to a dense pass (their slots join
 // list Q), as for collapses.
-__device__ __forceinline__ void swap_apply_one(const Store& S, bool ok, int v, const int4* opA,
-                                               const int* opK2, int* A, int* nA, int* amark,
-                                               int* Dn, int* nDn, int* dmark, int tag, int* Q,
-                                               int* nQ) {
-  {
-    int mi = 0, q1 = 0, q2 = 0;
-    int t[4] = {0, 0, 0, 0};
-    if (ok) {
-      MeshCtx c = ctx_of(S, v);
-      mi = c.mi;
-      int lv = v - c.vb;
-      int4 op = opA[v];
-      int K2 = opK2[v];
-      int4 t1 = make_int4(lv, op.z, op.y, 1);  // K1 = (v, d, c)
-      int4 t2 = make_int4(op.z, op.x, op.y, 1);  // K2 = (d, w, c)
-      S.EN[c.eb + op.w] = t1;
-      S.EN[c.eb + K2] = t2;
-      q1 = c.eb + op.w;
-      q2 = c.eb + K2;
-      t[0] = v;
-      t[1] = c.vb + op.x;
-      t[2] = c.vb + op.y;
-      t[3] = c.vb + op.z;
-    }
-    count_op(S, ok, mi);
-    bool fa[4], fd[4];
-    int na = 0, nd = 0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      fa[k] = ok && stamp_first(amark, t[k], tag);
-      fd[k] = ok && stamp_first(dmark, t[k], tag);
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      na += fa[k];
-      nd += fd[k];
-    }
-    int pa = warp_reserve(na, nA);
-    int pd = warp_reserve(nd, nDn);
-    int pq = warp_reserve(ok ? 2 : 0, nQ);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (fa[k]) A[pa++] = t[k];
-      if (fd[k]) Dn[pd++] = t[k];
-    }
-    if (ok) {
-      Q[pq] = q1;
-      Q[pq + 1] = q2;
-    }
-  }
-}
-
-// One round's independent set and its flips (see k_coarsen_select_apply).
 __device__ __forceinline__ void swap_select_apply_phase(Store S, const int* C, const int* nCp,
                                                         const int* cmark, int* smark, int tag,
                                                         const int4* opA, const int* opK2, int* A,
@@ -1844,15 +1845,60 @@ __device__ __forceinline__ void swap_select_apply_phase(Store S, const int* C, c
   for (int i0 = 0; i0 < n; i0 += gsize()) {
     int i = i0 + grank(il);
     bool win = false, lose = false;
-    int v = 0;
+    int v = 0, mi = 0, q1 = 0, q2 = 0;
+    int t[4] = {0, 0, 0, 0};
+    bool fa[4] = {false, false, false, false}, fd[4] = {false, false, false, false};
     if (i < n) {
       v = C[i];
+      const int4 op = opA[v];
+      const int K2 = opK2[v];
       win = local_max(S, v, cmark, tag);
-      if (win) smark[v] = tag;
-      else lose = stamp_first(dmark, v, tag);
+      if (win) {
+        smark[v] = tag;
+        const MeshCtx c = ctx_of(S, v);
+        mi = c.mi;
+        const int lv = v - c.vb;
+        q1 = c.eb + op.w;
+        q2 = c.eb + K2;
+        S.EN[q1] = make_int4(lv, op.z, op.y, 1);    // K1 = (v, d, c)
+        S.EN[q2] = make_int4(op.z, op.x, op.y, 1);  // K2 = (d, w, c)
+        t[0] = v;
+        t[1] = c.vb + op.x;
+        t[2] = c.vb + op.y;
+        t[3] = c.vb + op.z;
+        int oa[4], od[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          oa[k] = atomicExch(amark + t[k], tag);
+          od[k] = atomicExch(dmark + t[k], tag);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          fa[k] = oa[k] != tag;
+          fd[k] = od[k] != tag;
+        }
+      } else {
+        lose = stamp_first(dmark, v, tag);
+      }
     }
-    warp_append(lose, v, Dn, nDn);
-    swap_apply_one(S, win, v, opA, opK2, A, nA, amark, Dn, nDn, dmark, tag, Q, nQ);
+    count_op(S, win, mi);
+    int na = 0, nd = lose ? 1 : 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      na += fa[k];
+      nd += fd[k];
+    }
+    Room3 at = warp_reserve3(na, nA, nd, nDn, win ? 2 : 0, nQ);
+    if (lose) Dn[at.b] = v;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (fa[k]) A[at.a++] = t[k];
+      if (fd[k]) Dn[at.b++] = t[k];
+    }
+    if (win) {
+      Q[at.c] = q1;
+      Q[at.c + 1] = q2;
+    }
   }
 }
 
@@ -1863,6 +1909,47 @@ __global__ void k_swap_select_apply(Store S, const int* C, const int* nCp, const
   swap_select_apply_phase(S, C, nCp, cmark, smark, tag, opA, opK2, A, nA, amark, Dn, nDn, dmark,
                           Q, nQ);
   round_done(S, done);
+}
+
+// The commit below for rows of at most 16 entries that stay so (see
+// coarsen_commit_short).
+__device__ __forceinline__ bool swap_commit_short(const Store& S, int u, MeshCtx c, int lu,
+                                                  int nnl, int nel, const int4* opA,
+                                                  const int* opK2, const int* smark, int tag) {
+  int* nn = S.NN + (size_t)u * S.W;
+  int* ne = S.NE + (size_t)u * S.W;
+  Row16 R, Q;
+  R.load(nn, nnl);
+  Q.load(ne, nel);
+  unsigned sel = smark[u] == tag ? 1u << kRowReg : 0u;
+#pragma unroll
+  for (int k = 0; k < kRowReg; ++k)
+    if (k < nnl && smark[c.vb + R.a[k]] == tag) sel |= 1u << k;
+  bool ok = true;
+  for (; sel && ok; sel &= sel - 1u) {
+    const int k = __ffs(sel) - 1;
+    const int x = k == kRowReg ? lu : nn[k];
+    const int4 op = opA[c.vb + x];
+    const int K2 = opK2[c.vb + x];
+    // u is v (x itself), w, c or d of the flip, or not in it
+    if (x == lu || op.x == lu) {
+      R.erase(x == lu ? op.x : x);
+      Q.erase(x == lu ? K2 : op.w);
+    } else if (op.y == lu || op.z == lu) {
+      ok = R.insert(op.y == lu ? op.z : op.y);
+      ok &= Q.insert(op.y == lu ? K2 : op.w);
+    }
+  }
+  if (!ok) return false;
+  const int nn2 = R.len(), ne2 = Q.len();
+  R.store(nn, nn2);
+  Q.store(ne, ne2);
+  S.NNlen[u] = nn2;
+  S.NElen[u] = ne2;
+#pragma unroll
+  for (int k = 0; k < kRowReg; ++k)
+    if (k < nn2) S.ntouch[c.vb + R.a[k]] = tag + 1;
+  return true;
 }
 
 // Deferred-update commit of a swap round for affected vertex u, from the
@@ -1882,6 +1969,9 @@ __device__ __forceinline__ void swap_commit_phase(Store S, const int* A, const i
     int* nn = S.NN + (size_t)u * S.W;
     int* ne = S.NE + (size_t)u * S.W;
     int nnl = S.NNlen[u], nel = S.NElen[u];
+    if (nnl <= kRowReg && nel <= kRowReg &&
+        swap_commit_short(S, u, c, lu, nnl, nel, opA, opK2, smark, tag))
+      continue;
     int nb[MAXW], eb[MAXW];
     load_row(nn, nnl, nb);
     load_row(ne, nel, eb);
