@@ -336,7 +336,7 @@ pm_status pm_quality_arrays_noalloc_dev(const double* xy, const double* m, int32
  *     to this size (and at most one per 8-lane tile of the grid) are scanned
  *     and evaluated in one phase.
  * Defaults: 128 threads, 16 blocks per SM, 131072, 1 block, fuse_limit
- * {0, 2^30} (on the 2M workload the one-phase flip evaluation was slower). */
+ * {2^30, 2^30}. */
 typedef struct {
   int32_t block[4];
   int32_t blocks_per_sm[4];

@@ -1407,57 +1407,6 @@ __global__ void k_swap_scan(Store S, const int* D, const int* nDp, const int4* o
   swap_scan_phase(S, D, nDp, opA, C, nC, cmark, tag, pass0, E, nE, items, nI, icap, gains, st);
 }
 
-// Pass 2 (per listed edge, dense FP64): both flipped elements counter-
-// clockwise and their minimum quality above the old minimum -> the gain.
-// Gain of flipping edge (v, w) shared by K1 = (v, w, c) and K2 = (v, d, w)
-// (ball slots k1, k2 of v): both new elements counter-clockwise and their
-// minimum quality above the old minimum, else -1.  The flip's c and d go to
-// *cc and *d.
-__device__ __forceinline__ double flip_gain(const Store& S, MeshCtx c, int lv, const int* ne,
-                                            int k1, int k2, int* cc_out, int* d_out,
-                                            unsigned& ops) {
-  int K1 = ne[k1], K2 = ne[k2];
-  int4 e = S.EN[c.eb + K1];
-  int4 f = S.EN[c.eb + K2];
-  int w = (e.x == lv) ? e.y : (e.y == lv) ? e.z : e.x;
-  int cc = (e.x == lv) ? e.z : (e.y == lv) ? e.x : e.y;
-  int d = (f.x == lv) ? f.y : (f.y == lv) ? f.z : f.x;
-  *cc_out = cc;
-  *d_out = d;
-  double q1 = S.qK[c.eb + K1], q2 = S.qK[c.eb + K2];
-  double qold = dlt(q1, q2) ? q1 : q2;
-  VD dv = load_vd(S, c.vb + lv), dw = load_vd(S, c.vb + w), dc = load_vd(S, c.vb + cc),
-     dd = load_vd(S, c.vb + d);
-  // The gain is -1 unless all four hold: (v, d, c) and (d, w, c)
-  // counter-clockwise, n1 > qold, n2 > qold.  A conjunction may be decided in
-  // any order: the orientation filters first (a decided negative sign ends
-  // it), then the qualities, and only then the exact sign of an orientation
-  // the filter left open (nearly or exactly collinear points, whose element
-  // has quality near zero and so has almost always failed by then).  Every
-  // test is still made before a gain is returned, so the result is the one
-  // of the order orientations-then-qualities whatever the values.
-  const int s1 = orient_filter(dv, dd, dc);
-  ops += kOpsOrient;
-  if (s1 < 0) return -1.0;
-  const int s2 = orient_filter(dd, dw, dc);
-  ops += kOpsOrient;
-  if (s2 < 0) return -1.0;
-  ops += kOpsQuality;
-  const double n1 = quality_c(lv, d, cc, dv, dd, dc);
-  if (!dgt(n1, qold)) return -1.0;
-  ops += kOpsQuality;
-  const double n2 = quality_c(d, w, cc, dd, dw, dc);
-  if (!dgt(n2, qold)) return -1.0;
-  if (s1 == 0 || s2 == 0) {
-    const VD pv = load_xy_again(S, c.vb + lv), pw = load_xy_again(S, c.vb + w),
-             pc = load_xy_again(S, c.vb + cc), pd = load_xy_again(S, c.vb + d);
-    if (s1 == 0 && orient_resolve(pv, pd, pc) <= 0) return -1.0;
-    if (s2 == 0 && orient_resolve(pd, pw, pc) <= 0) return -1.0;
-  }
-  ops += 1;
-  return (dlt(n1, n2) ? n1 : n2) - qold;
-}
-
 // An edge both of whose end points are evaluated this round is listed from
 // both ends with the same two new elements: in canonical rotation their
 // qualities and orientations, hence the gain, are bitwise equal from either
@@ -1482,27 +1431,53 @@ constexpr int kEdgeQueueWarps = 8;
 // first vertex slot of the mesh, K2), vt = local ids (v, w, c, d).
 struct FlipQueue {
   int4 *id, *vt;
-  double* qold;
+  double *qold, *gain;
   int n;  // entries, the same in every lane
 };
 
-// Evaluates the first `cnt` (<= 16) queued flips; all lanes call.
-__device__ __forceinline__ void flip_run(const Store& S, FlipQueue& Q, int cnt, double* gains,
-                                         unsigned& ops) {
-  const int lane = threadIdx.x & 31, j = lane >> 1;
+// One queue per warp, in the block's shared memory.  The callers leave at most
+// 15 entries queued between turns and add at most 32 a turn.
+__device__ __forceinline__ FlipQueue flip_queue() {
+  __shared__ int4 s_id[kEdgeQueueWarps][48];
+  __shared__ int4 s_vt[kEdgeQueueWarps][48];
+  __shared__ double s_q[kEdgeQueueWarps][48];
+  __shared__ double s_g[kEdgeQueueWarps][48];
+  const int wq = (threadIdx.x >> 5) % kEdgeQueueWarps;
+  return FlipQueue{s_id[wq], s_vt[wq], s_q[wq], s_g[wq], 0};
+}
+
+// The FP32 part of the gain of flipping (v, w), K1 = (v, w, c), K2 = (v, d, w)
+// (slots and local ids): false when the flip certainly fails, else the queue
+// entry of what is left to decide.
+__device__ __forceinline__ bool flip_filter(const Store& S, MeshCtx c, int lv, int w, int cc, int d,
+                                            int K2, double qold, int low, int4& id, int4& vt) {
+  const VF fv = load_vf(S, c.vb + lv), fw = load_vf(S, c.vb + w), fc = load_vf(S, c.vb + cc),
+           fd = load_vf(S, c.vb + d);
+  // the flipped edge (c, d) must not exist already
+  const bool dup = row_has(nn_row(S, c.vb + d), S.NNlen[c.vb + d], cc);
+  const float floor = __double2float_rd(qold);
+  int s1, s2;
+  const float u1 = f_quality_up(fv, fd, fc, s1), u2 = f_quality_up(fd, fw, fc, s2);
+  id = make_int4(c.vb + lv, low | ((s1 == 0 ? 1 : 0) << 17) | ((s2 == 0 ? 1 : 0) << 18), c.vb, K2);
+  vt = make_int4(lv, w, cc, d);
+  return !dup && s1 >= 0 && s2 >= 0 && !(u1 < floor) && !(u2 < floor);
+}
+
+// The exact gains of queued flips at..at + 15 (those below n) into Q.gain, -1
+// for a flip that fails: flip j on lanes 2 j and 2 j + 1.  All lanes call.
+__device__ __forceinline__ void flip_gains16(const Store& S, const FlipQueue& Q, int at, int n,
+                                             unsigned& ops) {
+  const int lane = threadIdx.x & 31, j = at + (lane >> 1);
   const bool second = lane & 1;  // element (d, w, c); else (v, d, c)
   bool ok = false;
-  double q = 0.0, qold = 0.0;
-  int4 id = make_int4(0, 0, 0, 0), vt = make_int4(0, 0, 0, 0);
-  if (j < cnt) {
-    id = Q.id[j];
-    vt = Q.vt[j];
-    qold = Q.qold[j];
+  double q = 0.0;
+  if (j < n) {
+    const int4 id = Q.id[j], vt = Q.vt[j];
     const int i0 = second ? vt.w : vt.x, i1 = second ? vt.y : vt.w, i2 = vt.z;
-    const VD a = load_vd(S, id.z + i0), b = load_vd(S, id.z + i1), c = load_vd(S, id.z + i2);
-    q = quality_c(i0, i1, i2, a, b, c);
+    q = quality_c(i0, i1, i2, load_vd(S, id.z + i0), load_vd(S, id.z + i1),
+                  load_vd(S, id.z + i2));
     ops += kOpsQuality;
-    ok = dgt(q, qold);
+    ok = dgt(q, Q.qold[j]);
     if (ok && ((id.y >> (second ? 18 : 17)) & 1)) {
       ops += kOpsOrient;
       ok = orient_sign(load_xy_again(S, id.z + i0), load_xy_again(S, id.z + i1),
@@ -1511,16 +1486,28 @@ __device__ __forceinline__ void flip_run(const Store& S, FlipQueue& Q, int cnt, 
   }
   const unsigned okm = __ballot_sync(0xffffffffu, ok);
   const double q2 = __shfl_xor_sync(0xffffffffu, q, 1);
-  if (!second && ((okm >> lane) & 3u) == 3u) {
+  if (!second && j < n) {
+    const bool both = ((okm >> lane) & 3u) == 3u;
+    Q.gain[j] = both ? (dlt(q, q2) ? q : q2) - Q.qold[j] : -1.0;
     ++ops;
-    const double g = (dlt(q, q2) ? q : q2) - qold;
-    const int v = id.x;
-    gains[(size_t)v * S.W + (id.y & 0xFF)] = g;
+  }
+  __syncwarp();
+}
+
+// Evaluates the first `cnt` (<= 16) queued flips and stores the gains; all
+// lanes call.
+__device__ __forceinline__ void flip_run(const Store& S, FlipQueue& Q, int cnt, double* gains,
+                                         unsigned& ops) {
+  const int lane = threadIdx.x & 31;
+  flip_gains16(S, Q, 0, cnt, ops);
+  if (lane < cnt && dgt(Q.gain[lane], 0.0)) {
+    const int4 id = Q.id[lane], vt = Q.vt[lane];
+    const double g = Q.gain[lane];
+    gains[(size_t)id.x * S.W + (id.y & 0xFF)] = g;
     if ((id.y >> 16) & 1) {
       // from w's side the pair is (K2, K1): w's slot of K2
       const int ws = id.z + vt.y;
-      const int* nw = ne_row(S, ws);
-      const int kk = row_find(nw, S.NElen[ws], id.w);
+      const int kk = row_find(ne_row(S, ws), S.NElen[ws], id.w);
       if (kk >= 0) gains[(size_t)ws * S.W + kk] = g;
     }
   }
@@ -1546,14 +1533,9 @@ __device__ __forceinline__ void flip_run(const Store& S, FlipQueue& Q, int cnt, 
 __device__ __forceinline__ void swap_edge_phase(Store S, const int2* items, const int* nIp,
                                                 double* gains, int tag, unsigned long long* work,
                                                 bool il = false) {
-  // at most 15 entries stay queued between turns, a turn adds at most 32
-  __shared__ int4 s_id[kEdgeQueueWarps][48];
-  __shared__ int4 s_vt[kEdgeQueueWarps][48];
-  __shared__ double s_q[kEdgeQueueWarps][48];
   const int n = *nIp;
   const int lane = threadIdx.x & 31;
-  const int wq = (threadIdx.x >> 5) % kEdgeQueueWarps;
-  FlipQueue Q{s_id[wq], s_vt[wq], s_q[wq], 0};
+  FlipQueue Q = flip_queue();
   unsigned ops = 0;
   for (int i0 = 0; i0 < n; i0 += gsize()) {
     const int i = i0 + grank(il);
@@ -1574,19 +1556,9 @@ __device__ __forceinline__ void swap_edge_phase(Store S, const int2* items, cons
       const int d = (f.x == lv) ? f.y : (f.y == lv) ? f.z : f.x;
       const bool both = S.evs[c.vb + w] == tag;
       if (!both || lv < w) {
-        const VF fv = load_vf(S, v), fw = load_vf(S, c.vb + w), fc = load_vf(S, c.vb + cc),
-                 fd = load_vf(S, c.vb + d);
-        // the flipped edge (c, d) must not exist already
-        const bool dup = row_has(nn_row(S, c.vb + d), S.NNlen[c.vb + d], cc);
         qold = dlt(qa, qb) ? qa : qb;
-        const float floor = __double2float_rd(qold);
-        int s1, s2;
-        const float u1 = f_quality_up(fv, fd, fc, s1), u2 = f_quality_up(fd, fw, fc, s2);
-        need = !dup && s1 >= 0 && s2 >= 0 && !(u1 < floor) && !(u2 < floor);
-        id = make_int4(v, k1 | (k2 << 8) | ((both ? 1 : 0) << 16) | ((s1 == 0 ? 1 : 0) << 17) |
-                              ((s2 == 0 ? 1 : 0) << 18),
-                       c.vb, K2);
-        vt = make_int4(lv, w, cc, d);
+        need = flip_filter(S, c, lv, w, cc, d, K2, qold,
+                           k1 | (k2 << 8) | ((both ? 1 : 0) << 16), id, vt);
       }
     }
     const unsigned m = __ballot_sync(0xffffffffu, need);
@@ -1724,12 +1696,16 @@ __global__ void k_swap_pick(Store S, const int* E, const int* nEp, const double*
 
 // Passes 1-3 in one, for persistent rounds whose list fits one pass of the
 // grid's tiles: lane j of v's tile takes v's ball elements j, j + 8, ... as
-// K1 of the edge (v, w) that follows v in it, lists the edge by pass 1's rule
-// (interior, one of the pair below q_thresh, the flip duplicates no edge),
-// evaluates its gain (pass 2), and the tile keeps the largest positive gain,
-// ties to the smallest w (pass 3's order: a total order, w differs between
-// v's edges).  Each edge of v is the K1 edge of exactly one ball element, so
-// the candidate edges are those pass 1 lists.  Two barriers fewer per round.
+// K1 of the edge (v, w) that follows v in it, finds the element K2 = (v, d, w)
+// that follows K1 around v among the tile's elements (shuffles), lists the edge
+// by pass 1's rule (interior, one of the pair below q_thresh), filters it and,
+// when something is left to decide, gets its gain from the warp's queue (pass
+// 2); the tile keeps the largest positive gain, ties to the smallest w (pass
+// 3's order: a total order, w differs between v's edges).  Each edge of v is
+// the K1 edge of exactly one ball element, so the candidate edges are those
+// pass 1 lists.  An edge between two listed vertices is evaluated from both
+// ends; in exchange a round takes two barriers fewer and no trip of items and
+// gains through memory.
 __device__ __forceinline__ bool flip_better(bool f2, double g2, int w2, bool f, double g, int w) {
   return f2 && (!f || dgt(g2, g) || (dbits(g2) == dbits(g) && w2 < w));
 }
@@ -1739,15 +1715,20 @@ __device__ __forceinline__ void swap_scan_eval_phase(Store S, const int* D, cons
                                                      int* cmark, int tag, int pass0,
                                                      unsigned long long* work) {
   const Tile t = tile_of();
+  const int lane = threadIdx.x & 31;
+  FlipQueue Q = flip_queue();
   const int n = *nDp;
   unsigned ops = 0;
   for (int i0 = 0; i0 < n; i0 += tcount()) {
     const int i = i0 + trank(true);
-    int v = 0;
-    bool cand = false;
+    int v = 0, lv = 0, nel = 0;
+    bool cand = false, eval = false;
+    MeshCtx c{0, 0, 0};
+    const int* ne = nullptr;
+    double qt = 0.0;
     if (i < n) {
       v = D[i];
-      MeshCtx c = ctx_of(S, v);
+      c = ctx_of(S, v);
       const int et = __shfl_sync(t.mask, S.evs[v], 0, TW);
       if (unchanged(S, v, c.vb, et, pass0)) {
         cand = opA[v].x >= 0;
@@ -1756,76 +1737,115 @@ __device__ __forceinline__ void swap_scan_eval_phase(Store S, const int* D, cons
           S.tab.had[c.mi] = 1;
         }
       } else if (S.vflag[v] & VF_ALIVE) {
-        if (t.tl == 0) S.evs[v] = tag;
-        const int lv = v - c.vb;
-        const int* ne = ne_row(S, v);
-        const int nel = S.NElen[v];
-        const double qt = S.tab.q_thresh[c.mi];
-        bool found = false;
-        double best = 0.0;
-        int bw = 0, bk1 = -1, bk2 = -1, bc = 0, bd = 0;
-        for (int k = t.tl; k < nel; k += TW) {
-          const int K1 = ne[k];
-          const int4 e = S.EN[c.eb + K1];
-          const int w = (e.x == lv) ? e.y : (e.y == lv) ? e.z : e.x;   // after v
-          const int cc = (e.x == lv) ? e.z : (e.y == lv) ? e.x : e.y;  // before v
-          int k2 = -1, d = 0;
-          for (int j = 0; j < nel; ++j) {
-            if (j == k) continue;
-            const int4 f = S.EN[c.eb + ne[j]];
-            if (((f.x == lv) ? f.z : (f.y == lv) ? f.x : f.y) == w) {
-              k2 = j;
-              d = (f.x == lv) ? f.y : (f.y == lv) ? f.z : f.x;
-              break;
-            }
-          }
-          if (k2 < 0) continue;  // boundary edge
-          if (!dlt(S.qK[c.eb + K1], qt) && !dlt(S.qK[c.eb + ne[k2]], qt)) continue;
-          if (row_has(nn_row(S, c.vb + d), S.NNlen[c.vb + d], cc)) continue;
-          int c2, d2;
-          const double g = flip_gain(S, c, lv, ne, k, k2, &c2, &d2, ops);
-          if (!dgt(g, 0.0)) continue;
-          if (flip_better(true, g, w, found, best, bw)) {
-            found = true;
-            best = g;
-            bw = w;
-            bk1 = k;
-            bk2 = k2;
-            bc = cc;
-            bd = d;
-          }
-        }
-#pragma unroll
-        for (int o = TW / 2; o > 0; o >>= 1) {
-          const bool f2 = __shfl_xor_sync(t.mask, found ? 1 : 0, o, TW) != 0;
-          const double g2 = __shfl_xor_sync(t.mask, best, o, TW);
-          const int w2 = __shfl_xor_sync(t.mask, bw, o, TW);
-          const int k1b = __shfl_xor_sync(t.mask, bk1, o, TW);
-          const int k2b = __shfl_xor_sync(t.mask, bk2, o, TW);
-          const int cb = __shfl_xor_sync(t.mask, bc, o, TW);
-          const int db = __shfl_xor_sync(t.mask, bd, o, TW);
-          if (flip_better(f2, g2, w2, found, best, bw)) {
-            found = true;
-            best = g2;
-            bw = w2;
-            bk1 = k1b;
-            bk2 = k2b;
-            bc = cb;
-            bd = db;
-          }
-        }
-        if (t.tl == 0) {
-          if (found) {
-            opA[v] = make_int4(bw, bc, bd, ne[bk1]);
-            opK2[v] = ne[bk2];
-            cmark[v] = tag;
-            S.tab.had[c.mi] = 1;
-          } else {
-            opA[v].x = -1;
-          }
-        }
-        cand = found;
+        eval = true;
+        lv = v - c.vb;
+        ne = ne_row(S, v);
+        nel = S.NElen[v];
+        qt = S.tab.q_thresh[c.mi];
       }
+    }
+    if (eval && t.tl == 0) S.evs[v] = tag;
+    const int nelw = __reduce_max_sync(0xffffffffu, nel);
+    bool found = false;
+    double best = 0.0;
+    int bw = 0, bK1 = -1, bK2 = -1, bc = 0, bd = 0;
+    for (int base = 0; base < nelw; base += TW) {
+      const int k = base + t.tl;
+      int K1 = -1, w = -1, cc = -2;
+      double q1 = 0.0;
+      if (k < nel) {
+        K1 = ne[k];
+        const int4 e = S.EN[c.eb + K1];
+        q1 = S.qK[c.eb + K1];
+        w = (e.x == lv) ? e.y : (e.y == lv) ? e.z : e.x;   // after v
+        cc = (e.x == lv) ? e.z : (e.y == lv) ? e.x : e.y;  // before v
+      }
+      // K2: the element whose vertex before v is w (one at most)
+      int K2 = -1, d = 0;
+      double q2 = 0.0;
+      for (int other = 0; other < nelw; other += TW) {
+        int oK = K1, onx = w, opv = cc;
+        double oq = q1;
+        if (other != base) {
+          oK = -1;
+          opv = -2;
+          const int ko = other + t.tl;
+          if (ko < nel) {
+            oK = ne[ko];
+            const int4 f = S.EN[c.eb + oK];
+            oq = S.qK[c.eb + oK];
+            onx = (f.x == lv) ? f.y : (f.y == lv) ? f.z : f.x;
+            opv = (f.x == lv) ? f.z : (f.y == lv) ? f.x : f.y;
+          }
+        }
+        int src = -1;
+#pragma unroll
+        for (int j = TW - 1; j >= 0; --j)
+          if (__shfl_sync(0xffffffffu, opv, j, TW) == w) src = j;
+        const int from = src >= 0 ? src : 0;
+        const int sK = __shfl_sync(0xffffffffu, oK, from, TW);
+        const int sd = __shfl_sync(0xffffffffu, onx, from, TW);
+        const double sq = __shfl_sync(0xffffffffu, oq, from, TW);
+        if (src >= 0 && K2 < 0) {
+          K2 = sK;
+          d = sd;
+          q2 = sq;
+        }
+      }
+      bool need = false;
+      int4 id = make_int4(0, 0, 0, 0), vt = id;
+      double qold = 0.0;
+      if (k < nel && K2 >= 0 && K2 != K1 && (dlt(q1, qt) || dlt(q2, qt))) {
+        qold = dlt(q1, q2) ? q1 : q2;
+        need = flip_filter(S, c, lv, w, cc, d, K2, qold, 0, id, vt);
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, need);
+      const int at = __popc(m & ((1u << lane) - 1u)), cnt = __popc(m);
+      if (need) {
+        Q.id[at] = id;
+        Q.vt[at] = vt;
+        Q.qold[at] = qold;
+      }
+      __syncwarp();
+      for (int b = 0; b < cnt; b += 16) flip_gains16(S, Q, b, cnt, ops);
+      if (need) {
+        const double g = Q.gain[at];
+        if (dgt(g, 0.0) && flip_better(true, g, w, found, best, bw)) {
+          found = true;
+          best = g;
+          bw = w;
+          bK1 = K1;
+          bK2 = K2;
+          bc = cc;
+          bd = d;
+        }
+      }
+      __syncwarp();
+    }
+    // the tile's best: lane `src` holds it
+    int src = t.tl;
+#pragma unroll
+    for (int o = TW / 2; o > 0; o >>= 1) {
+      const bool f2 = __shfl_xor_sync(0xffffffffu, found ? 1 : 0, o, TW) != 0;
+      const double g2 = __shfl_xor_sync(0xffffffffu, best, o, TW);
+      const int w2 = __shfl_xor_sync(0xffffffffu, bw, o, TW);
+      const int s2 = __shfl_xor_sync(0xffffffffu, src, o, TW);
+      if (flip_better(f2, g2, w2, found, best, bw)) {
+        found = true;
+        best = g2;
+        bw = w2;
+        src = s2;
+      }
+    }
+    if (eval) {
+      if (found && src == t.tl) {
+        opA[v] = make_int4(bw, bc, bd, bK1);
+        opK2[v] = bK2;
+        cmark[v] = tag;
+        S.tab.had[c.mi] = 1;
+      }
+      if (!found && t.tl == 0) opA[v].x = -1;
+      cand = found;
     }
     warp_append(cand && t.tl == 0, v, C, nC);
   }

@@ -36,7 +36,7 @@ namespace pm {
 namespace {
 
 constexpr Tuning kDefaults = {{128, 128, 128, 128}, {16, 16, 16, 16}, {131072, 131072, 131072},
-                               {1, 1, 1}, {0, 1 << 30}};
+                               {1, 1, 1}, {1 << 30, 1 << 30}};
 
 std::mutex g_tmu;
 Tuning g_tune = kDefaults;

@@ -563,7 +563,7 @@ def set_tuning(t=None):
 
 def get_tuning_defaults():
     return {"block": [128] * 4, "blocks_per_sm": [16] * 4, "rounds_limit": [131072] * 3,
-            "rounds_blocks_per_sm": [1] * 3, "fuse_limit": [0, 1 << 30]}
+            "rounds_blocks_per_sm": [1] * 3, "fuse_limit": [1 << 30] * 2}
 
 
 def get_tuning():
