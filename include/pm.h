@@ -310,7 +310,7 @@ pm_status pm_selftest_orient_dev(const double* pts, int32_t* out, int64_t n, voi
  * allocation after start-up).  The paper has no counterpart: this is a
  * service of this library.  Same arguments, results, stream behaviour and
  * statuses as pm_quality_arrays_dev, but every temporary lives in one fixed array
- * (about 9.6 MB) compiled into the library, which each GPU that loads the
+ * (about 6.5 MB) compiled into the library, which each GPU that loads the
  * library keeps until the process exits; the call allocates and frees
  * nothing.  Limits: ne <= 65536 elements and nv <= 65536 vertices, else
  * PM_ERR_CAPACITY.  The first call on a device looks up the array's device

@@ -23,6 +23,8 @@ struct ScanWork {
 
 int scan_tiles(int n);
 void scan_exclusive(const int* in, int* out, int n, ScanWork& w, DevStatus* st, cudaStream_t s);
+void scan_exclusive_cleared(const int* in, int* out, int n, ScanWork& w, DevStatus* st,
+                            cudaStream_t s);
 void scan_alive_vertices(const Store& S, int* out, int n, ScanWork& w, DevStatus* st,
                          cudaStream_t s);
 void scan_alive_elements(const Store& S, int* out, int n, ScanWork& w, DevStatus* st,
@@ -120,6 +122,9 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
 void set_free(MeshSet& m);
 // Release the status word and the pinned read-back slot of a set.
 void set_release(MeshSet& m);
+// A slot of the process-wide pinned arena (16 KB; null when none can be had).
+void* pinned_slot();
+void pinned_slot_free(void* p);
 cudaError_t upload_tab(MeshSet& m);
 void set_used(MeshSet& m);
 cudaError_t grow(MeshSet& m, const std::vector<int>& vcap, const std::vector<int>& ecap, int W);
@@ -150,6 +155,36 @@ cudaError_t fetch_ops(MeshSet& m, std::vector<unsigned long long>& ops);
 int quality_mesh(MeshSet& m, double* qsum_host, double* dxy_host, double* dm_host);
 int quality_arrays(const double* xy, const double* mt, int nv, const int* tri, int ne,
                    double* qsum, double* dxy, double* dm, cudaStream_t s);
+
+// Partial derivatives of an element's quality: d/d(x, y) of its three
+// vertices, then the metric's three, which are the same for each vertex (the
+// element metric is their mean).
+struct EGrad {
+  double xy[6];
+  double m[3];
+};
+// Status, block counter and scan ticket of a call.
+struct QHead {
+  DevStatus st;
+  unsigned done;
+  int ticket;
+};
+// Workspace of one call on plain arrays; head, cnt and state start at zero.
+struct QualityWork {
+  QHead* head;
+  int* cnt;                   // 2 (nv + 1): corners per vertex, and beyond its 255th
+  unsigned long long* state;  // scan_tiles(nv + 1)
+  double* part;               // quality_blocks(ne)
+  EGrad* eg;                  // ne
+  int* off;                   // nv + 1
+  int* col;                   // 3 ne
+  uint8_t* pos;               // 3 ne
+};
+constexpr int kQualityBlocks = 152 * 8;
+int quality_blocks(int ne);
+cudaError_t quality_launch(const QualityWork& w, const double* xy, const double* mt, int nv,
+                           const int* tri, int ne, double* qsum, double* dxy, double* dm,
+                           DevStatus* out_st, cudaStream_t s);
 
 // ---- errors (pm_capi.cu) ----
 void set_last_error(const std::string& msg);

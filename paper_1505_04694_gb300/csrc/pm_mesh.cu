@@ -644,6 +644,9 @@ __global__ void k_out_e_set(Store S, const int* vscan, const int* escan, int32_t
 
 // ---------------------------------------------------------------------------
 
+void* pinned_slot() { return pinned_get(); }
+void pinned_slot_free(void* p) { pinned_put(p); }
+
 // Bounds below which every used slot lies (from the host mirror).
 void set_used(MeshSet& m) {
   int last = m.nmesh - 1;

@@ -17,9 +17,25 @@ namespace {
 constexpr int RED_BLOCKS = 256;
 constexpr int RED_THREADS = 256;
 
-struct EGrad {
-  double g[15];
-};
+__device__ __forceinline__ EGrad pack_grad(const double g[3][5]) {
+  EGrad out;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    out.xy[2 * k] = g[k][0];
+    out.xy[2 * k + 1] = g[k][1];
+    out.m[k] = g[0][2 + k];
+  }
+  return out;
+}
+
+// acc += the derivatives of corner i of an element
+__device__ __forceinline__ void add_corner(double acc[5], const EGrad& e, int i) {
+  acc[0] = acc[0] + e.xy[2 * i];
+  acc[1] = acc[1] + e.xy[2 * i + 1];
+  acc[2] = acc[2] + e.m[0];
+  acc[3] = acc[3] + e.m[1];
+  acc[4] = acc[4] + e.m[2];
+}
 
 __global__ void k_elem_qgrad_store(Store S, int mesh, double* qel, EGrad* eg) {
   int vb = S.tab.vbase[mesh], eb = S.tab.ebase[mesh], ne = S.tab.ne[mesh];
@@ -29,18 +45,14 @@ __global__ void k_elem_qgrad_store(Store S, int mesh, double* qel, EGrad* eg) {
       qel[l] = 0.0;
       continue;
     }
-    double g[3][5];
-    double q = quality_grad_c(e.x, e.y, e.z, load_vd(S, vb + e.x), load_vd(S, vb + e.y),
-                              load_vd(S, vb + e.z), g);
-    qel[l] = q;
-    if (eg) {
-      EGrad out;
-#pragma unroll
-      for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int j = 0; j < 5; ++j) out.g[5 * k + j] = g[k][j];
-      eg[l] = out;
+    const VD a = load_vd(S, vb + e.x), b = load_vd(S, vb + e.y), c = load_vd(S, vb + e.z);
+    if (!eg) {
+      qel[l] = quality_c(e.x, e.y, e.z, a, b, c);
+      continue;
     }
+    double g[3][5];
+    qel[l] = quality_grad_c(e.x, e.y, e.z, a, b, c, g);
+    eg[l] = pack_grad(g);
   }
 }
 
@@ -56,9 +68,7 @@ __global__ void k_vgather_store(Store S, int mesh, const EGrad* eg, double* dxy,
         int K = ne[k];
         int4 e = S.EN[eb + K];
         int i = (e.x == l) ? 0 : (e.y == l) ? 1 : 2;
-        const double* g = eg[K].g + 5 * i;
-#pragma unroll
-        for (int j = 0; j < 5; ++j) acc[j] = acc[j] + g[j];
+        add_corner(acc, eg[K], i);
       }
     }
     if (dxy) {
@@ -79,84 +89,148 @@ __device__ __forceinline__ VD arr_vd(const double* xy, const double* m, int v) {
   return VD{xy[2 * v], xy[2 * v + 1], m[3 * v], m[3 * v + 1], m[3 * v + 2]};
 }
 
-// An element with a vertex id outside [0, nv) records PM_ERR_INVALID_MESH
-// and contributes NaN (nothing is read through a bad id).
-__global__ void k_elem_qgrad_arr(const double* xy, const double* m, const int* tri, int ne,
-                                 int nv, double* qel, EGrad* eg, DevStatus* st) {
-  for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < ne; K += gridDim.x * blockDim.x) {
-    int a = tri[3 * K], b = tri[3 * K + 1], c = tri[3 * K + 2];
-    if ((unsigned)a >= (unsigned)nv || (unsigned)b >= (unsigned)nv || (unsigned)c >= (unsigned)nv) {
-      set_err(st, PM_ERR_INVALID_MESH);
-      qel[K] = __longlong_as_double(0x7ff8000000000000LL);
+// Sum over the block in a fixed order (blockDim.x: a power of two of at most
+// RED_THREADS); thread 0 gets it.
+__device__ __forceinline__ double block_sum(double x) {
+  __shared__ double sh[RED_THREADS];
+  sh[threadIdx.x] = x;
+  __syncthreads();
+  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+    if (threadIdx.x < o) sh[threadIdx.x] = sh[threadIdx.x] + sh[threadIdx.x + o];
+    __syncthreads();
+  }
+  const double r = sh[0];
+  __syncthreads();
+  return r;
+}
+
+// Quality (and, with GRAD, the derivatives) of every element, and the sum over
+// all of them: block b sums elements b T + t, b T + t + G T, ... (T threads, G
+// blocks), the last block to finish adds the blocks' sums; the shape of the sum
+// depends on the element count alone.  With GRAD each corner also takes its
+// place in its vertex's list (`pos`), under the FP64 work that bounds this
+// kernel; without it only the quality itself is evaluated (77 operations instead
+// of about 230).  An element with a vertex id outside [0, nv) records
+// PM_ERR_INVALID_MESH and contributes NaN (nothing is read through a bad id).
+// The status goes to `out_st` (pinned host memory) with the sum.
+constexpr int QT = 128;
+template <bool GRAD>
+__global__ void __launch_bounds__(QT)
+k_elem_quality_arr(const double* xy, const double* m, const int* tri, int ne, int nv, EGrad* eg,
+                   int* cnt, uint8_t* pos, double* part, double* qsum, QHead* head,
+                   DevStatus* out_st) {
+  const double nan = __longlong_as_double(0x7ff8000000000000LL);
+  double sum = 0.0;
+  for (int K = blockIdx.x * QT + threadIdx.x; K < ne; K += gridDim.x * QT) {
+    const int t[3] = {tri[3 * K], tri[3 * K + 1], tri[3 * K + 2]};
+    if ((unsigned)t[0] >= (unsigned)nv || (unsigned)t[1] >= (unsigned)nv ||
+        (unsigned)t[2] >= (unsigned)nv) {
+      set_err(&head->st, PM_ERR_INVALID_MESH);
+      sum = sum + nan;
       continue;
     }
-    double g[3][5];
-    double q = quality_grad_c(a, b, c, arr_vd(xy, m, a), arr_vd(xy, m, b), arr_vd(xy, m, c), g);
-    qel[K] = q;
-    if (eg) {
-      EGrad out;
+    const VD a = arr_vd(xy, m, t[0]), b = arr_vd(xy, m, t[1]), c = arr_vd(xy, m, t[2]);
+    if (GRAD) {
+      // (a vertex in more than 255 elements marks its later corners 255: the
+      // fill pass then takes places from the counter)
 #pragma unroll
-      for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int j = 0; j < 5; ++j) out.g[5 * k + j] = g[k][j];
-      eg[K] = out;
+      for (int i = 0; i < 3; ++i) {
+        const int p = atomicAdd(cnt + t[i], 1);
+        pos[3 * (size_t)K + i] = (uint8_t)(p < 255 ? p : 255);
+      }
+      double g[3][5];
+      sum = sum + quality_grad_c(t[0], t[1], t[2], a, b, c, g);
+      eg[K] = pack_grad(g);
+    } else {
+      sum = sum + quality_c(t[0], t[1], t[2], a, b, c);
+    }
+  }
+  const double bs = block_sum(sum);
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = bs;
+    __threadfence();
+    last = atomicAdd(&head->done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double s = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += QT) s = s + __ldcg(part + i);
+  s = block_sum(s);
+  if (threadIdx.x == 0) {
+    *qsum = s;
+    if (out_st) {
+      DevStatus r = head->st;
+      r.err = atomicAdd(&head->st.err, 0);
+      *out_st = r;
     }
   }
 }
 
-// Corners per vertex (ids outside [0, nv) are skipped: the element pass has
-// recorded them).
-__global__ void k_corner_count(const int* tri, int ne, int nv, int* cnt) {
-  for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < ne; K += gridDim.x * blockDim.x)
-    for (int i = 0; i < 3; ++i) {
-      int v = tri[3 * K + i];
-      if ((unsigned)v < (unsigned)nv) atomicAdd(cnt + v, 1);
-    }
-}
-
 // Corner list per vertex: entry = 3 * element + corner position; nothing is
 // written after a device error (the offsets may be unwritten) and no entry
-// leaves its vertex's range.
-__global__ void k_corner_fill(const int* tri, int ne, int nv, const int* off, int* fill, int* col,
-                              const DevStatus* st) {
+// leaves its vertex's range.  `more` counts the corners beyond a vertex's 255th.
+__global__ void k_corner_fill(const int* tri, int ne, int nv, const int* off, const uint8_t* pos,
+                              int* more, int* col, const DevStatus* st) {
   if (st->err) return;
   for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < ne; K += gridDim.x * blockDim.x) {
+#pragma unroll
     for (int i = 0; i < 3; ++i) {
-      int v = tri[3 * K + i];
+      const int v = tri[3 * K + i];
       if ((unsigned)v >= (unsigned)nv) continue;
-      int p = atomicAdd(fill + v, 1);
+      int p = pos[3 * (size_t)K + i];
+      if (p == 255) p += atomicAdd(more + v, 1);
       if (off[v] + p < off[v + 1]) col[off[v] + p] = 3 * K + i;
     }
   }
 }
 
 // Per vertex: its corners in ascending element id, contributions summed in
-// that order.  After a device error every output entry is NaN.
+// that order.  After a device error every output entry is NaN.  Up to 12
+// corners are sorted in registers (rank by comparison, all loads in flight);
+// more are sorted in place.  The status goes to `out_st` (pinned host memory).
+constexpr int kCornerFast = 12;
 __global__ void k_vgather_arr(const int* off, int* col, const EGrad* eg, int nv, double* dxy,
-                              double* dm, const DevStatus* st) {
+                              double* dm, const DevStatus* st, DevStatus* out_st) {
   const bool bad = st->err != 0;
   const double nan = __longlong_as_double(0x7ff8000000000000LL);
+  if (out_st && blockIdx.x == 0 && threadIdx.x == 0) *out_st = *st;
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += gridDim.x * blockDim.x) {
     double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     if (bad) {
 #pragma unroll
       for (int j = 0; j < 5; ++j) acc[j] = nan;
     } else {
-      int a = off[v], b = off[v + 1];
-      for (int k = a + 1; k < b; ++k) {  // ascending element id
-        int x = col[k];
-        int j = k - 1;
-        while (j >= a && col[j] > x) {
-          col[j + 1] = col[j];
-          --j;
-        }
-        col[j + 1] = x;
-      }
-      for (int k = a; k < b; ++k) {
-        int x = col[k];
-        const double* g = eg[x / 3].g + 5 * (x % 3);
+      const int a = off[v], b = off[v + 1];
+      if (b - a <= kCornerFast) {
+        int x[kCornerFast], o[kCornerFast];
 #pragma unroll
-        for (int j = 0; j < 5; ++j) acc[j] = acc[j] + g[j];
+        for (int k = 0; k < kCornerFast; ++k) {
+          x[k] = a + k < b ? col[a + k] : 0x7fffffff;
+          o[k] = 0x7fffffff;
+        }
+        // insertion through a minimum-maximum network keeps o sorted
+#pragma unroll
+        for (int k = 0; k < kCornerFast; ++k) {
+#pragma unroll
+          for (int j = kCornerFast - 1; j > 0; --j) o[j] = max(o[j - 1], min(o[j], x[k]));
+          o[0] = min(o[0], x[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < kCornerFast; ++k)
+          if (a + k < b) add_corner(acc, eg[o[k] / 3], o[k] % 3);
+      } else {
+        for (int k = a + 1; k < b; ++k) {  // ascending element id
+          int x = col[k];
+          int j = k - 1;
+          while (j >= a && col[j] > x) {
+            col[j + 1] = col[j];
+            --j;
+          }
+          col[j + 1] = x;
+        }
+        for (int k = a; k < b; ++k) add_corner(acc, eg[col[k] / 3], col[k] % 3);
       }
     }
     if (dxy) {
@@ -244,73 +318,97 @@ int quality_mesh(MeshSet& m, double* qsum_host, double* dxy_host, double* dm_hos
   return status ? status : err;
 }
 
+// Blocks of the element pass: 8 of 128 threads on each of the 152 SMs hide the
+// latency of the FP64 chains; the shape of the sum follows from the block count.
+int quality_blocks(int ne) {
+  return (int)std::max<long long>(1, std::min<long long>((ne + QT - 1LL) / QT, kQualityBlocks));
+}
+
+// The kernels of one call on a workspace whose head, counters and scan state
+// the caller has cleared.
+cudaError_t quality_launch(const QualityWork& w, const double* xy, const double* mt, int nv,
+                           const int* tri, int ne, double* qsum, double* dxy, double* dm,
+                           DevStatus* out_st, cudaStream_t s) {
+  const int blocks = quality_blocks(ne);
+  if (!dxy && !dm) {
+    PM_LAUNCH(k_elem_quality_arr<false>, blocks, QT, 0, s, xy, mt, tri, ne, nv, w.eg, w.cnt, w.pos,
+              w.part, qsum, w.head, out_st);
+    return cudaGetLastError();
+  }
+  PM_LAUNCH(k_elem_quality_arr<true>, blocks, QT, 0, s, xy, mt, tri, ne, nv, w.eg, w.cnt, w.pos,
+            w.part, qsum, w.head, (DevStatus*)nullptr);
+  ScanWork sw;
+  sw.state = w.state;
+  sw.ticket = &w.head->ticket;
+  sw.tiles_cap = scan_tiles(nv + 1);
+  scan_exclusive_cleared(w.cnt, w.off, nv, sw, &w.head->st, s);
+  PM_LAUNCH(k_corner_fill, gridn(ne), 128, 0, s, tri, ne, nv, (const int*)w.off,
+            (const uint8_t*)w.pos, w.cnt + (nv + 1), w.col, (const DevStatus*)&w.head->st);
+  PM_LAUNCH(k_vgather_arr, gridn(nv), 128, 0, s, (const int*)w.off, w.col, (const EGrad*)w.eg, nv,
+            dxy, dm, (const DevStatus*)&w.head->st, out_st);
+  return cudaGetLastError();
+}
+
 // Quality sum (and gradient) on plain device arrays.  Temporaries come from
-// one stream-ordered allocation; the call waits for its stream and returns
-// the device status (PM_ERR_INVALID_MESH for a vertex id outside [0, nv),
+// one stream-ordered allocation, of which one memset clears the part that starts
+// at zero; the kernels write the status straight into pinned host memory (a copy
+// into pageable memory cost 30 us a call); the call waits for its stream and
+// returns it (PM_ERR_INVALID_MESH for a vertex id outside [0, nv),
 // PM_ERR_TIMEOUT when the scan's bounded wait gave up; the outputs then hold
 // NaN).
 int quality_arrays(const double* xy, const double* mt, int nv, const int* tri, int ne,
                    double* qsum, double* dxy, double* dm, cudaStream_t s) {
   const bool grad = dxy || dm;
-  const int tiles = scan_tiles(nv + 1);
+  const int tiles = scan_tiles(nv + 1), blocks = quality_blocks(ne);
   auto r256 = [](size_t x) { return (x + 255) & ~size_t(255); };
-  const size_t b_qel = r256(std::max(ne, 1) * sizeof(double));
-  const size_t b_part = r256(RED_BLOCKS * sizeof(double));
-  const size_t b_st = r256(sizeof(DevStatus));
-  const size_t b_eg = grad ? r256(std::max(ne, 1) * sizeof(EGrad)) : 0;
+  const size_t b_head = r256(sizeof(QHead));
   const size_t b_cnt = grad ? r256(2 * ((size_t)nv + 1) * sizeof(int)) : 0;
+  const size_t b_state = grad ? r256((size_t)tiles * sizeof(unsigned long long)) : 0;
+  const size_t b_part = r256(blocks * sizeof(double));
+  const size_t b_eg = grad ? r256(std::max(ne, 1) * sizeof(EGrad)) : 0;
   const size_t b_off = grad ? r256(((size_t)nv + 1) * sizeof(int)) : 0;
   const size_t b_col = grad ? r256(std::max(3LL * ne, 1LL) * sizeof(int)) : 0;
-  const size_t b_state = grad ? r256((size_t)tiles * sizeof(unsigned long long)) : 0;
-  const size_t b_ticket = grad ? r256(sizeof(int)) : 0;
+  const size_t b_pos = grad ? r256(std::max(3LL * ne, 1LL)) : 0;
+  DevStatus* h = (DevStatus*)pinned_slot();
+  if (!h) {
+    set_last_error("pinned status word");
+    return PM_ERR_OOM;
+  }
+  h->err = PM_ERR_CUDA;  // overwritten by the last kernel
   char* base = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&base, b_qel + b_part + b_st + b_eg + b_cnt + b_off +
-                                                     b_col + b_state + b_ticket, s);
+  cudaError_t e = cudaMallocAsync((void**)&base, b_head + b_cnt + b_state + b_part + b_eg + b_off +
+                                                     b_col + b_pos, s);
   if (e != cudaSuccess) {
     set_last_error(std::string("quality workspace: ") + cudaGetErrorString(e));
     cudaGetLastError();
+    pinned_slot_free(h);
     return e == cudaErrorMemoryAllocation ? PM_ERR_OOM : PM_ERR_CUDA;
   }
   char* p = base;
-  double* qel = (double*)p; p += b_qel;
-  double* part = (double*)p; p += b_part;
-  DevStatus* st = (DevStatus*)p; p += b_st;
-  EGrad* eg = grad ? (EGrad*)p : nullptr; p += b_eg;
-  int* cnt = (int*)p; p += b_cnt;
-  int* off = (int*)p; p += b_off;
-  int* col = (int*)p; p += b_col;
-  ScanWork sw;
-  sw.state = (unsigned long long*)p; p += b_state;
-  sw.ticket = (int*)p;
-  sw.tiles_cap = tiles;
-  e = cudaMemsetAsync(st, 0, sizeof(DevStatus), s);
-  if (!e && grad) e = cudaMemsetAsync(cnt, 0, 2 * ((size_t)nv + 1) * sizeof(int), s);
-  if (!e && grad) e = cudaMemsetAsync(sw.state, 0, b_state, s);
-  if (!e) {
-    PM_LAUNCH(k_elem_qgrad_arr, gridn(ne), 128, 0, s, xy, mt, tri, ne, nv, qel, eg, st);
-    dsum(qel, ne, part, qsum, s);
-    if (grad) {
-      int* fill = cnt + (nv + 1);
-      PM_LAUNCH(k_corner_count, gridn(ne), 128, 0, s, tri, ne, nv, cnt);
-      scan_exclusive(cnt, off, nv, sw, st, s);
-      PM_LAUNCH(k_corner_fill, gridn(ne), 128, 0, s, tri, ne, nv, (const int*)off, fill, col,
-                (const DevStatus*)st);
-      PM_LAUNCH(k_vgather_arr, gridn(nv), 128, 0, s, (const int*)off, col, (const EGrad*)eg, nv,
-                dxy, dm, (const DevStatus*)st);
-    }
-    e = cudaGetLastError();
-  }
-  DevStatus h{};
-  if (!e) e = cudaMemcpyAsync(&h, st, sizeof(DevStatus), cudaMemcpyDeviceToHost, s);
+  QualityWork w;
+  w.head = (QHead*)p; p += b_head;
+  w.cnt = (int*)p; p += b_cnt;
+  w.state = (unsigned long long*)p; p += b_state;
+  w.part = (double*)p; p += b_part;
+  w.eg = (EGrad*)p; p += b_eg;
+  w.off = (int*)p; p += b_off;
+  w.col = (int*)p; p += b_col;
+  w.pos = (uint8_t*)p;
+  e = cudaMemsetAsync(base, 0, b_head + b_cnt + b_state, s);
+  if (!e) e = quality_launch(w, xy, mt, nv, tri, ne, qsum, dxy, dm, h, s);
   cudaFreeAsync(base, s);
-  if (!e) e = cudaStreamSynchronize(s);
+  // (waits also after an error: the status slot goes back)
+  const cudaError_t es = cudaStreamSynchronize(s);
+  if (!e) e = es;
+  const int err = h->err;
+  pinned_slot_free(h);
   if (e != cudaSuccess) {
     set_last_error(std::string("CUDA: ") + cudaGetErrorString(e));
     return PM_ERR_CUDA;
   }
-  if (h.err == PM_ERR_INVALID_MESH) set_last_error("vertex id outside [0, nv) in tri");
-  if (h.err == PM_ERR_TIMEOUT) set_last_error("the gradient's scan gave up waiting");
-  return h.err;
+  if (err == PM_ERR_INVALID_MESH) set_last_error("vertex id outside [0, nv) in tri");
+  if (err == PM_ERR_TIMEOUT) set_last_error("the gradient's scan gave up waiting");
+  return err;
 }
 
 }  // namespace pm

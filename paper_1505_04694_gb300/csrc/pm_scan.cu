@@ -202,13 +202,14 @@ int scan_tiles(int n) { return (n + SCAN_TILE - 1) / SCAN_TILE; }
 namespace {
 
 template <class Input>
-void scan_run(Input input, int* out, int n, ScanWork& w, DevStatus* st, cudaStream_t s) {
+void scan_run(Input input, int* out, int n, ScanWork& w, DevStatus* st, cudaStream_t s,
+              bool cleared = false) {
   if (n <= 0) {
     cudaMemsetAsync(out, 0, sizeof(int), s);
     return;
   }
   int tiles = scan_tiles(n);
-  cudaMemsetAsync(w.ticket, 0, sizeof(int), s);
+  if (!cleared) cudaMemsetAsync(w.ticket, 0, sizeof(int), s);
   w.epoch = (w.epoch + 1) & 0x3FFFFFFFu;
   if (w.epoch == 0) w.epoch = 1;
   PM_LAUNCH(k_scan<Input>, tiles, SCAN_THREADS, 0, s, input, out, n, w.state, w.ticket, w.epoch,
@@ -222,6 +223,12 @@ void scan_run(Input input, int* out, int n, ScanWork& w, DevStatus* st, cudaStre
 // apart); `ticket` is reset here.
 void scan_exclusive(const int* in, int* out, int n, ScanWork& w, DevStatus* st, cudaStream_t s) {
   scan_run(IntInput{in}, out, n, w, st, s);
+}
+
+// The same with a ticket (and state words) the caller has just cleared.
+void scan_exclusive_cleared(const int* in, int* out, int n, ScanWork& w, DevStatus* st,
+                            cudaStream_t s) {
+  scan_run(IntInput{in}, out, n, w, st, s, true);
 }
 
 // The same over the alive flags of the used vertex (element) slots [0, n).
