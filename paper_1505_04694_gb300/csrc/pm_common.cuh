@@ -342,9 +342,8 @@ struct Row16 {
     const int4* r4 = reinterpret_cast<const int4*>(row);
 #pragma unroll
     for (int q = 0; q < kRowReg / 4; ++q) {
-      int4 x = make_int4(kRowPad, kRowPad, kRowPad, kRowPad);
-      if (4 * q < len) x = r4[q];
-      a[4 * q] = x.x;
+      const int4 x = r4[q];  // (a row holds 16 entries at least: no wait for len)
+      a[4 * q] = 4 * q < len ? x.x : kRowPad;
       a[4 * q + 1] = 4 * q + 1 < len ? x.y : kRowPad;
       a[4 * q + 2] = 4 * q + 2 < len ? x.z : kRowPad;
       a[4 * q + 3] = 4 * q + 3 < len ? x.w : kRowPad;

@@ -33,10 +33,12 @@ struct MeshCtx {
 };
 
 __device__ __forceinline__ MeshCtx ctx_of(const Store& S, int slot) {
-  MeshCtx c;
-  c.mi = mesh_of_vslot(S, slot);
-  c.vb = S.tab.vbase[c.mi];
-  c.eb = S.tab.ebase[c.mi];
+  MeshCtx c{0, 0, 0};  // the regions of a single mesh start at 0: no loads
+  if (S.nmesh > 1) {
+    c.mi = mesh_of_vslot(S, slot);
+    c.vb = S.tab.vbase[c.mi];
+    c.eb = S.tab.ebase[c.mi];
+  }
   return c;
 }
 
@@ -50,6 +52,13 @@ __device__ __forceinline__ int grank(bool il) {
   return il ? threadIdx.x * gridDim.x + blockIdx.x : blockIdx.x * blockDim.x + threadIdx.x;
 }
 __device__ __forceinline__ int gsize() { return gridDim.x * blockDim.x; }
+
+// The list entry of a thread's first turn, loaded together with the list's
+// length instead of after it (any position below the list's capacity may be
+// read; the value is used only below the length).
+__device__ __forceinline__ int first_entry(const int* list, int i, int cap) {
+  return i < cap ? list[i] : 0;
+}
 
 __device__ __forceinline__ const int* nn_row(const Store& S, int slot) {
   return S.NN + (size_t)slot * S.W;
@@ -121,15 +130,17 @@ __device__ __forceinline__ void add_work(unsigned long long* work, unsigned ops)
 // qK of every listed element slot, one element per thread.
 __device__ __forceinline__ void elem_quality_phase(const Store& S, const int* list, const int* np,
                                                    unsigned long long* work, bool il = false) {
+  // in the persistent rounds from the last warp of every block backwards: the
+  // commit that shares the phase fills the blocks from their first warp
+  const int r0 = il ? (blockDim.x - 1 - threadIdx.x) * gridDim.x + blockIdx.x : grank(false);
+  const int first = first_entry(list, r0, S.eslots);
   const int n = *np;
   for (int i0 = 0; i0 < n; i0 += gsize()) {
-    // in the persistent rounds from the last warp of every block backwards: the
-    // commit that shares the phase fills the blocks from their first warp
-    int i = i0 + (il ? (blockDim.x - 1 - threadIdx.x) * gridDim.x + blockIdx.x : grank(false));
+    const int i = i0 + r0;
     unsigned ops = 0;
     if (i < n) {
-      int slot = list[i];
-      int vb = S.tab.vbase[mesh_of_eslot(S, slot)];
+      const int slot = i0 == 0 ? first : list[i];
+      const int vb = S.nmesh > 1 ? S.tab.vbase[mesh_of_eslot(S, slot)] : 0;
       int4 e = S.EN[slot];
       S.qK[slot] = quality_c(e.x, e.y, e.z, load_vd(S, vb + e.x), load_vd(S, vb + e.y),
                              load_vd(S, vb + e.z));
@@ -931,6 +942,7 @@ __device__ __forceinline__ void coarsen_eval_phase(Store S, const int* D, const 
                                                    int* nC, int* cmark, int tag, int pass0,
                                                    unsigned long long* work, bool il = false) {
   const Tile t = tile_of();
+  const int first = first_entry(D, trank(il), S.vslots);
   const int n = *nDp;
   unsigned ops = 0;
   for (int i0 = 0; i0 < n; i0 += tcount()) {
@@ -938,7 +950,7 @@ __device__ __forceinline__ void coarsen_eval_phase(Store S, const int* D, const 
     int v = 0;
     bool found = false;
     if (i < n) {
-      v = D[i];
+      v = i0 == 0 ? first : D[i];
       MeshCtx c = ctx_of(S, v);
       const int et = __shfl_sync(t.mask, S.evc[v], 0, TW);
       if (unchanged(S, v, c.vb, et, pass0)) {
@@ -985,6 +997,7 @@ __device__ __forceinline__ void coarsen_select_apply_phase(Store S, const int* C
                                                            int* dmark,
                                                            int* Q, int* nQ,
                                                            bool il = false) {
+  const int first = first_entry(C, grank(il), S.vslots);
   const int n = *nCp;
   for (int i0 = 0; i0 < n; i0 += gsize()) {
     int i = i0 + grank(il);
@@ -994,7 +1007,7 @@ __device__ __forceinline__ void coarsen_select_apply_phase(Store S, const int* C
     const int* ne = nullptr;
     RowMask qbits, fa, fd;
     if (i < n) {
-      v = C[i];
+      v = i0 == 0 ? first : C[i];
       win = local_max(S, v, cmark, tag);
       if (win) smark[v] = tag;
       else lose = stamp_first(dmark, v, tag);
@@ -1062,13 +1075,15 @@ __global__ void k_coarsen_select_apply(Store S, const int* C, const int* nCp, co
 // registers, edited in place (a row of dependent local-memory accesses per
 // edit otherwise).  False, with nothing written, when a row grows past 16.
 __device__ __forceinline__ bool coarsen_commit_short(const Store& S, int u, MeshCtx c, int lu,
-                                                     int nnl, int nel, const int* target,
-                                                     const int* smark, int tag) {
+                                                     const int* target, const int* smark,
+                                                     int tag) {
   int* nn = S.NN + (size_t)u * S.W;
   int* ne = S.NE + (size_t)u * S.W;
+  const int nnl = S.NNlen[u], nel = S.NElen[u];
   Row16 R, Q;
   R.load(nn, nnl);
   Q.load(ne, nel);
+  if (nnl > kRowReg || nel > kRowReg) return false;
   unsigned dead = 0, sel = 0;
 #pragma unroll
   for (int k = 0; k < kRowReg; ++k)
@@ -1118,18 +1133,17 @@ __device__ __forceinline__ bool coarsen_commit_short(const Store& S, int u, Mesh
 __device__ __forceinline__ void coarsen_commit_phase(Store S, const int* A, const int* nAp,
                                                      const int* target, const int* smark, int tag,
                                                      DevStatus* st, bool il = false) {
+  const int first = first_entry(A, grank(il), S.vslots);
   const int n = *nAp;
   for (int i = grank(il); i < n; i += gsize()) {
-    int u = A[i];
+    const int u = i < gsize() ? first : A[i];
     S.touch[u] = tag + 1;
     MeshCtx c = ctx_of(S, u);
     int lu = u - c.vb;
     const int* nn = nn_row(S, u);
     const int* ne = ne_row(S, u);
+    if (coarsen_commit_short(S, u, c, lu, target, smark, tag)) continue;
     int nnl = S.NNlen[u], nel = S.NElen[u];
-    if (nnl <= kRowReg && nel <= kRowReg &&
-        coarsen_commit_short(S, u, c, lu, nnl, nel, target, smark, tag))
-      continue;
     int nb[MAXW], eb[MAXW];
     int nn2 = 0, ne2 = 0;
     bool ok = true;
@@ -1531,9 +1545,9 @@ __device__ __forceinline__ void flip_run(const Store& S, FlipQueue& Q, int cnt, 
 }
 
 __device__ __forceinline__ void swap_edge_phase(Store S, const int2* items, const int* nIp,
-                                                double* gains, int tag, unsigned long long* work,
-                                                bool il = false) {
-  const int n = *nIp;
+                                                int icap, double* gains, int tag,
+                                                unsigned long long* work, bool il = false) {
+  const int n = min(*nIp, icap);
   const int lane = threadIdx.x & 31;
   FlipQueue Q = flip_queue();
   unsigned ops = 0;
@@ -1576,9 +1590,9 @@ __device__ __forceinline__ void swap_edge_phase(Store S, const int2* items, cons
   add_work(work, ops);
 }
 
-__global__ void k_swap_edge(Store S, const int2* items, const int* nIp, double* gains, int tag,
-                            unsigned long long* work) {
-  swap_edge_phase(S, items, nIp, gains, tag, work);
+__global__ void k_swap_edge(Store S, const int2* items, const int* nIp, int icap, double* gains,
+                            int tag, unsigned long long* work) {
+  swap_edge_phase(S, items, nIp, icap, gains, tag, work);
 }
 
 // Pass 3 (per evaluated vertex): largest strictly positive gain, ties to the
@@ -1717,30 +1731,36 @@ __device__ __forceinline__ void swap_scan_eval_phase(Store S, const int* D, cons
   const Tile t = tile_of();
   const int lane = threadIdx.x & 31;
   FlipQueue Q = flip_queue();
+  const int first = first_entry(D, trank(true), S.vslots);
   const int n = *nDp;
   unsigned ops = 0;
   for (int i0 = 0; i0 < n; i0 += tcount()) {
     const int i = i0 + trank(true);
-    int v = 0, lv = 0, nel = 0;
+    int v = 0, lv = 0, nel = 0, K0 = 0;
     bool cand = false, eval = false;
     MeshCtx c{0, 0, 0};
     const int* ne = nullptr;
     double qt = 0.0;
     if (i < n) {
-      v = D[i];
+      v = i0 == 0 ? first : D[i];
       c = ctx_of(S, v);
-      const int et = __shfl_sync(t.mask, S.evs[v], 0, TW);
-      if (unchanged(S, v, c.vb, et, pass0)) {
-        cand = opA[v].x >= 0;
+      ne = ne_row(S, v);
+      // everything the vertex itself holds, in flight together
+      const int evs = S.evs[v], tch = S.touch[v], ntch = S.ntouch[v], old = opA[v].x;
+      const int len = S.NElen[v];
+      K0 = ne[t.tl];
+      const bool alive = (S.vflag[v] & VF_ALIVE) != 0;
+      const int et = __shfl_sync(t.mask, evs, 0, TW);
+      if (et > pass0 && tch <= et && ntch <= et) {  // see unchanged()
+        cand = old >= 0;
         if (cand && t.tl == 0) {
           cmark[v] = tag;
           S.tab.had[c.mi] = 1;
         }
-      } else if (S.vflag[v] & VF_ALIVE) {
+      } else if (alive) {
         eval = true;
         lv = v - c.vb;
-        ne = ne_row(S, v);
-        nel = S.NElen[v];
+        nel = len;
         qt = S.tab.q_thresh[c.mi];
       }
     }
@@ -1754,7 +1774,7 @@ __device__ __forceinline__ void swap_scan_eval_phase(Store S, const int* D, cons
       int K1 = -1, w = -1, cc = -2;
       double q1 = 0.0;
       if (k < nel) {
-        K1 = ne[k];
+        K1 = base == 0 ? K0 : ne[k];
         const int4 e = S.EN[c.eb + K1];
         q1 = S.qK[c.eb + K1];
         w = (e.x == lv) ? e.y : (e.y == lv) ? e.z : e.x;   // after v
@@ -1861,6 +1881,7 @@ __device__ __forceinline__ void swap_select_apply_phase(Store S, const int* C, c
                                                         int* nA, int* amark, int* Dn, int* nDn,
                                                         int* dmark, int* Q, int* nQ,
                                                         bool il = false) {
+  const int first = first_entry(C, grank(il), S.vslots);
   const int n = *nCp;
   for (int i0 = 0; i0 < n; i0 += gsize()) {
     int i = i0 + grank(il);
@@ -1869,7 +1890,7 @@ __device__ __forceinline__ void swap_select_apply_phase(Store S, const int* C, c
     int t[4] = {0, 0, 0, 0};
     bool fa[4] = {false, false, false, false}, fd[4] = {false, false, false, false};
     if (i < n) {
-      v = C[i];
+      v = i0 == 0 ? first : C[i];
       const int4 op = opA[v];
       const int K2 = opK2[v];
       win = local_max(S, v, cmark, tag);
@@ -1934,14 +1955,16 @@ __global__ void k_swap_select_apply(Store S, const int* C, const int* nCp, const
 // The commit below for rows of at most 16 entries that stay so (see
 // coarsen_commit_short).
 __device__ __forceinline__ bool swap_commit_short(const Store& S, int u, MeshCtx c, int lu,
-                                                  int nnl, int nel, const int4* opA,
-                                                  const int* opK2, const int* smark, int tag) {
+                                                  const int4* opA, const int* opK2,
+                                                  const int* smark, int tag) {
   int* nn = S.NN + (size_t)u * S.W;
   int* ne = S.NE + (size_t)u * S.W;
+  const int nnl = S.NNlen[u], nel = S.NElen[u], own = smark[u];
   Row16 R, Q;
   R.load(nn, nnl);
   Q.load(ne, nel);
-  unsigned sel = smark[u] == tag ? 1u << kRowReg : 0u;
+  if (nnl > kRowReg || nel > kRowReg) return false;
+  unsigned sel = own == tag ? 1u << kRowReg : 0u;
 #pragma unroll
   for (int k = 0; k < kRowReg; ++k)
     if (k < nnl && smark[c.vb + R.a[k]] == tag) sel |= 1u << k;
@@ -1980,18 +2003,17 @@ __device__ __forceinline__ void swap_commit_phase(Store S, const int* A, const i
                                                   const int4* opA, const int* opK2,
                                                   const int* smark, int tag, DevStatus* st,
                                                   bool il = false) {
+  const int first = first_entry(A, grank(il), S.vslots);
   const int n = *nAp;
   for (int i = grank(il); i < n; i += gsize()) {
-    int u = A[i];
+    const int u = i < gsize() ? first : A[i];
     S.touch[u] = tag + 1;
     MeshCtx c = ctx_of(S, u);
     int lu = u - c.vb;
     int* nn = S.NN + (size_t)u * S.W;
     int* ne = S.NE + (size_t)u * S.W;
+    if (swap_commit_short(S, u, c, lu, opA, opK2, smark, tag)) continue;
     int nnl = S.NNlen[u], nel = S.NElen[u];
-    if (nnl <= kRowReg && nel <= kRowReg &&
-        swap_commit_short(S, u, c, lu, nnl, nel, opA, opK2, smark, tag))
-      continue;
     int nb[MAXW], eb[MAXW];
     load_row(nn, nnl, nb);
     load_row(ne, nel, eb);
@@ -2526,13 +2548,14 @@ __device__ __forceinline__ void smooth_select_apply_phase(Store S, const int* C,
                                                           const double* qball, int* P, int* nP,
                                                           int* pmark, int ptag, int stamp,
                                                           bool il = false) {
+  const int first = first_entry(C, grank(il), S.vslots);
   const int n = *nCp;
   for (int i0 = 0; i0 < n; i0 += gsize()) {
     int i = i0 + grank(il);
     bool win = false, lose = false;
     int v = 0;
     if (i < n) {
-      v = C[i];
+      v = i0 == 0 ? first : C[i];
       win = local_max(S, v, cmark, tag);
       if (win) smark[v] = tag;
       else lose = stamp_first(dmark, v, tag);
@@ -2980,11 +3003,15 @@ __device__ __forceinline__ int ld_volatile(const int* p) { return *(volatile con
 
 // Grid-wide barrier on a counter of arrivals that only grows (zeroed before
 // the launch): the k-th barrier waits for k * gridDim.x arrivals.  Thread 0
-// of each block publishes the block's writes (__syncthreads, then a
-// device-wide fence), arrives, waits, and fences again before the block
-// reads what the other blocks wrote.  Returns false (the caller leaves the
-// kernel) when the wait ran out (PM_ERR_TIMEOUT is recorded) or when any
-// phase recorded an error.
+// of each block arrives with a release after the block's __syncthreads (so
+// every write of the block is published with it) and waits with acquire loads;
+// nothing waits for the arrival's own round trip, and the error word travels
+// with the waiting loads.  Returns false (the caller leaves the kernel) when the
+// wait ran out (PM_ERR_TIMEOUT is recorded) or when an error had been recorded.
+// An error recorded in the phase just left may be seen only at the next barrier
+// (a block that leaves at once does not arrive there, and the others find the
+// error while they wait), so a phase bounds its own reads by what the one before
+// may have overrun.
 __device__ bool grid_barrier(unsigned* bar, unsigned& target, DevStatus* st,
                              unsigned long long limit_ns = kBarrierNs) {
   __shared__ int s_ok;
@@ -2992,25 +3019,29 @@ __device__ bool grid_barrier(unsigned* bar, unsigned& target, DevStatus* st,
   __syncthreads();
   if (threadIdx.x == 0) {
     int ok = 1;
-    __threadfence();
-    const unsigned arrived = atomicAdd(bar, 1u) + 1u;
-    if ((int)(arrived - target) < 0) {
-      const volatile unsigned* vb = bar;
-      const unsigned long long t0 = global_ns();
-      while ((int)(*vb - target) < 0) {
-        if (ld_volatile(&st->err) != 0) {
-          ok = 0;
-          break;
-        }
-        if (global_ns() - t0 > limit_ns) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    unsigned long long t0 = 0;
+    for (unsigned spin = 1;; ++spin) {
+      int err;
+      unsigned arrived;
+      asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(err) : "l"(&st->err) : "memory");
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(arrived) : "l"(bar) : "memory");
+      if (err != 0) {
+        ok = 0;
+        break;
+      }
+      if ((int)(arrived - target) >= 0) break;
+      if ((spin & 255u) == 0) {
+        const unsigned long long now = global_ns();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > limit_ns) {
           set_err(st, PM_ERR_TIMEOUT);
           ok = 0;
           break;
         }
       }
     }
-    __threadfence();
-    s_ok = ok && ld_volatile(&st->err) == 0;
+    s_ok = ok;
   }
   __syncthreads();
   return s_ok != 0;
@@ -3097,7 +3128,7 @@ __device__ __forceinline__ void topo_rounds(const RoundArgs& a) {
                       w.E, cnt + CN_E, w.items, cnt + CN_I, a.icap, w.gains, a.st, true);
       if (!grid_barrier(a.bar, target, a.st)) return;
       if (blockIdx.x == 0 && threadIdx.x == 0) *cand_count(cnt, r + 1) = 0;
-      swap_edge_phase(a.S, w.items, cnt + CN_I, w.gains, tag, a.work, true);
+      swap_edge_phase(a.S, w.items, cnt + CN_I, a.icap, w.gains, tag, a.work, true);
       if (!grid_barrier(a.bar, target, a.st)) return;
       swap_pick_phase(a.S, w.E, cnt + CN_E, w.gains, w.opA, w.opK2, w.C, nC, w.cmark, tag, true);
       if (!grid_barrier(a.bar, target, a.st)) return;
@@ -3512,7 +3543,7 @@ int op_swap(MeshSet& m, int max_rounds) {
               w.C, w.counts + CN_C, w.cmark, tag, pass0, w.E, w.counts + CN_E, w.items,
               w.counts + CN_I, icap, w.gains, m.st);
     PM_LAUNCH(k_swap_edge, grid_tuned(m, 6LL * m.S.vslots, bs, bps), bs, 0, m.stream, m.S, w.items,
-              w.counts + CN_I, w.gains, tag, prof_work("k_swap_edge"));
+              w.counts + CN_I, icap, w.gains, tag, prof_work("k_swap_edge"));
     PM_LAUNCH(k_swap_pick, gv, bs, 0, m.stream, m.S, w.E, w.counts + CN_E, w.gains, w.opA,
               w.opK2, w.C, w.counts + CN_C, w.cmark, tag);
     zero_counts(m, CN_CL, 1);
