@@ -72,12 +72,18 @@ struct Work {
 enum CountIdx {
   CN_D0 = 0, CN_C = 1, CN_S = 2, CN_A = 3, CN_E = 4, CN_I = 5, CN_I2 = 6, CN_D1 = 7,
   CN_P = 8, CN_EL = 9, CN_CL = 10, CN_DONE = 11,
-  CN_RES = 12,  // persistent rounds: rounds run, list index after, pass complete (3)
-  CN_BAR = 15,  // persistent rounds: grid barrier arrivals
-  CN_C2 = 16,   // persistent rounds: candidates of odd rounds
-  CN_RENUM = 17,  // renumbering: 1 when some mesh's compaction is not the identity
-  CN_NUM = 18
+  CN_RES = 12,  // persistent rounds: rounds run, list index after, pass complete; smoothing:
+                // see SmoothRes (8)
+  CN_BAR = 20,  // persistent rounds: grid barrier arrivals
+  CN_C2 = 21,   // persistent rounds: candidates of odd rounds
+  CN_RENUM = 22,  // renumbering: 1 when some mesh's compaction is not the identity
+  CN_NUM = 23
 };
+// What a persistent smoothing launch leaves at CN_RES: rounds with candidates,
+// sweeps finished, 1 when the sweeps are over, 1 when the current sweep has
+// moved a vertex, the buffers holding the current, the next and the pending list
+// (0, 1: D, 2: P; two bits each), tags used, the stamp of the pending list.
+enum SmoothRes { SR_ROUNDS = 0, SR_SWEEPS, SR_OVER, SR_MOVED, SR_PERM, SR_TAGS, SR_PTAG };
 constexpr int cn_list(int i) { return i == 0 ? CN_D0 : CN_D1; }
 
 // Everything the library keeps on the device for a set of meshes.

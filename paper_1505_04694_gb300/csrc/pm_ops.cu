@@ -2509,6 +2509,7 @@ __device__ __forceinline__ void smooth_apply_one(const Store& S, bool ok, int v,
   {
     int mi = 0, vb = 0, nnl = 0;
     const int* nn = nullptr;
+    RowMask take;
     if (ok) {
       MeshCtx c = ctx_of(S, v);
       mi = c.mi;
@@ -2522,19 +2523,22 @@ __device__ __forceinline__ void smooth_apply_one(const Store& S, bool ok, int v,
       S.touch[v] = stamp;
       const int* ne = ne_row(S, v);
       int nel = S.NElen[v];
+#pragma unroll 8
       for (int k = 0; k < nel; ++k) S.qK[c.eb + ne[k]] = qball[(size_t)v * S.W + k];
       nn = nn_row(S, v);
       nnl = S.NNlen[v];
       stamp_neighbours(S, nn, nnl, vb, stamp);
+      // (a stamp on a vertex that is not taken is harmless: only interior
+      // neighbours look at it)
+#pragma unroll 8
+      for (int k = 0; k < nnl; ++k) {
+        const int s = vb + nn[k];
+        const uint8_t f = S.vflag[s];
+        const bool first = stamp_first(pmark, s, ptag);
+        if (first && (f & VF_ALIVE) && !(f & VF_BND)) take.set(k);
+      }
     }
     count_op(S, ok, mi);
-    RowMask take;
-#pragma unroll 4
-    for (int k = 0; k < nnl; ++k) {
-      int s = vb + nn[k];
-      uint8_t f = S.vflag[s];
-      if ((f & VF_ALIVE) && !(f & VF_BND) && stamp_first(pmark, s, ptag)) take.set(k);
-    }
     int pp = warp_reserve(take.count(), nP);
     write_row_bits(take, nn, vb, P, pp);
   }
@@ -3067,6 +3071,8 @@ struct RoundArgs {
   int limit;           // leave when the next list holds more entries
   int icap;            // flips: capacity of the item list
   int ptag;            // smoothing: stamp of the next sweep's list
+  int sweeps;          // smoothing: sweeps left, the current one included
+  int moved;           // smoothing: the current sweep has moved a vertex
   int fuse;            // flips, smoothing: lists up to this size take the one-phase evaluation
   unsigned long long* work;  // counted FP64 work (measurement) or null
 };
@@ -3174,45 +3180,59 @@ __global__ void __launch_bounds__(256) k_coarsen_rounds(RoundArgs a) { topo_roun
 
 __global__ void __launch_bounds__(256) k_swap_rounds(RoundArgs a) { topo_rounds<true>(a); }
 
-// Rounds of smoothing moves.  A round whose list fits one pass of the grid's
+// Sweeps of smoothing rounds.  A round whose list fits one pass of the grid's
 // tiles: [scan + evaluate] B1 [select + apply] B2; a longer one: [scan] B1
 // [evaluate] B1' [select + apply] B2 (its tiles then go to the vertices that
-// need an evaluation only).  Block 0 clears, before B1 of round r: the list
-// round r fills (last read by round r - 1's scan and by its decision, both
-// before B1 of round r); after B1: the candidate slot of round r + 1 (last
-// read after B2 of round r - 1); after B1': E (read by the evaluation before
-// B1').  The round counters advance after B2 from the flag set of the round's
-// parity, so that round r + 1's evaluation can set the other set meanwhile.
+// need an evaluation only).  A sweep ends with a round that finds no candidate;
+// its pending list then becomes the current one and the next sweep starts in
+// the same launch (ten sweeps used to be ten launches and read-backs, most of
+// them for a handful of vertices).  The three lists trade places by index, each
+// with its own counter.  Block 0 clears, before B1 of round r: the list round
+// r fills and, in a sweep's first round, its pending list (both last read by a
+// scan and a decision before the last barrier); after B1: the candidate slot of
+// round r + 1 (last read after B2 of round r - 1); after B1': E (read by the
+// evaluation before B1').  The round counters advance after B2 from the flag
+// set of the round's parity, so that round r + 1's evaluation can set the other
+// set meanwhile.  The launch returns when the sweeps are over, after
+// `max_rounds` rounds with candidates, or when the next list outgrows `limit`;
+// the lists' counts are then put where the host expects them.
 __global__ void __launch_bounds__(256) k_smooth_rounds(RoundArgs a) {
   const Work& w = a.w;
   int* cnt = w.counts;
   unsigned target = 0;
-  int cur = a.cur, r = 0;
-  bool complete = false;
+  int cur = 0, nxt = 1, pen = 2;
+  auto list = [&](int b) { return b == 0 ? w.D[0] : (b == 1 ? w.D[1] : w.P); };
+  auto count = [&](int b) { return cnt + (b == 2 ? CN_P : cn_list(b)); };
+  int r = 0, rounds = 0, sweeps = 0, tag = a.tag0 - 2, ptag = a.ptag;
+  bool moved = a.moved != 0, over = false, fresh = false;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *cand_count(cnt, 0) = 0;
     cnt[CN_E] = 0;
   }
   if (!grid_barrier(a.bar, target, a.st)) return;
-  // a first list longer than the limit is left to the one-kernel-per-phase rounds
-  const bool too_long = ld_volatile(cnt + cn_list(cur)) > a.limit;
+  // a list longer than the limit is left to the one-kernel-per-phase rounds
+  int n = ld_volatile(count(cur));
   const int tiles = gridDim.x * (blockDim.x / TW);
-  while (!too_long && r < a.max_rounds) {
-    const int tag = a.tag0 + 2 * r, nxt = 1 - cur;
+  while (!over && n <= a.limit && rounds < a.max_rounds) {
+    tag += 2;
     int* nC = cand_count(cnt, r);
     Store S = a.S;
     S.tab.had = a.S.tab.had + (r & 1) * S.nmesh;
     // the list is complete since B2 of the last round: every block decides alike
-    const bool fused = ld_volatile(cnt + cn_list(cur)) <= min(a.fuse, tiles);
-    if (blockIdx.x == 0 && threadIdx.x == 0) cnt[cn_list(nxt)] = 0;
+    const bool fused = n <= min(a.fuse, tiles);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      *count(nxt) = 0;
+      if (fresh) *count(pen) = 0;
+    }
+    fresh = false;
     if (fused) {
-      smooth_scan_eval_phase(S, w.D[cur], cnt + cn_list(cur), w.mvxy, w.mvM, w.gains, w.C, nC,
-                             w.cmark, tag, a.pass0, a.work);
+      smooth_scan_eval_phase(S, list(cur), count(cur), w.mvxy, w.mvM, w.gains, w.C, nC, w.cmark,
+                             tag, a.pass0, a.work);
       if (!grid_barrier(a.bar, target, a.st)) return;
       if (blockIdx.x == 0 && threadIdx.x == 0) *cand_count(cnt, r + 1) = 0;
     } else {
-      smooth_scan_phase(S, w.D[cur], cnt + cn_list(cur), w.mvM, w.C, nC, w.cmark, tag, a.pass0,
-                        w.E, cnt + CN_E, true);
+      smooth_scan_phase(S, list(cur), count(cur), w.mvM, w.C, nC, w.cmark, tag, a.pass0, w.E,
+                        cnt + CN_E, true);
       if (!grid_barrier(a.bar, target, a.st)) return;
       if (blockIdx.x == 0 && threadIdx.x == 0) *cand_count(cnt, r + 1) = 0;
       smooth_eval_phase(S, w.E, cnt + CN_E, w.mvxy, w.mvM, w.gains, w.C, nC, w.cmark, tag, a.work,
@@ -3220,23 +3240,51 @@ __global__ void __launch_bounds__(256) k_smooth_rounds(RoundArgs a) {
       if (!grid_barrier(a.bar, target, a.st)) return;
       if (blockIdx.x == 0 && threadIdx.x == 0) cnt[CN_E] = 0;
     }
-    smooth_select_apply_phase(S, w.C, nC, w.cmark, w.smark, tag, w.D[nxt], cnt + cn_list(nxt),
-                              w.dmark, w.mvxy, w.mvM, w.gains, w.P, cnt + CN_P, w.pmark, a.ptag,
-                              tag + 1, true);
+    smooth_select_apply_phase(S, w.C, nC, w.cmark, w.smark, tag, list(nxt), count(nxt), w.dmark,
+                              w.mvxy, w.mvM, w.gains, list(pen), count(pen), w.pmark, ptag, tag + 1,
+                              true);
     if (!grid_barrier(a.bar, target, a.st)) return;
-    const int nc = ld_volatile(nC), nd = ld_volatile(cnt + cn_list(nxt));
+    const int nc = ld_volatile(nC), nd = ld_volatile(count(nxt)), np = ld_volatile(count(pen));
     advance_rounds(S);
     ++r;
-    if (nc == 0) {
-      complete = true;
-      break;
+    if (nc > 0) {
+      ++rounds;
+      moved = true;
+      const int t = cur;
+      cur = nxt;
+      nxt = t;
+      n = nd;
+    } else {
+      ++sweeps;
+      over = !moved || sweeps == a.sweeps;
+      if (!over) {
+        const int t = cur;
+        cur = pen;
+        pen = t;
+        n = np;
+        tag += 2;
+        ptag = tag;
+        moved = false;
+        fresh = true;
+      }
     }
-    cur = nxt;
-    if (nd > a.limit) break;
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0 && r > 0)
-    cnt[CN_C] = ld_volatile(cand_count(cnt, r - 1));
-  finish_rounds(a, r, cur, complete);
+  // every block has left the counters: the lists go to their places (D[0]
+  // current, D[1] next, P pending)
+  const int nn = ld_volatile(count(nxt)), np = fresh ? 0 : ld_volatile(count(pen));
+  if (!grid_barrier(a.bar, target, a.st)) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    cnt[CN_D0] = n;
+    cnt[CN_D1] = nn;
+    cnt[CN_P] = np;
+    a.res[SR_ROUNDS] = rounds;
+    a.res[SR_SWEEPS] = sweeps;
+    a.res[SR_OVER] = over ? 1 : 0;
+    a.res[SR_MOVED] = moved ? 1 : 0;
+    a.res[SR_PERM] = cur | (nxt << 2) | (pen << 4);
+    a.res[SR_TAGS] = (tag + 2 - a.tag0) / 2;
+    a.res[SR_PTAG] = ptag;
+  }
 }
 
 // ---- host helpers --------------------------------------------------------------
@@ -3368,6 +3416,8 @@ RoundArgs round_args(MeshSet& m, int cur, int pass0, long long max_rounds) {
   a.limit = tuning().rounds_limit[0];
   a.icap = 0;
   a.ptag = 0;
+  a.sweeps = 0;
+  a.moved = 0;
   a.fuse = 0;
   a.work = nullptr;
   return a;
@@ -3398,6 +3448,10 @@ int run_rounds(MeshSet& m, int which, const void* kernel, const char* name, Roun
   }
   out.io = read_round(m);
   if (out.io.err) return out.io.err;
+  if (which == 2) {
+    m.tag += 2 * m.hcounts[CN_RES + SR_TAGS];
+    return PM_OK;
+  }
   out.rounds = m.hcounts[CN_RES];
   out.cur = m.hcounts[CN_RES + 1];
   out.complete = m.hcounts[CN_RES + 2];
@@ -3679,52 +3733,72 @@ int op_smooth(MeshSet& m, int max_sweeps, int max_rounds) {
   PM_LAUNCH(k_init_list, gv, bs, 0, m.stream, m.S, 1, w.D[0], w.counts + CN_D0, nullptr, 0);
   int nlist = 0;  // unknown at first (see op_coarsen)
   long long nr = 0;
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    int ptag = (m.tag += 2);  // stamp of the next sweep's pending list
-    zero_counts(m, CN_P, 1);
-    int cur = 0;
-    bool moved = false;
-    while (max_rounds == 0 || nr < max_rounds) {
-      if (persist && nlist >= 0 && nlist <= rlimit) {
-        RoundArgs a = round_args(m, cur, pass0, max_rounds == 0 ? (1LL << 30) : max_rounds - nr);
-        a.ptag = ptag;
-        a.limit = rlimit;
-        a.fuse = tu.fuse_limit[1];
-        RoundsOut o;
-        int err = run_rounds(m, 2, (const void*)k_smooth_rounds, "k_smooth_rounds", a, o);
-        if (err) return err;
-        nr += o.rounds - o.complete;
-        if (o.rounds - o.complete > 0) moved = true;
-        cur = o.cur;
-        nlist = m.hcounts[cn_list(cur)];
-        if (o.complete) break;
-        continue;
+  int cur = 0, ptag = 0;
+  bool moved = false, fresh = true;
+  for (int sweep = 0; sweep < max_sweeps && (max_rounds == 0 || nr < max_rounds);) {
+    if (fresh) {
+      ptag = (m.tag += 2);  // stamp of the next sweep's pending list
+      if (sweep > 0) zero_counts(m, CN_P, 1);
+      moved = fresh = false;
+    }
+    if (persist && nlist >= 0 && nlist <= rlimit) {
+      if (cur == 1) {  // the launch starts from D[0]
+        std::swap(w.D[0], w.D[1]);
+        cudaMemcpyAsync(w.counts + CN_D0, w.counts + CN_D1, sizeof(int), cudaMemcpyDeviceToDevice,
+                        m.stream);
+        cur = 0;
       }
-      int tag = (m.tag += 2);
-      int nxt = 1 - cur;
-      zero_round(m, nxt);
-      PM_LAUNCH(k_smooth_scan, gv, bs, 0, m.stream, m.S, w.D[cur], w.counts + cn_list(cur),
-                w.mvM, w.C, w.counts + CN_C, w.cmark, tag, pass0, w.E, w.counts + CN_E);
-      PM_LAUNCH(k_smooth_eval, gv, bs, 0, m.stream, m.S, w.E, w.counts + CN_E, w.mvxy, w.mvM, w.gains, w.C, w.counts + CN_C, w.cmark, tag,
-                prof_work("k_smooth_eval"));
-      PM_LAUNCH(k_smooth_select_apply, gv, bs, 0, m.stream, m.S, w.C, w.counts + CN_C,
-                w.cmark, w.smark, tag, w.D[nxt], w.counts + cn_list(nxt), w.dmark, w.mvxy, w.mvM,
-                w.gains, w.P, w.counts + CN_P, w.pmark, ptag, tag + 1,
-                (unsigned*)(w.counts + CN_DONE));
-      RoundIO io = read_round(m);
-      if (io.err) return io.err;
-      if (io.nC == 0) break;
+      RoundArgs a = round_args(m, cur, pass0, max_rounds == 0 ? (1LL << 30) : max_rounds - nr);
+      a.ptag = ptag;
+      a.sweeps = max_sweeps - sweep;
+      a.moved = moved ? 1 : 0;
+      a.limit = rlimit;
+      a.fuse = tu.fuse_limit[1];
+      RoundsOut o;
+      int err = run_rounds(m, 2, (const void*)k_smooth_rounds, "k_smooth_rounds", a, o);
+      if (err) return err;
+      const int* res = m.hcounts + CN_RES;
+      nr += res[SR_ROUNDS];
+      sweep += res[SR_SWEEPS];
+      moved = res[SR_MOVED] != 0;
+      ptag = res[SR_PTAG];
+      int* const buf[3] = {w.D[0], w.D[1], w.P};
+      w.D[0] = buf[res[SR_PERM] & 3];
+      w.D[1] = buf[(res[SR_PERM] >> 2) & 3];
+      w.P = buf[(res[SR_PERM] >> 4) & 3];
+      nlist = m.hcounts[CN_D0];
+      if (res[SR_OVER]) break;
+      continue;
+    }
+    int tag = (m.tag += 2);
+    int nxt = 1 - cur;
+    zero_round(m, nxt);
+    PM_LAUNCH(k_smooth_scan, gv, bs, 0, m.stream, m.S, w.D[cur], w.counts + cn_list(cur),
+              w.mvM, w.C, w.counts + CN_C, w.cmark, tag, pass0, w.E, w.counts + CN_E);
+    PM_LAUNCH(k_smooth_eval, gv, bs, 0, m.stream, m.S, w.E, w.counts + CN_E, w.mvxy, w.mvM, w.gains,
+              w.C, w.counts + CN_C, w.cmark, tag, prof_work("k_smooth_eval"));
+    PM_LAUNCH(k_smooth_select_apply, gv, bs, 0, m.stream, m.S, w.C, w.counts + CN_C,
+              w.cmark, w.smark, tag, w.D[nxt], w.counts + cn_list(nxt), w.dmark, w.mvxy, w.mvM,
+              w.gains, w.P, w.counts + CN_P, w.pmark, ptag, tag + 1,
+              (unsigned*)(w.counts + CN_DONE));
+    RoundIO io = read_round(m);
+    if (io.err) return io.err;
+    if (io.nC > 0) {
       ++nr;
       moved = true;
       cur = nxt;
       nlist = m.hcounts[cn_list(cur)];
+      continue;
     }
+    ++sweep;
     if (!moved) break;
     // the next sweep's pending list becomes the current list
     std::swap(w.D[0], w.P);
     cudaMemcpyAsync(w.counts + CN_D0, w.counts + CN_P, sizeof(int), cudaMemcpyDeviceToDevice,
                     m.stream);
+    cur = 0;
     nlist = m.hcounts[CN_P];
+    fresh = true;
   }
   return PM_OK;
 }
