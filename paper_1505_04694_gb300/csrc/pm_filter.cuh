@@ -151,8 +151,10 @@ PM_HD int f_len_cmp(const FLen& l, float lo2, float hi2) {
 // |d ln h / d ln P| <= 5 (between -2 and 1 below the ideal perimeter, between
 // -5 and -2 above), so a relative error rP of P changes it by at most 5 rP to
 // first order (rP <= 0.04 is required, the rest of the series is inside the
-// factor 1.15).  `sign` receives the orientation's sign, 0 when undecided.
-PM_HD float f_quality_up(const VF& a, const VF& b, const VF& c, int& sign) {
+// factor 1.15).  `sign` receives the orientation's sign, 0 when undecided.  `kx`
+// bounds the relative error of one vertex's metric beyond its rounding (see
+// f_metric_at): it adds to that of the mean, and four times to the determinant's.
+PM_HD float f_quality_up(const VF& a, const VF& b, const VF& c, int& sign, float kx = 0.0f) {
   const float E = a.e + (b.e + c.e);
   const float dx0 = f_dx(a, b), dy0 = f_dy(a, b);
   const float dx1 = f_dx(b, c), dy1 = f_dy(b, c);
@@ -163,7 +165,7 @@ PM_HD float f_quality_up(const VF& a, const VF& b, const VF& c, int& sign) {
   const float k00 = ((a.m00 + b.m00) + c.m00) * third;
   const float k01 = ((a.m01 + b.m01) + c.m01) * third;
   const float k11 = ((a.m11 + b.m11) + c.m11) * third;
-  constexpr float ku = 5.0f * kU;
+  const float ku = 5.0f * kU + kx;
   const FLen q0 = f_len2(k00, k01, k11, dx0, dy0, E, ku);
   const FLen q1 = f_len2(k00, k01, k11, dx1, dy1, E, ku);
   const FLen q2 = f_len2(k00, k01, k11, dx2, dy2, E, ku);
@@ -175,9 +177,9 @@ PM_HD float f_quality_up(const VF& a, const VF& b, const VF& c, int& sign) {
   const float rP = eP * rp + 6.0f * kU;
   const float kk = k00 * k11;
   // (perimeters and metrics whose powers would underflow give no bound)
-  const bool fine = rP < 0.04f && q0.err < 0.4f * q0.L2 && q1.err < 0.4f * q1.L2 &&
+  const bool fine = rP < 0.04f && kx < 0.05f && q0.err < 0.4f * q0.L2 && q1.err < 0.4f * q1.L2 &&
                     q2.err < 0.4f * q2.L2 && P > 1e-6f && P < 1e6f && kk > 1e-30f;
-  const float D = (kk - k01 * k01) + 28.0f * kU * kk;
+  const float D = (kk - k01 * k01) + (28.0f * kU + 4.2f * kx) * kk;
   const float up = 0.5f * (d.det + d.err);
   const float area = up < 0.0f ? 0.0f : up;  // a negative quality is below 0 (a NaN stays)
   const float x = P * third;
@@ -185,6 +187,35 @@ PM_HD float f_quality_up(const VF& a, const VF& b, const VF& c, int& sign) {
   const float f = s * (2.0f - s);
   const float q = ((20.784612f * area) * f_sqrt(D)) * ((rp * rp) * ((f * f) * f));
   return fine ? q + (q * (5.75f * rP + 40.0f * kU) + 1e-30f) : nanf("");
+}
+
+// The barycentric metric at point x of element (a, b, d), into the metric part of
+// `out`; returns a bound of its relative error (of m01's bound sqrt(m00 m11) for
+// m01), NaN when the element's area is not known well enough.  A weight s / o
+// has the error (err_s + |s / o| err_o) / o and roundings; by Cauchy the error of
+// m01 stays below the larger of those of m00 and m11.
+PM_HD float f_metric_at(const VF& x, const VF& a, const VF& b, const VF& d, VF& out) {
+  const float E = (x.e + a.e) + (b.e + d.e);
+  const float abx = f_dx(a, b), aby = f_dy(a, b), adx = f_dx(a, d), ady = f_dy(a, d);
+  const float axx = f_dx(a, x), axy = f_dy(a, x);
+  const FDet o = f_det(abx, aby, adx, ady, E);
+  const FDet s0 = f_det(f_dx(x, b), f_dy(x, b), f_dx(x, d), f_dy(x, d), E);
+  const FDet s1 = f_det(axx, axy, adx, ady, E), s2 = f_det(abx, aby, axx, axy, E);
+  const float r = f_rcp(o.det);
+  const float l0 = s0.det * r, l1 = s1.det * r, l2 = s2.det * r;
+  const float e0 = 1.4f * (s0.err + fabsf(l0) * o.err) * r + 6.0f * kU * fabsf(l0);
+  const float e1 = 1.4f * (s1.err + fabsf(l1) * o.err) * r + 6.0f * kU * fabsf(l1);
+  const float e2 = 1.4f * (s2.err + fabsf(l2) * o.err) * r + 6.0f * kU * fabsf(l2);
+  out.m00 = (l0 * a.m00 + l1 * b.m00) + l2 * d.m00;
+  out.m01 = (l0 * a.m01 + l1 * b.m01) + l2 * d.m01;
+  out.m11 = (l0 * a.m11 + l1 * b.m11) + l2 * d.m11;
+  const float w0 = e0 + 5.0f * kU * fabsf(l0), w1 = e1 + 5.0f * kU * fabsf(l1),
+              w2 = e2 + 5.0f * kU * fabsf(l2);
+  const float k0 = ((w0 * a.m00 + w1 * b.m00) + w2 * d.m00) * f_rcp(out.m00);
+  const float k1 = ((w0 * a.m11 + w1 * b.m11) + w2 * d.m11) * f_rcp(out.m11);
+  const bool fine = o.det > 4.0f * o.err && out.m00 > 0.0f && out.m11 > 0.0f;
+  const float k = 1.1f * (k0 > k1 ? k0 : k1);
+  return fine && k0 == k0 && k1 == k1 ? k : nanf("");
 }
 
 }  // namespace pm

@@ -2169,40 +2169,22 @@ __device__ __forceinline__ double4 interpolate_in(const Store& S, int vb, int4 e
                       (l0 * a.m11 + l1 * b.m11) + l2 * d.m11, 0.0);
 }
 
-// Element e of v's ball with v moved to the record `fn`: certainly not
-// counter-clockwise, or its quality certainly below `floor`.
-__device__ __forceinline__ bool move_fails(const Store& S, int vb, int lv, int4 e, const VF& fn,
-                                           float floor) {
+// Upper bound of the quality of element e of v's ball with v at the record `fn`
+// (relative error kx of its metric), -1 when it is certainly not
+// counter-clockwise, NaN when there is no useful bound.
+__device__ __forceinline__ float moved_quality_up(const Store& S, int vb, int lv, int4 e,
+                                                  const VF& fn, float kx) {
   const VF a = e.x == lv ? fn : load_vf(S, vb + e.x), b = e.y == lv ? fn : load_vf(S, vb + e.y),
            c = e.z == lv ? fn : load_vf(S, vb + e.z);
   int sign;
-  const float up = f_quality_up(a, b, c, sign);
-  return sign < 0 || up < floor;
+  const float up = f_quality_up(a, b, c, sign, kx);
+  return sign < 0 ? -1.0f : up;
 }
 
-// First ball element (ascending id) that contains X, with v at its current
-// place: its barycentric metric interpolation.
-__device__ bool tile_interpolate(const Tile& t, const Store& S, MeshCtx c, const int* ne, int nel,
-                                 double X, double Y, double4& Mout) {
-  const VF fx = make_vf_xy(X, Y);
-  for (int base = 0; base < nel; base += TW) {
-    int k = base + t.tl;
-    int4 e = make_int4(0, 0, 0, 0);
-    bool inside = false;
-    if (k < nel) {
-      e = S.EN[c.eb + ne[k]];
-      inside = contains(S, fx, X, Y, c.vb + e.x, c.vb + e.y, c.vb + e.z);
-    }
-    unsigned bal = (__ballot_sync(t.mask, inside) >> t.shift) & 0xFFu;
-    if (bal) {
-      int src = __ffs(bal) - 1;
-      double4 m = make_double4(0.0, 0.0, 0.0, 0.0);
-      if (t.tl == src) m = interpolate_in(S, c.vb, e, X, Y);
-      Mout = make_double4(tshfl(t, m.x, src), tshfl(t, m.y, src), tshfl(t, m.z, src), 0.0);
-      return true;
-    }
-  }
-  return false;
+// The FP32 metric at X in element e into fn, its relative error bound.
+__device__ __forceinline__ float metric_at(const Store& S, int vb, int4 e, const VF& fx, VF& fn) {
+  fn = fx;
+  return f_metric_at(fx, load_vf(S, vb + e.x), load_vf(S, vb + e.y), load_vf(S, vb + e.z), fn);
 }
 
 // Ball with v moved to (X, Y, Mv): every element counter-clockwise, and every
@@ -2239,17 +2221,53 @@ __device__ bool tile_ball_exact(const Tile& t, const Store& S, MeshCtx c, int lv
   return tall(t, ok);
 }
 
-// The same after the FP32 bounds: most moves fail, and they mostly show it.
-__device__ bool tile_ball_after_move(const Tile& t, const Store& S, MeshCtx c, int lv,
-                                     const int* ne, int nel, double X, double Y, double4 Mv,
-                                     double floor, bool strict, double* qout, double* qsum) {
-  const VF fn = make_vf(X, Y, Mv.x, Mv.y, Mv.z);
+// A move of v to X, by v's tile: located in the first ball element (ascending
+// id) that contains X with v at its current place, its metric interpolated there,
+// and the ball checked.  Most moves fail, and the FP32 bounds mostly show it
+// before the metric is interpolated in FP64: a quality certainly below `floor`,
+// or (with qsum) a sum of the upper bounds below `sum_old`.
+__device__ bool tile_try_move(const Tile& t, const Store& S, MeshCtx c, int lv, const int* ne,
+                              int nel, double X, double Y, double floor, bool strict, double* qout,
+                              double* qsum, double sum_old, double4& Mout, unsigned& ops) {
+  const VF fx = make_vf_xy(X, Y);
+  int4 eat = make_int4(0, 0, 0, 0);
+  int src = -1;
+  for (int base = 0; base < nel && src < 0; base += TW) {
+    const int k = base + t.tl;
+    bool inside = false;
+    if (k < nel) {
+      eat = S.EN[c.eb + ne[k]];
+      inside = contains(S, fx, X, Y, c.vb + eat.x, c.vb + eat.y, c.vb + eat.z);
+    }
+    const unsigned bal = (__ballot_sync(t.mask, inside) >> t.shift) & 0xFFu;
+    if (bal) src = __ffs(bal) - 1;
+  }
+  if (src < 0) return false;
+  eat.x = __shfl_sync(t.mask, eat.x, src, TW);
+  eat.y = __shfl_sync(t.mask, eat.y, src, TW);
+  eat.z = __shfl_sync(t.mask, eat.z, src, TW);
+  VF fn;
+  const float kx = metric_at(S, c.vb, eat, fx, fn);
   const float ffloor = __double2float_rd(floor);
   bool fails = false;
-  for (int k = t.tl; k < nel; k += TW)
-    fails |= move_fails(S, c.vb, lv, S.EN[c.eb + ne[k]], fn, ffloor);
+  float up = 0.0f;
+  for (int k = t.tl; k < nel; k += TW) {
+    const float u = moved_quality_up(S, c.vb, lv, S.EN[c.eb + ne[k]], fn, kx);
+    fails |= u < ffloor;
+    up += u;
+  }
   if (!tall(t, !fails)) return false;
-  return tile_ball_exact(t, S, c, lv, ne, nel, X, Y, Mv, floor, strict, qout, qsum);
+  if (qsum) {
+#pragma unroll
+    for (int o = TW / 2; o > 0; o >>= 1) up += __shfl_xor_sync(t.mask, up, o, TW);
+    // (the sum of at most 128 bounds is short by 128 u of itself at most)
+    if (up * 1.00001f < __double2float_rd(sum_old)) return false;
+  }
+  double4 m = make_double4(0.0, 0.0, 0.0, 0.0);
+  if (t.tl == src) m = interpolate_in(S, c.vb, eat, X, Y);
+  Mout = make_double4(tshfl(t, m.x, src), tshfl(t, m.y, src), tshfl(t, m.z, src), 0.0);
+  if (t.tl == 0) ops += 46 + 85 * nel;
+  return tile_ball_exact(t, S, c, lv, ne, nel, X, Y, Mout, floor, strict, qout, qsum);
 }
 
 // Quality-constrained Laplacian move of v: metric-weighted neighbour mean,
@@ -2259,8 +2277,7 @@ __device__ bool tile_ball_after_move(const Tile& t, const Store& S, MeshCtx c, i
 // neighbour (Laplacian), 11 (solve), 46 (barycentrics and metric) and 85 per
 // element of the ball of an accepted move (orientation and quality).
 __device__ bool tile_smooth_eval(const Tile& t, const Store& S, int v, MeshCtx c, double2& Xo,
-                                 double4& Mo, double* qout, int& ops) {
-  ops = 0;
+                                 double4& Mo, double* qout, unsigned& ops) {
   uint8_t f = S.vflag[v];
   if (!(f & VF_ALIVE) || (f & VF_BND)) return false;
   const int* ne = ne_row(S, v);
@@ -2293,29 +2310,23 @@ __device__ bool tile_smooth_eval(const Tile& t, const Store& S, int v, MeshCtx c
       b1 = b1 + tshfl(t, t1, j);
     }
   }
-  ops = 17 * nnl + 3;
+  if (t.tl == 0) ops += 17 * nnl + 3;
   double det = a00 * a11 - a01 * a01;
   if (!dgt(det, 0.0)) return false;
   double x = (a11 * b0 - a01 * b1) / det;
   double y = (a00 * b1 - a01 * b0) / det;
-  ops += 8;
-  double4 Mn;
-  if (!tile_interpolate(t, S, c, ne, nel, x, y, Mn)) return false;
-  ops += 46;
-  if (!tile_ball_after_move(t, S, c, v - c.vb, ne, nel, x, y, Mn, qold, true, qout, nullptr))
-    return false;
-  ops += 85 * nel;
+  if (t.tl == 0) ops += 8;
   Xo = make_double2(x, y);
-  Mo = Mn;
-  return true;
+  return tile_try_move(t, S, c, v - c.vb, ne, nel, x, y, qold, true, qout, nullptr, 0.0, Mo, ops);
 }
 
 // Pass 2 of the longer lists, one listed vertex per thread: the Laplacian sums,
 // the 2x2 solve, the location and the interpolation run per thread (a tile of
 // lanes per vertex repeats the ordered sums in every lane: four vertices per
 // warp instruction of FP64 instead of 32), the FP32 bounds of the moved ball
-// drop the moves that certainly fail, and the remaining ones get the exact
-// ball check, four at a time on 8-lane tiles.  Every value is computed by the
+// (its metric interpolated in FP32) drop the moves that certainly fail, and the
+// remaining ones get the exact metric and the exact ball check, four at a time
+// on 8-lane tiles.  Every value is computed by the
 // same operations in the same order as in tile_smooth_eval.
 __device__ __forceinline__ void smooth_eval_phase(Store S, const int* E, const int* nEp,
                                                   double2* mvxy, double4* mvM, double* qball,
@@ -2374,13 +2385,17 @@ __device__ __forceinline__ void smooth_eval_phase(Store S, const int* E, const i
           may = contains(S, fx, x, y, c.vb + e.x, c.vb + e.y, c.vb + e.z);
         }
         if (may) {
-          Mn = interpolate_in(S, c.vb, e, x, y);
-          ops += 46;
-          const VF fn = make_vf(x, y, Mn.x, Mn.y, Mn.z);
+          VF fn;
+          const float kx = metric_at(S, c.vb, e, fx, fn);
           const float ffloor = __double2float_rd(qold);
 #pragma unroll 2
           for (int k = 0; k < nel; ++k)
-            may = may && !move_fails(S, c.vb, lv, S.EN[c.eb + ne[k]], fn, ffloor);
+            may = may &&
+                  !(moved_quality_up(S, c.vb, lv, S.EN[c.eb + ne[k]], fn, kx) < ffloor);
+          if (may) {
+            Mn = interpolate_in(S, c.vb, e, x, y);
+            ops += 46;
+          }
         }
       }
       if (!may) mvM[v].w = 0.0;
@@ -2447,16 +2462,18 @@ __device__ __forceinline__ void smooth_scan_eval_phase(Store S, const int* D, co
                                                        double2* mvxy, double4* mvM, double* qball,
                                                        int* C, int* nC, int* cmark, int tag,
                                                        int pass0, unsigned long long* work) {
-  const int n = *nDp;
   const Tile t = tile_of();
   const int tile_rank = (threadIdx.x / TW) * gridDim.x + blockIdx.x;
   const int tiles = gridDim.x * (blockDim.x / TW);
+  const int first = first_entry(D, tile_rank, S.vslots);
+  const int n = *nDp;
+  unsigned ops = 0;
   for (int j0 = 0; j0 < n; j0 += tiles) {
     int j = j0 + tile_rank;
-    int v = 0, ops = 0;
+    int v = 0;
     bool cand = false;
     if (j < n) {
-      v = D[j];
+      v = j0 == 0 ? first : D[j];
       MeshCtx c = ctx_of(S, v);
       bool keep = unchanged(S, v, c.vb, S.evm[v], pass0);
       keep = __shfl_sync(t.mask, keep, 0, TW);
@@ -2487,11 +2504,8 @@ __device__ __forceinline__ void smooth_scan_eval_phase(Store S, const int* D, co
       }
     }
     warp_append(cand && t.tl == 0, v, C, nC);
-    if (work) {  // measurement only: one atomic per warp
-      unsigned tot = __reduce_add_sync(0xffffffffu, t.tl == 0 ? (unsigned)ops : 0u);
-      if ((threadIdx.x & 31) == 0 && tot) atomicAdd(work, (unsigned long long)tot);
-    }
   }
+  add_work(work, ops);
 }
 
 __global__ void k_smooth_eval(Store S, const int* E, const int* nEp, double2* mvxy, double4* mvM,
@@ -2579,6 +2593,64 @@ __global__ void k_smooth_select_apply(Store S, const int* C, const int* nCp, con
   round_done(S, done);
 }
 
+// d/dx and d/dy of the quality of element (i0, i1, i2) with respect to its
+// vertex `own`: the operations of quality_grad_c that these two values need, in
+// its order (the metric's derivatives, the other vertices' and those of the edge
+// that does not touch the vertex are left out: about 200 FP64 instructions
+// instead of 270).
+__device__ __forceinline__ void quality_grad_xy(int i0, int i1, int i2, VD a, VD b, VD c, int own,
+                                                double& gx, double& gy) {
+  canon(i0, i1, i2, a, b, c);
+  const int at = own == i0 ? 0 : (own == i1 ? 1 : 2);
+  double k00 = div3((a.m00 + b.m00) + c.m00);
+  double k01 = div3((a.m01 + b.m01) + c.m01);
+  double k11 = div3((a.m11 + b.m11) + c.m11);
+  double dx[3] = {b.x - a.x, c.x - b.x, a.x - c.x};
+  double dy[3] = {b.y - a.y, c.y - b.y, a.y - c.y};
+  double l[3];
+#pragma unroll
+  for (int e = 0; e < 3; ++e) {
+    double L2 = ((k00 * dx[e]) * dx[e] + ((2.0 * k01) * dx[e]) * dy[e]) + (k11 * dy[e]) * dy[e];
+    l[e] = sqrt(L2);
+  }
+  double P = (l[0] + l[1]) + l[2];
+  double area = 0.5 * orient3(a, b, c);
+  double sd = sqrt(k00 * k11 - k01 * k01);
+  double AM = sd * area;
+  double xx = div3(P);
+  bool left = (xx <= 1.0);
+  double sv = left ? xx : 1.0 / xx;
+  double f = sv * (2.0 - sv);
+  double F = (f * f) * f;
+  double PP = P * P;
+  double t = (QC * AM) / PP;
+  double gAM = (F * QC) / PP;
+  double gP = -((2.0 * t) / P) * F;
+  double gf = (3.0 * (f * f)) * t;
+  double gs = (2.0 - 2.0 * sv) * gf;
+  double gxx = left ? gs : -(gs / (xx * xx));
+  gP = gP + div3(gxx);
+  double go = 0.5 * (sd * gAM);
+  // the edges before and after the vertex, and the opposite one's ends
+  const double lb = at == 0 ? l[2] : (at == 1 ? l[0] : l[1]);
+  const double la = at == 0 ? l[0] : (at == 1 ? l[1] : l[2]);
+  const double bx = at == 0 ? dx[2] : (at == 1 ? dx[0] : dx[1]);
+  const double by = at == 0 ? dy[2] : (at == 1 ? dy[0] : dy[1]);
+  const double ax = at == 0 ? dx[0] : (at == 1 ? dx[1] : dx[2]);
+  const double ay = at == 0 ? dy[0] : (at == 1 ? dy[1] : dy[2]);
+  const double ya = at == 0 ? b.y : (at == 1 ? c.y : a.y), yb = at == 0 ? c.y : (at == 1 ? a.y : b.y);
+  const double xa = at == 0 ? c.x : (at == 1 ? a.x : b.x), xb = at == 0 ? b.x : (at == 1 ? c.x : a.x);
+  const double gLb = gP / (2.0 * lb), gLa = gP / (2.0 * la);
+  const double bgx = ((2.0 * k00) * bx + (2.0 * k01) * by) * gLb;
+  const double bgy = ((2.0 * k01) * bx + (2.0 * k11) * by) * gLb;
+  const double agx = ((2.0 * k00) * ax + (2.0 * k01) * ay) * gLa;
+  const double agy = ((2.0 * k01) * ax + (2.0 * k11) * ay) * gLa;
+  // vertex 0 subtracts its own edge first, the others add the edge before first
+  const double x0 = go * (ya - yb), y0 = go * (xa - xb);
+  gx = at == 0 ? (x0 - agx) + bgx : (x0 + bgx) - agx;
+  gy = at == 0 ? (y0 - agy) + bgy : (y0 + bgy) - agy;
+}
+
 // Optimisation-based smoothing of one member of S (gradient ascent of the
 // ball's quality sum in v's coordinates, metric fixed; step 0.1 * shortest
 // incident edge / |g|, halved up to five times; kept when every element stays
@@ -2597,12 +2669,8 @@ __device__ bool tile_opt_eval(const Tile& t, const Store& S, int v, MeshCtx c, d
     double gxk = 0.0, gyk = 0.0;
     if (k < nel) {
       int4 e = S.EN[c.eb + ne[k]];
-      double g[3][5];
-      quality_grad_c(e.x, e.y, e.z, load_vd(S, c.vb + e.x), load_vd(S, c.vb + e.y),
-                     load_vd(S, c.vb + e.z), g);
-      int i = (e.x == lv) ? 0 : (e.y == lv) ? 1 : 2;
-      gxk = g[i][0];
-      gyk = g[i][1];
+      quality_grad_xy(e.x, e.y, e.z, load_vd(S, c.vb + e.x), load_vd(S, c.vb + e.y),
+                      load_vd(S, c.vb + e.z), lv, gxk, gyk);
     }
     int cnt = min(TW, nel - base);
     for (int j = 0; j < cnt; ++j) {
@@ -2627,18 +2695,18 @@ __device__ bool tile_opt_eval(const Tile& t, const Store& S, int v, MeshCtx c, d
   double qsum_old;
   double qmin_old = tile_ball_quality(t, S, c, ne, nel, &qsum_old);
   double alpha = (0.1 * lmin) / gn;
+  unsigned ops = 0;
   for (int k = 0; k < 6; ++k) {
     double X = pv.x + alpha * gx;
     double Y = pv.y + alpha * gy;
     double4 Mn;
-    if (tile_interpolate(t, S, c, ne, nel, X, Y, Mn)) {
-      double qsum;
-      if (tile_ball_after_move(t, S, c, lv, ne, nel, X, Y, Mn, qmin_old, false, qout, &qsum) &&
-          qsum > qsum_old) {
-        Xo = make_double2(X, Y);
-        Mo = Mn;
-        return true;
-      }
+    double qsum;
+    if (tile_try_move(t, S, c, lv, ne, nel, X, Y, qmin_old, false, qout, &qsum, qsum_old, Mn,
+                      ops) &&
+        qsum > qsum_old) {
+      Xo = make_double2(X, Y);
+      Mo = Mn;
+      return true;
     }
     alpha = alpha * 0.5;
   }

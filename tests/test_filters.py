@@ -16,6 +16,19 @@ SRC = r"""
 #include "pm_filter.cuh"
 using namespace pm;
 static VF vf(const double* p) { return make_vf(p[0], p[1], p[2], p[3], p[4]); }
+// the metric at points x of the triangles, and the quality bound of (x, b, c) with it
+extern "C" void at(const double* p, const double* x, int n, float* m, float* kx, float* up) {
+  for (int i = 0; i < n; ++i) {
+    const VF a = vf(p + 15 * i), b = vf(p + 15 * i + 5), c = vf(p + 15 * i + 10);
+    VF o = make_vf_xy(x[2 * i], x[2 * i + 1]);
+    kx[i] = f_metric_at(o, a, b, c, o);
+    m[3 * i] = o.m00;
+    m[3 * i + 1] = o.m01;
+    m[3 * i + 2] = o.m11;
+    int sign;
+    up[i] = f_quality_up(o, b, c, sign, kx[i]);
+  }
+}
 extern "C" void run(const double* p, const double* bound, int n, int32_t* orient, int32_t* len,
                     float* up, int32_t* osign, float* l2, float* el2) {
   for (int i = 0; i < n; ++i) {
@@ -119,3 +132,55 @@ def test_filters_decide_only_what_is_certain(lib, scale, offset, aspect, flat):
         ok = has & (det > 0) & (x < 10) & fat
         if aspect <= 30 and offset <= 1.0:
             assert np.median((out["up"][ok] - q[ok]) / q[ok]) < 0.01
+
+
+def quality_exact(a, b, c):
+    """The quality of (a, b, c) (columns x, y, m00, m01, m11) in extended precision."""
+    L = np.longdouble
+    k = [(a[:, j] + b[:, j] + c[:, j]) / 3 for j in (2, 3, 4)]
+    P = 0
+    for p, q in ((a, b), (b, c), (c, a)):
+        dx, dy = q[:, 0] - p[:, 0], q[:, 1] - p[:, 1]
+        P = P + np.sqrt(k[0] * dx * dx + 2 * k[1] * dx * dy + k[2] * dy * dy)
+    det = ((b[:, 0] - a[:, 0]) * (c[:, 1] - a[:, 1]) - (b[:, 1] - a[:, 1]) * (c[:, 0] - a[:, 0]))
+    s = np.minimum(P / 3, 3 / P)
+    return (12 * np.sqrt(L(3)) * np.sqrt(k[0] * k[2] - k[1] ** 2) * (det / 2) / P ** 2
+            * (s * (2 - s)) ** 3)
+
+
+@pytest.mark.parametrize("scale,offset,aspect,flat", CASES)
+def test_interpolated_metric_and_its_quality_bound(lib, scale, offset, aspect, flat):
+    """f_metric_at at points inside the triangles, on their edges and just outside: its error
+    bound holds, and so does the quality bound that carries it."""
+    rng = np.random.default_rng(int(abs(np.log10(scale)) * 11 + aspect))
+    n = 40000
+    tri = triangles(rng, n, scale, offset, aspect, flat)
+    w = rng.dirichlet([1.0, 1.0, 1.0], n)
+    w[: n // 4, 0] = rng.uniform(-1e-8, 1e-8, n // 4)  # on an edge line, within rounding
+    with np.errstate(all="ignore"):
+        x = np.ascontiguousarray(np.einsum("ij,ijk->ik", w, tri[:, :, :2]))
+        L = np.longdouble
+        a, b, c = (tri[:, k].astype(L) for k in range(3))
+        X = x.astype(L)
+
+        def det(p, q, r):
+            return ((q[:, 0] - p[:, 0]) * (r[:, 1] - p[:, 1])
+                    - (q[:, 1] - p[:, 1]) * (r[:, 0] - p[:, 0]))
+
+        o = det(a, b, c)
+        l0, l1, l2 = det(X, b, c) / o, det(a, X, c) / o, det(a, b, X) / o
+        m = [l0 * a[:, k] + l1 * b[:, k] + l2 * c[:, k] for k in (2, 3, 4)]
+        got, kx, up = np.zeros((n, 3), np.float32), np.zeros(n, np.float32), np.zeros(n, np.float32)
+        vp = C.c_void_p
+        lib.at(vp(tri.ctypes.data), vp(x.ctypes.data), n, vp(got.ctypes.data), vp(kx.ctypes.data),
+               vp(up.ctypes.data))
+        known = (kx < 0.05) & np.isfinite(o.astype(float))  # larger bounds are not used
+        bound = kx.astype(L)
+        root = np.sqrt(abs(m[0] * m[2]))
+        for j, ref in ((0, m[0]), (1, root), (2, m[2])):
+            assert not np.any(known & (abs(got[:, j].astype(L) - m[j]) > bound * abs(ref) * 1.01))
+        q = quality_exact(np.stack([X[:, 0], X[:, 1], *m], axis=1), b, c)
+        has = known & np.isfinite(up) & np.isfinite(q.astype(float))
+        assert not np.any(has & ~(up.astype(L) >= q))
+    if 1e-13 < scale < 1e10 and offset <= 1.0:
+        assert np.mean(known[(np.arange(n) >= n // 3) & (o > 0)]) > 0.95
