@@ -258,6 +258,21 @@ __device__ __forceinline__ bool stamp_first(int* stamp, int slot, int tag) {
   return atomicExch(stamp + slot, tag) != tag;
 }
 
+// Eight consecutive entries of an adjacency row from position `base` (a multiple
+// of 8) on: rows hold a multiple of 16 entries, so whole chunks may be read
+// whatever the row's length.  Loops over rows go by such chunks with their loads
+// predicated and issued together: a loop whose trip count is the row's length is
+// unrolled with a remainder loop, in which a typical row of six entries runs
+// alone, one round trip to memory per entry.
+struct Row8 {
+  int a[8];
+};
+__device__ __forceinline__ Row8 row8(const int* row, int base) {
+  const int4* r4 = reinterpret_cast<const int4*>(row + base);
+  const int4 p = r4[0], q = r4[1];
+  return Row8{{p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w}};
+}
+
 // Position of val in the first len entries of an adjacency row, or -1.  A
 // row starts on a 64-byte boundary (arrays are 256-byte aligned and the row
 // width is a power of two of at least 16), so it is read in 16-byte chunks
@@ -266,15 +281,11 @@ __device__ __forceinline__ bool stamp_first(int* stamp, int slot, int tag) {
 // chain of dependent loads.  Chunks never pass the row's end (len <= width,
 // a multiple of 4); entries at len and beyond are not compared.
 __device__ __forceinline__ int row_find(const int* row, int len, int val) {
-  const int4* r4 = reinterpret_cast<const int4*>(row);
   int at = -1;
-#pragma unroll 4
-  for (int k = 0; k < len; k += 4) {
-    const int4 q = r4[k >> 2];
-    at = (q.w == val && k + 3 < len) ? k + 3 : at;
-    at = (q.z == val && k + 2 < len) ? k + 2 : at;
-    at = (q.y == val && k + 1 < len) ? k + 1 : at;
-    at = (q.x == val) ? k : at;
+  for (int b = 0; b < len; b += 8) {
+    const Row8 r = row8(row, b);
+#pragma unroll
+    for (int k = 7; k >= 0; --k) at = (r.a[k] == val && b + k < len) ? b + k : at;
   }
   return at;
 }

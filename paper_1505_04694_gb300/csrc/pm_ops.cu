@@ -92,9 +92,14 @@ __device__ __forceinline__ void advance_rounds(const Store& S) {
 __device__ __forceinline__ int count_elems_with(const Store& S, const int* ne, int nel, int eb,
                                                 int lw) {
   int c = 0;
-  for (int k = 0; k < nel; ++k) {
-    int4 e = S.EN[eb + ne[k]];
-    if (e.x == lw || e.y == lw || e.z == lw) ++c;
+  for (int b = 0; b < nel; b += 8) {
+    const Row8 r = row8(ne, b);
+    int4 e[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      e[k] = b + k < nel ? S.EN[eb + r.a[k]] : make_int4(-1, -1, -1, 0);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) c += (e[k].x == lw || e[k].y == lw || e[k].z == lw) ? 1 : 0;
   }
   return c;
 }
@@ -153,8 +158,12 @@ __device__ __forceinline__ void elem_quality_phase(const Store& S, const int* li
 // Stamps the neighbours in `row` (local ids) after a change of their vertex.
 __device__ __forceinline__ void stamp_neighbours(const Store& S, const int* row, int len, int vb,
                                                  int stamp) {
-#pragma unroll 4
-  for (int k = 0; k < len; ++k) S.ntouch[vb + row[k]] = stamp;
+  for (int b = 0; b < len; b += 8) {
+    const Row8 r = row8(row, b);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (b + k < len) S.ntouch[vb + r.a[k]] = stamp;
+  }
 }
 
 // ---- worklist initialisation ---------------------------------------------------
@@ -224,14 +233,26 @@ __device__ __forceinline__ bool local_max(const Store& S, int v, const int* cmar
   if (by_colour && S.tab.col[v] != cls) return false;
   uint32_t pv = prio(vid_of(S, v, c.vb), seed, r);
   const int* nn = nn_row(S, v);
-  int nnl = S.NNlen[v];
+  Row8 nb = row8(nn, 0);
+  const int nnl = S.NNlen[v];
   bool win = true;
-#pragma unroll 8
-  for (int k = 0; k < nnl; ++k) {
-    int u = c.vb + nn[k];
-    int cu = cmark[u];
-    uint32_t iu = vid_of(S, u, c.vb);
-    win &= !(cu == tag && (!by_colour || S.tab.col[u] == cls) && prio(iu, seed, r) > pv);
+  for (int b = 0;;) {
+    int cu[8];
+    uint32_t iu[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const bool in = b + k < nnl;
+      cu[k] = in ? cmark[c.vb + nb.a[k]] : tag - 1;
+      iu[k] = in ? vid_of(S, c.vb + nb.a[k], c.vb) : 0u;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (cu[k] != tag) continue;
+      win &= !((!by_colour || S.tab.col[c.vb + nb.a[k]] == cls) && prio(iu[k], seed, r) > pv);
+    }
+    b += 8;
+    if (b >= nnl) break;
+    nb = row8(nn, b);
   }
   return win;
 }
@@ -594,22 +615,29 @@ __device__ __forceinline__ void coarsen_scan_phase(Store S, const int* D, const 
         float lo[MAXW];      // candidates: lower bound of the squared length
         float first = INFINITY;  // the smallest upper bound
         RowMask cm;
-#pragma unroll 4
-        for (int k = 0; k < nnl; ++k) {
-          const int us = c.vb + nn[k];
-          const VF fu = load_vf(S, us);
-          const FLen l = f_edge2(fv, fu);
-          const int r = f_len_cmp(l, bf.x, bf.y);
-          bool is = r < 0;
-          if (r == 0) is = edge_shorter(S, c.mi, fv, fu, v, us, ops);
-          // a boundary vertex collapses only along a boundary edge
-          if (is && (f & VF_BND))
-            is = count_elems_with(S, ne_row(S, v), S.NElen[v], c.eb, nn[k]) == 1;
-          if (is) {
-            cm.set(k);
-            lo[k] = l.L2 - l.err;
-            // (a NaN bound leaves `first` as it is and passes the test below)
-            first = l.L2 + l.err < first ? l.L2 + l.err : first;
+        for (int b = 0; b < nnl; b += 4) {
+          const int4 r4 = *reinterpret_cast<const int4*>(nn + b);
+          const int u4[4] = {r4.x, r4.y, r4.z, r4.w};
+          VF fu[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) fu[j] = b + j < nnl ? load_vf(S, c.vb + u4[j]) : VF{};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int k = b + j;
+            if (k >= nnl) continue;
+            const FLen l = f_edge2(fv, fu[j]);
+            const int r = f_len_cmp(l, bf.x, bf.y);
+            bool is = r < 0;
+            if (r == 0) is = edge_shorter(S, c.mi, fv, fu[j], v, c.vb + u4[j], ops);
+            // a boundary vertex collapses only along a boundary edge
+            if (is && (f & VF_BND))
+              is = count_elems_with(S, ne_row(S, v), S.NElen[v], c.eb, u4[j]) == 1;
+            if (is) {
+              cm.set(k);
+              lo[k] = l.L2 - l.err;
+              // (a NaN bound leaves `first` as it is and passes the test below)
+              first = l.L2 + l.err < first ? l.L2 + l.err : first;
+            }
           }
         }
         nc = cm.count();
@@ -794,38 +822,74 @@ __device__ __forceinline__ void check_len_chunk(const Store& S, const CheckQueue
 // elements and v's neighbours.
 __device__ __forceinline__ bool check_filter(const Store& S, const CoarsenCtx& x, int u,
                                              RowMask& oo, RowMask& ol) {
-  const bool bedge = count_elems_with(S, x.ne, x.nel, x.c.eb, u) == 1;
-  if (x.bnd && !bedge) return false;
   const int ws = x.c.vb + u;
   const int* nnw = nn_row(S, ws);
   const int nnwl = S.NNlen[ws];
-  RowMask common;
-#pragma unroll 2
-  for (int k = 0; k < x.nnl; ++k)
-    if (row_has(nnw, nnwl, x.nn[k])) common.set(k);
-  if (common.count() != (bedge ? 1 : 2)) return false;
   const VF fw = load_vf(S, ws);
+  const bool bedge = count_elems_with(S, x.ne, x.nel, x.c.eb, u) == 1;
+  if (x.bnd && !bedge) return false;
+  // v's neighbours in u's row
+  RowMask common;
+  for (int b = 0; b < nnwl; b += 8) {
+    const Row8 w8 = row8(nnw, b);
+    for (int a = 0; a < x.nnl; a += 8) {
+      const Row8 v8 = row8(x.nn, a);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        bool in = false;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) in |= b + j < nnwl && w8.a[j] == v8.a[k];
+        if (in && a + k < x.nnl) common.set(a + k);
+      }
+    }
+  }
+  if (common.count() != (bedge ? 1 : 2)) return false;
   bool ok = true;
-#pragma unroll 2
-  for (int k = 0; k < x.nel; ++k) {
-    const int4 e = S.EN[x.c.eb + x.ne[k]];
-    if (e.x == u || e.y == u || e.z == u) continue;
-    // the element in the order (u in place of v, next, before)
-    const int n1 = (e.x == x.lv) ? e.y : (e.y == x.lv) ? e.z : e.x;
-    const int n2 = (e.x == x.lv) ? e.z : (e.y == x.lv) ? e.x : e.y;
-    const int o = f_orient(fw, load_vf(S, x.c.vb + n1), load_vf(S, x.c.vb + n2));
-    ok &= o >= 0;
-    if (o == 0) oo.set(k);
+  for (int b = 0; b < x.nel; b += 4) {
+    const int4 r4 = *reinterpret_cast<const int4*>(x.ne + b);
+    const int K4[4] = {r4.x, r4.y, r4.z, r4.w};
+    int4 e[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      e[j] = b + j < x.nel ? S.EN[x.c.eb + K4[j]] : make_int4(u, u, u, 0);
+    VF p[4], q[4];
+    bool test[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      test[j] = e[j].x != u && e[j].y != u && e[j].z != u;
+      // the element in the order (u in place of v, next, before)
+      const int n1 = (e[j].x == x.lv) ? e[j].y : (e[j].y == x.lv) ? e[j].z : e[j].x;
+      const int n2 = (e[j].x == x.lv) ? e[j].z : (e[j].y == x.lv) ? e[j].x : e[j].y;
+      p[j] = test[j] ? load_vf(S, x.c.vb + n1) : VF{};
+      q[j] = test[j] ? load_vf(S, x.c.vb + n2) : VF{};
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (!test[j]) continue;
+      const int o = f_orient(fw, p[j], q[j]);
+      ok &= o >= 0;
+      if (o == 0) oo.set(b + j);
+    }
   }
   if (!ok) return false;
   const float4 bf = S.tab.bandf[x.c.mi];
-#pragma unroll 2
-  for (int k = 0; k < x.nnl; ++k) {
-    const int y = x.nn[k];
-    if (y == u || common.test(k)) continue;
-    const int r = edge_cmp(fw, load_vf(S, x.c.vb + y), bf.z, bf.w);
-    ok &= r <= 0;
-    if (r == 0) ol.set(k);
+  for (int b = 0; b < x.nnl; b += 4) {
+    const int4 r4 = *reinterpret_cast<const int4*>(x.nn + b);
+    const int y4[4] = {r4.x, r4.y, r4.z, r4.w};
+    VF p[4];
+    bool test[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      test[j] = b + j < x.nnl && y4[j] != u && !common.test(b + j);
+      p[j] = test[j] ? load_vf(S, x.c.vb + y4[j]) : VF{};
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (!test[j]) continue;
+      const int r = edge_cmp(fw, p[j], bf.z, bf.w);
+      ok &= r <= 0;
+      if (r == 0) ol.set(b + j);
+    }
   }
   return ok;
 }
@@ -1025,30 +1089,37 @@ __device__ __forceinline__ void coarsen_select_apply_phase(Store S, const int* C
       const int nel = S.NElen[v];
       // the ball is read first (all loads in flight), then only the words that
       // change are written: v's slot takes w, or the alive word is cleared in
-      // the elements that hold w.  Two bits per element: the word to write.
-      for (int k0 = 0; k0 < nel; k0 += 32) {
-        unsigned long long word = 0ull;
-        const int m = min(32, nel - k0);
-#pragma unroll 8
-        for (int k = 0; k < m; ++k) {
-          const int4 e = S.EN[c.eb + ne[k0 + k]];
-          const bool dies = e.x == w || e.y == w || e.z == w;
-          const unsigned f = dies ? 3u : (e.x == lv ? 0u : (e.y == lv ? 1u : 2u));
-          word |= (unsigned long long)f << (2 * k);
-          if (!dies) qbits.set(k0 + k);
-        }
-#pragma unroll 8
-        for (int k = 0; k < m; ++k) {
-          const int f = (int)(word >> (2 * k)) & 3;
-          reinterpret_cast<int*>(S.EN + c.eb + ne[k0 + k])[f] = f == 3 ? 0 : w;
+      // the elements that hold w
+      for (int b = 0; b < nel; b += 8) {
+        const Row8 r = row8(ne, b);
+        int4 e[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          e[k] = b + k < nel ? S.EN[c.eb + r.a[k]] : make_int4(0, 0, 0, 0);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          if (b + k >= nel) continue;
+          const bool dies = e[k].x == w || e[k].y == w || e[k].z == w;
+          const int f = dies ? 3 : (e[k].x == lv ? 0 : (e[k].y == lv ? 1 : 2));
+          reinterpret_cast<int*>(S.EN + c.eb + r.a[k])[f] = dies ? 0 : w;
+          if (!dies) qbits.set(b + k);
         }
       }
       S.vflag[v] = (uint8_t)(S.vflag[v] & ~VF_ALIVE);
-#pragma unroll 8
-      for (int k = 0; k < nnl; ++k) {
-        const int s = vb + nn[k];
-        if (stamp_first(amark, s, tag)) fa.set(k);
-        if (stamp_first(dmark, s, tag)) fd.set(k);
+      for (int b = 0; b < nnl; b += 8) {
+        const Row8 r = row8(nn, b);
+        int oa[8], od[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const bool in = b + k < nnl;
+          oa[k] = in ? atomicExch(amark + vb + r.a[k], tag) : tag;
+          od[k] = in ? atomicExch(dmark + vb + r.a[k], tag) : tag;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          if (oa[k] != tag) fa.set(b + k);
+          if (od[k] != tag) fd.set(b + k);
+        }
       }
     }
     count_op(S, win, mi);
@@ -2351,26 +2422,39 @@ __device__ __forceinline__ void smooth_eval_phase(Store S, const int* E, const i
       const int* nn = nn_row(S, v);
       const int nnl = S.NNlen[v];
       qold = 1e300;
-#pragma unroll 4
-      for (int k = 0; k < nel; ++k) {
-        const double q = S.qK[c.eb + ne[k]];
-        qold = dlt(q, qold) ? q : qold;
+      for (int b = 0; b < nel; b += 8) {
+        const Row8 r = row8(ne, b);
+        double q[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) q[k] = b + k < nel ? S.qK[c.eb + r.a[k]] : 1e300;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) qold = dlt(q[k], qold) ? q[k] : qold;
       }
       const double4 mv = S.M[v];
       double a00 = 0.0, a01 = 0.0, a11 = 0.0, b0 = 0.0, b1 = 0.0;
-#pragma unroll 2
-      for (int k = 0; k < nnl; ++k) {
-        const int js = c.vb + nn[k];
-        const double2 pj = S.xy[js];
-        const double4 mj = S.M[js];
-        const double w00 = 0.5 * (mv.x + mj.x);
-        const double w01 = 0.5 * (mv.y + mj.y);
-        const double w11 = 0.5 * (mv.z + mj.z);
-        a00 = a00 + w00;
-        a01 = a01 + w01;
-        a11 = a11 + w11;
-        b0 = b0 + (w00 * pj.x + w01 * pj.y);
-        b1 = b1 + (w01 * pj.x + w11 * pj.y);
+      for (int b = 0; b < nnl; b += 4) {
+        const int4 r4 = *reinterpret_cast<const int4*>(nn + b);
+        const int u4[4] = {r4.x, r4.y, r4.z, r4.w};
+        double2 p[4];
+        double4 mj[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int js = b + j < nnl ? c.vb + u4[j] : v;
+          p[j] = S.xy[js];
+          mj[j] = S.M[js];
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (b + j >= nnl) continue;
+          const double w00 = 0.5 * (mv.x + mj[j].x);
+          const double w01 = 0.5 * (mv.y + mj[j].y);
+          const double w11 = 0.5 * (mv.z + mj[j].z);
+          a00 = a00 + w00;
+          a01 = a01 + w01;
+          a11 = a11 + w11;
+          b0 = b0 + (w00 * p[j].x + w01 * p[j].y);
+          b1 = b1 + (w01 * p[j].x + w11 * p[j].y);
+        }
       }
       const double det = a00 * a11 - a01 * a01;
       ops += 17 * nnl + 3;
@@ -2537,19 +2621,33 @@ __device__ __forceinline__ void smooth_apply_one(const Store& S, bool ok, int v,
       S.touch[v] = stamp;
       const int* ne = ne_row(S, v);
       int nel = S.NElen[v];
-#pragma unroll 8
-      for (int k = 0; k < nel; ++k) S.qK[c.eb + ne[k]] = qball[(size_t)v * S.W + k];
+      for (int b = 0; b < nel; b += 8) {
+        const Row8 r = row8(ne, b);
+        double q[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) q[k] = b + k < nel ? qball[(size_t)v * S.W + b + k] : 0.0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (b + k < nel) S.qK[c.eb + r.a[k]] = q[k];
+      }
       nn = nn_row(S, v);
       nnl = S.NNlen[v];
-      stamp_neighbours(S, nn, nnl, vb, stamp);
       // (a stamp on a vertex that is not taken is harmless: only interior
       // neighbours look at it)
-#pragma unroll 8
-      for (int k = 0; k < nnl; ++k) {
-        const int s = vb + nn[k];
-        const uint8_t f = S.vflag[s];
-        const bool first = stamp_first(pmark, s, ptag);
-        if (first && (f & VF_ALIVE) && !(f & VF_BND)) take.set(k);
+      for (int b = 0; b < nnl; b += 8) {
+        const Row8 r = row8(nn, b);
+        int op[8], f[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const bool in = b + k < nnl;
+          const int s = vb + r.a[k];
+          f[k] = in ? S.vflag[s] : VF_BND;
+          op[k] = in ? atomicExch(pmark + s, ptag) : ptag;
+          if (in) S.ntouch[s] = stamp;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (op[k] != ptag && (f[k] & VF_ALIVE) && !(f[k] & VF_BND)) take.set(b + k);
       }
     }
     count_op(S, ok, mi);
@@ -2789,10 +2887,24 @@ __global__ void k_refine_mark(Store S, int* cnt, RowMask* mask, int tag, int pas
       // the row is sorted, so the neighbours above la form a suffix; four
       // lengths at a time so that their loads overlap
       int k0 = 0;
-      while (k0 < nnl && nn[k0] <= la) ++k0;
-#pragma unroll 4
-      for (int k = k0; k < nnl; ++k)
-        if (edge_longer(S, mi, fa, load_vf(S, vb + nn[k]), s, vb + nn[k], ops)) m.set(k);
+      for (int b = 0; b < nnl; b += 8) {
+        const Row8 r = row8(nn, b);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) k0 += b + k < nnl && r.a[k] <= la ? 1 : 0;
+      }
+      for (int b = k0 & ~3; b < nnl; b += 4) {
+        const int4 r4 = *reinterpret_cast<const int4*>(nn + b);
+        const int u4[4] = {r4.x, r4.y, r4.z, r4.w};
+        VF fu[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          fu[j] = b + j >= k0 && b + j < nnl ? load_vf(S, vb + u4[j]) : VF{};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (b + j >= k0 && b + j < nnl &&
+              edge_longer(S, mi, fa, fu[j], s, vb + u4[j], ops))
+            m.set(b + j);
+      }
       mask[s] = m;
     } else {
       mask[s] = RowMask();
