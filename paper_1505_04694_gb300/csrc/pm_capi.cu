@@ -80,8 +80,8 @@ __global__ void k_ingest(Store S, const double* xy, const int* tri, const uint8_
   int top = ne > nv ? ne : nv;
   for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < top; g += gridDim.x * blockDim.x) {
     if (g < nv) {
-      int mi = seg_of(pv, n, g);
-      int slot = S.tab.vbase[mi] + (g - pv[mi]);
+      const int mi = n == 1 ? 0 : seg_of(pv, n, g);
+      const int slot = n == 1 ? g : S.tab.vbase[mi] + (g - pv[mi]);
       const double2 p = make_double2(xy[2 * (size_t)g], xy[2 * (size_t)g + 1]);
       const double4 m = make_double4(1.0, 0.0, 1.0, 0.0);
       S.xy[slot] = p;
@@ -90,8 +90,8 @@ __global__ void k_ingest(Store S, const double* xy, const int* tri, const uint8_
       S.vflag[slot] = (uint8_t)(VF_ALIVE | ((corner && corner[g]) ? VF_CORNER : 0));
     }
     if (g < ne) {
-      int mi = seg_of(pe, n, g);
-      S.EN[S.tab.ebase[mi] + (g - pe[mi])] =
+      const int mi = n == 1 ? 0 : seg_of(pe, n, g);
+      S.EN[n == 1 ? g : S.tab.ebase[mi] + (g - pe[mi])] =
           make_int4(tri[3 * (size_t)g], tri[3 * (size_t)g + 1], tri[3 * (size_t)g + 2], 1);
     }
   }
@@ -107,11 +107,12 @@ __global__ void k_metric_check(const double* m, int nv, DevStatus* st) {
 
 // Concatenated metric (mesh after mesh, each in its used-slot order; offsets
 // in S.tab.pre) into the slots.
-__global__ void k_metric_set(Store S, const double* m, int nv) {
+__global__ void k_metric_set(Store S, const double* m, int nv, const DevStatus* st) {
+  if (st->err) return;  // a rejected metric changes nothing
   const int n = S.nmesh;
   for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < nv; g += gridDim.x * blockDim.x) {
-    int mi = seg_of(S.tab.pre, n, g);
-    int slot = S.tab.vbase[mi] + (g - S.tab.pre[mi]);
+    const int mi = n == 1 ? 0 : seg_of(S.tab.pre, n, g);
+    const int slot = n == 1 ? g : S.tab.vbase[mi] + (g - S.tab.pre[mi]);
     const double4 mv =
         make_double4(m[3 * (size_t)g], m[3 * (size_t)g + 1], m[3 * (size_t)g + 2], 0.0);
     S.M[slot] = mv;
@@ -139,6 +140,7 @@ void set_mem_pool_retain(int dev) {
 // the meshes' slots.
 cudaError_t upload_prefix(MeshSet& m, const std::vector<int>& nv, const std::vector<int>& ne) {
   const int n = m.nmesh;
+  if (n == 1) return cudaSuccess;  // a single mesh's offsets are zero
   std::vector<int> pre(2 * ((size_t)n + 1));
   for (int i = 0; i < n; ++i) {
     pre[i + 1] = pre[i] + nv[i];
@@ -211,20 +213,16 @@ pm_status create_set(const double* xy, const int32_t* nv, const int32_t* tri, co
   if (!s) {
     PM_LAUNCH(k_ingest, grid_for(m, std::max(nvt, net)), BLOCK, 0, m.stream, m.S, dxy, dtri,
               dcorner, (int)nvt, (int)net);
-    int err = validate_mesh(m);
+    validate_mesh(m);
+    // reads the status back: the input arrays have been read when it returns
+    const int err = rebuild_adjacency(m, true, corner != nullptr);
     if (err) s = (pm_status)err;
     if (s == PM_ERR_INVALID_ARG) set_last_error("non-finite coordinate");
     if (s == PM_ERR_INVALID_MESH)
-      set_last_error("invalid mesh: vertex id out of range, repeated in an element, or an "
-                     "element that is not counter-clockwise");
-    if (!s) {
-      err = rebuild_adjacency(m, true, corner != nullptr);
-      if (err) {
-        s = (pm_status)err;
-        if (s == PM_ERR_INVALID_MESH)
-          set_last_error("invalid mesh: overlapping elements, non-manifold or unused vertex");
-      }
-    }
+      set_last_error(m.hst->where ? "invalid mesh: vertex id out of range, repeated in an element, "
+                                    "or an element that is not counter-clockwise"
+                                  : "invalid mesh: overlapping elements, non-manifold or unused "
+                                    "vertex");
   }
   if (tmp) cudaFreeAsync(tmp, m.stream);
   if (s) {
@@ -235,6 +233,7 @@ pm_status create_set(const double* xy, const int32_t* nv, const int32_t* tri, co
     return s;
   }
   cudaMemsetAsync(m.st, 0, sizeof(DevStatus), m.stream);
+  m.dense = true;
   *out = h;
   return PM_OK;
 }
@@ -253,11 +252,10 @@ pm_status begin_call(MeshSet& m, const pm_params* P, int stride) {
   }
   pm_status s = cuda_status(upload_tab(m), "mesh table");
   if (s) return s;
-  cudaMemsetAsync(m.S.tab.r, 0, m.nmesh * sizeof(uint32_t), m.stream);
-  cudaMemsetAsync(m.S.tab.had, 0, 2 * m.nmesh * sizeof(int), m.stream);
+  // operation counts, round counters and candidate flags lie together
+  cudaMemsetAsync(m.ops, 0, (size_t)((char*)m.S.tab.active - (char*)m.ops), m.stream);
   cudaMemsetAsync(m.S.tab.active, 0xFF, m.nmesh * sizeof(int), m.stream);
   cudaMemsetAsync(m.st, 0, sizeof(DevStatus), m.stream);
-  zero_ops(m);
   // evaluations from earlier calls may predate a new metric or parameters
   m.lo_coarsen = m.lo_swap = m.lo_refine = m.tag;
   return PM_OK;
@@ -275,45 +273,13 @@ struct CallStats {
   }
 };
 
-// Run one operator and add its per-mesh operation counts to `acc`.
-template <class F>
-pm_status run_counted(MeshSet& m, F&& f, std::vector<long long>& acc,
-                      std::vector<unsigned long long>* last = nullptr) {
-  zero_ops(m);
-  int err = f();
-  if (err) return (pm_status)err;
-  std::vector<unsigned long long> ops;
-  pm_status s = cuda_status(fetch_ops(m, ops), "reading counters");
-  if (s) return s;
-  for (int i = 0; i < m.nmesh; ++i) acc[i] += (long long)ops[i];
-  if (last) *last = ops;
-  return PM_OK;
-}
-
-// Runs one operator and queues the read-back of its operation counts into
-// pinned slot `slot` without waiting (the caller reads them after its next
-// synchronisation).
-template <class F>
-pm_status run_counted_async(MeshSet& m, F&& f, int slot) {
-  zero_ops(m);
-  int err = f();
-  if (err) return (pm_status)err;
-  return cuda_status(cudaMemcpyAsync(m.hops + (size_t)slot * m.nmesh, m.S.tab.ops,
-                                     m.nmesh * sizeof(unsigned long long),
-                                     cudaMemcpyDeviceToHost, m.stream),
-                     "reading counters");
-}
-
-pm_status fill_stats(MeshSet& m, const CallStats& cs, double t0, pm_stats* out, int n) {
-  if (!out) return PM_OK;
-  std::vector<uint32_t> r(m.nmesh);
-  cudaError_t e = cudaMemcpyAsync(r.data(), m.S.tab.r, m.nmesh * sizeof(uint32_t),
-                                  cudaMemcpyDeviceToHost, m.stream);
-  if (!e) e = cudaStreamSynchronize(m.stream);
-  if (e) return cuda_status(e, "reading counters");
-  double ms = now_ms() - t0;
+// Round counters and operation counts of the call, as the last read-back of the
+// whole call state (sync_call) left them.
+void fill_stats(MeshSet& m, const CallStats& cs, double t0, pm_stats* out, int n) {
+  if (!out) return;
+  const double ms = now_ms() - t0;
   for (int i = 0; i < n; ++i) {
-    out[i].rounds = r[i];
+    out[i].rounds = m.hr[i];
     out[i].collapses = cs.collapses[i];
     out[i].splits = cs.splits[i];
     out[i].flips = cs.flips[i];
@@ -321,7 +287,6 @@ pm_status fill_stats(MeshSet& m, const CallStats& cs, double t0, pm_stats* out, 
     out[i].converged = cs.converged[i];
     out[i].ms = ms;
   }
-  return PM_OK;
 }
 
 enum OpKind { OP_COARSEN, OP_SWAP, OP_REFINE, OP_SMOOTH, OP_OPT, OP_ADAPT };
@@ -335,7 +300,16 @@ pm_status adapt_set(MeshSet& m, const pm_params* P, int stride, CallStats& cs) {
   if (int err = presize(m)) return (pm_status)err;
   int max_iter = 0;
   for (int i = 0; i < n; ++i) max_iter = std::max(max_iter, P[stride ? i : 0].max_iter);
-  std::vector<int> active(n, 1);
+  std::vector<int> active(n, 1), sent(n, 1);  // begin_call made every mesh active
+  std::vector<unsigned long long> seen(3 * (size_t)n, 0);
+  // the device flags follow `active` (a copy from pageable memory is staged)
+  auto send_active = [&](const std::vector<int>& a) {
+    if (a == sent) return;
+    cudaMemcpyAsync(m.S.tab.active, a.data(), n * sizeof(int), cudaMemcpyHostToDevice, m.stream);
+    sent = a;
+  };
+  const int mr = P[0].max_rounds;
+  int err;
   for (int it = 0; it < max_iter; ++it) {
     bool any = false;
     for (int i = 0; i < n; ++i) {
@@ -343,19 +317,19 @@ pm_status adapt_set(MeshSet& m, const pm_params* P, int stride, CallStats& cs) {
       any |= active[i] != 0;
     }
     if (!any) break;
-    cudaMemcpyAsync(m.S.tab.active, active.data(), n * sizeof(int), cudaMemcpyHostToDevice,
-                    m.stream);
-    pm_status s;
-    const int mr = P[0].max_rounds;
-    if ((s = run_counted_async(m, [&] { return op_coarsen(m, mr); }, 0))) return s;
-    if ((s = run_counted_async(m, [&] { return op_swap(m, mr); }, 1))) return s;
-    if ((s = run_counted_async(m, [&] { return op_refine(m, mr); }, 2))) return s;
-    int err = renumber(m, false);  // synchronises: the op counts have arrived
-    if (err) return (pm_status)err;
+    send_active(active);
+    select_ops(m, OS_COARSEN);
+    if ((err = op_coarsen(m, mr))) return (pm_status)err;
+    select_ops(m, OS_SWAP);
+    if ((err = op_swap(m, mr))) return (pm_status)err;
+    select_ops(m, OS_REFINE);
+    if ((err = op_refine(m, mr))) return (pm_status)err;
+    if ((err = renumber(m, false))) return (pm_status)err;  // reads the call state back
     const unsigned long long* h = m.hops;
     for (int i = 0; i < n; ++i) {
-      const long long c_i = (long long)h[i], sw_i = (long long)h[n + i];
-      const long long rf_i = (long long)h[2 * n + i];
+      const long long c_i = (long long)(h[i] - seen[i]);
+      const long long sw_i = (long long)(h[n + i] - seen[n + i]);
+      const long long rf_i = (long long)(h[2 * n + i] - seen[2 * n + i]);
       if (!active[i]) continue;
       cs.collapses[i] += c_i;
       cs.flips[i] += sw_i;
@@ -365,20 +339,20 @@ pm_status adapt_set(MeshSet& m, const pm_params* P, int stride, CallStats& cs) {
         active[i] = 0;
       }
     }
+    std::copy(h, h + 3 * (size_t)n, seen.begin());
   }
-  std::vector<int> all(n, 1);
-  cudaMemcpyAsync(m.S.tab.active, all.data(), n * sizeof(int), cudaMemcpyHostToDevice, m.stream);
+  send_active(std::vector<int>(n, 1));
   int sweeps = 0, opt = 0;
   for (int i = 0; i < n; ++i) {
     sweeps = std::max(sweeps, P[stride ? i : 0].max_smooth_sweeps);
     opt = std::max(opt, P[stride ? i : 0].opt_smooth_rounds);
   }
-  pm_status s;
-  const int mr = P[0].max_rounds;
-  if ((s = run_counted(m, [&] { return op_smooth(m, sweeps, mr); }, cs.moves))) return s;
+  select_ops(m, OS_SMOOTH);
+  if ((err = op_smooth(m, sweeps, mr))) return (pm_status)err;
   if (opt > 0)
-    if ((s = run_counted(m, [&] { return op_opt_smooth(m, opt, mr); }, cs.moves))) return s;
-  int err = renumber(m, true);
+    if ((err = op_opt_smooth(m, opt, mr))) return (pm_status)err;
+  err = renumber(m, true);
+  for (int i = 0; !err && i < n; ++i) cs.moves[i] = (long long)m.hops[3 * (size_t)n + i];
   return (pm_status)err;
 }
 
@@ -392,35 +366,46 @@ pm_status run_op(pm_mesh* h, const pm_params* P, pm_stats* st, OpKind kind) {
   if ((s = begin_call(m, P, 0))) return s;
   CallStats cs;
   cs.init(1);
+  if (kind == OP_COARSEN || kind == OP_SWAP || kind == OP_REFINE) m.dense = false;
+  int err = 0;
   switch (kind) {
     case OP_COARSEN:
-      s = run_counted(m, [&] { return op_coarsen(m, P->max_rounds); }, cs.collapses);
+      select_ops(m, OS_COARSEN);
+      err = op_coarsen(m, P->max_rounds);
       break;
     case OP_SWAP:
-      s = run_counted(m, [&] { return op_swap(m, P->max_rounds); }, cs.flips);
+      select_ops(m, OS_SWAP);
+      err = op_swap(m, P->max_rounds);
       break;
     case OP_REFINE:
-      s = run_counted(m, [&] { return op_refine(m, P->max_rounds); }, cs.splits);
+      select_ops(m, OS_REFINE);
+      err = op_refine(m, P->max_rounds);
       break;
     case OP_SMOOTH:
-      s = run_counted(m, [&] { return op_smooth(m, P->max_smooth_sweeps, P->max_rounds); },
-                      cs.moves);
-      if (!s && P->opt_smooth_rounds > 0)
-        s = run_counted(m, [&] { return op_opt_smooth(m, P->opt_smooth_rounds, P->max_rounds); },
-                        cs.moves);
+      select_ops(m, OS_SMOOTH);
+      err = op_smooth(m, P->max_smooth_sweeps, P->max_rounds);
+      if (!err && P->opt_smooth_rounds > 0)
+        err = op_opt_smooth(m, P->opt_smooth_rounds, P->max_rounds);
       break;
     case OP_OPT:
-      s = run_counted(m, [&] { return op_opt_smooth(m, P->opt_smooth_rounds, P->max_rounds); },
-                      cs.moves);
+      select_ops(m, OS_SMOOTH);
+      err = op_opt_smooth(m, P->opt_smooth_rounds, P->max_rounds);
       break;
     case OP_ADAPT:
-      s = adapt_set(m, P, 0, cs);
+      m.dense = false;
+      if ((s = adapt_set(m, P, 0, cs))) return s;
       break;
   }
-  if (s) return s;
-  int err = sync_status(m);
   if (err) return (pm_status)err;
-  return fill_stats(m, cs, t0, st, 1);
+  if (kind != OP_ADAPT) {  // (an adaptation ends with this read-back)
+    if ((err = sync_call(m))) return (pm_status)err;
+    cs.collapses[0] = (long long)m.hops[OS_COARSEN];
+    cs.flips[0] = (long long)m.hops[OS_SWAP];
+    cs.splits[0] = (long long)m.hops[OS_REFINE];
+    cs.moves[0] = (long long)m.hops[OS_SMOOTH];
+  }
+  fill_stats(m, cs, t0, st, 1);
+  return PM_OK;
 }
 
 // ---- batching ------------------------------------------------------------------
@@ -568,18 +553,21 @@ static pm_status set_metric_impl(pm_mesh* h, const double* M, bool host) {
     }
     src = tmp;
   }
-  // checked on the device, from host and device arrays alike
-  PM_LAUNCH(k_metric_check, grid_for(m, nv), BLOCK, 0, m.stream, src, nv, m.st);
-  if (int err = sync_status(m)) {
-    cudaMemsetAsync(m.st, 0, sizeof(DevStatus), m.stream);
-    if (tmp) cudaFreeAsync(tmp, m.stream);
-    return fail((pm_status)err, "metric must be finite and symmetric positive definite");
-  }
+  // checked on the device, from host and device arrays alike; a rejected metric
+  // leaves the mesh as it is
   pm_status s = cuda_status(upload_prefix(m, m.nv, m.ne), "mesh offsets");
-  if (!s) PM_LAUNCH(k_metric_set, grid_for(m, nv), BLOCK, 0, m.stream, m.S, src, nv);
+  if (!s) {
+    PM_LAUNCH(k_metric_check, grid_for(m, nv), BLOCK, 0, m.stream, src, nv, m.st);
+    PM_LAUNCH(k_metric_set, grid_for(m, nv), BLOCK, 0, m.stream, m.S, src, nv,
+              (const DevStatus*)m.st);
+  }
   if (tmp) cudaFreeAsync(tmp, m.stream);
   if (s) return s;
-  return (pm_status)refresh_quality(m);
+  if (int err = refresh_quality(m)) {
+    cudaMemsetAsync(m.st, 0, sizeof(DevStatus), m.stream);
+    return fail((pm_status)err, "metric must be finite and symmetric positive definite");
+  }
+  return PM_OK;
 }
 
 pm_status pm_set_metric(pm_mesh* h, const double* M) { return set_metric_impl(h, M, true); }
@@ -660,6 +648,7 @@ pm_status pm_adapt_batch(pm_mesh** meshes, int32_t n, const pm_params* params, p
   cs.init(n);
   if (!st) st = begin_call(b, params, 1);
   if (!st) st = adapt_set(b, params, 1, cs);
+  if (!st && stats) fill_stats(b, cs, t0, stats, n);
   // results back into each mesh (growing it where needed)
   for (int i = 0; i < n && !st; ++i) {
     MeshSet& s = meshes[i]->set;
@@ -673,11 +662,14 @@ pm_status pm_adapt_batch(pm_mesh** meshes, int32_t n, const pm_params* params, p
     if (st) break;
     s.nv[0] = b.nv[i];
     s.ne[0] = b.ne[i];
+    s.dense = b.dense;
+    s.S.lid = s.S.voff = nullptr;  // ids are the slot offsets of the compacted copy
     st = cuda_status(upload_tab(s), "mesh table");
     if (!st) st = copy_region(s, 0, b, i, b.stream);
   }
   if (!st) st = (pm_status)sync_status(b);
-  if (!st && stats) st = fill_stats(b, cs, t0, stats, n);
+  if (!st && stats)
+    for (int i = 0; i < n; ++i) stats[i].ms = now_ms() - t0;
   set_free(b);
   set_release(b);
   return st;
@@ -896,10 +888,10 @@ pm_status pm_batch_adapt(pm_mesh* h, const pm_params* params, pm_stats* stats) {
   if (s) return s;
   CallStats cs;
   cs.init(m.nmesh);
+  m.dense = false;
   if ((s = adapt_set(m, params, 1, cs))) return s;
-  int err = sync_status(m);
-  if (err) return (pm_status)err;
-  return fill_stats(m, cs, t0, stats, m.nmesh);
+  fill_stats(m, cs, t0, stats, m.nmesh);
+  return PM_OK;
 }
 
 static pm_status batch_get(pm_mesh* h, int32_t* nv, int32_t* ne, double* xy, int32_t* tri,

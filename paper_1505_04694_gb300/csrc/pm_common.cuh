@@ -33,8 +33,7 @@ struct MeshTab {
   uint32_t* r;  // round counter of the current call
   int* had;     // 1 when the mesh formed candidates this round (2 * nmesh)
   int* active;  // mesh takes part in the current phase
-  unsigned long long* ops;       // operations applied in the current call
-  unsigned long long* iter_ops;  // operations of the current outer iteration
+  unsigned long long* ops;       // operations applied in the current call, of the running operator
   double* L_low;                 // per-mesh parameters
   double* L_up;
   double* q_thresh;
@@ -97,7 +96,7 @@ struct DevStatus {
   int err;       // pm_status set by a kernel (first writer wins)
   int overflow;  // an adjacency row would exceed W
   int maxdeg;    // largest row length seen by the last adjacency build
-  int pad;
+  int where;     // 1: the error was found in the input elements themselves
 };
 
 // ---------------------------------------------------------------------------

@@ -23,8 +23,6 @@ struct ScanWork {
 
 int scan_tiles(int n);
 void scan_exclusive(const int* in, int* out, int n, ScanWork& w, DevStatus* st, cudaStream_t s);
-void scan_exclusive_cleared(const int* in, int* out, int n, ScanWork& w, DevStatus* st,
-                            cudaStream_t s);
 void scan_alive_vertices(const Store& S, int* out, int n, ScanWork& w, DevStatus* st,
                          cudaStream_t s);
 void scan_alive_elements(const Store& S, int* out, int n, ScanWork& w, DevStatus* st,
@@ -104,7 +102,10 @@ struct MeshSet {
   DevStatus* st = nullptr;     // device
   DevStatus* hst = nullptr;    // pinned host
   int* hcounts = nullptr;      // pinned host copy of w.counts
-  unsigned long long* hops = nullptr;  // pinned: operation counts of three operators (3 * nmesh)
+  unsigned long long* hops = nullptr;  // pinned: operation counts (see OpSlot, 4 * nmesh)
+  uint32_t* hr = nullptr;              // pinned: round counters
+  unsigned long long* ops = nullptr;   // device: operation counts of the call (4 * nmesh)
+  bool dense = false;  // no dead slot: ids are the slot offsets and the sizes are nv, ne
   char* hup = nullptr;                 // pinned: staging of the per-mesh table for upload_tab
   cudaEvent_t upev = nullptr;          // the last table upload has left the staging
   void* pinned = nullptr;      // slot of the process-wide pinned arena (hst, hcounts)
@@ -141,7 +142,11 @@ int compact_out(MeshSet& m, int mesh, double* xy, int32_t* tri, double* mt, int*
                 int* ne_out);
 int compact_out_set(MeshSet& m, double* xy, int32_t* tri, double* mt, int* nv_out, int* ne_out);
 int sync_status(MeshSet& m);
-int validate_mesh(MeshSet& m);
+// The status, the counters and the per-mesh words after them (`extra` ints) in
+// one copy; then the whole call state (operation counts and rounds too).
+int sync_counts(MeshSet& m, int extra);
+int sync_call(MeshSet& m);
+void validate_mesh(MeshSet& m);
 int refresh_quality(MeshSet& m);
 // The quality cache of every element, computed now when it is stale (a mesh
 // whose metric was never set gets it at its first operator call).
@@ -154,8 +159,9 @@ int op_swap(MeshSet& m, int max_rounds);
 int op_refine(MeshSet& m, int max_rounds);
 int op_smooth(MeshSet& m, int max_sweeps, int max_rounds);
 int op_opt_smooth(MeshSet& m, int nrounds, int max_rounds);
-void zero_ops(MeshSet& m);
-cudaError_t fetch_ops(MeshSet& m, std::vector<unsigned long long>& ops);
+// Operation counters of a call: one set per operator, selected before it runs.
+enum OpSlot { OS_COARSEN = 0, OS_SWAP, OS_REFINE, OS_SMOOTH };
+inline void select_ops(MeshSet& m, OpSlot k) { m.S.tab.ops = m.ops + (size_t)k * m.nmesh; }
 
 // ---- quality (pm_quality.cu) ----
 int quality_mesh(MeshSet& m, double* qsum_host, double* dxy_host, double* dm_host);

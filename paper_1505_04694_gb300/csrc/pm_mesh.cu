@@ -22,8 +22,8 @@ namespace {
 // process: page-locking is slow and gets slower after many allocate/free
 // cycles, so slots of one arena are handed out and recycled instead.
 constexpr size_t kPinnedSlot = 16384;
-// staging per mesh of upload_tab: band (double4, float4), L_low/L_up/q_thresh,
-// seven ints, the seed
+// staging per mesh of upload_tab, laid out like the device table's first part:
+// band (double4, float4), L_low/L_up/q_thresh, seven ints, the seed
 constexpr size_t kTabUploadBytes = sizeof(double4) + sizeof(float4) + 3 * sizeof(double) +
                                    7 * sizeof(int) + sizeof(uint32_t);
 constexpr size_t kPinnedBlock = 64 * kPinnedSlot;
@@ -213,6 +213,7 @@ __global__ void k_zero_nelen(Store S) {
 }
 
 __global__ void k_fill_ne(Store S, DevStatus* st) {
+  if (st->err) return;  // invalid input: ids may be out of range
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < S.eused; s += gridDim.x * blockDim.x) {
     int mi;
     if (!eslot_used(S, s, mi)) continue;
@@ -236,6 +237,7 @@ __global__ void k_fill_ne(Store S, DevStatus* st) {
 // flag (a vertex is on the boundary when it has one more neighbour than
 // incident elements).
 __global__ void k_finish_rows(Store S, int derive, DevStatus* st) {
+  if (st->err && st->where) return;  // invalid input: no rows were filled
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < S.vused; s += gridDim.x * blockDim.x) {
     int mi;
     if (!vslot_used(S, s, mi)) continue;
@@ -312,7 +314,8 @@ __device__ __forceinline__ int edge_elements(const Store& S, int slot, int eb, i
 
 // Corners: boundary vertices whose two boundary neighbours are not collinear
 // with them, or (given) the caller's flags, already set in vflag by the ingest.
-__global__ void k_corners(Store S, int given) {
+__global__ void k_corners(Store S, int given, const DevStatus* st) {
+  if (st->err || st->overflow) return;  // no rows, or rows to be built again
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < S.vused; s += gridDim.x * blockDim.x) {
     int mi;
     if (!vslot_used(S, s, mi)) continue;
@@ -348,12 +351,16 @@ __global__ void k_validate_coords(Store S, DevStatus* st) {
     const int mi = mesh_of_vslot(S, s);
     if (s - S.tab.vbase[mi] >= S.tab.nv[mi]) continue;
     const double2 p = S.xy[s];
-    if (!isfinite(p.x) || !isfinite(p.y)) set_err(st, PM_ERR_INVALID_ARG);
+    if (!isfinite(p.x) || !isfinite(p.y)) {
+      set_err(st, PM_ERR_INVALID_ARG);
+      st->where = 1;
+    }
   }
 }
 
 // Ids in range, distinct, and every element counter-clockwise (canonical).
 __global__ void k_validate_elems(Store S, DevStatus* st) {
+  if (st->err) return;  // orientations of non-finite points mean nothing
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < S.eused; s += gridDim.x * blockDim.x) {
     int mi;
     if (!eslot_used(S, s, mi)) continue;
@@ -363,15 +370,19 @@ __global__ void k_validate_elems(Store S, DevStatus* st) {
     if (e.x < 0 || e.y < 0 || e.z < 0 || e.x >= nv || e.y >= nv || e.z >= nv || e.x == e.y ||
         e.y == e.z || e.x == e.z) {
       set_err(st, PM_ERR_INVALID_MESH);
+      st->where = 1;
       continue;
     }
-    if (orient_sign(load_vd(S, vb + e.x), load_vd(S, vb + e.y), load_vd(S, vb + e.z)) <= 0)
+    if (orient_sign(load_vd(S, vb + e.x), load_vd(S, vb + e.y), load_vd(S, vb + e.z)) <= 0) {
       set_err(st, PM_ERR_INVALID_MESH);
+      st->where = 1;
+    }
   }
 }
 
-// Quality of every live element into the cache.
-__global__ void k_qcache_all(Store S) {
+// Quality of every live element into the cache (not after a rejected metric).
+__global__ void k_qcache_all(Store S, const DevStatus* st) {
+  if (st->err) return;
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < S.eused; s += gridDim.x * blockDim.x) {
     int mi;
     if (!eslot_used(S, s, mi)) continue;
@@ -391,6 +402,14 @@ __global__ void k_set_sizes(Store S, const int* tot) {
   if (i >= S.nmesh) return;
   S.tab.nv[i] = tot[2 * i];
   S.tab.ne[i] = tot[2 * i + 1];
+}
+
+// The table's sizes in the layout of k_mesh_totals (no dead slot).
+__global__ void k_table_totals(Store S, int* out) {
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= S.nmesh) return;
+  out[2 * i] = S.tab.nv[i];
+  out[2 * i + 1] = S.tab.ne[i];
 }
 
 // Live counts of every mesh; with `changed`, records whether any mesh has a
@@ -423,7 +442,7 @@ __device__ __forceinline__ void renum_row(const int* row, int len, int* out, con
 
 __global__ void k_renum_v(Store A, Store B, const int* vscan, const int* escan,
                           const int* changed) {
-  if (!*changed) return;  // nothing died since the last compaction
+  if (changed && !*changed) return;  // nothing died since the last compaction
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < A.vused; s += gridDim.x * blockDim.x) {
     int mi;
     if (!vslot_used(A, s, mi)) continue;
@@ -466,7 +485,7 @@ __global__ void k_renum_ids(Store S, const int* vscan, const int* tot, int* lid,
 
 __global__ void k_renum_e(Store A, Store B, const int* vscan, const int* escan,
                           const int* changed) {
-  if (!*changed) return;
+  if (changed && !*changed) return;
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < A.eused; s += gridDim.x * blockDim.x) {
     int mi;
     if (!eslot_used(A, s, mi)) continue;
@@ -481,13 +500,14 @@ __global__ void k_renum_e(Store A, Store B, const int* vscan, const int* escan,
 }
 
 // Compacted output of one mesh (canonical rotation of every triangle).
+// `vscan` / `escan` null: no slot is dead, positions are the slot offsets.
 __global__ void k_out_v(Store S, int mesh, const int* vscan, double* xy, double* mt) {
   int vb = S.tab.vbase[mesh], nv = S.tab.nv[mesh];
-  int v0 = vscan[vb];
+  int v0 = vscan ? vscan[vb] : 0;
   for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nv; l += gridDim.x * blockDim.x) {
     int s = vb + l;
     if (!(S.vflag[s] & VF_ALIVE)) continue;
-    int o = vscan[s] - v0;
+    int o = vscan ? vscan[s] - v0 : l;
     double2 p = S.xy[s];
     double4 m = S.M[s];
     if (xy) {
@@ -504,13 +524,18 @@ __global__ void k_out_v(Store S, int mesh, const int* vscan, double* xy, double*
 
 __global__ void k_out_e(Store S, int mesh, const int* vscan, const int* escan, int32_t* tri) {
   int vb = S.tab.vbase[mesh], eb = S.tab.ebase[mesh], ne = S.tab.ne[mesh];
-  int v0 = vscan[vb], e0 = escan[eb];
+  int v0 = vscan ? vscan[vb] : 0, e0 = escan ? escan[eb] : 0;
   for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < ne; l += gridDim.x * blockDim.x) {
     int s = eb + l;
     int4 e = S.EN[s];
     if (!e.w) continue;
-    int o = escan[s] - e0;
-    int a = vscan[vb + e.x] - v0, b = vscan[vb + e.y] - v0, c = vscan[vb + e.z] - v0;
+    int o = escan ? escan[s] - e0 : l;
+    int a = e.x, b = e.y, c = e.z;
+    if (vscan) {
+      a = vscan[vb + e.x] - v0;
+      b = vscan[vb + e.y] - v0;
+      c = vscan[vb + e.z] - v0;
+    }
     if (b < a && b < c) {
       int t = a; a = b; b = c; c = t;
     } else if (c < a && c < b) {
@@ -603,7 +628,7 @@ __global__ void k_out_v_set(Store S, const int* vscan, double* xy, double* mt) {
     if (!vslot_used(S, s, mi)) continue;
     if (!(S.vflag[s] & VF_ALIVE)) continue;
     int vb = S.tab.vbase[mi];
-    int o = S.tab.pre[mi] + (vscan[s] - vscan[vb]);
+    int o = S.tab.pre[mi] + (vscan ? vscan[s] - vscan[vb] : s - vb);
     double2 p = S.xy[s];
     double4 m = S.M[s];
     if (xy) {
@@ -626,9 +651,14 @@ __global__ void k_out_e_set(Store S, const int* vscan, const int* escan, int32_t
     int4 e = S.EN[s];
     if (!e.w) continue;
     int vb = S.tab.vbase[mi], eb = S.tab.ebase[mi];
-    int v0 = vscan[vb];
-    int o = S.tab.pre[n + 1 + mi] + (escan[s] - escan[eb]);
-    int a = vscan[vb + e.x] - v0, b = vscan[vb + e.y] - v0, c = vscan[vb + e.z] - v0;
+    int o = S.tab.pre[n + 1 + mi] + (escan ? escan[s] - escan[eb] : s - eb);
+    int a = e.x, b = e.y, c = e.z;
+    if (vscan) {
+      const int v0 = vscan[vb];
+      a = vscan[vb + e.x] - v0;
+      b = vscan[vb + e.y] - v0;
+      c = vscan[vb + e.z] - v0;
+    }
     if (b < a && b < c) {
       int t = a; a = b; b = c; c = t;
     } else if (c < a && c < b) {
@@ -690,14 +720,8 @@ cudaError_t upload_tab(MeshSet& m) {
                            std::nextafterf((float)band[i].z, -big),
                            std::nextafterf((float)band[i].w, big));
   }
-  cudaError_t e = cudaMemcpyAsync(m.S.tab.vbase, ints, 7 * n * sizeof(int), cudaMemcpyHostToDevice,
+  cudaError_t e = cudaMemcpyAsync(m.S.tab.band, band, n * kTabUploadBytes, cudaMemcpyHostToDevice,
                                   m.stream);
-  if (!e) e = cudaMemcpyAsync(m.S.tab.seed, seed, n * sizeof(uint32_t), cudaMemcpyHostToDevice,
-                              m.stream);
-  if (!e) e = cudaMemcpyAsync(m.S.tab.L_low, dbl, 3 * n * sizeof(double), cudaMemcpyHostToDevice,
-                              m.stream);
-  if (!e) e = cudaMemcpyAsync(m.S.tab.band, band, n * (sizeof(double4) + sizeof(float4)),
-                              cudaMemcpyHostToDevice, m.stream);
   if (!e && m.upev) e = cudaEventRecord(m.upev, m.stream);
   if (!e && !m.mesh_index_ok) {
     PM_LAUNCH(k_mesh_index, grid_for(m, m.S.vslots), BLOCK, 0, m.stream, n,
@@ -771,9 +795,7 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   Carver cv;
   carve_store(cv, S);
   carve_store(cv, m.B);
-  size_t tab_bytes = (size_t)n * (8 * sizeof(int) + 2 * sizeof(uint32_t) + 3 * sizeof(int) +
-                                  2 * sizeof(unsigned long long) + 3 * sizeof(double) +
-                                  sizeof(double4) + sizeof(float4)) +
+  size_t tab_bytes = (size_t)n * (kTabUploadBytes + sizeof(int)) +
                      2 * ((size_t)n + 1) * sizeof(int) + 64;
   char* t = nullptr;
   cv.add(&t, tab_bytes, true);
@@ -816,7 +838,6 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   cv.add(&w.E, vs);
   cv.add(&w.items2, vs);
   cv.add(&w.ncand, vs);
-  cv.add(&w.counts, CN_NUM + 2 * n + 8, true);
   cv.add(&w.cprop, vs);
   cv.add(&w.cstamp, vs, true);
   cv.add(&m.lidbuf, vs);
@@ -836,8 +857,6 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   T.L_low = (double*)t; t += n * sizeof(double);
   T.L_up = (double*)t; t += n * sizeof(double);
   T.q_thresh = (double*)t; t += n * sizeof(double);
-  T.ops = (unsigned long long*)t; t += n * sizeof(unsigned long long);
-  T.iter_ops = (unsigned long long*)t; t += n * sizeof(unsigned long long);
   T.vbase = (int*)t; t += n * sizeof(int);
   T.vcap = (int*)t; t += n * sizeof(int);
   T.ebase = (int*)t; t += n * sizeof(int);
@@ -845,23 +864,26 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   T.nv = (int*)t; t += n * sizeof(int);
   T.ne = (int*)t; t += n * sizeof(int);
   T.select = (int*)t; t += n * sizeof(int);
-  T.ncol = (int*)t; t += n * sizeof(int);
   T.seed = (uint32_t*)t; t += n * sizeof(uint32_t);
-  T.r = (uint32_t*)t; t += n * sizeof(uint32_t);
-  T.had = (int*)t; t += 2 * n * sizeof(int);  // two sets: persistent rounds alternate
-  T.active = (int*)t; t += n * sizeof(int);
+  T.ncol = (int*)t; t += n * sizeof(int);
   T.pre = (int*)t; t += 2 * ((size_t)n + 1) * sizeof(int);
   T.vmesh = vmesh;
   T.emesh = emesh;
   T.col = col;
   m.mesh_index_ok = n == 1;
-  m.B.tab = T;
+  // State of a call, kept over growths: status, counters (and two words per mesh
+  // after them), operation counts, round counters, candidate flags, active flags.
+  // The host reads it back in one copy, into a pinned image of its first part.
+  const size_t counts_bytes = (CN_NUM + 2 * (size_t)n + 8) * sizeof(int);
+  const size_t ops_off = 64 + ((counts_bytes + 7) & ~size_t(7));
+  const size_t r_off = ops_off + 4 * (size_t)n * sizeof(unsigned long long);
+  const size_t had_off = r_off + (size_t)n * sizeof(uint32_t);
+  const size_t act_off = had_off + 2 * (size_t)n * sizeof(int);
   if (!m.st) {
-    if ((e = cudaMallocAsync((void**)&m.st, sizeof(DevStatus), m.stream))) return e;
-    if ((e = cudaMemsetAsync(m.st, 0, sizeof(DevStatus), m.stream))) return e;
-    const size_t counts_bytes = (CN_NUM + 2 * (size_t)std::max(n, 1024) + 8) * sizeof(int);
-    const size_t ops_off = 64 + ((counts_bytes + 7) & ~size_t(7));
-    const size_t up_off = (ops_off + 3 * (size_t)n * sizeof(unsigned long long) + 63) & ~size_t(63);
+    const size_t bytes = act_off + (size_t)n * sizeof(int);
+    if ((e = cudaMallocAsync((void**)&m.st, bytes, m.stream))) return e;
+    if ((e = cudaMemsetAsync(m.st, 0, bytes, m.stream))) return e;
+    const size_t up_off = (had_off + 63) & ~size_t(63);
     size_t need = up_off + (size_t)n * kTabUploadBytes;
     if (need <= kPinnedSlot) {
       m.pinned = pinned_get();
@@ -874,9 +896,17 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
     m.hst = (DevStatus*)m.pinned;
     m.hcounts = (int*)((char*)m.pinned + 64);
     m.hops = (unsigned long long*)((char*)m.pinned + ops_off);
+    m.hr = (uint32_t*)((char*)m.pinned + r_off);
     m.hup = (char*)m.pinned + up_off;
     if ((e = cudaEventCreateWithFlags(&m.upev, cudaEventDisableTiming))) return e;
   }
+  char* call = (char*)m.st;
+  w.counts = (int*)(call + 64);
+  m.ops = T.ops = (unsigned long long*)(call + ops_off);
+  T.r = (uint32_t*)(call + r_off);
+  T.had = (int*)(call + had_off);  // two sets: persistent rounds alternate
+  T.active = (int*)(call + act_off);
+  m.B.tab = T;
   return cudaSuccess;
 }
 
@@ -898,6 +928,7 @@ void set_release(MeshSet& m) {
   m.hst = nullptr;
   m.hcounts = nullptr;
   m.hops = nullptr;
+  m.hr = nullptr;
   m.hup = nullptr;
   m.upev = nullptr;
 }
@@ -919,6 +950,7 @@ cudaError_t grow(MeshSet& m, const std::vector<int>& vcap, const std::vector<int
   n2.hst = m.hst;
   n2.hcounts = m.hcounts;
   n2.hops = m.hops;
+  n2.hr = m.hr;
   n2.hup = m.hup;
   n2.upev = m.upev;
   n2.num_sms = m.num_sms;
@@ -931,13 +963,7 @@ cudaError_t grow(MeshSet& m, const std::vector<int>& vcap, const std::vector<int
     set_free(n2);
     return e;
   }
-  // carry the per-call round counters and op counts
-  int nm = m.nmesh;
-  cudaMemcpyAsync(n2.S.tab.r, m.S.tab.r, nm * sizeof(uint32_t), cudaMemcpyDeviceToDevice, m.stream);
-  cudaMemcpyAsync(n2.S.tab.active, m.S.tab.active, nm * sizeof(int), cudaMemcpyDeviceToDevice,
-                  m.stream);
-  cudaMemcpyAsync(n2.S.tab.ops, m.S.tab.ops, 2 * nm * sizeof(unsigned long long),
-                  cudaMemcpyDeviceToDevice, m.stream);
+  const int nm = m.nmesh;
   if (m.S.lid) {  // ids that are not slot offsets move with their slots
     n2.S.lid = n2.lidbuf;
     n2.S.voff = n2.voffbuf;
@@ -950,6 +976,7 @@ cudaError_t grow(MeshSet& m, const std::vector<int>& vcap, const std::vector<int
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   set_free(m);
+  n2.S.tab.ops = m.S.tab.ops;  // the running operator's counters
   m.vbase = n2.vbase;
   m.vcap = n2.vcap;
   m.ebase = n2.ebase;
@@ -991,6 +1018,24 @@ int sync_status(MeshSet& m) {
   return m.hst->err;
 }
 
+static int sync_bytes(MeshSet& m, size_t bytes) {
+  cudaError_t e = cudaMemcpyAsync(m.hst, m.st, bytes, cudaMemcpyDeviceToHost, m.stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(m.stream);
+  if (e != cudaSuccess) {
+    set_last_error(std::string("CUDA: ") + cudaGetErrorString(e));
+    return PM_ERR_CUDA;
+  }
+  return m.hst->err;
+}
+
+int sync_counts(MeshSet& m, int extra) {
+  return sync_bytes(m, 64 + (CN_NUM + (size_t)extra) * sizeof(int));
+}
+
+int sync_call(MeshSet& m) {
+  return sync_bytes(m, (size_t)((char*)(m.S.tab.r + m.nmesh) - (char*)m.st));
+}
+
 // Build NN and NE from the element list for every mesh of the set.  With
 // `derive_flags` (creation) also derive boundary and corner flags and check
 // manifoldness.  Grows W (rebuilding) when a row does not fit.
@@ -1001,6 +1046,10 @@ int rebuild_adjacency(MeshSet& m, bool derive_flags, bool corners_given) {
     PM_LAUNCH(k_fill_ne, grid_for(m, m.S.eused), BLOCK, 0, m.stream, m.S, m.st);
     PM_LAUNCH(k_finish_rows, grid_for(m, m.S.vused), BLOCK, 0, m.stream, m.S, derive_flags ? 1 : 0,
                                                                   m.st);
+    // (skipped on the device when the rows have to be built again)
+    if (derive_flags)
+      PM_LAUNCH(k_corners, grid_for(m, m.S.vused), BLOCK, 0, m.stream, m.S, corners_given ? 1 : 0,
+                (const DevStatus*)m.st);
     int err = sync_status(m);
     if (err) return err;
     if (!m.hst->overflow) break;
@@ -1017,27 +1066,24 @@ int rebuild_adjacency(MeshSet& m, bool derive_flags, bool corners_given) {
       return e == cudaErrorMemoryAllocation ? PM_ERR_OOM : PM_ERR_CUDA;
     }
   }
-  if (derive_flags) {
-    PM_LAUNCH(k_corners, grid_for(m, m.S.vused), BLOCK, 0, m.stream, m.S, corners_given ? 1 : 0);
-    return sync_status(m);
-  }
   return PM_OK;
 }
 
 int refresh_quality(MeshSet& m) {
-  PM_LAUNCH(k_qcache_all, grid_for(m, m.S.eused), BLOCK, 0, m.stream, m.S);
-  m.qvalid = true;
-  return sync_status(m);
+  PM_LAUNCH(k_qcache_all, grid_for(m, m.S.eused), BLOCK, 0, m.stream, m.S,
+            (const DevStatus*)m.st);
+  const int err = sync_status(m);
+  if (!err) m.qvalid = true;
+  return err;
 }
 
 int ensure_quality(MeshSet& m) { return m.qvalid ? PM_OK : refresh_quality(m); }
 
-int validate_mesh(MeshSet& m) {
+// Queues the checks of the input; the adjacency build that follows skips what a
+// found error makes unsafe and reads the status back.
+void validate_mesh(MeshSet& m) {
   PM_LAUNCH(k_validate_coords, grid_for(m, m.S.vused), BLOCK, 0, m.stream, m.S, m.st);
-  int err = sync_status(m);
-  if (err) return err;  // orientations of non-finite points mean nothing
   PM_LAUNCH(k_validate_elems, grid_for(m, m.S.eused), BLOCK, 0, m.stream, m.S, m.st);
-  return sync_status(m);
 }
 
 // Renumbering of every mesh: live vertices and elements in ascending slot
@@ -1051,8 +1097,9 @@ int renumber(MeshSet& m, bool final) {
   scan_alive_vertices(m.S, w.vscan, m.S.vused, m.scan, m.st, m.stream);
   scan_alive_elements(m.S, w.escan, m.S.eused, m.scan, m.st, m.stream);
   int* tot = w.counts + CN_NUM;
-  int* changed = w.counts + CN_RENUM;
-  cudaMemsetAsync(changed, 0, sizeof(int), m.stream);
+  // (only the compaction queued below looks at the flag)
+  int* changed = final ? w.counts + CN_RENUM : nullptr;
+  if (final) cudaMemsetAsync(changed, 0, sizeof(int), m.stream);
   PM_LAUNCH(k_mesh_totals, (m.nmesh + 127) / 128, 128, 0, m.stream, m.S, w.vscan, w.escan, tot,
             changed);
   // compaction into the second buffer set (skipped on the device when no
@@ -1061,22 +1108,27 @@ int renumber(MeshSet& m, bool final) {
     // the second buffer's flags must read "dead" beyond the new counts
     cudaMemsetAsync(m.B.vflag, 0, m.S.vslots, m.stream);
     PM_LAUNCH(k_renum_v, grid_for(m, m.S.vused), BLOCK, 0, m.stream, m.S, m.B, w.vscan, w.escan,
-              changed);
+              (const int*)changed);
     PM_LAUNCH(k_renum_e, grid_for(m, m.S.eused), BLOCK, 0, m.stream, m.S, m.B, w.vscan, w.escan,
-              changed);
+              (const int*)changed);
     PM_LAUNCH(k_set_sizes, (m.nmesh + 127) / 128, 128, 0, m.stream, m.S, tot);
   };
   if (final) compact();  // queued before the read-back: one synchronisation
-  cudaMemcpyAsync(m.hcounts, tot, 2 * m.nmesh * sizeof(int), cudaMemcpyDeviceToHost, m.stream);
-  cudaMemcpyAsync(m.hcounts + 2 * m.nmesh, changed, sizeof(int), cudaMemcpyDeviceToHost, m.stream);
-  int err = sync_status(m);
+  // sizes, operation counts, rounds and status in one read-back
+  int err = sync_call(m);
   if (err) return err;
-  if (!m.hcounts[2 * m.nmesh]) return PM_OK;  // no dead slot: every id stays
+  const int* ht = m.hcounts + CN_NUM;
+  bool died = false;
+  for (int i = 0; i < m.nmesh; ++i) died |= ht[2 * i] != m.nv[i] || ht[2 * i + 1] != m.ne[i];
+  if (!died) {  // every id stays
+    if (final) m.dense = true;
+    return PM_OK;
+  }
   if (!final) {
     long long vdead = 0, edead = 0;
     for (int i = 0; i < m.nmesh; ++i) {
-      vdead += m.nv[i] - m.hcounts[2 * i];
-      edead += m.ne[i] - m.hcounts[2 * i + 1];
+      vdead += m.nv[i] - ht[2 * i];
+      edead += m.ne[i] - ht[2 * i + 1];
     }
     long long vu = 0, eu = 0;
     for (int i = 0; i < m.nmesh; ++i) {
@@ -1093,9 +1145,10 @@ int renumber(MeshSet& m, bool final) {
     compact();
   }
   for (int i = 0; i < m.nmesh; ++i) {
-    m.nv[i] = m.hcounts[2 * i];
-    m.ne[i] = m.hcounts[2 * i + 1];
+    m.nv[i] = ht[2 * i];
+    m.ne[i] = ht[2 * i + 1];
   }
+  if (final) m.dense = true;
   std::swap(m.S.xy, m.B.xy);
   std::swap(m.S.M, m.B.M);
   std::swap(m.S.F, m.B.F);
@@ -1123,6 +1176,17 @@ int renumber(MeshSet& m, bool final) {
 int compact_out(MeshSet& m, int mesh, double* xy, int32_t* tri, double* mt, int* nv_out,
                 int* ne_out) {
   Work& w = m.w;
+  if (m.dense) {  // nothing to count and nothing to move together
+    *nv_out = m.nv[mesh];
+    *ne_out = m.ne[mesh];
+    if (xy || mt)
+      PM_LAUNCH(k_out_v, grid_for(m, m.nv[mesh]), BLOCK, 0, m.stream, m.S, mesh,
+                (const int*)nullptr, xy, mt);
+    if (tri)
+      PM_LAUNCH(k_out_e, grid_for(m, m.ne[mesh]), BLOCK, 0, m.stream, m.S, mesh,
+                (const int*)nullptr, (const int*)nullptr, tri);
+    return xy || mt || tri ? sync_status(m) : PM_OK;
+  }
   scan_alive_vertices(m.S, w.vscan, m.S.vused, m.scan, m.st, m.stream);
   scan_alive_elements(m.S, w.escan, m.S.eused, m.scan, m.st, m.stream);
   int* tot = w.counts + CN_NUM;
@@ -1133,11 +1197,10 @@ int compact_out(MeshSet& m, int mesh, double* xy, int32_t* tri, double* mt, int*
   if (tri)
     PM_LAUNCH(k_out_e, grid_for(m, m.ne[mesh]), BLOCK, 0, m.stream, m.S, mesh, w.vscan, w.escan,
               tri);
-  cudaMemcpyAsync(m.hcounts, tot, 2 * m.nmesh * sizeof(int), cudaMemcpyDeviceToHost, m.stream);
-  int err = sync_status(m);
+  int err = sync_counts(m, 2 * m.nmesh);
   if (err) return err;
-  *nv_out = m.hcounts[2 * mesh];
-  *ne_out = m.hcounts[2 * mesh + 1];
+  *nv_out = m.hcounts[CN_NUM + 2 * mesh];
+  *ne_out = m.hcounts[CN_NUM + 2 * mesh + 1];
   return PM_OK;
 }
 
@@ -1147,6 +1210,23 @@ int compact_out(MeshSet& m, int mesh, double* xy, int32_t* tri, double* mt, int*
 int compact_out_set(MeshSet& m, double* xy, int32_t* tri, double* mt, int* nv_out, int* ne_out) {
   Work& w = m.w;
   const int n = m.nmesh;
+  if (m.dense) {
+    for (int i = 0; i < n; ++i) {
+      nv_out[i] = m.nv[i];
+      ne_out[i] = m.ne[i];
+    }
+    if (!xy && !mt && !tri) return PM_OK;
+    int* tot = w.counts + CN_NUM;
+    PM_LAUNCH(k_table_totals, (n + 127) / 128, 128, 0, m.stream, m.S, tot);
+    PM_LAUNCH(k_out_prefix, 1, 1024, 0, m.stream, n, (const int*)tot, m.S.tab.pre);
+    if (xy || mt)
+      PM_LAUNCH(k_out_v_set, grid_for(m, m.S.vused), BLOCK, 0, m.stream, m.S, (const int*)nullptr,
+                xy, mt);
+    if (tri)
+      PM_LAUNCH(k_out_e_set, grid_for(m, m.S.eused), BLOCK, 0, m.stream, m.S, (const int*)nullptr,
+                (const int*)nullptr, tri);
+    return sync_status(m);
+  }
   scan_alive_vertices(m.S, w.vscan, m.S.vused, m.scan, m.st, m.stream);
   scan_alive_elements(m.S, w.escan, m.S.eused, m.scan, m.st, m.stream);
   int* tot = w.counts + CN_NUM;
@@ -1160,12 +1240,11 @@ int compact_out_set(MeshSet& m, double* xy, int32_t* tri, double* mt, int* nv_ou
       PM_LAUNCH(k_out_e_set, grid_for(m, m.S.eused), BLOCK, 0, m.stream, m.S, w.vscan, w.escan,
                 tri);
   }
-  cudaMemcpyAsync(m.hcounts, tot, 2 * n * sizeof(int), cudaMemcpyDeviceToHost, m.stream);
-  int err = sync_status(m);
+  int err = sync_counts(m, 2 * n);
   if (err) return err;
   for (int i = 0; i < n; ++i) {
-    nv_out[i] = m.hcounts[2 * i];
-    ne_out[i] = m.hcounts[2 * i + 1];
+    nv_out[i] = m.hcounts[CN_NUM + 2 * i];
+    ne_out[i] = m.hcounts[CN_NUM + 2 * i + 1];
   }
   return PM_OK;
 }

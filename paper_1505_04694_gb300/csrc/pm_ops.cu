@@ -2913,24 +2913,14 @@ __global__ void k_refine_mark(Store S, int* cnt, RowMask* mask, int tag, int pas
   }
 }
 
-// Per-mesh number of new vertices (edges to split).
-__global__ void k_refine_newcount(Store S, const int* vscan, int* out) {
+// Per-mesh number of new vertices (edges to split), after the counters, with
+// the lists that the round's split fills cleared.
+__global__ void k_refine_newcount(Store S, const int* vscan, int* counts) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) counts[CN_EL] = counts[CN_CL] = 0;
   if (i >= S.nmesh) return;
   int vb = S.tab.vbase[i];
-  out[i] = vscan[vb + S.tab.nv[i]] - vscan[vb];
-}
-
-// A mesh that splits edges counts the round and its splits.
-__global__ void k_refine_vtotals(Store S, const int* vscan) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= S.nmesh) return;
-  int vb = S.tab.vbase[i];
-  int t = vscan[vb + S.tab.nv[i]] - vscan[vb];
-  if (t > 0) {
-    S.tab.r[i] += 1;
-    S.tab.ops[i] += (unsigned long long)t;
-  }
+  counts[CN_NUM + i] = vscan[vb + S.tab.nv[i]] - vscan[vb];
 }
 
 __device__ __forceinline__ int mid_id(const Store& S, int vb, int nv, const int* vscan,
@@ -3145,13 +3135,20 @@ __global__ void k_refine_rows_copy(Store S, Store B, int vend, int stamp) {
   }
 }
 
-__global__ void k_refine_sizes(Store S, const int* vscan, const int* escan) {
+// The sizes after the round, in the table and after the counters; a mesh that
+// splits edges counts the round and its splits.
+__global__ void k_refine_sizes(Store S, const int* vscan, const int* escan, int* counts) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= S.nmesh) return;
   int vb = S.tab.vbase[i], eb = S.tab.ebase[i];
   int nv = S.tab.nv[i], ne = S.tab.ne[i];
-  S.tab.nv[i] = nv + (vscan[vb + nv] - vscan[vb]);
-  S.tab.ne[i] = ne + (escan[eb + ne] - escan[eb]);
+  const int t = vscan[vb + nv] - vscan[vb];
+  S.tab.nv[i] = counts[CN_NUM + i] = nv + t;
+  S.tab.ne[i] = counts[CN_NUM + S.nmesh + i] = ne + (escan[eb + ne] - escan[eb]);
+  if (t > 0) {
+    S.tab.r[i] += 1;
+    S.tab.ops[i] += (unsigned long long)t;
+  }
 }
 
 // ---- persistent rounds ------------------------------------------------------------
@@ -3476,14 +3473,10 @@ struct RoundIO {
 };
 
 RoundIO read_round(MeshSet& m) {
-  cudaMemcpyAsync(m.hcounts, m.w.counts, CN_NUM * sizeof(int), cudaMemcpyDeviceToHost, m.stream);
-  cudaMemcpyAsync(m.hst, m.st, sizeof(DevStatus), cudaMemcpyDeviceToHost, m.stream);
-  cudaError_t e = cudaStreamSynchronize(m.stream);
   RoundIO io;
+  io.err = sync_counts(m, 0);
   io.nC = m.hcounts[CN_C];
   io.overflow = m.hst->overflow;
-  io.err = (e != cudaSuccess) ? PM_ERR_CUDA : m.hst->err;
-  if (e != cudaSuccess) set_last_error(std::string("CUDA: ") + cudaGetErrorString(e));
   return io;
 }
 
@@ -3613,10 +3606,12 @@ struct RoundsOut {
 // One cooperative launch of persistent rounds, then the read-back of every
 // counter and the status.  Advances the tag past the rounds that ran.
 int run_rounds(MeshSet& m, int which, const void* kernel, const char* name, RoundArgs& a,
-               RoundsOut& out) {
+               RoundsOut& out, bool& bar_clear) {
   a.work = prof_work(name);
   void* args[] = {&a};
-  cudaMemsetAsync(a.bar, 0, sizeof(unsigned), m.stream);
+  // (the first launch of an operator finds the counters cleared)
+  if (!bar_clear) cudaMemsetAsync(a.bar, 0, sizeof(unsigned), m.stream);
+  bar_clear = false;
   __atomic_fetch_add(&g_launches, 1ull, __ATOMIC_RELAXED);
   int slot = g_prof_on ? prof_begin(name, m.stream) : -1;
   cudaError_t e = cudaLaunchCooperativeKernel(kernel, dim3(rounds_grid(m, which)),
@@ -3645,18 +3640,6 @@ int run_rounds(MeshSet& m, int which, const void* kernel, const char* name, Roun
 // Operator loops (host)
 // ---------------------------------------------------------------------------
 
-void zero_ops(MeshSet& m) {
-  cudaMemsetAsync(m.S.tab.ops, 0, m.nmesh * sizeof(unsigned long long), m.stream);
-}
-
-cudaError_t fetch_ops(MeshSet& m, std::vector<unsigned long long>& ops) {
-  ops.resize(m.nmesh);
-  cudaError_t e = cudaMemcpyAsync(ops.data(), m.S.tab.ops, m.nmesh * sizeof(unsigned long long),
-                                  cudaMemcpyDeviceToHost, m.stream);
-  if (e != cudaSuccess) return e;
-  return cudaStreamSynchronize(m.stream);
-}
-
 // Rounds of collapses until no dirty vertex has a valid collapse.  The first
 // round's list leaves out vertices whose last collapse evaluation found
 // nothing and whose inputs have not changed since.
@@ -3669,6 +3652,7 @@ int op_coarsen(MeshSet& m, int max_rounds) {
   const int gv = grid_tuned(m, m.S.vused, bs, bps);
   int pass0 = m.tag;
   const bool persist = rounds_grid(m, 0) > 0;
+  bool bar_clear = true;
   zero_counts(m, 0, CN_NUM);
   PM_LAUNCH(k_init_list, gv, bs, 0, m.stream, m.S, 0, w.D[0], w.counts + CN_D0, m.S.evc,
             m.lo_coarsen);
@@ -3683,7 +3667,7 @@ int op_coarsen(MeshSet& m, int max_rounds) {
       RoundArgs a = round_args(m, cur, pass0, max_rounds == 0 ? (1LL << 30) : max_rounds - nr);
       a.limit = rlimit;
       RoundsOut o;
-      int err = run_rounds(m, 0, (const void*)k_coarsen_rounds, "k_coarsen_rounds", a, o);
+      int err = run_rounds(m, 0, (const void*)k_coarsen_rounds, "k_coarsen_rounds", a, o, bar_clear);
       if (err) return err;
       nr += o.rounds - o.complete;
       cur = o.cur;
@@ -3744,6 +3728,7 @@ int op_swap(MeshSet& m, int max_rounds) {
   int pass0 = m.tag;
   const int icap = m.S.vslots * 6 + 64;
   const bool persist = rounds_grid(m, 1) > 0;
+  bool bar_clear = true;
   zero_counts(m, 0, CN_NUM);
   PM_LAUNCH(k_init_list, gv, bs, 0, m.stream, m.S, 0, w.D[0], w.counts + CN_D0, m.S.evs,
             m.lo_swap);
@@ -3758,7 +3743,7 @@ int op_swap(MeshSet& m, int max_rounds) {
       a.limit = rlimit;
       a.fuse = tu.fuse_limit[0];
       RoundsOut o;
-      int err = run_rounds(m, 1, (const void*)k_swap_rounds, "k_swap_rounds", a, o);
+      int err = run_rounds(m, 1, (const void*)k_swap_rounds, "k_swap_rounds", a, o, bar_clear);
       if (err) return err;
       nr += o.rounds - o.complete;
       cur = o.cur;
@@ -3820,15 +3805,10 @@ int op_refine(MeshSet& m, int max_rounds) {
     PM_LAUNCH(k_refine_mark, gv, bs, 0, m.stream, m.S, w.vcnt, w.vmask, tag, pass0,
               m.lo_refine);
     scan_exclusive(w.vcnt, w.vscan, m.S.vused, m.scan, m.st, m.stream);
-    int* tot = w.counts + CN_NUM;
     std::vector<int> newv(m.nmesh);
-    PM_LAUNCH(k_refine_newcount, (m.nmesh + 127) / 128, 128, 0, m.stream, m.S, w.vscan, tot);
-    cudaMemcpyAsync(m.hcounts + CN_NUM, tot, m.nmesh * sizeof(int), cudaMemcpyDeviceToHost,
-                    m.stream);
-    {
-      int err = sync_status(m);
-      if (err) return err;
-    }
+    PM_LAUNCH(k_refine_newcount, (m.nmesh + 127) / 128, 128, 0, m.stream, m.S,
+              (const int*)w.vscan, w.counts);
+    if (int err = sync_counts(m, m.nmesh)) return err;
     for (int i = 0; i < m.nmesh; ++i) newv[i] = m.hcounts[CN_NUM + i];
     // A growth moves every mesh of the set, so when one mesh needs room, every
     // mesh that this round leaves with little gets half as much again as it
@@ -3865,9 +3845,7 @@ int op_refine(MeshSet& m, int max_rounds) {
     }
     const int stamp = tag + 1;
     const int vend = m.vbase.back() + m.nv.back() + newv.back();  // above every new vertex
-    PM_LAUNCH(k_refine_vtotals, (m.nmesh + 127) / 128, 128, 0, m.stream, m.S, w.vscan);
     PM_LAUNCH(k_refine_newverts, gv, bs, 0, m.stream, m.S, w.vscan, w.vmask, stamp, w.opA);
-    zero_counts(m, CN_EL, 2);
     PM_LAUNCH(k_refine_count, ge, bs, 0, m.stream, m.S, w.vscan, w.vmask, w.ecnt, w.emid,
               w.elist, w.counts + CN_EL);
     scan_exclusive(w.ecnt, w.escan, m.S.eused, m.scan, m.st, m.stream);
@@ -3878,20 +3856,17 @@ int op_refine(MeshSet& m, int max_rounds) {
     PM_LAUNCH(k_refine_rows, grid_tuned(m, vend, bs, bps), bs, 0, m.stream, m.S, m.B, vend, w.vscan,
               w.escan, w.opA, stamp, m.st);
     PM_LAUNCH(k_refine_rows_copy, grid_tuned(m, vend, bs, bps), bs, 0, m.stream, m.S, m.B, vend, stamp);
-    PM_LAUNCH(k_refine_sizes, (m.nmesh + 127) / 128, 128, 0, m.stream, m.S, w.vscan, w.escan);
+    PM_LAUNCH(k_refine_sizes, (m.nmesh + 127) / 128, 128, 0, m.stream, m.S, (const int*)w.vscan,
+              (const int*)w.escan, w.counts);
     // the new sizes and the status in one read-back
-    int* hsz = m.hcounts + CN_NUM;
-    cudaMemcpyAsync(hsz, m.S.tab.nv, 2 * m.nmesh * sizeof(int), cudaMemcpyDeviceToHost, m.stream);
-    int err = sync_status(m);
-    if (err) return err;
+    if (int err = sync_counts(m, 2 * m.nmesh)) return err;
     for (int i = 0; i < m.nmesh; ++i) {
-      m.nv[i] = hsz[i];
-      m.ne[i] = hsz[m.nmesh + i];
+      m.nv[i] = m.hcounts[CN_NUM + i];
+      m.ne[i] = m.hcounts[CN_NUM + m.nmesh + i];
     }
     set_used(m);
     if (m.hst->overflow) {  // a row outgrew W: rebuild every row with wider ones
-      err = after_overflow(m);
-      if (err) return err;
+      if (int err = after_overflow(m)) return err;
     }
   }
   if (!complete) m.lo_refine = m.tag;
@@ -3909,6 +3884,7 @@ int op_smooth(MeshSet& m, int max_sweeps, int max_rounds) {
   const int gv = grid_tuned(m, m.S.vused, bs, bps);
   const int pass0 = m.tag;
   const bool persist = rounds_grid(m, 2) > 0;
+  bool bar_clear = true;
   zero_counts(m, 0, CN_NUM);
   PM_LAUNCH(k_init_list, gv, bs, 0, m.stream, m.S, 1, w.D[0], w.counts + CN_D0, nullptr, 0);
   int nlist = 0;  // unknown at first (see op_coarsen)
@@ -3935,7 +3911,7 @@ int op_smooth(MeshSet& m, int max_sweeps, int max_rounds) {
       a.limit = rlimit;
       a.fuse = tu.fuse_limit[1];
       RoundsOut o;
-      int err = run_rounds(m, 2, (const void*)k_smooth_rounds, "k_smooth_rounds", a, o);
+      int err = run_rounds(m, 2, (const void*)k_smooth_rounds, "k_smooth_rounds", a, o, bar_clear);
       if (err) return err;
       const int* res = m.hcounts + CN_RES;
       nr += res[SR_ROUNDS];
@@ -4000,7 +3976,7 @@ int op_opt_smooth(MeshSet& m, int nrounds, int max_rounds) {
     PM_LAUNCH(k_opt_apply, grid_tuned(m, (long long)m.S.vused * TW, bs, bps), bs, 0, m.stream, m.S, w.Sl,
               w.counts + CN_S, w.gains, tag + 1);
   }
-  return sync_status(m);
+  return PM_OK;  // the caller's read-back waits
 }
 
 }  // namespace pm

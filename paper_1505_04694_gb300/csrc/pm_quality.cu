@@ -341,7 +341,7 @@ cudaError_t quality_launch(const QualityWork& w, const double* xy, const double*
   sw.state = w.state;
   sw.ticket = &w.head->ticket;
   sw.tiles_cap = scan_tiles(nv + 1);
-  scan_exclusive_cleared(w.cnt, w.off, nv, sw, &w.head->st, s);
+  scan_exclusive(w.cnt, w.off, nv, sw, &w.head->st, s);
   PM_LAUNCH(k_corner_fill, gridn(ne), 128, 0, s, tri, ne, nv, (const int*)w.off,
             (const uint8_t*)w.pos, w.cnt + (nv + 1), w.col, (const DevStatus*)&w.head->st);
   PM_LAUNCH(k_vgather_arr, gridn(nv), 128, 0, s, (const int*)w.off, w.col, (const EGrad*)w.eg, nv,

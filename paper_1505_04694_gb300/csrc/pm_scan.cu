@@ -97,6 +97,8 @@ k_scan(Input input, int* __restrict__ out, int n, unsigned long long* state, int
   __shared__ int s_fail;
   if (threadIdx.x == 0) {
     s_tile = atomicAdd(ticket, 1);
+    // tickets go out in order: whoever holds the last one re-arms the counter
+    if (s_tile == (int)gridDim.x - 1) *ticket = 0;
     s_fail = 0;
   }
   __syncthreads();
@@ -202,14 +204,12 @@ int scan_tiles(int n) { return (n + SCAN_TILE - 1) / SCAN_TILE; }
 namespace {
 
 template <class Input>
-void scan_run(Input input, int* out, int n, ScanWork& w, DevStatus* st, cudaStream_t s,
-              bool cleared = false) {
+void scan_run(Input input, int* out, int n, ScanWork& w, DevStatus* st, cudaStream_t s) {
   if (n <= 0) {
     cudaMemsetAsync(out, 0, sizeof(int), s);
     return;
   }
   int tiles = scan_tiles(n);
-  if (!cleared) cudaMemsetAsync(w.ticket, 0, sizeof(int), s);
   w.epoch = (w.epoch + 1) & 0x3FFFFFFFu;
   if (w.epoch == 0) w.epoch = 1;
   PM_LAUNCH(k_scan<Input>, tiles, SCAN_THREADS, 0, s, input, out, n, w.state, w.ticket, w.epoch,
@@ -220,15 +220,9 @@ void scan_run(Input input, int* out, int n, ScanWork& w, DevStatus* st, cudaStre
 
 // Exclusive scan of in[0..n) into out[0..n]; out[n] holds the total.
 // `state` needs scan_tiles(n) words and is never cleared (epochs tell runs
-// apart); `ticket` is reset here.
+// apart); `ticket` starts at zero and every scan leaves it there.
 void scan_exclusive(const int* in, int* out, int n, ScanWork& w, DevStatus* st, cudaStream_t s) {
   scan_run(IntInput{in}, out, n, w, st, s);
-}
-
-// The same with a ticket (and state words) the caller has just cleared.
-void scan_exclusive_cleared(const int* in, int* out, int n, ScanWork& w, DevStatus* st,
-                            cudaStream_t s) {
-  scan_run(IntInput{in}, out, n, w, st, s, true);
 }
 
 // The same over the alive flags of the used vertex (element) slots [0, n).
