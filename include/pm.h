@@ -333,10 +333,10 @@ pm_status pm_quality_arrays_noalloc_dev(const double* xy, const double* m, int32
  *   rounds_blocks_per_sm[3]: resident blocks per SM of those persistent
  *     launches (1 or 2; fewer when the kernel's registers allow fewer).
  *   fuse_limit[2]: flips, smoothing: inside the persistent launch, lists up
- *     to this size (and at most one per 8-lane tile of the grid) are scanned
+ *     to this size (and at most two per 8-lane tile of the grid) are scanned
  *     and evaluated in one phase.
- * Defaults: 128 threads, 16 blocks per SM, 131072, 1 block, fuse_limit
- * {2^30, 2^30}. */
+ * Defaults: 128 threads, 16 blocks per SM, rounds_limit {32768, 131072,
+ * 131072}, 1 block, fuse_limit {2^30, 2^30}. */
 typedef struct {
   int32_t block[4];
   int32_t blocks_per_sm[4];

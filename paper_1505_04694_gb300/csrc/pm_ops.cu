@@ -281,19 +281,26 @@ __global__ void k_colour_init(Store S, int* U, int* nU) {
   }
 }
 
-__global__ void k_colour_propose(Store S, const int* U, const int* nUp, int* prop, int* stamp,
-                                 int rt) {
+__device__ __forceinline__ void colour_propose_phase(const Store& S, const int* U, const int* nUp,
+                                                     int* prop, int* stamp, int rt, bool il) {
   const int n = *nUp;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  for (int i = grank(il); i < n; i += gsize()) {
     const int v = U[i];
-    const int vb = S.tab.vbase[mesh_of_vslot(S, v)];
+    const int vb = ctx_of(S, v).vb;
     const int* nn = nn_row(S, v);
+    Row8 r = row8(nn, 0);
     const int nnl = S.NNlen[v];
     RowMask used;  // colours 0..127 held by coloured neighbours
-#pragma unroll 4
-    for (int k = 0; k < nnl; ++k) {
-      const int c = S.tab.col[vb + nn[k]];
-      if (c >= 0 && c < MAXW) used.set(c);
+    for (int b = 0;;) {
+      int c[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) c[k] = b + k < nnl ? S.tab.col[vb + r.a[k]] : -1;
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (c[k] >= 0 && c[k] < MAXW) used.set(c[k]);
+      b += 8;
+      if (b >= nnl) break;
+      r = row8(nn, b);
     }
     int c = 0;
     if (~used.lo) c = __ffsll((long long)~used.lo) - 1;
@@ -304,36 +311,60 @@ __global__ void k_colour_propose(Store S, const int* U, const int* nUp, int* pro
   }
 }
 
-__global__ void k_colour_resolve(Store S, const int* U, const int* nUp, const int* prop,
-                                 const int* stamp, int rt, int* Un, int* nUn) {
+__device__ __forceinline__ void colour_resolve_phase(const Store& S, const int* U, const int* nUp,
+                                                     const int* prop, const int* stamp, int rt,
+                                                     int* Un, int* nUn, bool il) {
   const int n = *nUp;
-  for (int i0 = blockIdx.x * blockDim.x; i0 < n; i0 += gridDim.x * blockDim.x) {
-    const int i = i0 + threadIdx.x;
+  for (int i0 = 0; i0 < n; i0 += gsize()) {
+    const int i = i0 + grank(il);
     bool again = false;
     int v = 0;
     if (i < n) {
       v = U[i];
-      const int mi = mesh_of_vslot(S, v);
-      const int vb = S.tab.vbase[mi];
-      const uint32_t seed = S.tab.seed[mi], r = S.tab.r[mi];
-      const uint32_t pv = prio(vid_of(S, v, vb), seed, r);
+      const MeshCtx c = ctx_of(S, v);
+      const uint32_t seed = S.tab.seed[c.mi], r = S.tab.r[c.mi];
+      const uint32_t pv = prio(vid_of(S, v, c.vb), seed, r);
       const int pc = prop[v];
       const int* nn = nn_row(S, v);
+      Row8 nb = row8(nn, 0);
       const int nnl = S.NNlen[v];
       bool keep = true;
-#pragma unroll 4
-      for (int k = 0; k < nnl; ++k) {
-        const int u = vb + nn[k];
-        keep &= !(stamp[u] == rt && prop[u] == pc && prio(vid_of(S, u, vb), seed, r) > pv);
+      for (int b = 0;;) {
+        int su[8], pu[8];
+        uint32_t iu[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const bool in = b + k < nnl;
+          const int u = c.vb + nb.a[k];
+          su[k] = in ? stamp[u] : rt - 1;
+          pu[k] = in ? prop[u] : -1;
+          iu[k] = in ? vid_of(S, u, c.vb) : 0u;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          keep &= !(su[k] == rt && pu[k] == pc && prio(iu[k], seed, r) > pv);
+        b += 8;
+        if (b >= nnl) break;
+        nb = row8(nn, b);
       }
       if (keep) {
         S.tab.col[v] = pc;
-        atomicMax(S.tab.ncol + mi, pc + 1);
+        atomicMax(S.tab.ncol + c.mi, pc + 1);
       }
       again = !keep;
     }
     warp_append(again, v, Un, nUn);
   }
+}
+
+__global__ void k_colour_propose(Store S, const int* U, const int* nUp, int* prop, int* stamp,
+                                 int rt) {
+  colour_propose_phase(S, U, nUp, prop, stamp, rt, false);
+}
+
+__global__ void k_colour_resolve(Store S, const int* U, const int* nUp, const int* prop,
+                                 const int* stamp, int rt, int* Un, int* nUn) {
+  colour_resolve_phase(S, U, nUp, prop, stamp, rt, Un, nUn, false);
 }
 
 
@@ -1215,7 +1246,8 @@ __device__ __forceinline__ void coarsen_commit_phase(Store S, const int* A, cons
     const int* ne = ne_row(S, u);
     if (coarsen_commit_short(S, u, c, lu, target, smark, tag)) continue;
     int nnl = S.NNlen[u], nel = S.NElen[u];
-    int nb[MAXW], eb[MAXW];
+    __align__(16) int nb[MAXW];  // read in chunks below
+    int eb[MAXW];
     int nn2 = 0, ne2 = 0;
     bool ok = true;
     // gather the per-entry facts first so that their loads overlap
@@ -2085,7 +2117,8 @@ __device__ __forceinline__ void swap_commit_phase(Store S, const int* A, const i
     int* ne = S.NE + (size_t)u * S.W;
     if (swap_commit_short(S, u, c, lu, opA, opK2, smark, tag)) continue;
     int nnl = S.NNlen[u], nel = S.NElen[u];
-    int nb[MAXW], eb[MAXW];
+    __align__(16) int nb[MAXW];  // read in chunks below
+    int eb[MAXW];
     load_row(nn, nnl, nb);
     load_row(ne, nel, eb);
     int nn2 = nnl, ne2 = nel;
@@ -2393,35 +2426,29 @@ __device__ bool tile_smooth_eval(const Tile& t, const Store& S, int v, MeshCtx c
 
 // Pass 2 of the longer lists, one listed vertex per thread: the Laplacian sums,
 // the 2x2 solve, the location and the interpolation run per thread (a tile of
-// lanes per vertex repeats the ordered sums in every lane: four vertices per
-// warp instruction of FP64 instead of 32), the FP32 bounds of the moved ball
-// (its metric interpolated in FP32) drop the moves that certainly fail, and the
-// remaining ones get the exact metric and the exact ball check, four at a time
-// on 8-lane tiles.  Every value is computed by the
-// same operations in the same order as in tile_smooth_eval.
-__device__ __forceinline__ void smooth_eval_phase(Store S, const int* E, const int* nEp,
-                                                  double2* mvxy, double4* mvM, double* qball,
-                                                  int* C, int* nC, int* cmark, int tag,
-                                                  unsigned long long* work, bool il = false) {
+// lanes per vertex repeats them in every lane: four vertices per warp instruction
+// of FP64 instead of 32), and the FP32 bounds of the moved ball (its metric
+// interpolated in FP32 first) drop the moves that certainly fail.  The others are
+// listed for pass 3 with their target and metric.
+__device__ __forceinline__ void smooth_filter_phase(Store S, const int* E, const int* nEp,
+                                                    double2* mvxy, double4* mvM, int* R, int* nR,
+                                                    unsigned long long* work, bool il = false) {
+  const int first = first_entry(E, grank(il), S.vslots);
   const int n = *nEp;
-  const Tile t = tile_of();
   unsigned ops = 0;
   for (int j0 = 0; j0 < n; j0 += gsize()) {
     const int j = j0 + grank(il);
-    int v = 0, mi = 0;
+    int v = 0;
     bool may = false;
-    double x = 0.0, y = 0.0, qold = 0.0;
-    double4 Mn = make_double4(0.0, 0.0, 0.0, 0.0);
     if (j < n) {
-      v = E[j];
+      v = j0 == 0 ? first : E[j];
       const MeshCtx c = ctx_of(S, v);
-      mi = c.mi;
       const int lv = v - c.vb;
       const int* ne = ne_row(S, v);
       const int nel = S.NElen[v];
       const int* nn = nn_row(S, v);
       const int nnl = S.NNlen[v];
-      qold = 1e300;
+      double qold = 1e300;
       for (int b = 0; b < nel; b += 8) {
         const Row8 r = row8(ne, b);
         double q[8];
@@ -2438,29 +2465,29 @@ __device__ __forceinline__ void smooth_eval_phase(Store S, const int* E, const i
         double2 p[4];
         double4 mj[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int js = b + j < nnl ? c.vb + u4[j] : v;
-          p[j] = S.xy[js];
-          mj[j] = S.M[js];
+        for (int k = 0; k < 4; ++k) {
+          const int js = b + k < nnl ? c.vb + u4[k] : v;
+          p[k] = S.xy[js];
+          mj[k] = S.M[js];
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (b + j >= nnl) continue;
-          const double w00 = 0.5 * (mv.x + mj[j].x);
-          const double w01 = 0.5 * (mv.y + mj[j].y);
-          const double w11 = 0.5 * (mv.z + mj[j].z);
+        for (int k = 0; k < 4; ++k) {
+          if (b + k >= nnl) continue;
+          const double w00 = 0.5 * (mv.x + mj[k].x);
+          const double w01 = 0.5 * (mv.y + mj[k].y);
+          const double w11 = 0.5 * (mv.z + mj[k].z);
           a00 = a00 + w00;
           a01 = a01 + w01;
           a11 = a11 + w11;
-          b0 = b0 + (w00 * p[j].x + w01 * p[j].y);
-          b1 = b1 + (w01 * p[j].x + w11 * p[j].y);
+          b0 = b0 + (w00 * p[k].x + w01 * p[k].y);
+          b1 = b1 + (w01 * p[k].x + w11 * p[k].y);
         }
       }
       const double det = a00 * a11 - a01 * a01;
       ops += 17 * nnl + 3;
       if (dgt(det, 0.0)) {
-        x = (a11 * b0 - a01 * b1) / det;
-        y = (a00 * b1 - a01 * b0) / det;
+        const double x = (a11 * b0 - a01 * b1) / det;
+        const double y = (a00 * b1 - a01 * b0) / det;
         ops += 8;
         const VF fx = make_vf_xy(x, y);
         int4 e = make_int4(0, 0, 0, 0);
@@ -2477,63 +2504,56 @@ __device__ __forceinline__ void smooth_eval_phase(Store S, const int* E, const i
             may = may &&
                   !(moved_quality_up(S, c.vb, lv, S.EN[c.eb + ne[k]], fn, kx) < ffloor);
           if (may) {
-            Mn = interpolate_in(S, c.vb, e, x, y);
+            double4 Mn = interpolate_in(S, c.vb, e, x, y);
             ops += 46;
+            Mn.w = qold;  // for pass 3
+            mvxy[v] = make_double2(x, y);
+            mvM[v] = Mn;
           }
         }
       }
       if (!may) mvM[v].w = 0.0;
     }
-    // the exact check of the moves that may succeed: tile i of the warp takes
-    // the i-th of the next four
+    warp_append(may, v, R, nR);
+  }
+  add_work(work, ops);
+}
+
+// Pass 3 (one 8-lane tile per move that may succeed): the exact ball check.
+// Every value of a move is computed by the same operations in the same order as
+// in tile_smooth_eval.
+__device__ __forceinline__ void smooth_exact_phase(Store S, const int* R, const int* nRp,
+                                                   const double2* mvxy, double4* mvM,
+                                                   double* qball, int* C, int* nC, int* cmark,
+                                                   int tag, unsigned long long* work,
+                                                   bool il = false) {
+  const Tile t = tile_of();
+  const int first = first_entry(R, trank(il), S.vslots);
+  const int n = *nRp;
+  unsigned ops = 0;
+  for (int j0 = 0; j0 < n; j0 += tcount()) {
+    const int j = j0 + trank(il);
+    int v = 0;
     bool cand = false;
-    for (unsigned m = __ballot_sync(0xffffffffu, may); m;) {
-      int src = -1;
-      unsigned rest = m;
-#pragma unroll
-      for (int i = 0; i < 32 / TW; ++i) {
-        const int b = rest ? __ffs(rest) - 1 : -1;
-        if (i == t.shift / TW) src = b;
-        rest &= rest - 1u;
-      }
-      const int from = src >= 0 ? src : 0;
-      const int tv = __shfl_sync(0xffffffffu, v, from);
-      const double tx = __shfl_sync(0xffffffffu, x, from), ty = __shfl_sync(0xffffffffu, y, from);
-      const double tq = __shfl_sync(0xffffffffu, qold, from);
-      const double4 tm = make_double4(__shfl_sync(0xffffffffu, Mn.x, from),
-                                      __shfl_sync(0xffffffffu, Mn.y, from),
-                                      __shfl_sync(0xffffffffu, Mn.z, from), 0.0);
-      bool ok = false;
-      if (src >= 0) {
-        const MeshCtx c = ctx_of(S, tv);
-        const int nel = S.NElen[tv];
-        // the new ball qualities of an accepted move are kept for the apply
-        ok = tile_ball_exact(t, S, c, tv - c.vb, ne_row(S, tv), nel, tx, ty, tm, tq, true,
-                             qball + (size_t)tv * S.W, nullptr);
-        if (t.tl == 0) ops += 85 * nel;
-      }
-      const unsigned okm = __ballot_sync(0xffffffffu, ok && t.tl == 0);  // bit 8 i: tile i
-#pragma unroll
-      for (int i = 0; i < 32 / TW; ++i) {
-        if (m) {
-          const int b = __ffs(m) - 1;
-          m &= m - 1u;
-          if ((threadIdx.x & 31) == b) cand = (okm >> (TW * i)) & 1u;
+    if (j < n) {
+      v = j0 == 0 ? first : R[j];
+      const MeshCtx c = ctx_of(S, v);
+      const int nel = S.NElen[v];
+      const double2 X = mvxy[v];
+      const double4 Mn = mvM[v];
+      // the new ball qualities of an accepted move are kept for the apply
+      cand = tile_ball_exact(t, S, c, v - c.vb, ne_row(S, v), nel, X.x, X.y, Mn, Mn.w, true,
+                             qball + (size_t)v * S.W, nullptr);
+      if (t.tl == 0) {
+        ops += 85 * nel;
+        mvM[v].w = cand ? 1.0 : 0.0;  // marks a stored move
+        if (cand) {
+          cmark[v] = tag;
+          S.tab.had[c.mi] = 1;
         }
       }
     }
-    if (may) {
-      if (cand) {
-        mvxy[v] = make_double2(x, y);
-        Mn.w = 1.0;  // marks a stored move
-        mvM[v] = Mn;
-        cmark[v] = tag;
-        S.tab.had[mi] = 1;
-      } else {
-        mvM[v].w = 0.0;
-      }
-    }
-    warp_append(cand, v, C, nC);
+    warp_append(cand && t.tl == 0, v, C, nC);
   }
   add_work(work, ops);
 }
@@ -2592,10 +2612,15 @@ __device__ __forceinline__ void smooth_scan_eval_phase(Store S, const int* D, co
   add_work(work, ops);
 }
 
-__global__ void k_smooth_eval(Store S, const int* E, const int* nEp, double2* mvxy, double4* mvM,
-                              double* qball, int* C, int* nC, int* cmark, int tag,
+__global__ void k_smooth_filter(Store S, const int* E, const int* nEp, double2* mvxy,
+                                double4* mvM, int* R, int* nR, unsigned long long* work) {
+  smooth_filter_phase(S, E, nEp, mvxy, mvM, R, nR, work);
+}
+
+__global__ void k_smooth_eval(Store S, const int* R, const int* nRp, const double2* mvxy,
+                              double4* mvM, double* qball, int* C, int* nC, int* cmark, int tag,
                               unsigned long long* work) {
-  smooth_eval_phase(S, E, nEp, mvxy, mvM, qball, C, nC, cmark, tag, work);
+  smooth_exact_phase(S, R, nRp, mvxy, mvM, qball, C, nC, cmark, tag, work);
 }
 
 // Move the members of S; live interior neighbours become pending for the next
@@ -2887,24 +2912,12 @@ __global__ void k_refine_mark(Store S, int* cnt, RowMask* mask, int tag, int pas
       // the row is sorted, so the neighbours above la form a suffix; four
       // lengths at a time so that their loads overlap
       int k0 = 0;
-      for (int b = 0; b < nnl; b += 8) {
-        const Row8 r = row8(nn, b);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) k0 += b + k < nnl && r.a[k] <= la ? 1 : 0;
-      }
-      for (int b = k0 & ~3; b < nnl; b += 4) {
-        const int4 r4 = *reinterpret_cast<const int4*>(nn + b);
-        const int u4[4] = {r4.x, r4.y, r4.z, r4.w};
-        VF fu[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          fu[j] = b + j >= k0 && b + j < nnl ? load_vf(S, vb + u4[j]) : VF{};
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (b + j >= k0 && b + j < nnl &&
-              edge_longer(S, mi, fa, fu[j], s, vb + u4[j], ops))
-            m.set(b + j);
-      }
+      // (a sweep over every slot hides the latency with resident warps: fewer
+      // registers beat loads issued ahead, 150 against 187 us on 10M slots)
+      while (k0 < nnl && nn[k0] <= la) ++k0;
+#pragma unroll 4
+      for (int k = k0; k < nnl; ++k)
+        if (edge_longer(S, mi, fa, load_vf(S, vb + nn[k]), s, vb + nn[k], ops)) m.set(k);
       mask[s] = m;
     } else {
       mask[s] = RowMask();
@@ -3235,6 +3248,12 @@ __global__ void k_selftest_barrier(unsigned* bar, DevStatus* st, unsigned long l
   grid_barrier(bar, target, st, limit_ns);
 }
 
+// Flips and smoothing: lists of up to this many passes of the grid's tiles take
+// the one-phase form (measured on a 201 x 201 mesh adapted to 670k triangles:
+// flips 13.20 ms at one pass, 12.88 at two and three, 13.23 at eight; smoothing
+// 12.80, 12.58, 13.01 at one, two, three).
+constexpr int kFusePasses = 2;
+
 struct RoundArgs {
   Store S;
   Work w;
@@ -3250,7 +3269,8 @@ struct RoundArgs {
   int ptag;            // smoothing: stamp of the next sweep's list
   int sweeps;          // smoothing: sweeps left, the current one included
   int moved;           // smoothing: the current sweep has moved a vertex
-  int fuse;            // flips, smoothing: lists up to this size take the one-phase evaluation
+  int fuse;            // flips, smoothing: lists up to this size (and kFusePasses passes of
+                       // tiles) take the one-phase evaluation
   unsigned long long* work;  // counted FP64 work (measurement) or null
 };
 
@@ -3297,8 +3317,8 @@ __device__ __forceinline__ void topo_rounds(const RoundArgs& a) {
       cnt[cn_list(nxt)] = 0;
       cnt[CN_CL] = 0;  // elements whose quality changes
     }
-    if (FLIP && ld_volatile(cnt + cn_list(cur)) <= min(a.fuse, tcount())) {
-      // the list fits one pass of tiles: scan, gains and pick in one phase
+    if (FLIP && ld_volatile(cnt + cn_list(cur)) <= min(a.fuse, kFusePasses * tcount())) {
+      // the list fits two passes of tiles: scan, gains and pick in one phase
       // (the list is complete since the last barrier: every block decides alike)
       swap_scan_eval_phase(a.S, w.D[cur], cnt + cn_list(cur), w.opA, w.opK2, w.C, nC, w.cmark,
                            tag, a.pass0, a.work);
@@ -3357,10 +3377,36 @@ __global__ void __launch_bounds__(256) k_coarsen_rounds(RoundArgs a) { topo_roun
 
 __global__ void __launch_bounds__(256) k_swap_rounds(RoundArgs a) { topo_rounds<true>(a); }
 
+// Colouring rounds of a list of at most `limit` vertices: [propose] B1 [resolve]
+// B2, until no vertex is uncoloured.  (A colouring takes about 15 rounds, each of
+// which was two launches and a wait.)  Block 0 clears the list a round fills
+// before B1 (last read before the last round's B2).
+__global__ void __launch_bounds__(256) k_colour_rounds(RoundArgs a) {
+  const Work& w = a.w;
+  int* cnt = w.counts;
+  unsigned target = 0;
+  int cur = a.cur, r = 0;
+  int n = ld_volatile(cnt + cn_list(cur));
+  while (n > 0 && n <= a.limit && r < a.max_rounds) {
+    const int nxt = 1 - cur, rt = a.tag0 + 2 * r;
+    if (blockIdx.x == 0 && threadIdx.x == 0) cnt[cn_list(nxt)] = 0;
+    colour_propose_phase(a.S, w.D[cur], cnt + cn_list(cur), w.cprop, w.cstamp, rt, true);
+    if (!grid_barrier(a.bar, target, a.st)) return;
+    colour_resolve_phase(a.S, w.D[cur], cnt + cn_list(cur), w.cprop, w.cstamp, rt, w.D[nxt],
+                         cnt + cn_list(nxt), true);
+    if (!grid_barrier(a.bar, target, a.st)) return;
+    n = ld_volatile(cnt + cn_list(nxt));
+    cur = nxt;
+    ++r;
+  }
+  finish_rounds(a, r, cur, n == 0);
+}
+
 // Sweeps of smoothing rounds.  A round whose list fits one pass of the grid's
 // tiles: [scan + evaluate] B1 [select + apply] B2; a longer one: [scan] B1
-// [evaluate] B1' [select + apply] B2 (its tiles then go to the vertices that
-// need an evaluation only).  A sweep ends with a round that finds no candidate;
+// [filter] B1' [exact] B1'' [select + apply] B2 (its threads then go to the
+// vertices that need an evaluation, its tiles to the moves that may succeed).  A
+// sweep ends with a round that finds no candidate;
 // its pending list then becomes the current one and the next sweep starts in
 // the same launch (ten sweeps used to be ten launches and read-backs, most of
 // them for a handful of vertices).  The three lists trade places by index, each
@@ -3368,7 +3414,7 @@ __global__ void __launch_bounds__(256) k_swap_rounds(RoundArgs a) { topo_rounds<
 // r fills and, in a sweep's first round, its pending list (both last read by a
 // scan and a decision before the last barrier); after B1: the candidate slot of
 // round r + 1 (last read after B2 of round r - 1); after B1': E (read by the
-// evaluation before B1').  The round counters advance after B2 from the flag
+// filter before B1'); after B1'': the filtered list.  The round counters advance after B2 from the flag
 // set of the round's parity, so that round r + 1's evaluation can set the other
 // set meanwhile.  The launch returns when the sweeps are over, after
 // `max_rounds` rounds with candidates, or when the next list outgrows `limit`;
@@ -3384,7 +3430,7 @@ __global__ void __launch_bounds__(256) k_smooth_rounds(RoundArgs a) {
   bool moved = a.moved != 0, over = false, fresh = false;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *cand_count(cnt, 0) = 0;
-    cnt[CN_E] = 0;
+    cnt[CN_E] = cnt[CN_S] = 0;
   }
   if (!grid_barrier(a.bar, target, a.st)) return;
   // a list longer than the limit is left to the one-kernel-per-phase rounds
@@ -3396,7 +3442,7 @@ __global__ void __launch_bounds__(256) k_smooth_rounds(RoundArgs a) {
     Store S = a.S;
     S.tab.had = a.S.tab.had + (r & 1) * S.nmesh;
     // the list is complete since B2 of the last round: every block decides alike
-    const bool fused = n <= min(a.fuse, tiles);
+    const bool fused = n <= min(a.fuse, kFusePasses * tiles);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       *count(nxt) = 0;
       if (fresh) *count(pen) = 0;
@@ -3412,10 +3458,13 @@ __global__ void __launch_bounds__(256) k_smooth_rounds(RoundArgs a) {
                         cnt + CN_E, true);
       if (!grid_barrier(a.bar, target, a.st)) return;
       if (blockIdx.x == 0 && threadIdx.x == 0) *cand_count(cnt, r + 1) = 0;
-      smooth_eval_phase(S, w.E, cnt + CN_E, w.mvxy, w.mvM, w.gains, w.C, nC, w.cmark, tag, a.work,
-                        true);
+      smooth_filter_phase(S, w.E, cnt + CN_E, w.mvxy, w.mvM, w.Sl, cnt + CN_S, a.work, true);
       if (!grid_barrier(a.bar, target, a.st)) return;
       if (blockIdx.x == 0 && threadIdx.x == 0) cnt[CN_E] = 0;
+      smooth_exact_phase(S, w.Sl, cnt + CN_S, w.mvxy, w.mvM, w.gains, w.C, nC, w.cmark, tag,
+                         a.work, true);
+      if (!grid_barrier(a.bar, target, a.st)) return;
+      if (blockIdx.x == 0 && threadIdx.x == 0) cnt[CN_S] = 0;
     }
     smooth_select_apply_phase(S, w.C, nC, w.cmark, w.smark, tag, list(nxt), count(nxt), w.dmark,
                               w.mvxy, w.mvM, w.gains, list(pen), count(pen), w.pmark, ptag, tag + 1,
@@ -3484,36 +3533,6 @@ void zero_counts(MeshSet& m, int first, int num) {
   cudaMemsetAsync(m.w.counts + first, 0, num * sizeof(int), m.stream);
 }
 
-// Colours every active mesh whose parameters ask for colour-class sets, at
-// the start of a collapse, flip or smoothing pass: speculative rounds until
-// no vertex is left uncoloured (each round keeps at least the proposal of
-// the highest priority; the cap is far beyond any mesh's rounds).
-int colour_set(MeshSet& m) {
-  bool any = false;
-  for (int x : m.select) any |= x == PM_SELECT_COLOUR;
-  if (!any) return PM_OK;
-  Work& w = m.w;
-  const int g = grid_for(m, m.S.vused);
-  zero_counts(m, CN_D0, 1);
-  PM_LAUNCH(k_colour_init, g, BLOCK, 0, m.stream, m.S, w.D[0], w.counts + CN_D0);
-  int cur = 0;
-  for (int it = 0; it < (1 << 20); ++it) {
-    const int nxt = 1 - cur;
-    const int rt = (m.tag += 2);
-    zero_counts(m, cn_list(nxt), 1);
-    PM_LAUNCH(k_colour_propose, g, BLOCK, 0, m.stream, m.S, w.D[cur], w.counts + cn_list(cur),
-              w.cprop, w.cstamp, rt);
-    PM_LAUNCH(k_colour_resolve, g, BLOCK, 0, m.stream, m.S, w.D[cur], w.counts + cn_list(cur),
-              w.cprop, w.cstamp, rt, w.D[nxt], w.counts + cn_list(nxt));
-    RoundIO io = read_round(m);
-    if (io.err) return io.err;
-    if (m.hcounts[cn_list(nxt)] == 0) return PM_OK;
-    cur = nxt;
-  }
-  set_last_error("colouring did not finish");
-  return PM_ERR_INVALID_MESH;
-}
-
 // The counters of a new round (C, S, A, E, I, I2) and of the list it fills
 // (D[nxt]); the list it reads keeps its count.
 void zero_round(MeshSet& m, int nxt) {
@@ -3538,29 +3557,34 @@ int after_round(MeshSet& m, const RoundIO& io) {
 
 // Persistent rounds take over once a pass's list holds at most
 // Tuning::rounds_limit vertices (and hand back when the next list outgrows
-// it); default 131072 for each operator, measured best of 8k to 1M on the
-// 2M workload.
+// it).  Defaults, measured on meshes of 8k to 20M triangles: 131072 for flips and
+// smoothing (12.88 ms at 131072 against 13.2 at 32768 on the 201 x 201 mesh), 32768
+// for collapses, whose longer lists run faster one vertex per thread on a full
+// chip (8.08 against 8.80 ms on a 317 x 317 grid coarsened to 18k triangles).
 constexpr int kRoundsThreads = 256;
+// Colouring rounds are light (gathers and a mask), and each costs two launches
+// and a wait outside the persistent kernel.
+constexpr int kColourLimit = 131072;
 
 // Blocks of a cooperative launch of the persistent round kernel `which`
-// (0 collapse, 1 flip, 2 smoothing) on this device: the tuning's blocks per
+// (0 collapse, 1 flip, 2 smoothing, 3 colouring) on this device: the tuning's blocks per
 // SM (Tuning::rounds_blocks_per_sm, at most what its registers allow) on
 // every SM, or 0 when the device cannot run it cooperatively (rounds stay one
 // kernel per phase).
 int rounds_grid(MeshSet& m, int which) {
   static std::mutex mu;
-  static int occ[64][3];
+  static int occ[64][4];
   static bool known[64];
   const int dev = m.device;
-  if (dev < 0 || dev >= 64 || which < 0 || which > 2) return 0;
+  if (dev < 0 || dev >= 64 || which < 0 || which > 3) return 0;
   {
     std::lock_guard<std::mutex> lk(mu);
     if (!known[dev]) {
       int coop = 0;
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
       const void* ks[] = {(const void*)k_coarsen_rounds, (const void*)k_swap_rounds,
-                          (const void*)k_smooth_rounds};
-      for (int k = 0; k < 3; ++k) {
+                          (const void*)k_smooth_rounds, (const void*)k_colour_rounds};
+      for (int k = 0; k < 4; ++k) {
         int b = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, ks[k], kRoundsThreads, 0) !=
             cudaSuccess)
@@ -3571,7 +3595,7 @@ int rounds_grid(MeshSet& m, int which) {
       known[dev] = true;
     }
   }
-  const int b = std::min(occ[dev][which], tuning().rounds_blocks_per_sm[which]);
+  const int b = std::min(occ[dev][which], tuning().rounds_blocks_per_sm[which == 3 ? 0 : which]);
   return b >= 1 ? m.num_sms * b : 0;
 }
 
@@ -3632,6 +3656,52 @@ int run_rounds(MeshSet& m, int which, const void* kernel, const char* name, Roun
   out.complete = m.hcounts[CN_RES + 2];
   m.tag += 2 * out.rounds;
   return PM_OK;
+}
+
+// Colours every active mesh whose parameters ask for colour-class sets, at
+// the start of a collapse, flip or smoothing pass: speculative rounds until
+// no vertex is left uncoloured (each round keeps at least the proposal of
+// the highest priority; the cap is far beyond any mesh's rounds).
+int colour_set(MeshSet& m) {
+  bool any = false;
+  for (int x : m.select) any |= x == PM_SELECT_COLOUR;
+  if (!any) return PM_OK;
+  Work& w = m.w;
+  const int g = grid_for(m, m.S.vused);
+  const bool persist = rounds_grid(m, 3) > 0;
+  const int limit = kColourLimit;
+  bool bar_clear = true;
+  zero_counts(m, 0, CN_NUM);
+  PM_LAUNCH(k_colour_init, g, BLOCK, 0, m.stream, m.S, w.D[0], w.counts + CN_D0);
+  int cur = 0, nlist = 0;  // entries of the list; unknown (0) at first
+  for (int it = 0; it < (1 << 20); ++it) {
+    if (persist && nlist <= limit) {
+      RoundArgs a = round_args(m, cur, 0, 1 << 20);
+      a.limit = limit;
+      RoundsOut o;
+      int err =
+          run_rounds(m, 3, (const void*)k_colour_rounds, "k_colour_rounds", a, o, bar_clear);
+      if (err) return err;
+      if (o.complete) return PM_OK;
+      cur = o.cur;
+      nlist = m.hcounts[cn_list(cur)];
+      if (nlist <= limit) continue;  // the round cap
+    }
+    const int nxt = 1 - cur;
+    const int rt = (m.tag += 2);
+    zero_counts(m, cn_list(nxt), 1);
+    PM_LAUNCH(k_colour_propose, g, BLOCK, 0, m.stream, m.S, w.D[cur], w.counts + cn_list(cur),
+              w.cprop, w.cstamp, rt);
+    PM_LAUNCH(k_colour_resolve, g, BLOCK, 0, m.stream, m.S, w.D[cur], w.counts + cn_list(cur),
+              w.cprop, w.cstamp, rt, w.D[nxt], w.counts + cn_list(nxt));
+    RoundIO io = read_round(m);
+    if (io.err) return io.err;
+    cur = nxt;
+    nlist = m.hcounts[cn_list(cur)];
+    if (nlist == 0) return PM_OK;
+  }
+  set_last_error("colouring did not finish");
+  return PM_ERR_INVALID_MESH;
 }
 
 }  // namespace
@@ -3931,8 +4001,11 @@ int op_smooth(MeshSet& m, int max_sweeps, int max_rounds) {
     zero_round(m, nxt);
     PM_LAUNCH(k_smooth_scan, gv, bs, 0, m.stream, m.S, w.D[cur], w.counts + cn_list(cur),
               w.mvM, w.C, w.counts + CN_C, w.cmark, tag, pass0, w.E, w.counts + CN_E);
-    PM_LAUNCH(k_smooth_eval, gv, bs, 0, m.stream, m.S, w.E, w.counts + CN_E, w.mvxy, w.mvM, w.gains,
-              w.C, w.counts + CN_C, w.cmark, tag, prof_work("k_smooth_eval"));
+    PM_LAUNCH(k_smooth_filter, gv, bs, 0, m.stream, m.S, w.E, w.counts + CN_E, w.mvxy, w.mvM,
+              w.Sl, w.counts + CN_S, prof_work("k_smooth_filter"));
+    PM_LAUNCH(k_smooth_eval, grid_tuned(m, (long long)m.S.vused * TW, bs, bps), bs, 0, m.stream,
+              m.S, w.Sl, w.counts + CN_S, w.mvxy, w.mvM, w.gains, w.C, w.counts + CN_C, w.cmark,
+              tag, prof_work("k_smooth_eval"));
     PM_LAUNCH(k_smooth_select_apply, gv, bs, 0, m.stream, m.S, w.C, w.counts + CN_C,
               w.cmark, w.smark, tag, w.D[nxt], w.counts + cn_list(nxt), w.dmark, w.mvxy, w.mvM,
               w.gains, w.P, w.counts + CN_P, w.pmark, ptag, tag + 1,

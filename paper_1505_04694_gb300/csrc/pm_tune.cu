@@ -35,7 +35,7 @@ namespace pm {
 
 namespace {
 
-constexpr Tuning kDefaults = {{128, 128, 128, 128}, {16, 16, 16, 16}, {131072, 131072, 131072},
+constexpr Tuning kDefaults = {{128, 128, 128, 128}, {16, 16, 16, 16}, {32768, 131072, 131072},
                                {1, 1, 1}, {1 << 30, 1 << 30}};
 
 std::mutex g_tmu;

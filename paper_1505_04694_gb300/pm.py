@@ -562,7 +562,7 @@ def set_tuning(t=None):
 
 
 def get_tuning_defaults():
-    return {"block": [128] * 4, "blocks_per_sm": [16] * 4, "rounds_limit": [131072] * 3,
+    return {"block": [128] * 4, "blocks_per_sm": [16] * 4, "rounds_limit": [32768, 131072, 131072],
             "rounds_blocks_per_sm": [1] * 3, "fuse_limit": [1 << 30] * 2}
 
 
