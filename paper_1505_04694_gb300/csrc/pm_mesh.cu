@@ -102,8 +102,7 @@ struct Carver {
 // Everything whose size follows the row width W, in one allocation of its own
 // (a change of W replaces it and leaves no hole in the store): the rows of both
 // buffer sets and the collapse candidates.  The spare set's rows are written
-// only by a refinement round and by a compaction, both of which read no flip
-// gain, collapse length or moved ball quality, so those W doubles per vertex
+// only by a compaction, which reads no flip gain, collapse length or moved ball quality, so those W doubles per vertex
 // (Work::gains) share them.
 cudaError_t rows_alloc(MeshSet& m, int W) {
   const size_t n = (size_t)m.S.vslots * W;
@@ -550,23 +549,26 @@ __global__ void k_out_e(Store S, int mesh, const int* vscan, const int* escan, i
 // Element count each mesh's metric asks for, before the factor 4/sqrt(3):
 // the sum over live elements of area * mean sqrt(det M) of its vertices (the
 // number of unit equilateral metric triangles that tile the mesh).  Only
-// sizes storage, so the order of the atomic sums does not matter.
+// sizes storage, so single precision serves (its FP64 form was bound by the FP64
+// pipe, 2.5 ms on 19M elements) and the order of the atomic sums does not matter.
 __global__ void k_estimate(Store S, double* est) {
   const int lane = threadIdx.x & 31;
   for (int s0 = blockIdx.x * blockDim.x; s0 < S.eused; s0 += gridDim.x * blockDim.x) {
     const int s = s0 + (int)threadIdx.x;
     int mi = -1;
-    double x = 0.0;
+    float x = 0.0f;
     if (s < S.eused && eslot_used(S, s, mi)) {
       int4 e = S.EN[s];
       if (e.w) {
         int vb = S.tab.vbase[mi];
-        VD a = load_vd(S, vb + e.x), b = load_vd(S, vb + e.y), c = load_vd(S, vb + e.z);
-        double area = 0.5 * fabs(orient3(a, b, c));
-        double sd = sqrt(fmax(a.m00 * a.m11 - a.m01 * a.m01, 0.0)) +
-                    sqrt(fmax(b.m00 * b.m11 - b.m01 * b.m01, 0.0)) +
-                    sqrt(fmax(c.m00 * c.m11 - c.m01 * c.m01, 0.0));
-        x = area * sd / 3.0;
+        const VF a = load_vf(S, vb + e.x), b = load_vf(S, vb + e.y), c = load_vf(S, vb + e.z);
+        const float area =
+            0.5f * fabsf(f_dx(a, b) * f_dy(a, c) - f_dy(a, b) * f_dx(a, c));
+        const float sd = sqrtf(fmaxf(a.m00 * a.m11 - a.m01 * a.m01, 0.0f)) +
+                         sqrtf(fmaxf(b.m00 * b.m11 - b.m01 * b.m01, 0.0f)) +
+                         sqrtf(fmaxf(c.m00 * c.m11 - c.m01 * c.m01, 0.0f));
+        x = area * sd / 3.0f;
+        if (!isfinite(x)) x = 0.0f;  // (metrics beyond single precision: no estimate)
       }
     }
     // a warp whose slots all belong to one mesh (meshes are contiguous runs
@@ -574,9 +576,9 @@ __global__ void k_estimate(Store S, double* est) {
     const int m0 = __shfl_sync(0xffffffffu, mi, 0);
     if (__all_sync(0xffffffffu, mi == m0) && m0 >= 0) {
       for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-      if (lane == 0) atomicAdd(est + m0, x);
+      if (lane == 0) atomicAdd(est + m0, (double)x);
     } else if (mi >= 0) {
-      atomicAdd(est + mi, x);
+      atomicAdd(est + mi, (double)x);
     }
   }
 }

@@ -155,7 +155,8 @@ __device__ __forceinline__ void elem_quality_phase(const Store& S, const int* li
   }
 }
 
-// Stamps the neighbours in `row` (local ids) after a change of their vertex.
+// Stamps the neighbours in `row` (local ids, whole chunks of 8 readable) after a
+// change of their vertex.
 __device__ __forceinline__ void stamp_neighbours(const Store& S, const int* row, int len, int vb,
                                                  int stamp) {
   for (int b = 0; b < len; b += 8) {
@@ -3087,24 +3088,70 @@ __device__ __forceinline__ int refine_children(const Store& S, int mi, int eb, c
   return 1 + extra;
 }
 
-// New rows of every vertex whose elements changed in this refinement round
-// (stamped), written to the spare buffer B: NE = the children of its old
-// elements that contain it (a new vertex: the children of the elements of its
-// split edge), NN = the other vertices of those, both sorted.
-__global__ void k_refine_rows(Store S, Store B, int vend, const int* vscan, const int* escan,
+// New rows of vertex slot s of a refinement round, from the old element row of
+// `src`: NE = the children of those elements that contain the vertex, NN = the
+// other vertices of those, both sorted.  Rows of up to 16 entries are made in
+// registers; false, with nothing written, when one is longer.
+__device__ __forceinline__ bool refine_row_short(const Store& S, int s, int src, int mi, int vb,
+                                                 int eb, const int* escan, int stamp) {
+  const int lu = s - vb;
+  const int nel = S.NElen[src];
+  Row16 P;
+  P.load(S.NE + (size_t)src * S.W, nel);
+  if (nel > kRowReg) return false;
+  const int base = S.tab.ne[mi] - escan[eb];
+  Row16 N, E;
+#pragma unroll
+  for (int k = 0; k < kRowReg; ++k) N.a[k] = E.a[k] = kRowPad;
+  bool ok = true;
+  for (int k = 0; k < nel; ++k) {
+    // (the row again, in cache: P is indexed by constants only)
+    const int K = S.NE[(size_t)src * S.W + k];
+    const int e0 = escan[eb + K], extra = escan[eb + K + 1] - e0;
+    int4 e[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      e[j] = j <= extra ? S.EN[eb + (j == 0 ? K : base + e0 + j - 1)] : make_int4(-1, -1, -1, 0);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (e[j].x != lu && e[j].y != lu && e[j].z != lu) continue;
+      ok &= E.insert(j == 0 ? K : base + e0 + j - 1);
+      ok &= N.insert((e[j].x == lu) ? e[j].y : e[j].x);
+      ok &= N.insert((e[j].z == lu) ? e[j].y : e[j].z);
+    }
+  }
+  if (!ok) return false;
+  const int nn2 = N.len(), ne2 = E.len();
+  N.store(S.NN + (size_t)s * S.W, nn2);
+  E.store(S.NE + (size_t)s * S.W, ne2);
+  S.NNlen[s] = nn2;
+  S.NElen[s] = ne2;
+#pragma unroll
+  for (int k = 0; k < kRowReg; ++k)
+    if (k < nn2) S.ntouch[vb + N.a[k]] = stamp;
+  return true;
+}
+
+// Rows of the vertices whose elements changed in this refinement round
+// (stamped), in place, in two launches: the new vertices first (`fresh`), which
+// read the old element row of their split edge's first end (the children that
+// contain the new vertex are exactly those of the two parents on that edge), then
+// the old ones, which read and write their own rows alone.
+__global__ void k_refine_rows(Store S, int vfirst, int vend, int fresh, const int* escan,
                               const int4* owner, int stamp, DevStatus* st) {
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < vend; s += gridDim.x * blockDim.x) {
+  for (int s = vfirst + blockIdx.x * blockDim.x + threadIdx.x; s < vend;
+       s += gridDim.x * blockDim.x) {
     if (S.touch[s] != stamp) continue;
-    int mi = mesh_of_vslot(S, s);
-    int vb = S.tab.vbase[mi], eb = S.tab.ebase[mi], nv = S.tab.nv[mi];
-    int lu = s - vb;
-    // the old element row holding the parents: v's own, or for a new vertex
-    // that of its split edge's first end (the children that contain the new
-    // vertex are exactly those of the two parents on that edge)
-    int src = (lu < nv) ? s : vb + owner[s].x;
+    const int mi = mesh_of_vslot(S, s);
+    const int vb = S.tab.vbase[mi], eb = S.tab.ebase[mi], nv = S.tab.nv[mi];
+    const int lu = s - vb;
+    if ((lu >= nv) != (fresh != 0)) continue;
+    const int src = fresh ? vb + owner[s].x : s;
+    if (refine_row_short(S, s, src, mi, vb, eb, escan, stamp)) continue;
     const int* ne = S.NE + (size_t)src * S.W;
-    int nel = S.NElen[src];
-    int eb_[MAXW], nb_[MAXW];
+    const int nel = S.NElen[src];
+    __align__(16) int nb_[MAXW];  // read in chunks below
+    int eb_[MAXW];
     int ne2 = 0, nn2 = 0;
     bool ok = true;
     for (int k = 0; k < nel; ++k) {
@@ -3126,25 +3173,13 @@ __global__ void k_refine_rows(Store S, Store B, int vend, const int* vscan, cons
       atomicMax(&st->maxdeg, max(ne2, nn2));
       continue;
     }
-    int* wn = B.NN + (size_t)s * B.W;
-    int* we = B.NE + (size_t)s * B.W;
+    int* wn = S.NN + (size_t)s * S.W;
+    int* we = S.NE + (size_t)s * S.W;
     for (int k = 0; k < nn2; ++k) wn[k] = nb_[k];
     for (int k = 0; k < ne2; ++k) we[k] = eb_[k];
-    B.NNlen[s] = nn2;
-    B.NElen[s] = ne2;
-  }
-}
-
-__global__ void k_refine_rows_copy(Store S, Store B, int vend, int stamp) {
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < vend; s += gridDim.x * blockDim.x) {
-    if (S.touch[s] != stamp) continue;
-    int a = B.NNlen[s], b = B.NElen[s];
-    const int* nn = B.NN + (size_t)s * B.W;
-    for (int k = 0; k < a; ++k) S.NN[(size_t)s * S.W + k] = nn[k];
-    for (int k = 0; k < b; ++k) S.NE[(size_t)s * S.W + k] = B.NE[(size_t)s * B.W + k];
-    S.NNlen[s] = a;
-    S.NElen[s] = b;
-    stamp_neighbours(S, nn, a, S.tab.vbase[mesh_of_vslot(S, s)], stamp);
+    S.NNlen[s] = nn2;
+    S.NElen[s] = ne2;
+    stamp_neighbours(S, nb_, nn2, vb, stamp);
   }
 }
 
@@ -3922,10 +3957,12 @@ int op_refine(MeshSet& m, int max_rounds) {
     PM_LAUNCH(k_refine_split, ge, bs, 0, m.stream, m.S, w.escan, w.emid, w.elist,
               w.counts + CN_EL, w.clist, w.counts + CN_CL, stamp);
     PM_LAUNCH(k_refine_quality, ge, bs, 0, m.stream, m.S, w.clist, w.counts + CN_CL, nullptr);
-    // rows of the vertices whose elements changed, through the spare buffer
-    PM_LAUNCH(k_refine_rows, grid_tuned(m, vend, bs, bps), bs, 0, m.stream, m.S, m.B, vend, w.vscan,
-              w.escan, w.opA, stamp, m.st);
-    PM_LAUNCH(k_refine_rows_copy, grid_tuned(m, vend, bs, bps), bs, 0, m.stream, m.S, m.B, vend, stamp);
+    // rows of the vertices whose elements changed: the new ones, then the old ones
+    const int vnew = m.nmesh == 1 ? m.nv[0] : 0;
+    PM_LAUNCH(k_refine_rows, grid_tuned(m, vend - vnew, bs, bps), bs, 0, m.stream, m.S, vnew, vend, 1,
+              (const int*)w.escan, (const int4*)w.opA, stamp, m.st);
+    PM_LAUNCH(k_refine_rows, gv, bs, 0, m.stream, m.S, 0, m.S.vused, 0, (const int*)w.escan,
+              (const int4*)w.opA, stamp, m.st);
     PM_LAUNCH(k_refine_sizes, (m.nmesh + 127) / 128, 128, 0, m.stream, m.S, (const int*)w.vscan,
               (const int*)w.escan, w.counts);
     // the new sizes and the status in one read-back
