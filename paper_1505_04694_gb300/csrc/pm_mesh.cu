@@ -1286,7 +1286,12 @@ int presize(MeshSet& m) {
     et += ecap[i];
   }
   if (!need || vt >= (1LL << 31) - 4 || et >= (1LL << 31) - 4) return PM_OK;
-  e = grow(m, vcap, ecap, m.S.W);
+  // A set of many vertices nearly always meets one of more than 16 neighbours, and
+  // widening the rows later rebuilds every row in storage of its own: such sets
+  // start with 32 (20M slots: 100.2 -> 95.1 ms, 42M slots: 260 -> 255 ms; at 3M
+  // slots, where the rebuild is cheap, rows of 16 are faster, 10.93 against 11.09).
+  constexpr long long kWideRowsFrom = 1LL << 23;
+  e = grow(m, vcap, ecap, vt >= kWideRowsFrom ? std::max(m.S.W, 32) : m.S.W);
   if (e) {
     set_last_error(std::string("growing mesh storage: ") + cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? PM_ERR_OOM : PM_ERR_CUDA;
