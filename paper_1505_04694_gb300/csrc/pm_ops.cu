@@ -397,6 +397,7 @@ __device__ __forceinline__ void round_done(const Store& S, unsigned* done) {
 // depend on order.  All lanes of a tile end with the same result.
 
 constexpr int TW = 8;
+constexpr int kTileMax = 32;  // tiles per block (blocks hold at most 256 threads)
 
 struct Tile {
   int tl;          // lane within the tile
@@ -2274,6 +2275,25 @@ __device__ __forceinline__ double4 interpolate_in(const Store& S, int vb, int4 e
                       (l0 * a.m11 + l1 * b.m11) + l2 * d.m11, 0.0);
 }
 
+// The same by the lanes of a tile, which all hold e: lanes 0 to 3 take one of the
+// four areas each, lanes 0 to 2 one weight and one entry (about 24 FP64
+// instructions of the warp instead of 73, the values by the same operations).
+__device__ __forceinline__ double4 tile_interpolate_in(const Tile& t, const Store& S, int vb, int4 e,
+                                                       double X, double Y) {
+  const VD px{X, Y, 0.0, 0.0, 0.0};
+  int i0 = e.x, i1 = e.y, i2 = e.z;
+  VD a = load_vd(S, vb + i0), b = load_vd(S, vb + i1), d = load_vd(S, vb + i2);
+  canon(i0, i1, i2, a, b, d);
+  const double det = orient3(t.tl == 0 ? px : a, t.tl == 1 ? px : b, t.tl == 2 ? px : d);
+  const double l = det / tshfl(t, det, 3);
+  const double l0 = tshfl(t, l, 0), l1 = tshfl(t, l, 1), l2 = tshfl(t, l, 2);
+  const double ma = t.tl == 0 ? a.m00 : (t.tl == 1 ? a.m01 : a.m11);
+  const double mb = t.tl == 0 ? b.m00 : (t.tl == 1 ? b.m01 : b.m11);
+  const double md = t.tl == 0 ? d.m00 : (t.tl == 1 ? d.m01 : d.m11);
+  const double m = (l0 * ma + l1 * mb) + l2 * md;
+  return make_double4(tshfl(t, m, 0), tshfl(t, m, 1), tshfl(t, m, 2), 0.0);
+}
+
 // Upper bound of the quality of element e of v's ball with v at the record `fn`
 // (relative error kx of its metric), -1 when it is certainly not
 // counter-clockwise, NaN when there is no useful bound.
@@ -2368,9 +2388,7 @@ __device__ bool tile_try_move(const Tile& t, const Store& S, MeshCtx c, int lv, 
     // (the sum of at most 128 bounds is short by 128 u of itself at most)
     if (up * 1.00001f < __double2float_rd(sum_old)) return false;
   }
-  double4 m = make_double4(0.0, 0.0, 0.0, 0.0);
-  if (t.tl == src) m = interpolate_in(S, c.vb, eat, X, Y);
-  Mout = make_double4(tshfl(t, m.x, src), tshfl(t, m.y, src), tshfl(t, m.z, src), 0.0);
+  Mout = tile_interpolate_in(t, S, c.vb, eat, X, Y);
   if (t.tl == 0) ops += 46 + 85 * nel;
   return tile_ball_exact(t, S, c, lv, ne, nel, X, Y, Mout, floor, strict, qout, qsum);
 }
@@ -2392,34 +2410,41 @@ __device__ bool tile_smooth_eval(const Tile& t, const Store& S, int v, MeshCtx c
   const int* nn = nn_row(S, v);
   int nnl = S.NNlen[v];
   double4 mv = S.M[v];
-  double a00 = 0.0, a01 = 0.0, a11 = 0.0, b0 = 0.0, b1 = 0.0;
+  // Five ordered sums over the neighbours, one on each of five lanes (through
+  // shared memory: a sixth of the FP64 instructions of every lane adding all
+  // five), then x on the even lanes and y on the odd ones.
+  __shared__ double s_lap[kTileMax][TW][5];
+  double (*lap)[5] = s_lap[(threadIdx.x / TW) % kTileMax];
+  double acc = 0.0;
   for (int base = 0; base < nnl; base += TW) {
-    int k = base + t.tl;
-    double w00 = 0.0, w01 = 0.0, w11 = 0.0, t0 = 0.0, t1 = 0.0;
+    const int k = base + t.tl;
     if (k < nnl) {
-      int js = c.vb + nn[k];
-      double2 pj = S.xy[js];
-      double4 mj = S.M[js];
-      w00 = 0.5 * (mv.x + mj.x);
-      w01 = 0.5 * (mv.y + mj.y);
-      w11 = 0.5 * (mv.z + mj.z);
-      t0 = w00 * pj.x + w01 * pj.y;
-      t1 = w01 * pj.x + w11 * pj.y;
+      const int js = c.vb + nn[k];
+      const double2 pj = S.xy[js];
+      const double4 mj = S.M[js];
+      const double w00 = 0.5 * (mv.x + mj.x);
+      const double w01 = 0.5 * (mv.y + mj.y);
+      const double w11 = 0.5 * (mv.z + mj.z);
+      lap[t.tl][0] = w00;
+      lap[t.tl][1] = w01;
+      lap[t.tl][2] = w11;
+      lap[t.tl][3] = w00 * pj.x + w01 * pj.y;
+      lap[t.tl][4] = w01 * pj.x + w11 * pj.y;
     }
-    int cnt = min(TW, nnl - base);
-    for (int j = 0; j < cnt; ++j) {
-      a00 = a00 + tshfl(t, w00, j);
-      a01 = a01 + tshfl(t, w01, j);
-      a11 = a11 + tshfl(t, w11, j);
-      b0 = b0 + tshfl(t, t0, j);
-      b1 = b1 + tshfl(t, t1, j);
-    }
+    __syncwarp(t.mask);
+    const int cnt = min(TW, nnl - base);
+    if (t.tl < 5)
+      for (int j = 0; j < cnt; ++j) acc = acc + lap[j][t.tl];
+    __syncwarp(t.mask);
   }
+  const double a00 = tshfl(t, acc, 0), a01 = tshfl(t, acc, 1), a11 = tshfl(t, acc, 2),
+               b0 = tshfl(t, acc, 3), b1 = tshfl(t, acc, 4);
   if (t.tl == 0) ops += 17 * nnl + 3;
-  double det = a00 * a11 - a01 * a01;
+  const double det = a00 * a11 - a01 * a01;
   if (!dgt(det, 0.0)) return false;
-  double x = (a11 * b0 - a01 * b1) / det;
-  double y = (a00 * b1 - a01 * b0) / det;
+  const bool odd = t.tl & 1;
+  const double z = ((odd ? a00 : a11) * (odd ? b1 : b0) - a01 * (odd ? b0 : b1)) / det;
+  const double x = tshfl(t, z, 0), y = tshfl(t, z, 1);
   if (t.tl == 0) ops += 8;
   Xo = make_double2(x, y);
   return tile_try_move(t, S, c, v - c.vb, ne, nel, x, y, qold, true, qout, nullptr, 0.0, Mo, ops);
@@ -2613,6 +2638,94 @@ __device__ __forceinline__ void smooth_scan_eval_phase(Store S, const int* D, co
   add_work(work, ops);
 }
 
+// Pass 3 of the large rounds: the same with the ball elements of five or so moves
+// side by side in a warp (a tile of 8 lanes per move leaves a quarter of them idle
+// at six elements a ball, and the FP64 pipe is what bounds this pass).  Each warp
+// walks a range of the list and takes as many moves at a time as fit 32 lanes; a
+// ball of more than 32 elements takes the warp alone.
+__device__ __forceinline__ void smooth_exact_packed(Store S, const int* R, const int* nRp,
+                                                    const double2* mvxy, double4* mvM,
+                                                    double* qball, int* C, int* nC, int* cmark,
+                                                    int tag, unsigned long long* work) {
+  const int n = *nRp;
+  const int lane = threadIdx.x & 31;
+  const int warps = gridDim.x * (blockDim.x >> 5);
+  const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int per = (n + warps - 1) / warps;
+  const int end = min(n, (w + 1) * per);
+  unsigned ops = 0;
+  for (int pos = w * per; pos < end;) {
+    // lanes 0..7: the next moves and their balls' places among the 32 lanes
+    int v = 0, nel = 0;
+    if (lane < 8 && pos + lane < end) {
+      v = R[pos + lane];
+      nel = S.NElen[v];
+    }
+    int incl = nel;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
+    }
+    const unsigned fit = __ballot_sync(0xffffffffu, lane < 8 && nel > 0 && incl <= 32);
+    int cnt = __ffs(~fit) - 1;  // moves taken: the leading ones that fit
+    if (cnt == 0) cnt = 1;
+    // my move and element
+    int own = -1, k = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int hi = __shfl_sync(0xffffffffu, incl, j), len = __shfl_sync(0xffffffffu, nel, j);
+      if (j < cnt && lane >= hi - len && lane < hi) {
+        own = j;
+        k = lane - (hi - len);
+      }
+    }
+    const int from = own >= 0 ? own : 0;
+    const int mv_v = __shfl_sync(0xffffffffu, v, from);
+    const int mv_n = __shfl_sync(0xffffffffu, nel, from);
+    bool ok = true;
+    if (own >= 0) {
+      const MeshCtx c = ctx_of(S, mv_v);
+      const int lv = mv_v - c.vb;
+      const double2 X = mvxy[mv_v];
+      const double4 M = mvM[mv_v];  // (its w holds the old minimum quality)
+      const VD nvd{X.x, X.y, M.x, M.y, M.z};
+      for (; k < mv_n; k += 32) {  // (one turn unless the ball takes the warp alone)
+        const int4 e = S.EN[c.eb + ne_row(S, mv_v)[k]];
+        const VD a = (e.x == lv) ? nvd : load_vd(S, c.vb + e.x);
+        const VD b = (e.y == lv) ? nvd : load_vd(S, c.vb + e.y);
+        const VD d = (e.z == lv) ? nvd : load_vd(S, c.vb + e.z);
+        ops += kOpsOrient + kOpsQuality;
+        if (orient_sign(a, b, d) > 0) {
+          const double q = quality_c(e.x, e.y, e.z, a, b, d);
+          ok &= dgt(q, M.w);
+          // the new ball qualities of an accepted move are kept for the apply
+          qball[(size_t)mv_v * S.W + k] = q;
+        } else {
+          ok = false;
+        }
+      }
+    }
+    const unsigned bad = __ballot_sync(0xffffffffu, !ok);
+    // lane j < cnt: the answer of move j
+    bool cand = false;
+    if (lane < cnt) {
+      const int lo = min(incl - nel, 32), hi = min(incl, 32);
+      const unsigned mask = (hi >= 32 ? 0xffffffffu : (1u << hi) - 1u) &
+                            ~(lo >= 32 ? 0xffffffffu : (1u << lo) - 1u);
+      cand = (bad & mask) == 0u;
+      mvM[v].w = cand ? 1.0 : 0.0;  // marks a stored move
+      if (cand) {
+        cmark[v] = tag;
+        S.tab.had[ctx_of(S, v).mi] = 1;
+      }
+    }
+    warp_append(cand, v, C, nC);
+    pos += cnt;
+  }
+  add_work(work, ops);
+}
+
 __global__ void k_smooth_filter(Store S, const int* E, const int* nEp, double2* mvxy,
                                 double4* mvM, int* R, int* nR, unsigned long long* work) {
   smooth_filter_phase(S, E, nEp, mvxy, mvM, R, nR, work);
@@ -2621,68 +2734,13 @@ __global__ void k_smooth_filter(Store S, const int* E, const int* nEp, double2* 
 __global__ void k_smooth_eval(Store S, const int* R, const int* nRp, const double2* mvxy,
                               double4* mvM, double* qball, int* C, int* nC, int* cmark, int tag,
                               unsigned long long* work) {
-  smooth_exact_phase(S, R, nRp, mvxy, mvM, qball, C, nC, cmark, tag, work);
+  smooth_exact_packed(S, R, nRp, mvxy, mvM, qball, C, nC, cmark, tag, work);
 }
 
-// Move the members of S; live interior neighbours become pending for the next
-// sweep (stamp pmark with the sweep tag).
-__device__ __forceinline__ void smooth_apply_one(const Store& S, bool ok, int v,
-                                                 const double2* mvxy, const double4* mvM,
-                                                 const double* qball, int* P, int* nP,
-                                                 int* pmark, int ptag, int stamp) {
-  {
-    int mi = 0, vb = 0, nnl = 0;
-    const int* nn = nullptr;
-    RowMask take;
-    if (ok) {
-      MeshCtx c = ctx_of(S, v);
-      mi = c.mi;
-      vb = c.vb;
-      const double2 p = mvxy[v];
-      double4 mv = mvM[v];
-      mv.w = 0.0;
-      S.xy[v] = p;
-      S.M[v] = mv;
-      store_vf(S, v, p, mv);
-      S.touch[v] = stamp;
-      const int* ne = ne_row(S, v);
-      int nel = S.NElen[v];
-      for (int b = 0; b < nel; b += 8) {
-        const Row8 r = row8(ne, b);
-        double q[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) q[k] = b + k < nel ? qball[(size_t)v * S.W + b + k] : 0.0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-          if (b + k < nel) S.qK[c.eb + r.a[k]] = q[k];
-      }
-      nn = nn_row(S, v);
-      nnl = S.NNlen[v];
-      // (a stamp on a vertex that is not taken is harmless: only interior
-      // neighbours look at it)
-      for (int b = 0; b < nnl; b += 8) {
-        const Row8 r = row8(nn, b);
-        int op[8], f[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const bool in = b + k < nnl;
-          const int s = vb + r.a[k];
-          f[k] = in ? S.vflag[s] : VF_BND;
-          op[k] = in ? atomicExch(pmark + s, ptag) : ptag;
-          if (in) S.ntouch[s] = stamp;
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-          if (op[k] != ptag && (f[k] & VF_ALIVE) && !(f[k] & VF_BND)) take.set(b + k);
-      }
-    }
-    count_op(S, ok, mi);
-    int pp = warp_reserve(take.count(), nP);
-    write_row_bits(take, nn, vb, P, pp);
-  }
-}
-
-// One round's independent set and its moves (see k_coarsen_select_apply).
+// One round's independent set and its moves (see k_coarsen_select_apply); live
+// interior neighbours of a moved vertex become pending for the next sweep (stamp
+// pmark with the sweep tag).  What the move needs is loaded beside the
+// independent set's gathers, and the round's two lists share a reservation.
 __device__ __forceinline__ void smooth_select_apply_phase(Store S, const int* C, const int* nCp,
                                                           const int* cmark, int* smark, int tag,
                                                           int* Dn, int* nDn, int* dmark,
@@ -2695,15 +2753,64 @@ __device__ __forceinline__ void smooth_select_apply_phase(Store S, const int* C,
   for (int i0 = 0; i0 < n; i0 += gsize()) {
     int i = i0 + grank(il);
     bool win = false, lose = false;
-    int v = 0;
+    int v = 0, mi = 0, vb = 0, nnl = 0;
+    const int* nn = nullptr;
+    RowMask take;
     if (i < n) {
       v = i0 == 0 ? first : C[i];
+      const double2 p = mvxy[v];
+      double4 mv = mvM[v];
+      const MeshCtx c = ctx_of(S, v);
+      const int* ne = ne_row(S, v);
+      Row8 er = row8(ne, 0);
+      const int nel = S.NElen[v];
       win = local_max(S, v, cmark, tag);
-      if (win) smark[v] = tag;
-      else lose = stamp_first(dmark, v, tag);
+      if (!win) lose = stamp_first(dmark, v, tag);
+      if (win) {
+        mi = c.mi;
+        vb = c.vb;
+        nn = nn_row(S, v);
+        nnl = S.NNlen[v];
+        for (int b = 0; b < nnl; b += 8) {
+          const Row8 r = row8(nn, b);
+          int op[8], f[8];
+          // (a stamp on a vertex that is not taken is harmless: only interior
+          // neighbours look at it)
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const bool in = b + k < nnl;
+            const int s = vb + r.a[k];
+            f[k] = in ? S.vflag[s] : VF_BND;
+            op[k] = in ? atomicExch(pmark + s, ptag) : ptag;
+            if (in) S.ntouch[s] = stamp;
+          }
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            if (op[k] != ptag && (f[k] & VF_ALIVE) && !(f[k] & VF_BND)) take.set(b + k);
+        }
+        smark[v] = tag;
+        mv.w = 0.0;
+        S.xy[v] = p;
+        S.M[v] = mv;
+        store_vf(S, v, p, mv);
+        S.touch[v] = stamp;
+        for (int b = 0;;) {
+          double q[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) q[k] = b + k < nel ? qball[(size_t)v * S.W + b + k] : 0.0;
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            if (b + k < nel) S.qK[c.eb + er.a[k]] = q[k];
+          b += 8;
+          if (b >= nel) break;
+          er = row8(ne, b);
+        }
+      }
     }
-    warp_append(lose, v, Dn, nDn);
-    smooth_apply_one(S, win, v, mvxy, mvM, qball, P, nP, pmark, ptag, stamp);
+    count_op(S, win, mi);
+    const Room3 at = warp_reserve3(take.count(), nP, lose ? 1 : 0, nDn, 0, nullptr);
+    write_row_bits(take, nn, vb, P, at.a);
+    if (lose) Dn[at.b] = v;
   }
 }
 
