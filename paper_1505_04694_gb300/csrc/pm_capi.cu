@@ -254,6 +254,7 @@ pm_status begin_call(MeshSet& m, const pm_params* P, int stride) {
   if (s) return s;
   // operation counts, round counters and candidate flags lie together
   cudaMemsetAsync(m.ops, 0, (size_t)((char*)m.S.tab.active - (char*)m.ops), m.stream);
+  std::fill(m.seen_dead.begin(), m.seen_dead.end(), 0);
   cudaMemsetAsync(m.S.tab.active, 0xFF, m.nmesh * sizeof(int), m.stream);
   cudaMemsetAsync(m.st, 0, sizeof(DevStatus), m.stream);
   // evaluations from earlier calls may predate a new metric or parameters
@@ -323,8 +324,10 @@ pm_status adapt_set(MeshSet& m, const pm_params* P, int stride, CallStats& cs) {
     select_ops(m, OS_SWAP);
     if ((err = op_swap(m, mr))) return (pm_status)err;
     select_ops(m, OS_REFINE);
-    if ((err = op_refine(m, mr))) return (pm_status)err;
-    if ((err = renumber(m, false))) return (pm_status)err;  // reads the call state back
+    bool queued = false;
+    if ((err = op_refine(m, mr, &queued))) return (pm_status)err;
+    // reads the call state back, unless the refinement has
+    if ((err = renumber(m, false, queued))) return (pm_status)err;
     const unsigned long long* h = m.hops;
     for (int i = 0; i < n; ++i) {
       const long long c_i = (long long)(h[i] - seen[i]);
@@ -644,6 +647,7 @@ pm_status pm_adapt_batch(pm_mesh** meshes, int32_t n, const pm_params* params, p
     if (!st) st = copy_region(b, i, meshes[i]->set, 0, b.stream);
   }
   b.qvalid = true;  // the copied cache of every mesh is current
+  for (int i = 0; i < n && !st; ++i) b.edead[i] = meshes[i]->set.edead[0];
   CallStats cs;
   cs.init(n);
   if (!st) st = begin_call(b, params, 1);
@@ -663,6 +667,7 @@ pm_status pm_adapt_batch(pm_mesh** meshes, int32_t n, const pm_params* params, p
     s.nv[0] = b.nv[i];
     s.ne[0] = b.ne[i];
     s.dense = b.dense;
+    s.edead[0] = 0;  // the copy is compacted
     s.S.lid = s.S.voff = nullptr;  // ids are the slot offsets of the compacted copy
     st = cuda_status(upload_tab(s), "mesh table");
     if (!st) st = copy_region(s, 0, b, i, b.stream);

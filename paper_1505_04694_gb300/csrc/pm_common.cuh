@@ -34,6 +34,7 @@ struct MeshTab {
   int* had;     // 1 when the mesh formed candidates this round (2 * nmesh)
   int* active;  // mesh takes part in the current phase
   unsigned long long* ops;       // operations applied in the current call, of the running operator
+  unsigned long long* bnd;       // collapses of boundary edges in the current call
   double* L_low;                 // per-mesh parameters
   double* L_up;
   double* q_thresh;

@@ -77,6 +77,11 @@ enum CountIdx {
   CN_RENUM = 22,  // renumbering: 1 when some mesh's compaction is not the identity
   CN_NUM = 23
 };
+// Words per mesh after the counters: live counts (vertices, elements; two per
+// mesh), the new vertices of a refinement round, the sizes after it.
+constexpr int kMeshWords = 5;
+constexpr int cn_newv(int n) { return CN_NUM + 2 * n; }
+constexpr int cn_sizes(int n) { return CN_NUM + 3 * n; }
 // What a persistent smoothing launch leaves at CN_RES: rounds with candidates,
 // sweeps finished, 1 when the sweeps are over, 1 when the current sweep has
 // moved a vertex, the buffers holding the current, the next and the pending list
@@ -102,9 +107,11 @@ struct MeshSet {
   DevStatus* st = nullptr;     // device
   DevStatus* hst = nullptr;    // pinned host
   int* hcounts = nullptr;      // pinned host copy of w.counts
-  unsigned long long* hops = nullptr;  // pinned: operation counts (see OpSlot, 4 * nmesh)
+  unsigned long long* hops = nullptr;  // pinned: operation counts (see OpSlot, OS_NUM * nmesh)
   uint32_t* hr = nullptr;              // pinned: round counters
-  unsigned long long* ops = nullptr;   // device: operation counts of the call (4 * nmesh)
+  unsigned long long* ops = nullptr;   // device: operation counts of the call
+  std::vector<long long> edead;        // dead element slots of each mesh
+  std::vector<long long> seen_dead;    // those of the current call counted so far
   bool dense = false;  // no dead slot: ids are the slot offsets and the sizes are nv, ne
   char* hup = nullptr;                 // pinned: staging of the per-mesh table for upload_tab
   cudaEvent_t upev = nullptr;          // the last table upload has left the staging
@@ -137,7 +144,12 @@ void set_used(MeshSet& m);
 cudaError_t grow(MeshSet& m, const std::vector<int>& vcap, const std::vector<int>& ecap, int W);
 int rebuild_adjacency(MeshSet& m, bool derive_flags, bool corners_given);
 int presize(MeshSet& m);
-int renumber(MeshSet& m, bool final);
+// The part of a renumbering inside the outer loop that runs before its
+// read-back (sync_call); `renumber` does it unless it has been queued.
+// The scan of the live vertices goes to `vscan` (vslots + 1), which has to be
+// Work::vscan when `renumber` runs.
+void renumber_queue(MeshSet& m, int* vscan);
+int renumber(MeshSet& m, bool final, bool queued = false);
 int compact_out(MeshSet& m, int mesh, double* xy, int32_t* tri, double* mt, int* nv_out,
                 int* ne_out);
 int compact_out_set(MeshSet& m, double* xy, int32_t* tri, double* mt, int* nv_out, int* ne_out);
@@ -156,11 +168,13 @@ cudaError_t refresh_sizes(MeshSet& m);
 // ---- operators (pm_ops.cu) ----
 int op_coarsen(MeshSet& m, int max_rounds);
 int op_swap(MeshSet& m, int max_rounds);
-int op_refine(MeshSet& m, int max_rounds);
+int op_refine(MeshSet& m, int max_rounds, bool* renumber_queued = nullptr);
 int op_smooth(MeshSet& m, int max_sweeps, int max_rounds);
 int op_opt_smooth(MeshSet& m, int nrounds, int max_rounds);
 // Operation counters of a call: one set per operator, selected before it runs.
-enum OpSlot { OS_COARSEN = 0, OS_SWAP, OS_REFINE, OS_SMOOTH };
+// OS_BND counts the collapses that kill one element (a boundary edge) instead of
+// two, so that the host knows the dead elements without a pass over them.
+enum OpSlot { OS_COARSEN = 0, OS_SWAP, OS_REFINE, OS_SMOOTH, OS_BND, OS_NUM };
 inline void select_ops(MeshSet& m, OpSlot k) { m.S.tab.ops = m.ops + (size_t)k * m.nmesh; }
 
 // ---- quality (pm_quality.cu) ----

@@ -411,15 +411,16 @@ __global__ void k_table_totals(Store S, int* out) {
   out[2 * i + 1] = S.tab.ne[i];
 }
 
-// Live counts of every mesh; with `changed`, records whether any mesh has a
-// dead slot (its compaction is not the identity).
+// Live counts of every mesh (without `escan` the used element slots); with
+// `changed`, records whether any mesh has a dead slot (its compaction is not the
+// identity).
 __global__ void k_mesh_totals(Store S, const int* vscan, const int* escan, int* out,
                               int* changed) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= S.nmesh) return;
   int vb = S.tab.vbase[i], eb = S.tab.ebase[i];
   out[2 * i] = vscan[vb + S.tab.nv[i]] - vscan[vb];
-  out[2 * i + 1] = escan[eb + S.tab.ne[i]] - escan[eb];
+  out[2 * i + 1] = escan ? escan[eb + S.tab.ne[i]] - escan[eb] : S.tab.ne[i];
   if (changed && (out[2 * i] != S.tab.nv[i] || out[2 * i + 1] != S.tab.ne[i]))
     atomicOr(changed, 1);
 }
@@ -873,12 +874,12 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   T.emesh = emesh;
   T.col = col;
   m.mesh_index_ok = n == 1;
-  // State of a call, kept over growths: status, counters (and two words per mesh
+  // State of a call, kept over growths: status, counters (and some words per mesh
   // after them), operation counts, round counters, candidate flags, active flags.
   // The host reads it back in one copy, into a pinned image of its first part.
-  const size_t counts_bytes = (CN_NUM + 2 * (size_t)n + 8) * sizeof(int);
+  const size_t counts_bytes = (CN_NUM + kMeshWords * (size_t)n + 8) * sizeof(int);
   const size_t ops_off = 64 + ((counts_bytes + 7) & ~size_t(7));
-  const size_t r_off = ops_off + 4 * (size_t)n * sizeof(unsigned long long);
+  const size_t r_off = ops_off + OS_NUM * (size_t)n * sizeof(unsigned long long);
   const size_t had_off = r_off + (size_t)n * sizeof(uint32_t);
   const size_t act_off = had_off + 2 * (size_t)n * sizeof(int);
   if (!m.st) {
@@ -905,6 +906,9 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   char* call = (char*)m.st;
   w.counts = (int*)(call + 64);
   m.ops = T.ops = (unsigned long long*)(call + ops_off);
+  T.bnd = m.ops + (size_t)OS_BND * n;
+  m.edead.resize(n, 0);
+  m.seen_dead.resize(n, 0);
   T.r = (uint32_t*)(call + r_off);
   T.had = (int*)(call + had_off);  // two sets: persistent rounds alternate
   T.active = (int*)(call + act_off);
@@ -1035,7 +1039,16 @@ int sync_counts(MeshSet& m, int extra) {
 }
 
 int sync_call(MeshSet& m) {
-  return sync_bytes(m, (size_t)((char*)(m.S.tab.r + m.nmesh) - (char*)m.st));
+  const int err = sync_bytes(m, (size_t)((char*)(m.S.tab.r + m.nmesh) - (char*)m.st));
+  // a collapse kills the two elements of its edge, one at the boundary
+  const size_t n = m.nmesh;
+  for (size_t i = 0; !err && i < n; ++i) {
+    const long long dead =
+        2 * (long long)m.hops[OS_COARSEN * n + i] - (long long)m.hops[OS_BND * n + i];
+    m.edead[i] += dead - m.seen_dead[i];
+    m.seen_dead[i] = dead;
+  }
+  return err;
 }
 
 // Build NN and NE from the element list for every mesh of the set.  With
@@ -1094,16 +1107,26 @@ void validate_mesh(MeshSet& m) {
 // the live slots together (compaction); the others leave every slot in place
 // and record the new vertex ids (only the priorities read id values; every
 // other use of an id is an order, which both numberings share).
-int renumber(MeshSet& m, bool final) {
+void renumber_queue(MeshSet& m, int* vscan) {
+  scan_alive_vertices(m.S, vscan, m.S.vused, m.scan, m.st, m.stream);
+  PM_LAUNCH(k_mesh_totals, (m.nmesh + 127) / 128, 128, 0, m.stream, m.S, (const int*)vscan,
+            (const int*)nullptr, m.w.counts + CN_NUM, (int*)nullptr);
+}
+
+int renumber(MeshSet& m, bool final, bool queued) {
   Work& w = m.w;
-  scan_alive_vertices(m.S, w.vscan, m.S.vused, m.scan, m.st, m.stream);
-  scan_alive_elements(m.S, w.escan, m.S.eused, m.scan, m.st, m.stream);
   int* tot = w.counts + CN_NUM;
   // (only the compaction queued below looks at the flag)
   int* changed = final ? w.counts + CN_RENUM : nullptr;
-  if (final) cudaMemsetAsync(changed, 0, sizeof(int), m.stream);
-  PM_LAUNCH(k_mesh_totals, (m.nmesh + 127) / 128, 128, 0, m.stream, m.S, w.vscan, w.escan, tot,
-            changed);
+  auto count_all = [&] {
+    if (final) scan_alive_vertices(m.S, w.vscan, m.S.vused, m.scan, m.st, m.stream);
+    scan_alive_elements(m.S, w.escan, m.S.eused, m.scan, m.st, m.stream);
+    if (final) cudaMemsetAsync(changed, 0, sizeof(int), m.stream);
+    PM_LAUNCH(k_mesh_totals, (m.nmesh + 127) / 128, 128, 0, m.stream, m.S, w.vscan,
+              (const int*)w.escan, tot, changed);
+  };
+  if (final) count_all();
+  else if (!queued) renumber_queue(m, w.vscan);
   // compaction into the second buffer set (skipped on the device when no
   // slot died); the host swaps the sets afterwards
   auto compact = [&] {
@@ -1117,11 +1140,12 @@ int renumber(MeshSet& m, bool final) {
   };
   if (final) compact();  // queued before the read-back: one synchronisation
   // sizes, operation counts, rounds and status in one read-back
-  int err = sync_call(m);
+  int err = queued ? PM_OK : sync_call(m);
   if (err) return err;
   const int* ht = m.hcounts + CN_NUM;
   bool died = false;
-  for (int i = 0; i < m.nmesh; ++i) died |= ht[2 * i] != m.nv[i] || ht[2 * i + 1] != m.ne[i];
+  for (int i = 0; i < m.nmesh; ++i)
+    died |= ht[2 * i] != m.nv[i] || (final && ht[2 * i + 1] != m.ne[i]);
   if (!died) {  // every id stays
     if (final) m.dense = true;
     return PM_OK;
@@ -1130,7 +1154,7 @@ int renumber(MeshSet& m, bool final) {
     long long vdead = 0, edead = 0;
     for (int i = 0; i < m.nmesh; ++i) {
       vdead += m.nv[i] - ht[2 * i];
-      edead += m.ne[i] - ht[2 * i + 1];
+      edead += m.edead[i];
     }
     long long vu = 0, eu = 0;
     for (int i = 0; i < m.nmesh; ++i) {
@@ -1144,8 +1168,11 @@ int renumber(MeshSet& m, bool final) {
                 m.lidbuf, m.voffbuf);
       return PM_OK;
     }
+    count_all();
     compact();
+    if ((err = sync_call(m))) return err;
   }
+  std::fill(m.edead.begin(), m.edead.end(), 0);
   for (int i = 0; i < m.nmesh; ++i) {
     m.nv[i] = ht[2 * i];
     m.ne[i] = ht[2 * i + 1];

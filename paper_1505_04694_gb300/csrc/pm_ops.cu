@@ -1123,6 +1123,7 @@ __device__ __forceinline__ void coarsen_select_apply_phase(Store S, const int* C
       // the ball is read first (all loads in flight), then only the words that
       // change are written: v's slot takes w, or the alive word is cleared in
       // the elements that hold w
+      int dead = 0;
       for (int b = 0; b < nel; b += 8) {
         const Row8 r = row8(ne, b);
         int4 e[8];
@@ -1136,8 +1137,10 @@ __device__ __forceinline__ void coarsen_select_apply_phase(Store S, const int* C
           const int f = dies ? 3 : (e[k].x == lv ? 0 : (e[k].y == lv ? 1 : 2));
           reinterpret_cast<int*>(S.EN + c.eb + r.a[k])[f] = dies ? 0 : w;
           if (!dies) qbits.set(b + k);
+          else ++dead;
         }
       }
+      if (dead == 1) atomicAdd(S.tab.bnd + mi, 1ull);
       S.vflag[v] = (uint8_t)(S.vflag[v] & ~VF_ALIVE);
       for (int b = 0; b < nnl; b += 8) {
         const Row8 r = row8(nn, b);
@@ -3041,7 +3044,7 @@ __global__ void k_refine_newcount(Store S, const int* vscan, int* counts) {
   if (i == 0) counts[CN_EL] = counts[CN_CL] = 0;
   if (i >= S.nmesh) return;
   int vb = S.tab.vbase[i];
-  counts[CN_NUM + i] = vscan[vb + S.tab.nv[i]] - vscan[vb];
+  counts[cn_newv(S.nmesh) + i] = vscan[vb + S.tab.nv[i]] - vscan[vb];
 }
 
 __device__ __forceinline__ int mid_id(const Store& S, int vb, int nv, const int* vscan,
@@ -3278,6 +3281,9 @@ __global__ void k_refine_rows(Store S, int vfirst, int vend, int fresh, const in
     if (!ok || ne2 > S.W || nn2 > S.W) {
       atomicExch(&st->overflow, 1);
       atomicMax(&st->maxdeg, max(ne2, nn2));
+      // until the rows are rebuilt a new vertex has none (the marks queued behind
+      // this round read them)
+      if (fresh) S.NNlen[s] = S.NElen[s] = 0;
       continue;
     }
     int* wn = S.NN + (size_t)s * S.W;
@@ -3298,8 +3304,8 @@ __global__ void k_refine_sizes(Store S, const int* vscan, const int* escan, int*
   int vb = S.tab.vbase[i], eb = S.tab.ebase[i];
   int nv = S.tab.nv[i], ne = S.tab.ne[i];
   const int t = vscan[vb + nv] - vscan[vb];
-  S.tab.nv[i] = counts[CN_NUM + i] = nv + t;
-  S.tab.ne[i] = counts[CN_NUM + S.nmesh + i] = ne + (escan[eb + ne] - escan[eb]);
+  S.tab.nv[i] = counts[cn_sizes(S.nmesh) + i] = nv + t;
+  S.tab.ne[i] = counts[cn_sizes(S.nmesh) + S.nmesh + i] = ne + (escan[eb + ne] - escan[eb]);
   if (t > 0) {
     S.tab.r[i] += 1;
     S.tab.ops[i] += (unsigned long long)t;
@@ -4002,59 +4008,89 @@ int op_swap(MeshSet& m, int max_rounds) {
 }
 
 // Rounds of splits until no edge is longer than L_up.  Capacity is checked
-// (and grown) before any new vertex or element is written.
-int op_refine(MeshSet& m, int max_rounds) {
+// (and grown) before any new vertex or element is written.  A round's split is
+// not waited for: the next round's marks are queued behind it, and one read-back
+// brings the sizes after the split and the new marks' count (a row that outgrew W
+// in the split voids those marks).  With `renumber_queued`, marks behind a split
+// (which mostly find nothing) also take the renumbering's counts along.
+int op_refine(MeshSet& m, int max_rounds, bool* renumber_queued) {
   const Tuning tu = tuning();
   const int bs = tu.block[TO_REFINE], bps = tu.blocks_per_sm[TO_REFINE];
   Work& w = m.w;
+  const int n = m.nmesh;
   int pass0 = m.tag;
   bool complete = false;
-  for (long long nr = 0; max_rounds == 0 || nr < max_rounds; ++nr) {
+  bool split = false;  // a split is queued whose sizes have not been read back
+  std::vector<int> newv(n);
+  // the sizes after a queued split; rows rebuilt wider when one outgrew W
+  auto settle = [&](bool& again) -> int {
+    for (int i = 0; i < n; ++i) {
+      m.nv[i] = m.hcounts[cn_sizes(n) + i];
+      m.ne[i] = m.hcounts[cn_sizes(n) + n + i];
+    }
+    set_used(m);
+    split = false;
+    again = m.hst->overflow != 0;
+    return again ? after_overflow(m) : PM_OK;
+  };
+  for (long long nr = 0; max_rounds == 0 || nr < max_rounds;) {
     const int gv = grid_tuned(m, m.S.vused, bs, bps);
-    const int ge = grid_tuned(m, m.S.eused, bs, bps);
     int tag = (m.tag += 2);
     if (m.lo_refine > pass0) pass0 = m.lo_refine;  // storage was regrown
     PM_LAUNCH(k_refine_mark, gv, bs, 0, m.stream, m.S, w.vcnt, w.vmask, tag, pass0,
               m.lo_refine);
     scan_exclusive(w.vcnt, w.vscan, m.S.vused, m.scan, m.st, m.stream);
-    std::vector<int> newv(m.nmesh);
-    PM_LAUNCH(k_refine_newcount, (m.nmesh + 127) / 128, 128, 0, m.stream, m.S,
-              (const int*)w.vscan, w.counts);
-    if (int err = sync_counts(m, m.nmesh)) return err;
-    for (int i = 0; i < m.nmesh; ++i) newv[i] = m.hcounts[CN_NUM + i];
+    PM_LAUNCH(k_refine_newcount, (n + 127) / 128, 128, 0, m.stream, m.S, (const int*)w.vscan,
+              w.counts);
+    const bool ahead = renumber_queued && split;
+    // (beside the marks' scan, which a split still needs; the counts are spent)
+    if (ahead) renumber_queue(m, w.vcnt);
+    if (int err = ahead ? sync_call(m) : sync_counts(m, kMeshWords * n)) return err;
+    std::copy(m.hcounts + cn_newv(n), m.hcounts + cn_newv(n) + n, newv.begin());
+    if (split) {
+      bool again = false;
+      if (int err = settle(again)) return err;
+      if (again) continue;
+    }
     // A growth moves every mesh of the set, so when one mesh needs room, every
     // mesh that this round leaves with little gets half as much again as it
-    // needs now, and some thousands at least (the next rounds of a refinement pass usually split again).
+    // needs now, and some thousands at least (the next rounds of a refinement pass
+    // usually split again).
     long long total = 0;
     bool need_grow = false;
-    for (int i = 0; i < m.nmesh; ++i) {
+    for (int i = 0; i < n; ++i) {
       total += newv[i];
       if ((long long)m.nv[i] + newv[i] > m.vcap[i] || (long long)m.ne[i] + 2LL * newv[i] > m.ecap[i])
         need_grow = true;
     }
-    std::vector<int> vcap = m.vcap, ecap = m.ecap;
-    for (int i = 0; need_grow && i < m.nmesh; ++i) {
-      if (newv[i] == 0) continue;
-      const long long vneed = (long long)m.nv[i] + newv[i] + 64;
-      const long long eneed = (long long)m.ne[i] + 2LL * newv[i] + 64;
-      if (vneed + vneed / 8 > m.vcap[i])
-        vcap[i] = (int)std::min<long long>(std::max(vneed + vneed / 2, vneed + 8192), (1LL << 30));
-      if (eneed + eneed / 8 > m.ecap[i])
-        ecap[i] = (int)std::min<long long>(std::max(eneed + eneed / 2, eneed + 16384), (1LL << 30));
-    }
     if (total == 0) {
       complete = true;
+      if (ahead) {
+        *renumber_queued = true;
+        std::swap(w.vcnt, w.vscan);
+      }
       break;
     }
     if (need_grow) {
+      std::vector<int> vcap = m.vcap, ecap = m.ecap;
+      for (int i = 0; i < n; ++i) {
+        if (newv[i] == 0) continue;
+        const long long vneed = (long long)m.nv[i] + newv[i] + 64;
+        const long long eneed = (long long)m.ne[i] + 2LL * newv[i] + 64;
+        if (vneed + vneed / 8 > m.vcap[i])
+          vcap[i] = (int)std::min<long long>(std::max(vneed + vneed / 2, vneed + 8192), (1LL << 30));
+        if (eneed + eneed / 8 > m.ecap[i])
+          ecap[i] =
+              (int)std::min<long long>(std::max(eneed + eneed / 2, eneed + 16384), (1LL << 30));
+      }
       cudaError_t e = grow(m, vcap, ecap, m.S.W);
       if (e != cudaSuccess) {
         set_last_error(std::string("growing mesh storage: ") + cudaGetErrorString(e));
         return e == cudaErrorMemoryAllocation ? PM_ERR_OOM : PM_ERR_CUDA;
       }
-      --nr;  // redo this round on the new layout
-      continue;
+      continue;  // redo this round on the new layout
     }
+    const int ge = grid_tuned(m, m.S.eused, bs, bps);
     const int stamp = tag + 1;
     const int vend = m.vbase.back() + m.nv.back() + newv.back();  // above every new vertex
     PM_LAUNCH(k_refine_newverts, gv, bs, 0, m.stream, m.S, w.vscan, w.vmask, stamp, w.opA);
@@ -4065,23 +4101,24 @@ int op_refine(MeshSet& m, int max_rounds) {
               w.counts + CN_EL, w.clist, w.counts + CN_CL, stamp);
     PM_LAUNCH(k_refine_quality, ge, bs, 0, m.stream, m.S, w.clist, w.counts + CN_CL, nullptr);
     // rows of the vertices whose elements changed: the new ones, then the old ones
-    const int vnew = m.nmesh == 1 ? m.nv[0] : 0;
+    const int vnew = n == 1 ? m.nv[0] : 0;
     PM_LAUNCH(k_refine_rows, grid_tuned(m, vend - vnew, bs, bps), bs, 0, m.stream, m.S, vnew, vend, 1,
               (const int*)w.escan, (const int4*)w.opA, stamp, m.st);
     PM_LAUNCH(k_refine_rows, gv, bs, 0, m.stream, m.S, 0, m.S.vused, 0, (const int*)w.escan,
               (const int4*)w.opA, stamp, m.st);
-    PM_LAUNCH(k_refine_sizes, (m.nmesh + 127) / 128, 128, 0, m.stream, m.S, (const int*)w.vscan,
+    PM_LAUNCH(k_refine_sizes, (n + 127) / 128, 128, 0, m.stream, m.S, (const int*)w.vscan,
               (const int*)w.escan, w.counts);
-    // the new sizes and the status in one read-back
-    if (int err = sync_counts(m, 2 * m.nmesh)) return err;
-    for (int i = 0; i < m.nmesh; ++i) {
-      m.nv[i] = m.hcounts[CN_NUM + i];
-      m.ne[i] = m.hcounts[CN_NUM + m.nmesh + i];
-    }
-    set_used(m);
-    if (m.hst->overflow) {  // a row outgrew W: rebuild every row with wider ones
-      if (int err = after_overflow(m)) return err;
-    }
+    split = true;
+    // every slot lies below these bounds (the exact element sizes follow with the
+    // next read-back)
+    m.S.vused = vend;
+    m.S.eused = m.S.eused + 2 * newv.back();
+    ++nr;
+  }
+  if (split) {
+    if (int err = sync_counts(m, kMeshWords * n)) return err;
+    bool again = false;
+    if (int err = settle(again)) return err;
   }
   if (!complete) m.lo_refine = m.tag;
   return PM_OK;
