@@ -319,13 +319,15 @@ pm_status adapt_set(MeshSet& m, const pm_params* P, int stride, CallStats& cs) {
     }
     if (!any) break;
     send_active(active);
+    Ahead done;
+    if (mr == 0 && (err = ops_ahead(m, done))) return (pm_status)err;
     select_ops(m, OS_COARSEN);
-    if ((err = op_coarsen(m, mr))) return (pm_status)err;
+    if ((err = op_coarsen(m, mr, done))) return (pm_status)err;
     select_ops(m, OS_SWAP);
-    if ((err = op_swap(m, mr))) return (pm_status)err;
+    if ((err = op_swap(m, mr, done))) return (pm_status)err;
     select_ops(m, OS_REFINE);
     bool queued = false;
-    if ((err = op_refine(m, mr, &queued))) return (pm_status)err;
+    if ((err = op_refine(m, mr, done, &queued))) return (pm_status)err;
     // reads the call state back, unless the refinement has
     if ((err = renumber(m, false, queued))) return (pm_status)err;
     const unsigned long long* h = m.hops;

@@ -82,6 +82,8 @@ enum CountIdx {
 constexpr int kMeshWords = 5;
 constexpr int cn_newv(int n) { return CN_NUM + 2 * n; }
 constexpr int cn_sizes(int n) { return CN_NUM + 3 * n; }
+// A second set of counters behind them, for flips queued behind collapses.
+constexpr int cn_second(int n) { return CN_NUM + kMeshWords * n; }
 // What a persistent smoothing launch leaves at CN_RES: rounds with candidates,
 // sweeps finished, 1 when the sweeps are over, 1 when the current sweep has
 // moved a vertex, the buffers holding the current, the next and the pending list
@@ -166,9 +168,21 @@ int ensure_quality(MeshSet& m);
 cudaError_t refresh_sizes(MeshSet& m);
 
 // ---- operators (pm_ops.cu) ----
-int op_coarsen(MeshSet& m, int max_rounds);
-int op_swap(MeshSet& m, int max_rounds);
-int op_refine(MeshSet& m, int max_rounds, bool* renumber_queued = nullptr);
+// What ops_ahead has done of an iteration: collapse rounds, flip rounds (0: none
+// run, 1: the pass is complete, 2: to be continued) and the first split marks.
+struct Ahead {
+  int coarsen = 0, swap = 0, mark_tag = 0;
+  int cur_c = 0, cur_s = 0;        // list the next round of a pass reads
+  int pass0_c = 0, pass0_s = 0;    // tag at the start of each pass
+};
+// Collapse rounds, flip rounds and the first split marks of an iteration queued one
+// behind the other with one read-back; each starts on the device only when the one
+// before is complete.
+int ops_ahead(MeshSet& m, Ahead& h);
+int op_coarsen(MeshSet& m, int max_rounds, const Ahead& h = Ahead());
+int op_swap(MeshSet& m, int max_rounds, const Ahead& h = Ahead());
+int op_refine(MeshSet& m, int max_rounds, const Ahead& h = Ahead(),
+              bool* renumber_queued = nullptr);
 int op_smooth(MeshSet& m, int max_sweeps, int max_rounds);
 int op_opt_smooth(MeshSet& m, int nrounds, int max_rounds);
 // Operation counters of a call: one set per operator, selected before it runs.

@@ -877,7 +877,7 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   // State of a call, kept over growths: status, counters (and some words per mesh
   // after them), operation counts, round counters, candidate flags, active flags.
   // The host reads it back in one copy, into a pinned image of its first part.
-  const size_t counts_bytes = (CN_NUM + kMeshWords * (size_t)n + 8) * sizeof(int);
+  const size_t counts_bytes = (cn_second(0) + kMeshWords * (size_t)n + CN_NUM + 8) * sizeof(int);
   const size_t ops_off = 64 + ((counts_bytes + 7) & ~size_t(7));
   const size_t r_off = ops_off + OS_NUM * (size_t)n * sizeof(unsigned long long);
   const size_t had_off = r_off + (size_t)n * sizeof(uint32_t);

@@ -173,7 +173,20 @@ __device__ __forceinline__ void stamp_neighbours(const Store& S, const int* row,
 // With `ev`, vertices whose last evaluation (newer than `lo`) found nothing
 // and whose inputs are unchanged since are left out: they would find
 // nothing again.
-__global__ void k_init_list(Store S, int mode, int* list, int* count, const int* ev, int lo) {
+// A pass queued behind another's persistent rounds, whose results are `before`
+// (rounds run, list, complete): it does nothing unless those are complete and no
+// row has outgrown its width, and its tags follow theirs.
+__device__ __forceinline__ bool may_go(const int* before, const DevStatus* st) {
+  return !before || (before[2] != 0 && *(volatile const int*)&st->overflow == 0 &&
+                     *(volatile const int*)&st->err == 0);
+}
+__device__ __forceinline__ int tags_of(const int* before) {
+  return before ? 2 * before[0] : 0;
+}
+
+__global__ void k_init_list(Store S, int mode, int* list, int* count, const int* ev, int lo,
+                            const int* before, const DevStatus* st) {
+  if (!may_go(before, st)) return;
   for (int i0 = blockIdx.x * blockDim.x; i0 < S.vused; i0 += gridDim.x * blockDim.x) {
     int s = i0 + threadIdx.x;
     bool take = false;
@@ -3001,7 +3014,11 @@ __global__ void k_stamp_list(Store S, const int* L, const int* nLp, int* cmark, 
 // inside one call vertices keep their positions and metrics until the
 // operator loop ends (smoothing runs after it), so a's own stamp tells
 // whether anything the mask read has changed: every change of a's row stamps a.
-__global__ void k_refine_mark(Store S, int* cnt, RowMask* mask, int tag, int pass0, int lo) {
+__global__ void k_refine_mark(Store S, int* cnt, RowMask* mask, int tag, int pass0, int lo,
+                              const int* before, const int* before2, const DevStatus* st) {
+  if (!may_go(before, st)) return;
+  tag += tags_of(before) + tags_of(before2);
+  pass0 += tags_of(before) + tags_of(before2);
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < S.vused; s += gridDim.x * blockDim.x) {
     int mi = mesh_of_vslot(S, s);
     int vb = S.tab.vbase[mi];
@@ -3417,6 +3434,7 @@ struct RoundArgs {
   int ptag;            // smoothing: stamp of the next sweep's list
   int sweeps;          // smoothing: sweeps left, the current one included
   int moved;           // smoothing: the current sweep has moved a vertex
+  const int* before;   // flips: results of the rounds this launch is queued behind (may_go)
   int fuse;            // flips, smoothing: lists up to this size (and kFusePasses passes of
                        // tiles) take the one-phase evaluation
   unsigned long long* work;  // counted FP64 work (measurement) or null
@@ -3450,6 +3468,8 @@ __device__ __forceinline__ void topo_rounds(const RoundArgs& a) {
   unsigned target = 0;
   int cur = a.cur, r = 0;
   bool complete = false;
+  if (!may_go(a.before, a.st)) return;  // (the same answer in every block: all wait at B1 first)
+  const int tag0 = a.tag0 + tags_of(a.before), pass0 = a.pass0 + tags_of(a.before);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *cand_count(cnt, 0) = 0;
     cnt[CN_E] = cnt[CN_I] = 0;
@@ -3458,7 +3478,7 @@ __device__ __forceinline__ void topo_rounds(const RoundArgs& a) {
   // a first list longer than the limit is left to the one-kernel-per-phase rounds
   const bool too_long = ld_volatile(cnt + cn_list(cur)) > a.limit;
   while (!too_long && r < a.max_rounds) {
-    const int tag = a.tag0 + 2 * r, nxt = 1 - cur;
+    const int tag = tag0 + 2 * r, nxt = 1 - cur;
     int* nC = cand_count(cnt, r);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       cnt[CN_A] = 0;
@@ -3469,13 +3489,13 @@ __device__ __forceinline__ void topo_rounds(const RoundArgs& a) {
       // the list fits two passes of tiles: scan, gains and pick in one phase
       // (the list is complete since the last barrier: every block decides alike)
       swap_scan_eval_phase(a.S, w.D[cur], cnt + cn_list(cur), w.opA, w.opK2, w.C, nC, w.cmark,
-                           tag, a.pass0, a.work);
+                           tag, pass0, a.work);
       if (!grid_barrier(a.bar, target, a.st)) return;
       if (blockIdx.x == 0 && threadIdx.x == 0) *cand_count(cnt, r + 1) = 0;
     } else if (FLIP) {
       // a longer list keeps the three passes: item-parallel FP64 gains beat
       // two barriers saved
-      swap_scan_phase(a.S, w.D[cur], cnt + cn_list(cur), w.opA, w.C, nC, w.cmark, tag, a.pass0,
+      swap_scan_phase(a.S, w.D[cur], cnt + cn_list(cur), w.opA, w.C, nC, w.cmark, tag, pass0,
                       w.E, cnt + CN_E, w.items, cnt + CN_I, a.icap, w.gains, a.st, true);
       if (!grid_barrier(a.bar, target, a.st)) return;
       if (blockIdx.x == 0 && threadIdx.x == 0) *cand_count(cnt, r + 1) = 0;
@@ -3486,7 +3506,7 @@ __device__ __forceinline__ void topo_rounds(const RoundArgs& a) {
       if (blockIdx.x == 0 && threadIdx.x == 0) cnt[CN_E] = cnt[CN_I] = 0;
     } else {
       coarsen_eval_phase(a.S, w.D[cur], cnt + cn_list(cur), w.target, w.cand, w.ncand, w.C, nC,
-                         w.cmark, tag, a.pass0, a.work, true);
+                         w.cmark, tag, pass0, a.work, true);
       if (!grid_barrier(a.bar, target, a.st)) return;
       if (blockIdx.x == 0 && threadIdx.x == 0) *cand_count(cnt, r + 1) = 0;
     }
@@ -3763,6 +3783,7 @@ RoundArgs round_args(MeshSet& m, int cur, int pass0, long long max_rounds) {
   a.ptag = 0;
   a.sweeps = 0;
   a.moved = 0;
+  a.before = nullptr;
   a.fuse = 0;
   a.work = nullptr;
   return a;
@@ -3775,15 +3796,10 @@ struct RoundsOut {
   RoundIO io{0, 0, 0};
 };
 
-// One cooperative launch of persistent rounds, then the read-back of every
-// counter and the status.  Advances the tag past the rounds that ran.
-int run_rounds(MeshSet& m, int which, const void* kernel, const char* name, RoundArgs& a,
-               RoundsOut& out, bool& bar_clear) {
+// One cooperative launch of persistent rounds.
+int launch_rounds(MeshSet& m, int which, const void* kernel, const char* name, RoundArgs& a) {
   a.work = prof_work(name);
   void* args[] = {&a};
-  // (the first launch of an operator finds the counters cleared)
-  if (!bar_clear) cudaMemsetAsync(a.bar, 0, sizeof(unsigned), m.stream);
-  bar_clear = false;
   __atomic_fetch_add(&g_launches, 1ull, __ATOMIC_RELAXED);
   int slot = g_prof_on ? prof_begin(name, m.stream) : -1;
   cudaError_t e = cudaLaunchCooperativeKernel(kernel, dim3(rounds_grid(m, which)),
@@ -3793,6 +3809,17 @@ int run_rounds(MeshSet& m, int which, const void* kernel, const char* name, Roun
     set_last_error(std::string("cooperative launch: ") + cudaGetErrorString(e));
     return PM_ERR_CUDA;
   }
+  return PM_OK;
+}
+
+// The same, then the read-back of every counter and the status.  Advances the tag
+// past the rounds that ran.
+int run_rounds(MeshSet& m, int which, const void* kernel, const char* name, RoundArgs& a,
+               RoundsOut& out, bool& bar_clear) {
+  // (the first launch of an operator finds the counters cleared)
+  if (!bar_clear) cudaMemsetAsync(a.bar, 0, sizeof(unsigned), m.stream);
+  bar_clear = false;
+  if (int err = launch_rounds(m, which, kernel, name, a)) return err;
   out.io = read_round(m);
   if (out.io.err) return out.io.err;
   if (which == 2) {
@@ -3858,10 +3885,87 @@ int colour_set(MeshSet& m) {
 // Operator loops (host)
 // ---------------------------------------------------------------------------
 
+// An iteration's collapses, flips and first split marks waited on the host three
+// times (10-20 us each on small meshes, the chip idle); queued one behind the other
+// they wait once: 1140 against 1205 us on a 41 x 41 mesh, 11.80 against 11.92 ms at
+// 201 x 201.  A launch that finds the pass before it incomplete (list too long, or a
+// row that outgrew its width) does nothing, and the operators go on from there.
+int ops_ahead(MeshSet& m, Ahead& h) {
+  const Tuning tu = tuning();
+  for (int x : m.select)
+    if (x == PM_SELECT_COLOUR) return PM_OK;  // a colouring comes before each pass
+  if (rounds_grid(m, 0) == 0 || rounds_grid(m, 1) == 0) return PM_OK;
+  // the first lists of a call hold every vertex; the later ones are known only on the
+  // device, where a pass whose list is too long hands back at once
+  if (m.lo_coarsen == m.tag && m.S.vused > tu.rounds_limit[0]) return PM_OK;
+  Work& w = m.w;
+  const int n = m.nmesh;
+  int* const second = w.counts + cn_second(n);
+  const int* const none = nullptr;
+  const int* const rounds_c = w.counts + CN_RES;
+  const int* const rounds_s = second + CN_RES;
+  const DevStatus* const st = m.st;
+  zero_counts(m, 0, CN_NUM);
+  cudaMemsetAsync(second, 0, CN_NUM * sizeof(int), m.stream);
+  const int tag = m.tag;
+
+  int bs = tu.block[TO_COARSEN];
+  select_ops(m, OS_COARSEN);
+  PM_LAUNCH(k_init_list, grid_tuned(m, m.S.vused, bs, tu.blocks_per_sm[TO_COARSEN]), bs, 0,
+            m.stream, m.S, 0, w.D[0], w.counts + CN_D0, m.S.evc, m.lo_coarsen, none, st);
+  RoundArgs a = round_args(m, 0, tag, 1 << 30);
+  a.limit = tu.rounds_limit[0];
+  if (int err = launch_rounds(m, 0, (const void*)k_coarsen_rounds, "k_coarsen_rounds", a))
+    return err;
+
+  bs = tu.block[TO_SWAP];
+  select_ops(m, OS_SWAP);
+  PM_LAUNCH(k_init_list, grid_tuned(m, m.S.vused, bs, tu.blocks_per_sm[TO_SWAP]), bs, 0, m.stream,
+            m.S, 0, w.D[0], second + CN_D0, m.S.evs, m.lo_swap, rounds_c, st);
+  a = round_args(m, 0, tag, 1 << 30);
+  a.w.counts = second;
+  a.bar = (unsigned*)(second + CN_BAR);
+  a.res = second + CN_RES;
+  a.icap = m.S.vslots * 6 + 64;
+  a.limit = tu.rounds_limit[1];
+  a.fuse = tu.fuse_limit[0];
+  a.before = rounds_c;
+  if (int err = launch_rounds(m, 1, (const void*)k_swap_rounds, "k_swap_rounds", a)) return err;
+
+  bs = tu.block[TO_REFINE];
+  select_ops(m, OS_REFINE);
+  PM_LAUNCH(k_refine_mark, grid_tuned(m, m.S.vused, bs, tu.blocks_per_sm[TO_REFINE]), bs, 0,
+            m.stream, m.S, w.vcnt, w.vmask, tag + 2, tag, m.lo_refine, rounds_s, rounds_c, st);
+  scan_exclusive(w.vcnt, w.vscan, m.S.vused, m.scan, m.st, m.stream);
+  PM_LAUNCH(k_refine_newcount, (n + 127) / 128, 128, 0, m.stream, m.S, (const int*)w.vscan,
+            w.counts);
+  if (int err = sync_counts(m, kMeshWords * n + CN_NUM)) return err;
+
+  const int* rc = m.hcounts + CN_RES;
+  const int* rs = m.hcounts + cn_second(n) + CN_RES;
+  m.tag = tag + 2 * rc[0];
+  h.coarsen = rc[2] ? 1 : 2;
+  h.pass0_c = tag;
+  h.cur_c = rc[1];
+  if (h.coarsen != 1) return PM_OK;
+  h.swap = rs[2] ? 1 : 2;
+  h.pass0_s = m.tag;
+  h.cur_s = rs[1];
+  m.tag += 2 * rs[0];
+  if (h.swap == 1) {
+    h.mark_tag = (m.tag += 2);
+  } else {  // op_swap goes on with the first set of counters
+    cudaMemcpyAsync(w.counts, second, CN_NUM * sizeof(int), cudaMemcpyDeviceToDevice, m.stream);
+    std::copy(m.hcounts + cn_second(n), m.hcounts + cn_second(n) + CN_NUM, m.hcounts);
+  }
+  return PM_OK;
+}
+
 // Rounds of collapses until no dirty vertex has a valid collapse.  The first
 // round's list leaves out vertices whose last collapse evaluation found
 // nothing and whose inputs have not changed since.
-int op_coarsen(MeshSet& m, int max_rounds) {
+int op_coarsen(MeshSet& m, int max_rounds, const Ahead& h) {
+  if (h.coarsen == 1) return PM_OK;
   if (int err = colour_set(m)) return err;
   const Tuning tu = tuning();
   const int bs = tu.block[TO_COARSEN], bps = tu.blocks_per_sm[TO_COARSEN];
@@ -3870,15 +3974,23 @@ int op_coarsen(MeshSet& m, int max_rounds) {
   const int gv = grid_tuned(m, m.S.vused, bs, bps);
   int pass0 = m.tag;
   const bool persist = rounds_grid(m, 0) > 0;
-  bool bar_clear = true;
-  zero_counts(m, 0, CN_NUM);
-  PM_LAUNCH(k_init_list, gv, bs, 0, m.stream, m.S, 0, w.D[0], w.counts + CN_D0, m.S.evc,
-            m.lo_coarsen);
+  bool bar_clear = h.coarsen == 0;
+  if (h.coarsen == 0) zero_counts(m, 0, CN_NUM);
+  if (h.coarsen == 0)
+    PM_LAUNCH(k_init_list, gv, bs, 0, m.stream, m.S, 0, w.D[0], w.counts + CN_D0, m.S.evc,
+            m.lo_coarsen, (const int*)nullptr, (const DevStatus*)m.st);
   // entries of the list the next round reads; unknown (0) at first: the
   // persistent launch itself hands a long first list back
   int nlist = 0;
   int cur = 0;
   bool complete = false;
+  if (h.coarsen == 2) {  // behind the rounds of ops_ahead
+    pass0 = h.pass0_c;
+    cur = h.cur_c;
+    if (m.hst->overflow)
+      if (int err = after_overflow(m)) return err;
+    nlist = m.hcounts[cn_list(cur)];
+  }
   for (long long nr = 0; max_rounds == 0 || nr < max_rounds;) {
     if (m.lo_coarsen > pass0) pass0 = m.lo_coarsen;  // rows were rebuilt after an overflow
     if (persist && nlist >= 0 && nlist <= rlimit) {
@@ -3936,7 +4048,8 @@ int op_coarsen(MeshSet& m, int max_rounds) {
 }
 
 // Rounds of flips until no dirty vertex has an improving flip.
-int op_swap(MeshSet& m, int max_rounds) {
+int op_swap(MeshSet& m, int max_rounds, const Ahead& h) {
+  if (h.swap == 1) return PM_OK;
   if (int err = colour_set(m)) return err;
   const Tuning tu = tuning();
   const int bs = tu.block[TO_SWAP], bps = tu.blocks_per_sm[TO_SWAP];
@@ -3946,13 +4059,21 @@ int op_swap(MeshSet& m, int max_rounds) {
   int pass0 = m.tag;
   const int icap = m.S.vslots * 6 + 64;
   const bool persist = rounds_grid(m, 1) > 0;
-  bool bar_clear = true;
-  zero_counts(m, 0, CN_NUM);
-  PM_LAUNCH(k_init_list, gv, bs, 0, m.stream, m.S, 0, w.D[0], w.counts + CN_D0, m.S.evs,
-            m.lo_swap);
+  bool bar_clear = h.swap == 0;
+  if (h.swap == 0) zero_counts(m, 0, CN_NUM);
+  if (h.swap == 0)
+    PM_LAUNCH(k_init_list, gv, bs, 0, m.stream, m.S, 0, w.D[0], w.counts + CN_D0, m.S.evs,
+            m.lo_swap, (const int*)nullptr, (const DevStatus*)m.st);
   int nlist = 0;  // unknown at first (see op_coarsen)
   int cur = 0;
   bool complete = false;
+  if (h.swap == 2) {  // behind the rounds of ops_ahead
+    pass0 = h.pass0_s;
+    cur = h.cur_s;
+    if (m.hst->overflow)
+      if (int err = after_overflow(m)) return err;
+    nlist = m.hcounts[cn_list(cur)];
+  }
   for (long long nr = 0; max_rounds == 0 || nr < max_rounds;) {
     if (m.lo_swap > pass0) pass0 = m.lo_swap;  // rows were rebuilt after an overflow
     if (persist && nlist >= 0 && nlist <= rlimit) {
@@ -4013,12 +4134,13 @@ int op_swap(MeshSet& m, int max_rounds) {
 // brings the sizes after the split and the new marks' count (a row that outgrew W
 // in the split voids those marks).  With `renumber_queued`, marks behind a split
 // (which mostly find nothing) also take the renumbering's counts along.
-int op_refine(MeshSet& m, int max_rounds, bool* renumber_queued) {
+int op_refine(MeshSet& m, int max_rounds, const Ahead& h, bool* renumber_queued) {
   const Tuning tu = tuning();
   const int bs = tu.block[TO_REFINE], bps = tu.blocks_per_sm[TO_REFINE];
   Work& w = m.w;
   const int n = m.nmesh;
-  int pass0 = m.tag;
+  int pass0 = h.mark_tag ? h.mark_tag - 2 : m.tag;
+  int marked = h.mark_tag;  // the first marks are there already, with their count
   bool complete = false;
   bool split = false;  // a split is queued whose sizes have not been read back
   std::vector<int> newv(n);
@@ -4035,17 +4157,20 @@ int op_refine(MeshSet& m, int max_rounds, bool* renumber_queued) {
   };
   for (long long nr = 0; max_rounds == 0 || nr < max_rounds;) {
     const int gv = grid_tuned(m, m.S.vused, bs, bps);
-    int tag = (m.tag += 2);
+    const int tag = marked ? marked : (m.tag += 2);
     if (m.lo_refine > pass0) pass0 = m.lo_refine;  // storage was regrown
-    PM_LAUNCH(k_refine_mark, gv, bs, 0, m.stream, m.S, w.vcnt, w.vmask, tag, pass0,
-              m.lo_refine);
-    scan_exclusive(w.vcnt, w.vscan, m.S.vused, m.scan, m.st, m.stream);
-    PM_LAUNCH(k_refine_newcount, (n + 127) / 128, 128, 0, m.stream, m.S, (const int*)w.vscan,
-              w.counts);
+    if (!marked) PM_LAUNCH(k_refine_mark, gv, bs, 0, m.stream, m.S, w.vcnt, w.vmask, tag, pass0,
+              m.lo_refine, (const int*)nullptr, (const int*)nullptr, (const DevStatus*)m.st);
     const bool ahead = renumber_queued && split;
-    // (beside the marks' scan, which a split still needs; the counts are spent)
-    if (ahead) renumber_queue(m, w.vcnt);
-    if (int err = ahead ? sync_call(m) : sync_counts(m, kMeshWords * n)) return err;
+    if (!marked) {
+      scan_exclusive(w.vcnt, w.vscan, m.S.vused, m.scan, m.st, m.stream);
+      PM_LAUNCH(k_refine_newcount, (n + 127) / 128, 128, 0, m.stream, m.S, (const int*)w.vscan,
+                w.counts);
+      // (beside the marks' scan, which a split still needs; the counts are spent)
+      if (ahead) renumber_queue(m, w.vcnt);
+      if (int err = ahead ? sync_call(m) : sync_counts(m, kMeshWords * n)) return err;
+    }
+    marked = 0;
     std::copy(m.hcounts + cn_newv(n), m.hcounts + cn_newv(n) + n, newv.begin());
     if (split) {
       bool again = false;
@@ -4137,7 +4262,8 @@ int op_smooth(MeshSet& m, int max_sweeps, int max_rounds) {
   const bool persist = rounds_grid(m, 2) > 0;
   bool bar_clear = true;
   zero_counts(m, 0, CN_NUM);
-  PM_LAUNCH(k_init_list, gv, bs, 0, m.stream, m.S, 1, w.D[0], w.counts + CN_D0, nullptr, 0);
+  PM_LAUNCH(k_init_list, gv, bs, 0, m.stream, m.S, 1, w.D[0], w.counts + CN_D0, nullptr, 0,
+            (const int*)nullptr, (const DevStatus*)m.st);
   int nlist = 0;  // unknown at first (see op_coarsen)
   long long nr = 0;
   int cur = 0, ptag = 0;
@@ -4220,7 +4346,8 @@ int op_opt_smooth(MeshSet& m, int nrounds, int max_rounds) {
   Work& w = m.w;
   const int gv = grid_tuned(m, m.S.vused, bs, bps);
   zero_counts(m, 0, CN_NUM);
-  PM_LAUNCH(k_init_list, gv, bs, 0, m.stream, m.S, 1, w.C, w.counts + CN_C, nullptr, 0);
+  PM_LAUNCH(k_init_list, gv, bs, 0, m.stream, m.S, 1, w.C, w.counts + CN_C, nullptr, 0,
+            (const int*)nullptr, (const DevStatus*)m.st);
   for (int it = 0; it < nrounds && (max_rounds == 0 || it < max_rounds); ++it) {
     int tag = (m.tag += 2);
     zero_counts(m, CN_S, 1);
