@@ -179,6 +179,10 @@ struct RowMask {
     if (k < 64) lo |= 1ull << k;
     else hi |= 1ull << (k - 64);
   }
+  __device__ __forceinline__ void clear(int k) {
+    if (k < 64) lo &= ~(1ull << k);
+    else hi &= ~(1ull << (k - 64));
+  }
   __device__ __forceinline__ bool test(int k) const {
     return k < 64 ? ((lo >> k) & 1ull) != 0ull : ((hi >> (k - 64)) & 1ull) != 0ull;
   }
@@ -238,18 +242,6 @@ __device__ __forceinline__ Room3 warp_reserve3(int na, int* pa, int nb, int* pb,
   r.b = __shfl_sync(0xffffffffu, base, 1) + ((int)(excl >> 21) & 0x1FFFFF);
   r.c = __shfl_sync(0xffffffffu, base, 2) + (int)(excl >> 42);
   return r;
-}
-
-template <class T>
-__device__ __forceinline__ void warp_append_t(bool pred, T val, T* list, int* count) {
-  unsigned m = __ballot_sync(0xffffffffu, pred);
-  if (m == 0) return;
-  int lane = threadIdx.x & 31;
-  int leader = __ffs(m) - 1;
-  int base = 0;
-  if (lane == leader) base = atomicAdd(count, __popc(m));
-  base = __shfl_sync(0xffffffffu, base, leader);
-  if (pred) list[base + __popc(m & ((1u << lane) - 1u))] = val;
 }
 
 // Append once per round: the stamp array holds the tag of the last round in

@@ -57,9 +57,7 @@ struct Work {
   int2* items = nullptr;           // flip candidates (vertex, edge slots) of this round
   double* gains = nullptr;         // gain of each (vertex, ball-element slot), vslots * W (in the
                                    // spare rows)
-  int2* items2 = nullptr;          // second wave list (vertex, candidate rank)
-  int* cand = nullptr;             // collapse candidates of each vertex by (length, id), vslots * W
-  int* ncand = nullptr;
+  int* cand = nullptr;             // collapse candidates of each vertex (see kCandRest), vslots * W
   int* counts = nullptr;           // device counters (see CountIdx)
   int* cprop = nullptr;            // colouring: proposed colour per vertex slot
   int* cstamp = nullptr;           // colouring: round in which the slot was uncoloured
@@ -68,7 +66,7 @@ struct Work {
 // The per-round counters sit between the two dirty-list counts so that one
 // memset clears them together with the next round's list (zero_round).
 enum CountIdx {
-  CN_D0 = 0, CN_C = 1, CN_S = 2, CN_A = 3, CN_E = 4, CN_I = 5, CN_I2 = 6, CN_D1 = 7,
+  CN_D0 = 0, CN_C = 1, CN_S = 2, CN_A = 3, CN_E = 4, CN_I = 5, CN_D1 = 7,
   CN_P = 8, CN_EL = 9, CN_CL = 10, CN_DONE = 11,
   CN_RES = 12,  // persistent rounds: rounds run, list index after, pass complete; smoothing:
                 // see SmoothRes (8)

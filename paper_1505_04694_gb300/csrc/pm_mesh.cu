@@ -102,7 +102,7 @@ struct Carver {
 // Everything whose size follows the row width W, in one allocation of its own
 // (a change of W replaces it and leaves no hole in the store): the rows of both
 // buffer sets and the collapse candidates.  The spare set's rows are written
-// only by a compaction, which reads no flip gain, collapse length or moved ball quality, so those W doubles per vertex
+// only by a compaction, which reads no flip gain or moved ball quality, so those W doubles per vertex
 // (Work::gains) share them.
 cudaError_t rows_alloc(MeshSet& m, int W) {
   const size_t n = (size_t)m.S.vslots * W;
@@ -820,8 +820,8 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   cv.add(&w.target, vs);
   cv.add(&w.opA, vs);
   cv.add(&w.opK2, vs);
-  // smoothing moves (16 + 32 bytes a vertex), and in the same place the flip and
-  // collapse work items (each interior edge gives at most two items and a
+  // smoothing moves (16 + 32 bytes a vertex), and in the same place the flip
+  // work items (each interior edge gives at most two items and a
   // planar mesh has < 3V edges): no operator uses both
   cv.add(&w.mvxy, vs);
   cv.add(&w.mvM, (size_t)vs + 16);
@@ -839,8 +839,6 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   cv.add(&w.elist, es);
   cv.add(&w.clist, es);
   cv.add(&w.E, vs);
-  cv.add(&w.items2, vs);
-  cv.add(&w.ncand, vs);
   cv.add(&w.cprop, vs);
   cv.add(&w.cstamp, vs, true);
   cv.add(&m.lidbuf, vs);

@@ -621,19 +621,57 @@ __device__ __forceinline__ CoarsenCtx coarsen_ctx(const Store& S, int v, MeshCtx
 // length, id), whose collapse is valid.  Pass 1 (per dirty vertex) reuses an
 // unchanged earlier result or finds v's first candidate; a dense pass then
 // checks every listed vertex's first candidate (one work item each), and a
-// last pass puts the candidates of the vertices whose first one failed in
-// order and goes through the rest of them.
-//
+// last pass checks all other candidates of the vertices whose first one failed
+// and takes the first of the valid ones.  A vertex's row of `cand` holds its first
+// candidate and, from kCandRest on, the others as bits over its neighbours.
+constexpr int kCandRest = 4;
+
+__device__ __forceinline__ ulonglong2* cand_rest(int* cand, const Store& S, int v) {
+  return reinterpret_cast<ulonglong2*>(cand + (size_t)v * S.W + kCandRest);
+}
+
+// The first of the neighbours `cm` (not empty) of v by (metric length, position in
+// the row, hence id).  It is mostly plain from the FP32 lengths: only neighbours
+// whose error intervals overlap that of the shortest (equal lengths on regular
+// grids) are compared by their exact lengths.  `first` is the smallest upper
+// bound of the squared lengths (a NaN bound leaves it as it is, and passes here).
+__device__ __forceinline__ int first_by_length(const Store& S, int v, int vb, const int* nn,
+                                               const VF& fv, RowMask cm, float first,
+                                               unsigned& ops) {
+  int best = cm.pop();
+  if (!cm.any()) return best;
+  cm.set(best);
+  RowMask near;
+  while (cm.any()) {
+    const int k = cm.pop();
+    const FLen l = f_edge2(fv, load_vf(S, vb + nn[k]));
+    if (!(l.L2 - l.err > first)) near.set(k);
+  }
+  best = near.pop();
+  if (!near.any()) return best;
+  const VD dv = load_vd(S, v);
+  double Lb = sqrt(metric_len2(dv, load_vd(S, vb + nn[best])));
+  ops += kOpsLen2 + 1;
+  while (near.any()) {  // ascending position
+    const int k = near.pop();
+    const double L = sqrt(metric_len2(dv, load_vd(S, vb + nn[k])));
+    ops += kOpsLen2 + 1;
+    if (dlt(L, Lb)) {
+      Lb = L;
+      best = k;
+    }
+  }
+  return best;
+}
+
 // Pass 1 of the large rounds, one dirty vertex per thread.  Which neighbours
 // are candidates is a length against L_low, and which of them comes first is
-// mostly plain from the FP32 lengths too: only candidates whose error
-// intervals overlap that of the shortest (equal lengths on regular grids) are
-// compared by their exact lengths.  A length that is certainly above another's
-// stays above it after rounding, so the order is the exact one.
+// mostly plain from the FP32 lengths too.  A length that is certainly above
+// another's stays above it after rounding, so the order is the exact one.
 __device__ __forceinline__ void coarsen_scan_phase(Store S, const int* D, const int* nDp,
-                                                   int* target, int* cand, int* ncand, int* C,
-                                                   int* nC, int* cmark, int tag, int pass0,
-                                                   int2* W0, int* nW0) {
+                                                   int* target, int* cand, int* C, int* nC,
+                                                   int* cmark, int tag, int pass0, int* W0,
+                                                   int* nW0) {
   const int n = *nDp;
   unsigned ops = 0;
   for (int i0 = blockIdx.x * blockDim.x; i0 < n; i0 += gridDim.x * blockDim.x) {
@@ -658,7 +696,6 @@ __device__ __forceinline__ void coarsen_scan_phase(Store S, const int* D, const 
         const int* nn = nn_row(S, v);
         const VF fv = load_vf(S, v);
         const float4 bf = S.tab.bandf[c.mi];
-        float lo[MAXW];      // candidates: lower bound of the squared length
         float first = INFINITY;  // the smallest upper bound
         RowMask cm;
         for (int b = 0; b < nnl; b += 4) {
@@ -680,137 +717,32 @@ __device__ __forceinline__ void coarsen_scan_phase(Store S, const int* D, const 
               is = count_elems_with(S, ne_row(S, v), S.NElen[v], c.eb, u4[j]) == 1;
             if (is) {
               cm.set(k);
-              lo[k] = l.L2 - l.err;
-              // (a NaN bound leaves `first` as it is and passes the test below)
               first = l.L2 + l.err < first ? l.L2 + l.err : first;
             }
           }
         }
         nc = cm.count();
-        int best = -1;
         if (nc > 0) {
-          RowMask near;
-          RowMask a = cm;
-          while (a.any()) {
-            const int k = a.pop();
-            if (!(lo[k] > first)) near.set(k);
-          }
-          best = near.pop();
-          if (near.any()) {
-            const VD dv = load_vd(S, v);
-            double Lb = sqrt(metric_len2(dv, load_vd(S, c.vb + nn[best])));
-            ops += kOpsLen2 + 1;
-            while (near.any()) {  // ascending position, hence id
-              const int k = near.pop();
-              const double L = sqrt(metric_len2(dv, load_vd(S, c.vb + nn[k])));
-              ops += kOpsLen2 + 1;
-              if (dlt(L, Lb)) {
-                Lb = L;
-                best = k;
-              }
-            }
-          }
+          const int best = first_by_length(S, v, c.vb, nn, fv, cm, first, ops);
           cand[(size_t)v * S.W] = nn[best];
+          cm.clear(best);
+          *cand_rest(cand, S, v) = make_ulonglong2(cm.lo, cm.hi);
         }
-        ncand[v] = nc;
         if (nc == 0) target[v] = -1;
       }
     }
     warp_append(reuse_cand, v, C, nC);
-    warp_append_t(eval && nc > 0, make_int2(v, 0), W0, nW0);
+    warp_append(eval && nc > 0, v, W0, nW0);
   }
 }
 
-__global__ void k_coarsen_scan(Store S, const int* D, const int* nDp, int* target, int* cand,
-                               int* ncand, int* C, int* nC, int* cmark, int tag, int pass0,
-                               int2* W0, int* nW0) {
-  coarsen_scan_phase(S, D, nDp, target, cand, ncand, C, nC, cmark, tag, pass0, W0, nW0);
+__global__ void __launch_bounds__(256, 3)
+k_coarsen_scan(Store S, const int* D, const int* nDp, int* target, int* cand, int* C, int* nC,
+               int* cmark, int tag, int pass0, int* W0, int* nW0) {
+  coarsen_scan_phase(S, D, nDp, target, cand, C, nC, cmark, tag, pass0, W0, nW0);
 }
 
-// The candidates of the warp's vertices (one per lane, `eval` lanes) by
-// (exact length, id) into their rows of `cand`.  The exact lengths are
-// evaluated 32 at a time from a per-warp queue, each candidate's length
-// stored in a scratch row and its bit in a per-lane mask; then each thread
-// places its own candidates by rank.
-__device__ __forceinline__ void coarsen_len_chunk(const Store& S, const int2* q, int cnt, int v,
-                                                  MeshCtx c, unsigned long long (*cm)[2],
-                                                  double* Lbuf) {
-  const int lane = threadIdx.x & 31;
-  const int2 r = lane < cnt ? q[lane] : make_int2(lane, 0);
-  const int ov = __shfl_sync(0xffffffffu, v, r.x);
-  const int ovb = __shfl_sync(0xffffffffu, c.vb, r.x);
-  const int oeb = __shfl_sync(0xffffffffu, c.eb, r.x);
-  const int omi = __shfl_sync(0xffffffffu, c.mi, r.x);
-  if (lane < cnt) {
-    const int u = nn_row(S, ov)[r.y];
-    const double L2 = metric_len2(load_vd(S, ov), load_vd(S, ovb + u));
-    const double4 band = S.tab.band[omi];
-    bool is = len_lt(L2, band.x, band.y, S.tab.L_low[omi]);
-    // a boundary vertex collapses only along a boundary edge
-    if (is && (S.vflag[ov] & VF_BND)) is = count_elems_with(S, ne_row(S, ov), S.NElen[ov], oeb, u) == 1;
-    if (is) {
-      Lbuf[(size_t)ov * S.W + r.y] = sqrt(L2);
-      atomicOr(&cm[r.x][r.y >> 6], 1ull << (r.y & 63));
-    }
-  }
-}
-
-__device__ __forceinline__ void coarsen_rank(const Store& S, bool eval, int v, MeshCtx c, int2* q,
-                                             unsigned long long (*scm)[2], int* cand,
-                                             double* Lbuf) {
-  const int lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  scm[lane][0] = scm[lane][1] = 0ull;
-  __syncwarp();
-  const int nnl = eval ? S.NNlen[v] : 0;
-  const float4 bf = eval ? S.tab.bandf[c.mi] : make_float4(0.f, 0.f, 0.f, 0.f);
-  VF fv{};
-  if (eval) fv = load_vf(S, v);
-  const int tmax = __reduce_max_sync(0xffffffffu, nnl);
-  int qn = 0;  // the same in every lane
-  for (int t = 0; t < tmax; ++t) {
-    const bool p =
-        t < nnl && edge_cmp(fv, load_vf(S, c.vb + nn_row(S, v)[t]), bf.x, bf.y) <= 0;
-    const unsigned m = __ballot_sync(0xffffffffu, p);
-    if (p) q[qn + __popc(m & lt)] = make_int2(lane, t);
-    qn += __popc(m);
-    __syncwarp();
-    if (qn >= 32) {
-      coarsen_len_chunk(S, q, 32, v, c, scm, Lbuf);
-      __syncwarp();
-      if (lane < qn - 32) q[lane] = q[32 + lane];
-      qn -= 32;
-      __syncwarp();
-    }
-  }
-  if (qn > 0) coarsen_len_chunk(S, q, qn, v, c, scm, Lbuf);
-  __syncwarp();
-  if (eval) {
-    RowMask cm;
-    cm.lo = scm[lane][0];
-    cm.hi = scm[lane][1];
-    const int* nn = nn_row(S, v);
-    const double* L = Lbuf + (size_t)v * S.W;
-    int* out = cand + (size_t)v * S.W;
-    RowMask a = cm;
-    while (a.any()) {
-      const int k = a.pop();
-      const double Lk = L[k];
-      int rank = 0;
-      RowMask b = cm;
-      while (b.any()) {
-        const int k2 = b.pop();
-        const double Lo = L[k2];
-        if (dlt(Lo, Lk) || (dbits(Lo) == dbits(Lk) && k2 < k)) ++rank;
-      }
-      out[rank] = nn[k];
-    }
-  }
-  __syncwarp();
-}
-
-// The check passes, one work item (v, k) per thread: is collapsing v onto
-// its k-th candidate valid (in the last pass: the first valid one from k on)?
+// The check passes, one candidate per thread: is collapsing v onto it valid?
 // Validity is the conjunction of the link condition (|NN(v) & NN(u)| = 2 for
 // an interior edge, 1 for a boundary edge; a boundary vertex only along a
 // boundary edge) and, for the collapse with v on u, every remaining ball
@@ -940,116 +872,206 @@ __device__ __forceinline__ bool check_filter(const Store& S, const CoarsenCtx& x
   return ok;
 }
 
-template <bool LAST>
-__device__ __forceinline__ void coarsen_check_phase(Store S, const int2* Win, const int* nWin,
-                                                    int2* Wout, int* nWout, int* target,
-                                                    int* cand, const int* ncand, int* C,
-                                                    int* nC, int* cmark, int tag, double* Lbuf,
+// The warp's candidates, one per lane (`have` lanes): u for x.v.  Whole warps call.
+__device__ __forceinline__ bool check_candidates(const Store& S, const CheckQueues& Q,
+                                                 const CoarsenCtx& x, int u, bool have,
+                                                 unsigned& ops) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  RowMask oo, ol;
+  const bool may = have && check_filter(S, x, u, oo, ol);
+  Q.ok[lane] = may ? 1 : 0;
+  if (!may) oo = ol = RowMask();
+  const int ws = x.c.vb + u;
+  int no = 0, nl = 0;  // queue lengths, the same in every lane
+  __syncwarp();
+  while (__ballot_sync(0xffffffffu, oo.any() || ol.any())) {
+    const bool po = oo.any(), pl = ol.any();
+    const unsigned mo = __ballot_sync(0xffffffffu, po);
+    const unsigned ml = __ballot_sync(0xffffffffu, pl);
+    if (po) {
+      const int4 e = S.EN[x.c.eb + x.ne[oo.pop()]];
+      Q.qo[no + __popc(mo & lt)] = make_int4(lane, e.x, e.y, e.z);
+    }
+    if (pl) Q.ql[nl + __popc(ml & lt)] = make_int2(lane, x.nn[ol.pop()]);
+    no += __popc(mo);
+    nl += __popc(ml);
+    __syncwarp();
+    if (no >= 32) {
+      check_orient_chunk(S, Q, 32, x.c.vb, x.lv, ws, ops);
+      __syncwarp();
+      if (lane < no - 32) Q.qo[lane] = Q.qo[32 + lane];
+      no -= 32;
+      __syncwarp();
+    }
+    if (nl >= 32) {
+      check_len_chunk(S, Q, 32, x.c.vb, ws, x.c.mi, ops);
+      __syncwarp();
+      if (lane < nl - 32) Q.ql[lane] = Q.ql[32 + lane];
+      nl -= 32;
+      __syncwarp();
+    }
+  }
+  if (no > 0) check_orient_chunk(S, Q, no, x.c.vb, x.lv, ws, ops);
+  if (nl > 0) check_len_chunk(S, Q, nl, x.c.vb, ws, x.c.mi, ops);
+  __syncwarp();
+  const bool ok = Q.ok[lane] != 0;
+  __syncwarp();
+  return ok;
+}
+
+// Pass 2: every listed vertex's first candidate.
+__device__ __forceinline__ void coarsen_check_phase(Store S, const int* Win, const int* nWin,
+                                                    int* Wout, int* nWout, int* target, int* cand,
+                                                    int* C, int* nC, int* cmark, int tag,
                                                     unsigned long long* work) {
   __shared__ int4 sqo[kCheckWarps][64];
   __shared__ int2 sql[kCheckWarps][64];
   __shared__ int sok[kCheckWarps][32];
-  __shared__ unsigned long long scm[LAST ? kCheckWarps : 1][32][2];
-  const int lane = threadIdx.x & 31, wq = (threadIdx.x >> 5) % kCheckWarps;
-  CheckQueues Q{sqo[wq], sql[wq], sok[wq]};
-  const unsigned lt = (1u << lane) - 1u;
+  const int wq = (threadIdx.x >> 5) % kCheckWarps;
+  const CheckQueues Q{sqo[wq], sql[wq], sok[wq]};
   unsigned ops = 0;
   const int n = *nWin;
   for (int i0 = blockIdx.x * blockDim.x; i0 < n; i0 += gridDim.x * blockDim.x) {
     const int i = i0 + threadIdx.x;
-    int v = 0, k = 0, nc = 0;
-    bool found = false, done = i >= n;
+    const bool have = i < n;
+    int v = 0, u = 0;
     CoarsenCtx x{};
-    const int* cv = nullptr;
-    if (!done) {
-      const int2 it = Win[i];
-      v = it.x;
-      k = it.y;
+    if (have) {
+      v = Win[i];
       x = coarsen_ctx(S, v, ctx_of(S, v));
-      cv = cand + (size_t)v * S.W;
-      nc = ncand[v];
+      u = cand[(size_t)v * S.W];
     }
-    if (LAST) coarsen_rank(S, !done, v, x.c, Q.ql, scm[LAST ? wq : 0], cand, Lbuf);
-    // one candidate per lane and turn; the last pass moves on to the next
-    // candidate of each lane whose candidate failed
-    while (__ballot_sync(0xffffffffu, !done)) {
-      const int u = done ? 0 : cv[k];
-      RowMask oo, ol;
-      const bool may = !done && check_filter(S, x, u, oo, ol);
-      Q.ok[lane] = may ? 1 : 0;
-      if (!may) oo = ol = RowMask();
-      const int ws = x.c.vb + u;
-      int no = 0, nl = 0;  // queue lengths, the same in every lane
-      __syncwarp();
-      while (__ballot_sync(0xffffffffu, oo.any() || ol.any())) {
-        const bool po = oo.any(), pl = ol.any();
-        const unsigned mo = __ballot_sync(0xffffffffu, po);
-        const unsigned ml = __ballot_sync(0xffffffffu, pl);
-        if (po) {
-          const int4 e = S.EN[x.c.eb + x.ne[oo.pop()]];
-          Q.qo[no + __popc(mo & lt)] = make_int4(lane, e.x, e.y, e.z);
-        }
-        if (pl) Q.ql[nl + __popc(ml & lt)] = make_int2(lane, x.nn[ol.pop()]);
-        no += __popc(mo);
-        nl += __popc(ml);
-        __syncwarp();
-        if (no >= 32) {
-          check_orient_chunk(S, Q, 32, x.c.vb, x.lv, ws, ops);
-          __syncwarp();
-          if (lane < no - 32) Q.qo[lane] = Q.qo[32 + lane];
-          no -= 32;
-          __syncwarp();
-        }
-        if (nl >= 32) {
-          check_len_chunk(S, Q, 32, x.c.vb, ws, x.c.mi, ops);
-          __syncwarp();
-          if (lane < nl - 32) Q.ql[lane] = Q.ql[32 + lane];
-          nl -= 32;
-          __syncwarp();
-        }
-      }
-      if (no > 0) check_orient_chunk(S, Q, no, x.c.vb, x.lv, ws, ops);
-      if (nl > 0) check_len_chunk(S, Q, nl, x.c.vb, ws, x.c.mi, ops);
-      __syncwarp();
-      if (!done) {
-        found = Q.ok[lane] != 0;
-        if (found || !LAST || k + 1 >= nc) done = true;
-        else ++k;
-      }
-      __syncwarp();
-    }
+    const bool found = check_candidates(S, Q, x, u, have, ops);
     bool next = false;
-    if (i < n) {
+    if (found) {
+      target[v] = u;
+      cmark[v] = tag;
+      S.tab.had[x.c.mi] = 1;
+    } else if (have) {
+      const ulonglong2 rest = *cand_rest(cand, S, v);
+      next = (rest.x | rest.y) != 0;
+      if (!next) target[v] = -1;
+    }
+    warp_append(found, v, C, nC);
+    warp_append(next, v, Wout, nWout);
+  }
+  add_work(work, ops);
+}
+
+__global__ void k_coarsen_check(Store S, const int* Win, const int* nWin, int* Wout, int* nWout,
+                                int* target, int* cand, int* C, int* nC, int* cmark, int tag,
+                                unsigned long long* work) {
+  coarsen_check_phase(S, Win, nWin, Wout, nWout, target, cand, C, nC, cmark, tag, work);
+}
+
+// Pass 3: all other candidates of the vertices whose first one failed, one per lane.
+// Most of these vertices have no valid candidate at all, so checking one after
+// the other by length (a thread per vertex) was a chain of up to six checks in a
+// few warps (9-16% of the warp slots held); eight vertices a warp fill its lanes
+// once, and lengths are compared only where several candidates are valid.
+constexpr int kRestOwners = 8;
+
+__device__ __forceinline__ void coarsen_rest_phase(Store S, const int* Win, const int* nWin,
+                                                   int* target, int* cand, int* C, int* nC,
+                                                   int* cmark, int tag,
+                                                   unsigned long long* work) {
+  __shared__ int4 sqo[kCheckWarps][64];
+  __shared__ int2 sql[kCheckWarps][64];
+  __shared__ int sok[kCheckWarps][32];
+  __shared__ unsigned long long svalid[kCheckWarps][kRestOwners][2];
+  const int lane = threadIdx.x & 31, wq = (threadIdx.x >> 5) % kCheckWarps;
+  const CheckQueues Q{sqo[wq], sql[wq], sok[wq]};
+  unsigned long long (*valid)[2] = svalid[wq];
+  unsigned ops = 0;
+  const int n = *nWin;
+  const int warps = gridDim.x * (blockDim.x >> 5);
+  for (int i0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kRestOwners; i0 < n;
+       i0 += warps * kRestOwners) {
+    const bool own = lane < kRestOwners && i0 + lane < n;
+    int v = 0;
+    RowMask rest;
+    if (own) {
+      v = Win[i0 + lane];
+      const ulonglong2 r = *cand_rest(cand, S, v);
+      rest.lo = r.x;
+      rest.hi = r.y;
+    }
+    if (lane < kRestOwners) valid[lane][0] = valid[lane][1] = 0ull;
+    int end = rest.count();  // of the owner's candidates in the warp's sequence
+#pragma unroll
+    for (int o = 1; o < kRestOwners; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, end, o);
+      if (lane >= o) end += y;
+    }
+    const int total = __shfl_sync(0xffffffffu, end, kRestOwners - 1);
+    __syncwarp();
+    for (int p0 = 0; p0 < total; p0 += 32) {
+      const int p = p0 + lane;
+      const bool have = p < total;
+      int o = 0, start = 0;  // the owner of candidate p, its first candidate
+#pragma unroll
+      for (int q = 0; q < kRestOwners - 1; ++q) {
+        const int e = __shfl_sync(0xffffffffu, end, q);
+        if (p >= e) {
+          o = q + 1;
+          start = e;
+        }
+      }
+      const int ov = __shfl_sync(0xffffffffu, v, o);
+      RowMask r;
+      r.lo = __shfl_sync(0xffffffffu, rest.lo, o);
+      r.hi = __shfl_sync(0xffffffffu, rest.hi, o);
+      int k = 0, u = 0;
+      CoarsenCtx x{};
+      if (have) {
+        for (int j = p - start; j >= 0; --j) k = r.pop();
+        x = coarsen_ctx(S, ov, ctx_of(S, ov));
+        u = x.nn[k];
+      }
+      if (check_candidates(S, Q, x, u, have, ops)) atomicOr(&valid[o][k >> 6], 1ull << (k & 63));
+    }
+    __syncwarp();
+    bool found = false;
+    if (own) {
+      RowMask ok;
+      ok.lo = valid[lane][0];
+      ok.hi = valid[lane][1];
+      found = ok.any();
       if (found) {
-        target[v] = cv[k];
+        const MeshCtx c = ctx_of(S, v);
+        const int* nn = nn_row(S, v);
+        const VF fv = load_vf(S, v);
+        float first = INFINITY;
+        RowMask a = ok;
+        while (a.any()) {
+          const FLen l = f_edge2(fv, load_vf(S, c.vb + nn[a.pop()]));
+          first = l.L2 + l.err < first ? l.L2 + l.err : first;
+        }
+        target[v] = nn[first_by_length(S, v, c.vb, nn, fv, ok, first, ops)];
         cmark[v] = tag;
-        S.tab.had[x.c.mi] = 1;
-      } else if (!LAST && k + 1 < nc) {
-        next = true;
+        S.tab.had[c.mi] = 1;
       } else {
         target[v] = -1;
       }
     }
     warp_append(found, v, C, nC);
-    if (!LAST) warp_append_t(next, make_int2(v, k + 1), Wout, nWout);
+    __syncwarp();
   }
   add_work(work, ops);
 }
 
-template <bool LAST>
-__global__ void k_coarsen_check(Store S, const int2* Win, const int* nWin, int2* Wout, int* nWout,
-                                int* target, int* cand, const int* ncand, int* C, int* nC,
-                                int* cmark, int tag, double* Lbuf, unsigned long long* work) {
-  coarsen_check_phase<LAST>(S, Win, nWin, Wout, nWout, target, cand, ncand, C, nC, cmark, tag,
-                            Lbuf, work);
+__global__ void k_coarsen_rest(Store S, const int* Win, const int* nWin, int* target, int* cand,
+                               int* C, int* nC, int* cmark, int tag, unsigned long long* work) {
+  coarsen_rest_phase(S, Win, nWin, target, cand, C, nC, cmark, tag, work);
 }
 
 // One tile per listed vertex, listing and checking at once (persistent
 // rounds): reuse or re-evaluate, then the candidates in order until one is a
 // valid collapse.  Same results as coarsen_scan_phase and the two check passes.
 __device__ __forceinline__ void coarsen_eval_phase(Store S, const int* D, const int* nDp,
-                                                   int* target, int* cand, int* ncand, int* C,
-                                                   int* nC, int* cmark, int tag, int pass0,
+                                                   int* target, int* cand, int* C, int* nC,
+                                                   int* cmark, int tag, int pass0,
                                                    unsigned long long* work, bool il = false) {
   const Tile t = tile_of();
   const int first = first_entry(D, trank(il), S.vslots);
@@ -1069,7 +1091,6 @@ __device__ __forceinline__ void coarsen_eval_phase(Store S, const int* D, const 
         if (t.tl == 0) S.evc[v] = tag;
         int* cv = cand + (size_t)v * S.W;
         int nc = tile_coarsen_candidates(t, S, v, c, cv, ops);
-        if (t.tl == 0) ncand[v] = nc;
         __syncwarp(t.mask);  // the candidates written by every lane
         if (nc > 0) {
           CoarsenCtx x = coarsen_ctx(S, v, c);
@@ -1711,7 +1732,7 @@ __device__ __forceinline__ void swap_edge_phase(Store S, const int2* items, cons
   add_work(work, ops);
 }
 
-__global__ void k_swap_edge(Store S, const int2* items, const int* nIp, int icap, double* gains,
+__global__ void __launch_bounds__(256, 4) k_swap_edge(Store S, const int2* items, const int* nIp, int icap, double* gains,
                             int tag, unsigned long long* work) {
   swap_edge_phase(S, items, nIp, icap, gains, tag, work);
 }
@@ -3264,7 +3285,7 @@ __device__ __forceinline__ bool refine_row_short(const Store& S, int s, int src,
 // read the old element row of their split edge's first end (the children that
 // contain the new vertex are exactly those of the two parents on that edge), then
 // the old ones, which read and write their own rows alone.
-__global__ void k_refine_rows(Store S, int vfirst, int vend, int fresh, const int* escan,
+__global__ void __launch_bounds__(256, 4) k_refine_rows(Store S, int vfirst, int vend, int fresh, const int* escan,
                               const int4* owner, int stamp, DevStatus* st) {
   for (int s = vfirst + blockIdx.x * blockDim.x + threadIdx.x; s < vend;
        s += gridDim.x * blockDim.x) {
@@ -3505,7 +3526,7 @@ __device__ __forceinline__ void topo_rounds(const RoundArgs& a) {
       if (!grid_barrier(a.bar, target, a.st)) return;
       if (blockIdx.x == 0 && threadIdx.x == 0) cnt[CN_E] = cnt[CN_I] = 0;
     } else {
-      coarsen_eval_phase(a.S, w.D[cur], cnt + cn_list(cur), w.target, w.cand, w.ncand, w.C, nC,
+      coarsen_eval_phase(a.S, w.D[cur], cnt + cn_list(cur), w.target, w.cand, w.C, nC,
                          w.cmark, tag, pass0, a.work, true);
       if (!grid_barrier(a.bar, target, a.st)) return;
       if (blockIdx.x == 0 && threadIdx.x == 0) *cand_count(cnt, r + 1) = 0;
@@ -3701,10 +3722,10 @@ void zero_counts(MeshSet& m, int first, int num) {
   cudaMemsetAsync(m.w.counts + first, 0, num * sizeof(int), m.stream);
 }
 
-// The counters of a new round (C, S, A, E, I, I2) and of the list it fills
+// The counters of a new round (C, S, A, E, I) and of the list it fills
 // (D[nxt]); the list it reads keeps its count.
 void zero_round(MeshSet& m, int nxt) {
-  static_assert(CN_D0 == 0 && CN_C == 1 && CN_I2 == 6 && CN_D1 == 7, "counter layout");
+  static_assert(CN_D0 == 0 && CN_C == 1 && CN_I == 5 && CN_D1 == 7, "counter layout");
   zero_counts(m, nxt == 0 ? CN_D0 : CN_C, 7);
 }
 
@@ -4013,16 +4034,15 @@ int op_coarsen(MeshSet& m, int max_rounds, const Ahead& h) {
     int nxt = 1 - cur;
     zero_round(m, nxt);
     PM_LAUNCH(k_coarsen_scan, gv, bs, 0, m.stream, m.S, w.D[cur], w.counts + cn_list(cur),
-              w.target, w.cand, w.ncand, w.C, w.counts + CN_C, w.cmark, tag, pass0, w.items,
-              w.counts + CN_I);
-    // one dense wave checking every vertex's best candidate, then the
-    // remaining candidates of the vertices whose best one failed
-    PM_LAUNCH(k_coarsen_check<false>, gv, bs, 0, m.stream, m.S, w.items, w.counts + CN_I, w.items2,
-              w.counts + CN_I2, w.target, w.cand, w.ncand, w.C, w.counts + CN_C, w.cmark, tag,
-              w.gains, prof_work("k_coarsen_check"));
-    PM_LAUNCH(k_coarsen_check<true>, gv, bs, 0, m.stream, m.S, w.items2, w.counts + CN_I2, w.items,
-              w.counts + CN_I, w.target, w.cand, w.ncand, w.C, w.counts + CN_C, w.cmark, tag,
-              w.gains, prof_work("k_coarsen_check"));
+              w.target, w.cand, w.C, w.counts + CN_C, w.cmark, tag, pass0, w.E,
+              w.counts + CN_E);
+    // one dense wave checking every vertex's first candidate, then the other
+    // candidates of the vertices whose first one failed
+    PM_LAUNCH(k_coarsen_check, gv, bs, 0, m.stream, m.S, w.E, w.counts + CN_E, w.Sl,
+              w.counts + CN_S, w.target, w.cand, w.C, w.counts + CN_C, w.cmark, tag,
+              prof_work("k_coarsen_check"));
+    PM_LAUNCH(k_coarsen_rest, gv, bs, 0, m.stream, m.S, w.Sl, w.counts + CN_S, w.target, w.cand,
+              w.C, w.counts + CN_C, w.cmark, tag, prof_work("k_coarsen_rest"));
     zero_counts(m, CN_CL, 1);
     PM_LAUNCH(k_coarsen_select_apply, gv, bs, 0, m.stream, m.S, w.C, w.counts + CN_C, w.cmark,
               w.smark, tag, w.target, w.A, w.counts + CN_A, w.amark, w.D[nxt],
