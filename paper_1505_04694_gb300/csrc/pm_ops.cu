@@ -2259,7 +2259,7 @@ __device__ __forceinline__ void smooth_scan_phase(Store S, const int* D, const i
   }
 }
 
-__global__ void k_smooth_scan(Store S, const int* D, const int* nDp, double4* mvM, int* C, int* nC,
+__global__ void __launch_bounds__(256, 3) k_smooth_scan(Store S, const int* D, const int* nDp, double4* mvM, int* C, int* nC,
                               int* cmark, int tag, int pass0, int* E, int* nE) {
   smooth_scan_phase(S, D, nDp, mvM, C, nC, cmark, tag, pass0, E, nE);
 }
@@ -2768,7 +2768,7 @@ __global__ void k_smooth_filter(Store S, const int* E, const int* nEp, double2* 
   smooth_filter_phase(S, E, nEp, mvxy, mvM, R, nR, work);
 }
 
-__global__ void k_smooth_eval(Store S, const int* R, const int* nRp, const double2* mvxy,
+__global__ void __launch_bounds__(256, 3) k_smooth_eval(Store S, const int* R, const int* nRp, const double2* mvxy,
                               double4* mvM, double* qball, int* C, int* nC, int* cmark, int tag,
                               unsigned long long* work) {
   smooth_exact_packed(S, R, nRp, mvxy, mvM, qball, C, nC, cmark, tag, work);
@@ -3035,7 +3035,7 @@ __global__ void k_stamp_list(Store S, const int* L, const int* nLp, int* cmark, 
 // inside one call vertices keep their positions and metrics until the
 // operator loop ends (smoothing runs after it), so a's own stamp tells
 // whether anything the mask read has changed: every change of a's row stamps a.
-__global__ void k_refine_mark(Store S, int* cnt, RowMask* mask, int tag, int pass0, int lo,
+__global__ void __launch_bounds__(256, 5) k_refine_mark(Store S, int* cnt, RowMask* mask, int tag, int pass0, int lo,
                               const int* before, const int* before2, const DevStatus* st) {
   if (!may_go(before, st)) return;
   tag += tags_of(before) + tags_of(before2);
