@@ -144,17 +144,21 @@ PM_HD int f_len_cmp(const FLen& l, float lo2, float hi2) {
   return l.L2 - l.err > hi2 ? 1 : (l.L2 + l.err < lo2 ? -1 : 0);
 }
 
-// An upper bound of the quality (12 sqrt 3 A / P^2) F(P / 3) of element
-// (a, b, c) in its mean metric, or NaN when the bound would be loose.  The
-// quality grows with the area and the metric's determinant, which are taken at
-// their upper bounds; as a function of P it is h(P) = F(P / 3) / P^2 with
+// Bounds of the quality (12 sqrt 3 A / P^2) F(P / 3) of element (a, b, c) in its
+// mean metric: `up` is NaN and `lo` -1 when they would be loose, and `lo` is -1
+// unless the element is certainly counter-clockwise.  The quality grows with the
+// area and the metric's determinant, which are taken at their bounds; as a function of P it is h(P) = F(P / 3) / P^2 with
 // |d ln h / d ln P| <= 5 (between -2 and 1 below the ideal perimeter, between
 // -5 and -2 above), so a relative error rP of P changes it by at most 5 rP to
 // first order (rP <= 0.04 is required, the rest of the series is inside the
 // factor 1.15).  `sign` receives the orientation's sign, 0 when undecided.  `kx`
 // bounds the relative error of one vertex's metric beyond its rounding (see
 // f_metric_at): it adds to that of the mean, and four times to the determinant's.
-PM_HD float f_quality_up(const VF& a, const VF& b, const VF& c, int& sign, float kx = 0.0f) {
+struct FQual {
+  float lo, up;
+};
+
+PM_HD FQual f_quality(const VF& a, const VF& b, const VF& c, int& sign, float kx = 0.0f) {
   const float E = a.e + (b.e + c.e);
   const float dx0 = f_dx(a, b), dy0 = f_dy(a, b);
   const float dx1 = f_dx(b, c), dy1 = f_dy(b, c);
@@ -179,14 +183,23 @@ PM_HD float f_quality_up(const VF& a, const VF& b, const VF& c, int& sign, float
   // (perimeters and metrics whose powers would underflow give no bound)
   const bool fine = rP < 0.04f && kx < 0.05f && q0.err < 0.4f * q0.L2 && q1.err < 0.4f * q1.L2 &&
                     q2.err < 0.4f * q2.L2 && P > 1e-6f && P < 1e6f && kk > 1e-30f;
-  const float D = (kk - k01 * k01) + (28.0f * kU + 4.2f * kx) * kk;
+  const float D = kk - k01 * k01, eD = (28.0f * kU + 4.2f * kx) * kk;
   const float up = 0.5f * (d.det + d.err);
   const float area = up < 0.0f ? 0.0f : up;  // a negative quality is below 0 (a NaN stays)
   const float x = P * third;
   const float s = x > 1.0f ? 3.0f * rp : x;
   const float f = s * (2.0f - s);
-  const float q = ((20.784612f * area) * f_sqrt(D)) * ((rp * rp) * ((f * f) * f));
-  return fine ? q + (q * (5.75f * rP + 40.0f * kU) + 1e-30f) : nanf("");
+  const float h = (rp * rp) * ((f * f) * f), eh = 5.75f * rP + 40.0f * kU;
+  const float q = ((20.784612f * area) * f_sqrt(D + eD)) * h;
+  const float p = ((20.784612f * (0.5f * (d.det - d.err))) * f_sqrt(D - eD)) * h;
+  FQual r;
+  r.up = fine ? q + (q * eh + 1e-30f) : nanf("");
+  r.lo = fine && sign > 0 && D > eD ? p - (p * eh + 1e-30f) : -1.0f;
+  return r;
+}
+
+PM_HD float f_quality_up(const VF& a, const VF& b, const VF& c, int& sign, float kx = 0.0f) {
+  return f_quality(a, b, c, sign, kx).up;
 }
 
 // The barycentric metric at point x of element (a, b, d), into the metric part of

@@ -2223,13 +2223,20 @@ __device__ __forceinline__ double ball_min_quality(const Store& S, MeshCtx c, co
   return qmin;
 }
 
+// The w of a stored move (mvM): 0 no move; 1 its new ball qualities are stored too;
+// 2 it certainly holds and they are evaluated after the move.  The last only in the
+// rounds with a kernel per phase, whose filter leaves them open (`defer`): in a
+// persistent round they would be one more phase and barrier, which lost 1% on
+// meshes of up to 130k triangles; it evaluates again what it finds of them.
+constexpr double kMoveEvaluated = 1.0, kMoveUnevaluated = 2.0;
+
 // Smoothing evaluation in two passes.  Pass 1 (per pending vertex): reuse an
 // unchanged earlier result, drop vertices whose ball is already good enough
 // (cached qualities), list the rest for the full move evaluation.
 __device__ __forceinline__ void smooth_scan_phase(Store S, const int* D, const int* nDp,
                                                   double4* mvM, int* C, int* nC, int* cmark,
                                                   int tag, int pass0, int* E, int* nE,
-                                                  bool il = false) {
+                                                  bool defer, bool il = false) {
   const int n = *nDp;
   for (int i0 = 0; i0 < n; i0 += gsize()) {
     int i = i0 + grank(il);
@@ -2238,8 +2245,9 @@ __device__ __forceinline__ void smooth_scan_phase(Store S, const int* D, const i
     if (i < n) {
       v = D[i];
       MeshCtx c = ctx_of(S, v);
-      if (unchanged(S, v, c.vb, S.evm[v], pass0)) {
-        reuse_cand = mvM[v].w != 0.0;
+      const double move = mvM[v].w;
+      if (unchanged(S, v, c.vb, S.evm[v], pass0) && (defer || move != kMoveUnevaluated)) {
+        reuse_cand = move != 0.0;
         if (reuse_cand) {
           cmark[v] = tag;
           S.tab.had[c.mi] = 1;
@@ -2261,7 +2269,7 @@ __device__ __forceinline__ void smooth_scan_phase(Store S, const int* D, const i
 
 __global__ void __launch_bounds__(256, 3) k_smooth_scan(Store S, const int* D, const int* nDp, double4* mvM, int* C, int* nC,
                               int* cmark, int tag, int pass0, int* E, int* nE) {
-  smooth_scan_phase(S, D, nDp, mvM, C, nC, cmark, tag, pass0, E, nE);
+  smooth_scan_phase(S, D, nDp, mvM, C, nC, cmark, tag, pass0, E, nE, true);
 }
 
 // Minimum cached quality of v's ball (and, if asked, its sum in ascending
@@ -2331,16 +2339,18 @@ __device__ __forceinline__ double4 tile_interpolate_in(const Tile& t, const Stor
   return make_double4(tshfl(t, m, 0), tshfl(t, m, 1), tshfl(t, m, 2), 0.0);
 }
 
-// Upper bound of the quality of element e of v's ball with v at the record `fn`
-// (relative error kx of its metric), -1 when it is certainly not
-// counter-clockwise, NaN when there is no useful bound.
-__device__ __forceinline__ float moved_quality_up(const Store& S, int vb, int lv, int4 e,
+// Bounds of the quality of element e of v's ball with v at the record `fn`
+// (relative error kx of its metric): the upper one is -1 when it is certainly not
+// counter-clockwise, NaN when there is no useful bound; the lower one is -1 unless it
+// is certainly counter-clockwise and the bound useful.
+__device__ __forceinline__ FQual moved_quality(const Store& S, int vb, int lv, int4 e,
                                                   const VF& fn, float kx) {
   const VF a = e.x == lv ? fn : load_vf(S, vb + e.x), b = e.y == lv ? fn : load_vf(S, vb + e.y),
            c = e.z == lv ? fn : load_vf(S, vb + e.z);
   int sign;
-  const float up = f_quality_up(a, b, c, sign, kx);
-  return sign < 0 ? -1.0f : up;
+  FQual q = f_quality(a, b, c, sign, kx);
+  if (sign < 0) q.up = -1.0f;
+  return q;
 }
 
 // The FP32 metric at X in element e into fn, its relative error bound.
@@ -2414,7 +2424,7 @@ __device__ bool tile_try_move(const Tile& t, const Store& S, MeshCtx c, int lv, 
   bool fails = false;
   float up = 0.0f;
   for (int k = t.tl; k < nel; k += TW) {
-    const float u = moved_quality_up(S, c.vb, lv, S.EN[c.eb + ne[k]], fn, kx);
+    const float u = moved_quality(S, c.vb, lv, S.EN[c.eb + ne[k]], fn, kx).up;
     fails |= u < ffloor;
     up += u;
   }
@@ -2491,18 +2501,22 @@ __device__ bool tile_smooth_eval(const Tile& t, const Store& S, int v, MeshCtx c
 // the 2x2 solve, the location and the interpolation run per thread (a tile of
 // lanes per vertex repeats them in every lane: four vertices per warp instruction
 // of FP64 instead of 32), and the FP32 bounds of the moved ball (its metric
-// interpolated in FP32 first) drop the moves that certainly fail.  The others are
-// listed for pass 3 with their target and metric.
+// interpolated in FP32 first) drop the moves that certainly fail.  With `defer` those
+// that certainly hold become candidates at once: their new qualities are evaluated
+// when the move is made (half the candidates lose to a neighbour, and most of those
+// are evaluated again after it has moved).  The others are listed for pass 3.
 __device__ __forceinline__ void smooth_filter_phase(Store S, const int* E, const int* nEp,
                                                     double2* mvxy, double4* mvM, int* R, int* nR,
-                                                    unsigned long long* work, bool il = false) {
+                                                    int* C, int* nC, int* cmark, int tag,
+                                                    bool defer, unsigned long long* work,
+                                                    bool il = false) {
   const int first = first_entry(E, grank(il), S.vslots);
   const int n = *nEp;
   unsigned ops = 0;
   for (int j0 = 0; j0 < n; j0 += gsize()) {
     const int j = j0 + grank(il);
     int v = 0;
-    bool may = false;
+    bool may = false, sure = defer;
     if (j < n) {
       v = j0 == 0 ? first : E[j];
       const MeshCtx c = ctx_of(S, v);
@@ -2561,15 +2575,22 @@ __device__ __forceinline__ void smooth_filter_phase(Store S, const int* E, const
         if (may) {
           VF fn;
           const float kx = metric_at(S, c.vb, e, fx, fn);
-          const float ffloor = __double2float_rd(qold);
+          const float ffloor = __double2float_rd(qold), fceil = __double2float_ru(qold);
 #pragma unroll 2
           for (int k = 0; k < nel; ++k)
-            may = may &&
-                  !(moved_quality_up(S, c.vb, lv, S.EN[c.eb + ne[k]], fn, kx) < ffloor);
+            if (may) {
+              const FQual q = moved_quality(S, c.vb, lv, S.EN[c.eb + ne[k]], fn, kx);
+              may = !(q.up < ffloor);
+              sure = sure && q.lo > fceil;
+            }
           if (may) {
             double4 Mn = interpolate_in(S, c.vb, e, x, y);
             ops += 46;
-            Mn.w = qold;  // for pass 3
+            Mn.w = sure ? kMoveUnevaluated : qold;  // (for pass 3)
+            if (sure) {
+              cmark[v] = tag;
+              S.tab.had[c.mi] = 1;
+            }
             mvxy[v] = make_double2(x, y);
             mvM[v] = Mn;
           }
@@ -2577,7 +2598,9 @@ __device__ __forceinline__ void smooth_filter_phase(Store S, const int* E, const
       }
       if (!may) mvM[v].w = 0.0;
     }
-    warp_append(may, v, R, nR);
+    const Room3 at = warp_reserve3(may && !sure ? 1 : 0, nR, may && sure ? 1 : 0, nC, 0, nullptr);
+    if (may && !sure) R[at.a] = v;
+    if (may && sure) C[at.b] = v;
   }
   add_work(work, ops);
 }
@@ -2609,7 +2632,7 @@ __device__ __forceinline__ void smooth_exact_phase(Store S, const int* R, const 
                              qball + (size_t)v * S.W, nullptr);
       if (t.tl == 0) {
         ops += 85 * nel;
-        mvM[v].w = cand ? 1.0 : 0.0;  // marks a stored move
+        mvM[v].w = cand ? kMoveEvaluated : 0.0;
         if (cand) {
           cmark[v] = tag;
           S.tab.had[c.mi] = 1;
@@ -2642,11 +2665,12 @@ __device__ __forceinline__ void smooth_scan_eval_phase(Store S, const int* D, co
     if (j < n) {
       v = j0 == 0 ? first : D[j];
       MeshCtx c = ctx_of(S, v);
-      bool keep = unchanged(S, v, c.vb, S.evm[v], pass0);
+      const double move = mvM[v].w;
+      bool keep = unchanged(S, v, c.vb, S.evm[v], pass0) && move != kMoveUnevaluated;
       keep = __shfl_sync(t.mask, keep, 0, TW);
       if (keep) {
         if (t.tl == 0) {
-          cand = mvM[v].w != 0.0;
+          cand = move != 0.0;
           if (cand) {
             cmark[v] = tag;
             S.tab.had[c.mi] = 1;
@@ -2659,7 +2683,7 @@ __device__ __forceinline__ void smooth_scan_eval_phase(Store S, const int* D, co
         if (t.tl == 0) {
           S.evm[v] = tag;
           if (cand) {
-            Mv.w = 1.0;  // marks a stored move
+            Mv.w = kMoveEvaluated;
             mvxy[v] = X;
             mvM[v] = Mv;
             cmark[v] = tag;
@@ -2751,7 +2775,7 @@ __device__ __forceinline__ void smooth_exact_packed(Store S, const int* R, const
       const unsigned mask = (hi >= 32 ? 0xffffffffu : (1u << hi) - 1u) &
                             ~(lo >= 32 ? 0xffffffffu : (1u << lo) - 1u);
       cand = (bad & mask) == 0u;
-      mvM[v].w = cand ? 1.0 : 0.0;  // marks a stored move
+      mvM[v].w = cand ? kMoveEvaluated : 0.0;
       if (cand) {
         cmark[v] = tag;
         S.tab.had[ctx_of(S, v).mi] = 1;
@@ -2764,8 +2788,9 @@ __device__ __forceinline__ void smooth_exact_packed(Store S, const int* R, const
 }
 
 __global__ void k_smooth_filter(Store S, const int* E, const int* nEp, double2* mvxy,
-                                double4* mvM, int* R, int* nR, unsigned long long* work) {
-  smooth_filter_phase(S, E, nEp, mvxy, mvM, R, nR, work);
+                                double4* mvM, int* R, int* nR, int* C, int* nC, int* cmark,
+                                int tag, unsigned long long* work) {
+  smooth_filter_phase(S, E, nEp, mvxy, mvM, R, nR, C, nC, cmark, tag, true, work);
 }
 
 __global__ void __launch_bounds__(256, 3) k_smooth_eval(Store S, const int* R, const int* nRp, const double2* mvxy,
@@ -2783,22 +2808,23 @@ __device__ __forceinline__ void smooth_select_apply_phase(Store S, const int* C,
                                                           int* Dn, int* nDn, int* dmark,
                                                           const double2* mvxy, const double4* mvM,
                                                           const double* qball, int* P, int* nP,
-                                                          int* pmark, int ptag, int stamp,
-                                                          bool il = false) {
+                                                          int* pmark, int ptag, int stamp, int* Q,
+                                                          int* nQ, bool il = false) {
   const int first = first_entry(C, grank(il), S.vslots);
   const int n = *nCp;
   for (int i0 = 0; i0 < n; i0 += gsize()) {
     int i = i0 + grank(il);
     bool win = false, lose = false;
-    int v = 0, mi = 0, vb = 0, nnl = 0;
+    int v = 0, mi = 0, vb = 0, nnl = 0, eb = 0, nq = 0;
     const int* nn = nullptr;
+    const int* ne = nullptr;
     RowMask take;
     if (i < n) {
       v = i0 == 0 ? first : C[i];
       const double2 p = mvxy[v];
       double4 mv = mvM[v];
       const MeshCtx c = ctx_of(S, v);
-      const int* ne = ne_row(S, v);
+      ne = ne_row(S, v);
       Row8 er = row8(ne, 0);
       const int nel = S.NElen[v];
       win = local_max(S, v, cmark, tag);
@@ -2826,12 +2852,14 @@ __device__ __forceinline__ void smooth_select_apply_phase(Store S, const int* C,
             if (op[k] != ptag && (f[k] & VF_ALIVE) && !(f[k] & VF_BND)) take.set(b + k);
         }
         smark[v] = tag;
+        if (mv.w == kMoveUnevaluated) nq = nel;
+        eb = c.eb;
         mv.w = 0.0;
         S.xy[v] = p;
         S.M[v] = mv;
         store_vf(S, v, p, mv);
         S.touch[v] = stamp;
-        for (int b = 0;;) {
+        for (int b = 0; nq == 0;) {
           double q[8];
 #pragma unroll
           for (int k = 0; k < 8; ++k) q[k] = b + k < nel ? qball[(size_t)v * S.W + b + k] : 0.0;
@@ -2845,19 +2873,20 @@ __device__ __forceinline__ void smooth_select_apply_phase(Store S, const int* C,
       }
     }
     count_op(S, win, mi);
-    const Room3 at = warp_reserve3(take.count(), nP, lose ? 1 : 0, nDn, 0, nullptr);
+    const Room3 at = warp_reserve3(take.count(), nP, lose ? 1 : 0, nDn, nq, nQ);
     write_row_bits(take, nn, vb, P, at.a);
     if (lose) Dn[at.b] = v;
+    for (int k = 0; k < nq; ++k) Q[at.c + k] = eb + ne[k];
   }
 }
 
 __global__ void k_smooth_select_apply(Store S, const int* C, const int* nCp, const int* cmark,
                                       int* smark, int tag, int* Dn, int* nDn, int* dmark,
                                       const double2* mvxy, const double4* mvM, const double* qball,
-                                      int* P, int* nP, int* pmark, int ptag, int stamp,
-                                      unsigned* done) {
+                                      int* P, int* nP, int* pmark, int ptag, int stamp, int* Q,
+                                      int* nQ, unsigned* done) {
   smooth_select_apply_phase(S, C, nCp, cmark, smark, tag, Dn, nDn, dmark, mvxy, mvM, qball, P, nP,
-                            pmark, ptag, stamp);
+                            pmark, ptag, stamp, Q, nQ);
   round_done(S, done);
 }
 
@@ -3644,10 +3673,11 @@ __global__ void __launch_bounds__(256) k_smooth_rounds(RoundArgs a) {
       if (blockIdx.x == 0 && threadIdx.x == 0) *cand_count(cnt, r + 1) = 0;
     } else {
       smooth_scan_phase(S, list(cur), count(cur), w.mvM, w.C, nC, w.cmark, tag, a.pass0, w.E,
-                        cnt + CN_E, true);
+                        cnt + CN_E, false, true);
       if (!grid_barrier(a.bar, target, a.st)) return;
       if (blockIdx.x == 0 && threadIdx.x == 0) *cand_count(cnt, r + 1) = 0;
-      smooth_filter_phase(S, w.E, cnt + CN_E, w.mvxy, w.mvM, w.Sl, cnt + CN_S, a.work, true);
+      smooth_filter_phase(S, w.E, cnt + CN_E, w.mvxy, w.mvM, w.Sl, cnt + CN_S, w.C, nC, w.cmark,
+                          tag, false, a.work, true);
       if (!grid_barrier(a.bar, target, a.st)) return;
       if (blockIdx.x == 0 && threadIdx.x == 0) cnt[CN_E] = 0;
       smooth_exact_phase(S, w.Sl, cnt + CN_S, w.mvxy, w.mvM, w.gains, w.C, nC, w.cmark, tag,
@@ -3657,7 +3687,7 @@ __global__ void __launch_bounds__(256) k_smooth_rounds(RoundArgs a) {
     }
     smooth_select_apply_phase(S, w.C, nC, w.cmark, w.smark, tag, list(nxt), count(nxt), w.dmark,
                               w.mvxy, w.mvM, w.gains, list(pen), count(pen), w.pmark, ptag, tag + 1,
-                              true);
+                              nullptr, nullptr, true);
     if (!grid_barrier(a.bar, target, a.st)) return;
     const int nc = ld_volatile(nC), nd = ld_volatile(count(nxt)), np = ld_volatile(count(pen));
     advance_rounds(S);
@@ -4329,14 +4359,17 @@ int op_smooth(MeshSet& m, int max_sweeps, int max_rounds) {
     PM_LAUNCH(k_smooth_scan, gv, bs, 0, m.stream, m.S, w.D[cur], w.counts + cn_list(cur),
               w.mvM, w.C, w.counts + CN_C, w.cmark, tag, pass0, w.E, w.counts + CN_E);
     PM_LAUNCH(k_smooth_filter, gv, bs, 0, m.stream, m.S, w.E, w.counts + CN_E, w.mvxy, w.mvM,
-              w.Sl, w.counts + CN_S, prof_work("k_smooth_filter"));
+              w.Sl, w.counts + CN_S, w.C, w.counts + CN_C, w.cmark, tag,
+              prof_work("k_smooth_filter"));
     PM_LAUNCH(k_smooth_eval, grid_tuned(m, (long long)m.S.vused * TW, bs, bps), bs, 0, m.stream,
               m.S, w.Sl, w.counts + CN_S, w.mvxy, w.mvM, w.gains, w.C, w.counts + CN_C, w.cmark,
               tag, prof_work("k_smooth_eval"));
+    zero_counts(m, CN_CL, 1);
     PM_LAUNCH(k_smooth_select_apply, gv, bs, 0, m.stream, m.S, w.C, w.counts + CN_C,
               w.cmark, w.smark, tag, w.D[nxt], w.counts + cn_list(nxt), w.dmark, w.mvxy, w.mvM,
-              w.gains, w.P, w.counts + CN_P, w.pmark, ptag, tag + 1,
+              w.gains, w.P, w.counts + CN_P, w.pmark, ptag, tag + 1, w.clist, w.counts + CN_CL,
               (unsigned*)(w.counts + CN_DONE));
+    PM_LAUNCH(k_refine_quality, gv, bs, 0, m.stream, m.S, w.clist, w.counts + CN_CL, nullptr);
     RoundIO io = read_round(m);
     if (io.err) return io.err;
     if (io.nC > 0) {

@@ -29,6 +29,18 @@ extern "C" void at(const double* p, const double* x, int n, float* m, float* kx,
     up[i] = f_quality_up(o, b, c, sign, kx[i]);
   }
 }
+// both quality bounds of (x, b, c) with the metric at x
+extern "C" void bounds(const double* p, const double* x, int n, float* lo, float* up,
+                       int32_t* sign) {
+  for (int i = 0; i < n; ++i) {
+    const VF a = vf(p + 15 * i), b = vf(p + 15 * i + 5), c = vf(p + 15 * i + 10);
+    VF o = make_vf_xy(x[2 * i], x[2 * i + 1]);
+    const float kx = f_metric_at(o, a, b, c, o);
+    const FQual q = f_quality(o, b, c, sign[i], kx);
+    lo[i] = q.lo;
+    up[i] = q.up;
+  }
+}
 extern "C" void run(const double* p, const double* bound, int n, int32_t* orient, int32_t* len,
                     float* up, int32_t* osign, float* l2, float* el2) {
   for (int i = 0; i < n; ++i) {
@@ -184,3 +196,40 @@ def test_interpolated_metric_and_its_quality_bound(lib, scale, offset, aspect, f
         assert not np.any(has & ~(up.astype(L) >= q))
     if 1e-13 < scale < 1e10 and offset <= 1.0:
         assert np.mean(known[(np.arange(n) >= n // 3) & (o > 0)]) > 0.95
+
+
+@pytest.mark.parametrize("scale,offset,aspect,flat", CASES)
+def test_lower_quality_bound(lib, scale, offset, aspect, flat):
+    """f_quality with an interpolated metric: the lower bound is -1 unless the element is certainly
+    counter-clockwise, lies below the quality and close to it where the upper one is close."""
+    rng = np.random.default_rng(int(abs(np.log10(scale)) * 13 + aspect))
+    n = 40000
+    tri = triangles(rng, n, scale, offset, aspect, flat)
+    w = rng.dirichlet([1.0, 1.0, 1.0], n)
+    with np.errstate(all="ignore"):
+        x = np.ascontiguousarray(np.einsum("ij,ijk->ik", w, tri[:, :, :2]))
+        L = np.longdouble
+        a, b, c = (tri[:, k].astype(L) for k in range(3))
+        X = x.astype(L)
+
+        def det(p, q, r):
+            return ((q[:, 0] - p[:, 0]) * (r[:, 1] - p[:, 1])
+                    - (q[:, 1] - p[:, 1]) * (r[:, 0] - p[:, 0]))
+
+        o = det(a, b, c)
+        l0, l1, l2 = det(X, b, c) / o, det(a, X, c) / o, det(a, b, X) / o
+        m = [l0 * a[:, k] + l1 * b[:, k] + l2 * c[:, k] for k in (2, 3, 4)]
+        lo, up, sign = np.zeros(n, np.float32), np.zeros(n, np.float32), np.zeros(n, np.int32)
+        vp = C.c_void_p
+        lib.bounds(vp(tri.ctypes.data), vp(x.ctypes.data), n, vp(lo.ctypes.data),
+                   vp(up.ctypes.data), vp(sign.ctypes.data))
+        q = quality_exact(np.stack([X[:, 0], X[:, 1], *m], axis=1), b, c)
+        has = lo > -1
+        assert not np.any(has & (sign <= 0)) and not np.any(np.isnan(lo))
+        assert not np.any(has & ~((lo.astype(L) < q) & (det(X, b, c) > 0)))
+        ok = has & (q > 1e-3)
+        width = (up[ok] - q[ok]) / q[ok]
+        assert np.all((q[ok] - lo[ok]) / q[ok] <= 3 * width + 1e-5)
+    if aspect <= 30 and offset <= 1.0 and 1e-13 < scale < 1e10:
+        fat = (np.arange(n) >= n // 3) & (q > 1e-3)
+        assert np.mean(has[fat]) > 0.95
