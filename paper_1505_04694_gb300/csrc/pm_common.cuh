@@ -161,16 +161,6 @@ __device__ __forceinline__ int warp_reserve(int cnt, int* count) {
   return base + incl - cnt;
 }
 
-// Writes vb + row[k] for every set bit k of `bits`, from slot `pos` on.
-__device__ __forceinline__ void write_row_bits(unsigned long long bits, const int* row, int vb,
-                                               int* list, int pos) {
-  while (bits) {
-    int k = __ffsll((long long)bits) - 1;
-    bits &= bits - 1ull;
-    list[pos++] = vb + row[k];
-  }
-}
-
 // A set of entries of one adjacency row (rows hold at most 128 entries): one
 // bit per entry, in two named words so that it stays in registers.
 struct RowMask {
@@ -284,17 +274,6 @@ __device__ __forceinline__ int row_find(const int* row, int len, int val) {
 
 __device__ __forceinline__ bool row_has(const int* row, int len, int val) {
   return row_find(row, len, val) >= 0;
-}
-
-// Position of val in a sorted array a[0..len) (binary search), or -1.
-__device__ __forceinline__ int sorted_pos(const int* a, int len, int val) {
-  int lo = 0, hi = len;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (a[mid] < val) lo = mid + 1;
-    else hi = mid;
-  }
-  return (lo < len && a[lo] == val) ? lo : -1;
 }
 
 // Copies the first len entries of an adjacency row into out (capacity: the

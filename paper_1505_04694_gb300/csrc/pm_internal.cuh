@@ -163,7 +163,6 @@ int refresh_quality(MeshSet& m);
 // The quality cache of every element, computed now when it is stale (a mesh
 // whose metric was never set gets it at its first operator call).
 int ensure_quality(MeshSet& m);
-cudaError_t refresh_sizes(MeshSet& m);
 
 // ---- operators (pm_ops.cu) ----
 // What ops_ahead has done of an iteration: collapse rounds, flip rounds (0: none

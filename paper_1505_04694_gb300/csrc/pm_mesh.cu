@@ -737,21 +737,6 @@ cudaError_t upload_tab(MeshSet& m) {
   return e;
 }
 
-// Read back the per-mesh used-slot counts (nv, ne) into the host mirror.
-cudaError_t refresh_sizes(MeshSet& m) {
-  std::vector<int> t(2 * m.nmesh);
-  cudaError_t e = cudaMemcpyAsync(t.data(), m.S.tab.nv, 2 * m.nmesh * sizeof(int),
-                                  cudaMemcpyDeviceToHost, m.stream);
-  if (e != cudaSuccess) return e;
-  e = cudaStreamSynchronize(m.stream);
-  for (int i = 0; i < m.nmesh; ++i) {
-    m.nv[i] = t[i];
-    m.ne[i] = t[m.nmesh + i];
-  }
-  set_used(m);
-  return e;
-}
-
 static void carve_store(Carver& cv, Store& S) {
   size_t V = S.vslots, E = S.eslots;
   cv.add(&S.xy, V);

@@ -1353,21 +1353,6 @@ __global__ void k_coarsen_commit(Store S, const int* A, const int* nAp, const in
 // scan (the ball's vertices gathered once); larger ones search the elements.
 constexpr int kBallFast = 16;
 
-// Warp-aggregated append of a work item into a list of capacity `cap`.
-__device__ __forceinline__ void append_item(bool pred, int2 val, int2* list, int* count, int cap,
-                                            DevStatus* st) {
-  unsigned m = __ballot_sync(0xffffffffu, pred);
-  if (m == 0) return;
-  int lane = threadIdx.x & 31, leader = __ffs(m) - 1, base = 0;
-  if (lane == leader) base = atomicAdd(count, __popc(m));
-  base = __shfl_sync(0xffffffffu, base, leader);
-  if (pred) {
-    int pos = base + __popc(m & ((1u << lane) - 1u));
-    if (pos < cap) list[pos] = val;
-    else set_err(st, PM_ERR_CAPACITY);
-  }
-}
-
 // A vertex whose ball holds more than kBallFast elements, listed by the whole
 // warp (all lanes call): lane l gathers elements l, l + 32, ... into the
 // warp's shared arrays and then finds the partner elements of its own poor
