@@ -133,6 +133,8 @@ __device__ __forceinline__ void add_work(unsigned long long* work, unsigned ops)
 }
 
 // qK of every listed element slot, one element per thread.
+// 77 FP64 operations on 32 lanes: the FP64 pipe bounds it (83% active); 114 bytes
+// gathered per element are a tenth of the memory's rate beside that.
 __device__ __forceinline__ void elem_quality_phase(const Store& S, const int* list, const int* np,
                                                    unsigned long long* work, bool il = false) {
   // in the persistent rounds from the last warp of every block backwards: the
@@ -668,6 +670,9 @@ __device__ __forceinline__ int first_by_length(const Store& S, int v, int vb, co
 // are candidates is a length against L_low, and which of them comes first is
 // mostly plain from the FP32 lengths too.  A length that is certainly above
 // another's stays above it after rounding, so the order is the exact one.
+// Dependent gathers bound it (DRAM 21-27%, FP64 pipe below 10%; with exact lengths
+// it was 80%): 36 ms of a 512-mesh batch's collapses, 12.1 with the FP32 lengths, 11.3
+// held to 80 registers (24 warps an SM instead of 16; at 64 it spills: 12.3).
 __device__ __forceinline__ void coarsen_scan_phase(Store S, const int* D, const int* nDp,
                                                    int* target, int* cand, int* C, int* nC,
                                                    int* cmark, int tag, int pass0, int* W0,
@@ -798,6 +803,7 @@ __device__ __forceinline__ void check_len_chunk(const Store& S, const CheckQueue
 // The integer part and the FP32 filters for collapsing x.v onto u: false when
 // it is certainly invalid; else the tests left open, as bits over the ball's
 // elements and v's neighbours.
+// All its loads run in chunks whose addresses do not wait on one another.
 __device__ __forceinline__ bool check_filter(const Store& S, const CoarsenCtx& x, int u,
                                              RowMask& oo, RowMask& ol) {
   const int ws = x.c.vb + u;
@@ -920,7 +926,9 @@ __device__ __forceinline__ bool check_candidates(const Store& S, const CheckQueu
   return ok;
 }
 
-// Pass 2: every listed vertex's first candidate.
+// Pass 2: every listed vertex's first candidate.  Gathers bound it (L1 50-60%, DRAM
+// 31-48%, FP64 pipe below 1%); with every test in FP64 the two check passes took 47
+// ms of a 512-mesh batch, 26.4 with the filters, 20.7 with pass 3 as it is.
 __device__ __forceinline__ void coarsen_check_phase(Store S, const int* Win, const int* nWin,
                                                     int* Wout, int* nWout, int* target, int* cand,
                                                     int* C, int* nC, int* cmark, int tag,
@@ -1215,6 +1223,10 @@ __global__ void k_coarsen_select_apply(Store S, const int* C, const int* nCp, co
 // The commit below for rows of at most 16 entries that stay so: both rows in
 // registers, edited in place (a row of dependent local-memory accesses per
 // edit otherwise).  False, with nothing written, when a row grows past 16.
+// A commit waits for its gathers (long-scoreboard stalls, DRAM 20-30%); with the rows
+// in registers, one reservation for all lists and the qualities on the idle warps, a
+// 317 x 317 grid coarsens in 11.9 instead of 13.7 ms, 16 small meshes adapt in 17.9
+// instead of 20.6.
 __device__ __forceinline__ bool coarsen_commit_short(const Store& S, int u, MeshCtx c, int lu,
                                                      const int* target, const int* smark,
                                                      int tag) {
@@ -1671,6 +1683,10 @@ __device__ __forceinline__ void flip_run(const Store& S, FlipQueue& Q, int cnt, 
   __syncwarp();
 }
 
+// Pass 2: the gains, by stages, full warps of items in each.  FP64 in full bound it
+// (57 ms of a 512-mesh batch); the FP32 bounds end most items, and the exact rest
+// runs at 64 registers, four blocks of 256 an SM (16.5 ms at three, 14.5 at four,
+// 17.9 at five, which spill).
 __device__ __forceinline__ void swap_edge_phase(Store S, const int2* items, const int* nIp,
                                                 int icap, double* gains, int tag,
                                                 unsigned long long* work, bool il = false) {
@@ -1835,8 +1851,8 @@ __global__ void k_swap_pick(Store S, const int* E, const int* nEp, const double*
   swap_pick_phase(S, E, nEp, gains, opA, opK2, C, nC, cmark, tag);
 }
 
-// Passes 1-3 in one, for persistent rounds whose list fits one pass of the
-// grid's tiles: lane j of v's tile takes v's ball elements j, j + 8, ... as
+// Passes 1-3 in one, for persistent rounds whose list fits kFusePasses passes of
+// the grid's tiles: lane j of v's tile takes v's ball elements j, j + 8, ... as
 // K1 of the edge (v, w) that follows v in it, finds the element K2 = (v, d, w)
 // that follows K1 around v among the tile's elements (shuffles), lists the edge
 // by pass 1's rule (interior, one of the pair below q_thresh), filters it and,
@@ -1846,7 +1862,9 @@ __global__ void k_swap_pick(Store S, const int* E, const int* nEp, const double*
 // the K1 edge of exactly one ball element, so the candidate edges are those
 // pass 1 lists.  An edge between two listed vertices is evaluated from both
 // ends; in exchange a round takes two barriers fewer and no trip of items and
-// gains through memory.
+// gains through memory.  A short round is a chain of latencies (about 5 us of this
+// phase's 10 are two dependent gathers and the first FP64 stage): 15.8 -> 15.0 ms on
+// the 201 x 201 mesh, 17.9 -> 16.4 on 16 small ones against five phases.
 __device__ __forceinline__ bool flip_better(bool f2, double g2, int w2, bool f, double g, int w) {
   return f2 && (!f || dgt(g2, g) || (dbits(g2) == dbits(g) && w2 < w));
 }
@@ -2490,6 +2508,9 @@ __device__ bool tile_smooth_eval(const Tile& t, const Store& S, int v, MeshCtx c
 // that certainly hold become candidates at once: their new qualities are evaluated
 // when the move is made (half the candidates lose to a neighbour, and most of those
 // are evaluated again after it has moved).  The others are listed for pass 3.
+// The sums' and the solve's FP64 bounds it (pipe 76% active; the FP32 bounds run
+// beside them).  Steps on 20M triangles, whole adaptation: a tile of lanes for all
+// 171 ms, a thread per vertex and the filter 152, two passes 105, `defer` 87.9 -> 83.8.
 __device__ __forceinline__ void smooth_filter_phase(Store S, const int* E, const int* nEp,
                                                     double2* mvxy, double4* mvM, int* R, int* nR,
                                                     int* C, int* nC, int* cmark, int tag,
@@ -2629,8 +2650,8 @@ __device__ __forceinline__ void smooth_exact_phase(Store S, const int* R, const 
   add_work(work, ops);
 }
 
-// Passes 1 and 2 in one (persistent rounds whose list fits one tile per
-// listed vertex): an evaluation whose inputs carry no newer stamp stands, the
+// Passes 1 to 3 in one (persistent rounds whose list fits kFusePasses passes of the
+// grid's tiles): an evaluation whose inputs carry no newer stamp stands, the
 // others are made again.  The tile takes the stamp decision from lane 0, after every
 // lane has read the stamp (the shuffle) and before lane 0 overwrites it.
 __device__ __forceinline__ void smooth_scan_eval_phase(Store S, const int* D, const int* nDp,
@@ -2688,7 +2709,8 @@ __device__ __forceinline__ void smooth_scan_eval_phase(Store S, const int* D, co
 // side by side in a warp (a tile of 8 lanes per move leaves a quarter of them idle
 // at six elements a ball, and the FP64 pipe is what bounds this pass).  Each warp
 // walks a range of the list and takes as many moves at a time as fit 32 lanes; a
-// ball of more than 32 elements takes the warp alone.
+// ball of more than 32 elements takes the warp alone.  FP64 pipe 84% active; with the
+// ordered sums of the tile form 94.8 -> 91.4 ms on 20M triangles.
 __device__ __forceinline__ void smooth_exact_packed(Store S, const int* R, const int* nRp,
                                                     const double2* mvxy, double4* mvM,
                                                     double* qball, int* C, int* nC, int* cmark,
@@ -2787,7 +2809,9 @@ __global__ void __launch_bounds__(256, 3) k_smooth_eval(Store S, const int* R, c
 // One round's independent set and its moves (see k_coarsen_select_apply); live
 // interior neighbours of a moved vertex become pending for the next sweep (stamp
 // pmark with the sweep tag).  What the move needs is loaded beside the
-// independent set's gathers, and the round's two lists share a reservation.
+// independent set's gathers, and the round's lists share a reservation.  The elements
+// of a move whose qualities were left open join list Q.  Gathers bound it
+// (long-scoreboard stalls, DRAM 38%).
 __device__ __forceinline__ void smooth_select_apply_phase(Store S, const int* C, const int* nCp,
                                                           const int* cmark, int* smark, int tag,
                                                           int* Dn, int* nDn, int* dmark,
@@ -2997,6 +3021,10 @@ __device__ bool tile_opt_eval(const Tile& t, const Store& S, int v, MeshCtx c, d
 
 // Evaluate and apply in one pass (one tile per member of S): members are
 // pairwise non-adjacent, so no member reads a vertex another member moves.
+// FP64 bounds it (pipe 80% active).  20 rounds on 131k vertices: 11.9 ms with every
+// trial step evaluated in full, 6.0 with the FP32 metric and quality bounds in front
+// and the gradient of the moved vertex alone, 5.4 with the ordered sums spread over
+// the tile's lanes.
 __global__ void k_opt_apply(Store S, const int* Sl, const int* nSp, double* qball, int stamp) {
   advance_rounds(S);
   const int n = *nSp;
@@ -3049,6 +3077,8 @@ __global__ void k_stamp_list(Store S, const int* L, const int* nLp, int* cmark, 
 // inside one call vertices keep their positions and metrics until the
 // operator loop ends (smoothing runs after it), so a's own stamp tells
 // whether anything the mask read has changed: every change of a's row stamps a.
+// A sweep over every slot that waits for its gathers: 48 registers, 40 warps an SM
+// (9.7 -> 9.5 ms over the 29 launches of a 512-mesh batch; 80 registers 11.7).
 __global__ void __launch_bounds__(256, 5) k_refine_mark(Store S, int* cnt, RowMask* mask, int tag, int pass0, int lo,
                               const int* before, const int* before2, const DevStatus* st) {
   if (!may_go(before, st)) return;
@@ -3254,6 +3284,8 @@ __device__ __forceinline__ int refine_children(const Store& S, int mi, int eb, c
 // `src`: NE = the children of those elements that contain the vertex, NN = the
 // other vertices of those, both sorted.  Rows of up to 16 entries are made in
 // registers; false, with nothing written, when one is longer.
+// (They were built in a second buffer through local memory: a tenth of the adaptation
+// of 20M triangles, 104.8 -> 99.6 ms, with the estimate of pm_mesh.cu in FP32.)
 __device__ __forceinline__ bool refine_row_short(const Store& S, int s, int src, int mi, int vb,
                                                  int eb, const int* escan, int stamp) {
   const int lu = s - vb;
@@ -3298,7 +3330,8 @@ __device__ __forceinline__ bool refine_row_short(const Store& S, int s, int src,
 // (stamped), in place, in two launches: the new vertices first (`fresh`), which
 // read the old element row of their split edge's first end (the children that
 // contain the new vertex are exactly those of the two parents on that edge), then
-// the old ones, which read and write their own rows alone.
+// the old ones, which read and write their own rows alone.  64 registers: 7.8 -> 6.5
+// ms over the 28 launches of a 512-mesh batch (latency, not the 12 spilled bytes).
 __global__ void __launch_bounds__(256, 4) k_refine_rows(Store S, int vfirst, int vend, int fresh, const int* escan,
                               const int4* owner, int stamp, DevStatus* st) {
   for (int s = vfirst + blockIdx.x * blockDim.x + threadIdx.x; s < vend;
@@ -3488,7 +3521,7 @@ __device__ __forceinline__ void finish_rounds(const RoundArgs& a, int r, int cur
 }
 
 // Rounds of collapses: [evaluate] B1 [select + apply] B2 [commit] B3; rounds
-// of flips whose list fits one pass of the grid's tiles: [scan + gains +
+// of flips whose list fits kFusePasses passes of the grid's tiles: [scan + gains +
 // pick] B1 [select + apply] B2 [commit] B3; longer flip lists: [scan] B1
 // [gains] [pick] [select + apply] [commit], five barriers.  Block 0 clears,
 // before B1 of round r: A and the list round r
@@ -3583,7 +3616,8 @@ __global__ void __launch_bounds__(256) k_swap_rounds(RoundArgs a) { topo_rounds<
 // Colouring rounds of a list of at most `limit` vertices: [propose] B1 [resolve]
 // B2, until no vertex is uncoloured.  (A colouring takes about 15 rounds, each of
 // which was two launches and a wait.)  Block 0 clears the list a round fills
-// before B1 (last read before the last round's B2).
+// before B1 (last read before the last round's B2).  A 129 x 129 mesh adapted by
+// colour classes: 16.2 -> 13.3 ms, with the smoothing's longer lists in two passes.
 __global__ void __launch_bounds__(256) k_colour_rounds(RoundArgs a) {
   const Work& w = a.w;
   int* cnt = w.counts;
@@ -3605,14 +3639,14 @@ __global__ void __launch_bounds__(256) k_colour_rounds(RoundArgs a) {
   finish_rounds(a, r, cur, n == 0);
 }
 
-// Sweeps of smoothing rounds.  A round whose list fits one pass of the grid's
+// Sweeps of smoothing rounds.  A round whose list fits kFusePasses passes of the grid's
 // tiles: [scan + evaluate] B1 [select + apply] B2; a longer one: [scan] B1
 // [filter] B1' [exact] B1'' [select + apply] B2 (its threads then go to the
 // vertices that need an evaluation, its tiles to the moves that may succeed).  A
 // sweep ends with a round that finds no candidate;
 // its pending list then becomes the current one and the next sweep starts in
 // the same launch (ten sweeps used to be ten launches and read-backs, most of
-// them for a handful of vertices).  The three lists trade places by index, each
+// them for a handful of vertices: 1.86 -> 1.48 ms on a 41 x 41 mesh).  The three lists trade places by index, each
 // with its own counter.  Block 0 clears, before B1 of round r: the list round
 // r fills and, in a sweep's first round, its pending list (both last read by a
 // scan and a decision before the last barrier); after B1: the candidate slot of
