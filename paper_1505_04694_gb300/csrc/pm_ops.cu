@@ -670,8 +670,8 @@ __device__ __forceinline__ int first_by_length(const Store& S, int v, int vb, co
 // are candidates is a length against L_low, and which of them comes first is
 // mostly plain from the FP32 lengths too.  A length that is certainly above
 // another's stays above it after rounding, so the order is the exact one.
-// Dependent gathers bound it (DRAM 21-27%, FP64 pipe below 10%; with exact lengths
-// it was 80%): 36 ms of a 512-mesh batch's collapses, 12.1 with the FP32 lengths, 11.3
+// Dependent gathers bound it (DRAM 21-27%, FP64 pipe below 10%, on regular grids whose
+// equal lengths are compared exactly 39-63%; with all lengths exact it was 80%): 36 ms of a 512-mesh batch's collapses, 12.1 with the FP32 lengths, 11.3
 // held to 80 registers (24 warps an SM instead of 16; at 64 it spills: 12.3).
 __device__ __forceinline__ void coarsen_scan_phase(Store S, const int* D, const int* nDp,
                                                    int* target, int* cand, int* C, int* nC,
@@ -926,8 +926,8 @@ __device__ __forceinline__ bool check_candidates(const Store& S, const CheckQueu
   return ok;
 }
 
-// Pass 2: every listed vertex's first candidate.  Gathers bound it (L1 50-60%, DRAM
-// 31-48%, FP64 pipe below 1%); with every test in FP64 the two check passes took 47
+// Pass 2: every listed vertex's first candidate.  Gathers bound it (L1 50-65%, DRAM
+// 31-48%, FP64 pipe below 1%, on regular grids 33%); with every test in FP64 the two check passes took 47
 // ms of a 512-mesh batch, 26.4 with the filters, 20.7 with pass 3 as it is.
 __device__ __forceinline__ void coarsen_check_phase(Store S, const int* Win, const int* nWin,
                                                     int* Wout, int* nWout, int* target, int* cand,
