@@ -5,9 +5,10 @@
 // no (a quality not above a bound, an edge longer than L_up, a point on one
 // side of a line), most of which single precision with a rigorous error bound
 // can give (a batch of 512 meshes: 445 -> 414 ms with the flip gains', 377 with the
-// collapses', 323 with the smoothing's filters).  Every filter returns "undecided" unless its answer is certain
-// for the value the FP64 code computes; the caller then runs that code.  So
-// no result changes, only the number of FP64 instructions behind it.
+// collapses', 323 with the smoothing's filters).  Every filter returns "undecided"
+// unless its answer is certain for the value the FP64 code computes; the caller then
+// runs that code.  So no result changes, only the number of FP64 instructions behind
+// it.
 //
 // Input: one 32-byte record per vertex (one DRAM sector; position and metric
 // in double take 48 bytes in two sectors): each coordinate as two floats
@@ -148,11 +149,11 @@ PM_HD int f_len_cmp(const FLen& l, float lo2, float hi2) {
 // Bounds of the quality (12 sqrt 3 A / P^2) F(P / 3) of element (a, b, c) in its
 // mean metric: `up` is NaN and `lo` -1 when they would be loose, and `lo` is -1
 // unless the element is certainly counter-clockwise.  The quality grows with the
-// area and the metric's determinant, which are taken at their bounds; as a function of P it is h(P) = F(P / 3) / P^2 with
-// |d ln h / d ln P| <= 5 (between -2 and 1 below the ideal perimeter, between
-// -5 and -2 above), so a relative error rP of P changes it by at most 5 rP to
-// first order (rP <= 0.04 is required, the rest of the series is inside the
-// factor 1.15).  `sign` receives the orientation's sign, 0 when undecided.  `kx`
+// area and the metric's determinant, which are taken at their bounds; as a function of
+// P it is h(P) = F(P / 3) / P^2 with |d ln h / d ln P| <= 5 (between -2 and 1 below the
+// ideal perimeter, between -5 and -2 above), so a relative error rP of P changes it by
+// at most 5 rP to first order (rP <= 0.04 is required, the rest of the series is inside
+// the factor 1.15).  `sign` receives the orientation's sign, 0 when undecided.  `kx`
 // bounds the relative error of one vertex's metric beyond its rounding (see
 // f_metric_at): it adds to that of the mean, and four times to the determinant's.
 struct FQual {

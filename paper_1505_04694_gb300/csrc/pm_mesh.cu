@@ -102,8 +102,8 @@ struct Carver {
 // Everything whose size follows the row width W, in one allocation of its own
 // (a change of W replaces it and leaves no hole in the store): the rows of both
 // buffer sets and the collapse candidates.  The spare set's rows are written
-// only by a compaction, which reads no flip gain or moved ball quality, so those W doubles per vertex
-// (Work::gains) share them.
+// only by a compaction, which reads no flip gain or moved ball quality, so those W
+// doubles per vertex (Work::gains) share them.
 cudaError_t rows_alloc(MeshSet& m, int W) {
   const size_t n = (size_t)m.S.vslots * W;
   char* base = nullptr;

@@ -671,8 +671,9 @@ __device__ __forceinline__ int first_by_length(const Store& S, int v, int vb, co
 // mostly plain from the FP32 lengths too.  A length that is certainly above
 // another's stays above it after rounding, so the order is the exact one.
 // Dependent gathers bound it (DRAM 21-27%, FP64 pipe below 10%, on regular grids whose
-// equal lengths are compared exactly 39-63%; with all lengths exact it was 80%): 36 ms of a 512-mesh batch's collapses, 12.1 with the FP32 lengths, 11.3
-// held to 80 registers (24 warps an SM instead of 16; at 64 it spills: 12.3).
+// equal lengths are compared exactly 39-63%; with all lengths exact it was 80%): 36
+// ms of a 512-mesh batch's collapses, 12.1 with the FP32 lengths, 11.3 held to 80
+// registers (24 warps an SM instead of 16; at 64 it spills: 12.3).
 __device__ __forceinline__ void coarsen_scan_phase(Store S, const int* D, const int* nDp,
                                                    int* target, int* cand, int* C, int* nC,
                                                    int* cmark, int tag, int pass0, int* W0,
@@ -927,8 +928,9 @@ __device__ __forceinline__ bool check_candidates(const Store& S, const CheckQueu
 }
 
 // Pass 2: every listed vertex's first candidate.  Gathers bound it (L1 50-65%, DRAM
-// 31-48%, FP64 pipe below 1%, on regular grids 33%); with every test in FP64 the two check passes took 47
-// ms of a 512-mesh batch, 26.4 with the filters, 20.7 with pass 3 as it is.
+// 31-48%, FP64 pipe below 1%, on regular grids 33%); with every test in FP64 the
+// two check passes took 47 ms of a 512-mesh batch, 26.4 with the filters, 20.7 with
+// pass 3 as it is.
 __device__ __forceinline__ void coarsen_check_phase(Store S, const int* Win, const int* nWin,
                                                     int* Wout, int* nWout, int* target, int* cand,
                                                     int* C, int* nC, int* cmark, int tag,
@@ -1733,8 +1735,9 @@ __device__ __forceinline__ void swap_edge_phase(Store S, const int2* items, cons
   add_work(work, ops);
 }
 
-__global__ void __launch_bounds__(256, 4) k_swap_edge(Store S, const int2* items, const int* nIp, int icap, double* gains,
-                            int tag, unsigned long long* work) {
+__global__ void __launch_bounds__(256, 4)
+k_swap_edge(Store S, const int2* items, const int* nIp, int icap, double* gains, int tag,
+            unsigned long long* work) {
   swap_edge_phase(S, items, nIp, icap, gains, tag, work);
 }
 
@@ -2270,8 +2273,9 @@ __device__ __forceinline__ void smooth_scan_phase(Store S, const int* D, const i
   }
 }
 
-__global__ void __launch_bounds__(256, 3) k_smooth_scan(Store S, const int* D, const int* nDp, double4* mvM, int* C, int* nC,
-                              int* cmark, int tag, int pass0, int* E, int* nE) {
+__global__ void __launch_bounds__(256, 3)
+k_smooth_scan(Store S, const int* D, const int* nDp, double4* mvM, int* C, int* nC, int* cmark,
+              int tag, int pass0, int* E, int* nE) {
   smooth_scan_phase(S, D, nDp, mvM, C, nC, cmark, tag, pass0, E, nE, true);
 }
 
@@ -2800,9 +2804,9 @@ __global__ void k_smooth_filter(Store S, const int* E, const int* nEp, double2* 
   smooth_filter_phase(S, E, nEp, mvxy, mvM, R, nR, C, nC, cmark, tag, true, work);
 }
 
-__global__ void __launch_bounds__(256, 3) k_smooth_eval(Store S, const int* R, const int* nRp, const double2* mvxy,
-                              double4* mvM, double* qball, int* C, int* nC, int* cmark, int tag,
-                              unsigned long long* work) {
+__global__ void __launch_bounds__(256, 3)
+k_smooth_eval(Store S, const int* R, const int* nRp, const double2* mvxy, double4* mvM,
+              double* qball, int* C, int* nC, int* cmark, int tag, unsigned long long* work) {
   smooth_exact_packed(S, R, nRp, mvxy, mvM, qball, C, nC, cmark, tag, work);
 }
 
@@ -3079,8 +3083,9 @@ __global__ void k_stamp_list(Store S, const int* L, const int* nLp, int* cmark, 
 // whether anything the mask read has changed: every change of a's row stamps a.
 // A sweep over every slot that waits for its gathers: 48 registers, 40 warps an SM
 // (9.7 -> 9.5 ms over the 29 launches of a 512-mesh batch; 80 registers 11.7).
-__global__ void __launch_bounds__(256, 5) k_refine_mark(Store S, int* cnt, RowMask* mask, int tag, int pass0, int lo,
-                              const int* before, const int* before2, const DevStatus* st) {
+__global__ void __launch_bounds__(256, 5)
+k_refine_mark(Store S, int* cnt, RowMask* mask, int tag, int pass0, int lo, const int* before,
+              const int* before2, const DevStatus* st) {
   if (!may_go(before, st)) return;
   tag += tags_of(before) + tags_of(before2);
   pass0 += tags_of(before) + tags_of(before2);
@@ -3332,8 +3337,9 @@ __device__ __forceinline__ bool refine_row_short(const Store& S, int s, int src,
 // contain the new vertex are exactly those of the two parents on that edge), then
 // the old ones, which read and write their own rows alone.  64 registers: 7.8 -> 6.5
 // ms over the 28 launches of a 512-mesh batch (latency, not the 12 spilled bytes).
-__global__ void __launch_bounds__(256, 4) k_refine_rows(Store S, int vfirst, int vend, int fresh, const int* escan,
-                              const int4* owner, int stamp, DevStatus* st) {
+__global__ void __launch_bounds__(256, 4)
+k_refine_rows(Store S, int vfirst, int vend, int fresh, const int* escan, const int4* owner,
+              int stamp, DevStatus* st) {
   for (int s = vfirst + blockIdx.x * blockDim.x + threadIdx.x; s < vend;
        s += gridDim.x * blockDim.x) {
     if (S.touch[s] != stamp) continue;
@@ -3646,16 +3652,16 @@ __global__ void __launch_bounds__(256) k_colour_rounds(RoundArgs a) {
 // sweep ends with a round that finds no candidate;
 // its pending list then becomes the current one and the next sweep starts in
 // the same launch (ten sweeps used to be ten launches and read-backs, most of
-// them for a handful of vertices: 1.86 -> 1.48 ms on a 41 x 41 mesh).  The three lists trade places by index, each
-// with its own counter.  Block 0 clears, before B1 of round r: the list round
-// r fills and, in a sweep's first round, its pending list (both last read by a
-// scan and a decision before the last barrier); after B1: the candidate slot of
-// round r + 1 (last read after B2 of round r - 1); after B1': E (read by the
-// filter before B1'); after B1'': the filtered list.  The round counters advance after B2 from the flag
-// set of the round's parity, so that round r + 1's evaluation can set the other
-// set meanwhile.  The launch returns when the sweeps are over, after
-// `max_rounds` rounds with candidates, or when the next list outgrows `limit`;
-// the lists' counts are then put where the host expects them.
+// them for a handful of vertices: 1.86 -> 1.48 ms on a 41 x 41 mesh).  The three
+// lists trade places by index, each with its own counter.  Block 0 clears, before B1 of
+// round r: the list round r fills and, in a sweep's first round, its pending list (both
+// last read by a scan and a decision before the last barrier); after B1: the candidate
+// slot of round r + 1 (last read after B2 of round r - 1); after B1': E (read by the
+// filter before B1'); after B1'': the filtered list.  The round counters advance after
+// B2 from the flag set of the round's parity, so that round r + 1's evaluation can set
+// the other set meanwhile.  The launch returns when the sweeps are over, after
+// `max_rounds` rounds with candidates, or when the next list outgrows `limit`; the
+// lists' counts are then put where the host expects them.
 __global__ void __launch_bounds__(256) k_smooth_rounds(RoundArgs a) {
   const Work& w = a.w;
   int* cnt = w.counts;
@@ -4045,10 +4051,11 @@ int op_coarsen(MeshSet& m, int max_rounds, const Ahead& h) {
   int pass0 = m.tag;
   const bool persist = rounds_grid(m, 0) > 0;
   bool bar_clear = h.coarsen == 0;
-  if (h.coarsen == 0) zero_counts(m, 0, CN_NUM);
-  if (h.coarsen == 0)
+  if (h.coarsen == 0) {
+    zero_counts(m, 0, CN_NUM);
     PM_LAUNCH(k_init_list, gv, bs, 0, m.stream, m.S, 0, w.D[0], w.counts + CN_D0, m.S.evc,
-            m.lo_coarsen, (const int*)nullptr, (const DevStatus*)m.st);
+              m.lo_coarsen, (const int*)nullptr, (const DevStatus*)m.st);
+  }
   // entries of the list the next round reads; unknown (0) at first: the
   // persistent launch itself hands a long first list back
   int nlist = 0;
@@ -4129,10 +4136,11 @@ int op_swap(MeshSet& m, int max_rounds, const Ahead& h) {
   const int icap = m.S.vslots * 6 + 64;
   const bool persist = rounds_grid(m, 1) > 0;
   bool bar_clear = h.swap == 0;
-  if (h.swap == 0) zero_counts(m, 0, CN_NUM);
-  if (h.swap == 0)
+  if (h.swap == 0) {
+    zero_counts(m, 0, CN_NUM);
     PM_LAUNCH(k_init_list, gv, bs, 0, m.stream, m.S, 0, w.D[0], w.counts + CN_D0, m.S.evs,
-            m.lo_swap, (const int*)nullptr, (const DevStatus*)m.st);
+              m.lo_swap, (const int*)nullptr, (const DevStatus*)m.st);
+  }
   int nlist = 0;  // unknown at first (see op_coarsen)
   int cur = 0;
   bool complete = false;
@@ -4228,10 +4236,10 @@ int op_refine(MeshSet& m, int max_rounds, const Ahead& h, bool* renumber_queued)
     const int gv = grid_tuned(m, m.S.vused, bs, bps);
     const int tag = marked ? marked : (m.tag += 2);
     if (m.lo_refine > pass0) pass0 = m.lo_refine;  // storage was regrown
-    if (!marked) PM_LAUNCH(k_refine_mark, gv, bs, 0, m.stream, m.S, w.vcnt, w.vmask, tag, pass0,
-              m.lo_refine, (const int*)nullptr, (const int*)nullptr, (const DevStatus*)m.st);
     const bool ahead = renumber_queued && split;
     if (!marked) {
+      PM_LAUNCH(k_refine_mark, gv, bs, 0, m.stream, m.S, w.vcnt, w.vmask, tag, pass0, m.lo_refine,
+                (const int*)nullptr, (const int*)nullptr, (const DevStatus*)m.st);
       scan_exclusive(w.vcnt, w.vscan, m.S.vused, m.scan, m.st, m.stream);
       PM_LAUNCH(k_refine_newcount, (n + 127) / 128, 128, 0, m.stream, m.S, (const int*)w.vscan,
                 w.counts);
