@@ -1315,7 +1315,13 @@ int presize(MeshSet& m) {
   // start with 32 (20M slots: 100.2 -> 95.1 ms, 42M slots: 260 -> 255 ms; at 3M
   // slots, where the rebuild is cheap, rows of 16 are faster, 10.93 against 11.09).
   constexpr long long kWideRowsFrom = 1LL << 23;
-  e = grow(m, vcap, ecap, vt >= kWideRowsFrom ? std::max(m.S.W, 32) : m.S.W);
+  const int W = vt >= kWideRowsFrom ? std::max(m.S.W, 32) : m.S.W;
+  e = grow(m, vcap, ecap, W);
+  if (e == cudaErrorMemoryAllocation && W > m.S.W) {
+    // no room for the wider rows (320 bytes a vertex more): as they are
+    cudaGetLastError();
+    e = grow(m, vcap, ecap, m.S.W);
+  }
   if (e) {
     set_last_error(std::string("growing mesh storage: ") + cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? PM_ERR_OOM : PM_ERR_CUDA;

@@ -1,0 +1,31 @@
+"""Storage where device memory is short: what fits without an optional extra is not refused."""
+import numpy as np
+import pytest
+
+from mempool import MemPool
+from paper_1505_04694_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+pm = pytest.importorskip("paper_1505_04694_gb300.pm")
+
+
+def make_room(limit=0):
+    """A mesh given room for 6M elements (over 2^23 vertex slots); the most bytes in use."""
+    xy, tri = inputs.grid_mesh(65)
+    d = 6.0e6 * np.sqrt(3.0) / 4.0  # sqrt(det): 6M unit triangles on the unit square
+    with MemPool(limit) as pool:
+        with pm.Mesh.from_host(xy, tri, device=0) as g:
+            g.set_metric(np.tile([d, 0.0, d], (xy.shape[0], 1)))
+            g.adapt(pm.Params(seed=1, max_iter=0, max_smooth_sweeps=0))
+            out = g.get_mesh()
+        high = pool.high()
+    return high, out
+
+
+def test_wide_rows_are_given_up_when_memory_is_short():
+    """From 2^23 vertex slots on rows are made 32 entries wide, 320 bytes a slot more than needed: with
+    half of that missing the rows stay as they are."""
+    high, (xy, tri, _) = make_room()
+    _, (xy1, tri1, _) = make_room(high - 160 * 2 ** 23)
+    assert np.array_equal(xy1, xy) and np.array_equal(tri1, tri)
