@@ -144,6 +144,7 @@ void set_used(MeshSet& m);
 cudaError_t grow(MeshSet& m, const std::vector<int>& vcap, const std::vector<int>& ecap, int W);
 int rebuild_adjacency(MeshSet& m, bool derive_flags, bool corners_given);
 int presize(MeshSet& m);
+int spare_slots(long long need, int most, int nmesh);
 // The part of a renumbering inside the outer loop that runs before its
 // read-back (sync_call); `renumber` does it unless it has been queued.
 // The scan of the live vertices goes to `vscan` (vslots + 1), which has to be

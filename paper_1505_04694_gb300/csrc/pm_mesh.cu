@@ -1275,13 +1275,20 @@ int compact_out_set(MeshSet& m, double* xy, int32_t* tri, double* mt, int* nv_ou
   return PM_OK;
 }
 
+// Slots beyond the `need` of a mesh in a growth: `most`, but in a set of more than
+// 512 meshes as many as it needs or its share of 512 times `most` if that is less (a
+// set of 50,000 tiny meshes would take 200 GB for 4096 vertices each).
+int spare_slots(long long need, int most, int nmesh) {
+  return (int)std::min<long long>(most, std::max<long long>(need, 512LL * most / nmesh));
+}
+
 // Capacity for the adaptation ahead, in one growth: while adapting, a mesh
 // holds at most about 2.2 times the larger of its element count and the
 // element count its metric asks for (refinement overshoots before the
 // collapses that follow), so every mesh below 2.5 times the estimate grows
 // now, together, instead of round after round of refinement (and some
-// thousands more: the estimate knows nothing of the boundary, which dominates
-// a coarse mesh of long elements).
+// thousands more, see spare_slots: the estimate knows nothing of the boundary,
+// which dominates a coarse mesh of long elements).
 int presize(MeshSet& m) {
   const int n = m.nmesh;
   double* est = m.w.gains;  // scratch: no evaluation is kept across calls
@@ -1302,8 +1309,9 @@ int presize(MeshSet& m) {
     const double ne_est = 4.0 / std::sqrt(3.0) * h[i];
     const double want_e = 2.5 * std::max(ne_est, (double)m.ne[i]);
     if (std::isfinite(want_e) && want_e > ecap[i] && want_e < (double)(1 << 29)) {
-      ecap[i] = (int)want_e + 8192;
-      vcap[i] = std::max(vcap[i], (int)(0.6 * want_e) + 4096);
+      ecap[i] = (int)want_e + spare_slots((long long)want_e, 8192, n);
+      vcap[i] = std::max(vcap[i], (int)(0.6 * want_e) +
+                                      spare_slots((long long)(0.6 * want_e), 4096, n));
       need = true;
     }
     vt += vcap[i];

@@ -4256,8 +4256,8 @@ int op_refine(MeshSet& m, int max_rounds, const Ahead& h, bool* renumber_queued)
     }
     // A growth moves every mesh of the set, so when one mesh needs room, every
     // mesh that this round leaves with little gets half as much again as it
-    // needs now, and some thousands at least (the next rounds of a refinement pass
-    // usually split again).
+    // needs now, and some thousands at least (spare_slots; the next rounds of a
+    // refinement pass usually split again).
     long long total = 0;
     bool need_grow = false;
     for (int i = 0; i < n; ++i) {
@@ -4280,10 +4280,11 @@ int op_refine(MeshSet& m, int max_rounds, const Ahead& h, bool* renumber_queued)
         const long long vneed = (long long)m.nv[i] + newv[i] + 64;
         const long long eneed = (long long)m.ne[i] + 2LL * newv[i] + 64;
         if (vneed + vneed / 8 > m.vcap[i])
-          vcap[i] = (int)std::min<long long>(std::max(vneed + vneed / 2, vneed + 8192), (1LL << 30));
+          vcap[i] = (int)std::min<long long>(
+              vneed + std::max<long long>(vneed / 2, spare_slots(vneed, 8192, n)), 1LL << 30);
         if (eneed + eneed / 8 > m.ecap[i])
-          ecap[i] =
-              (int)std::min<long long>(std::max(eneed + eneed / 2, eneed + 16384), (1LL << 30));
+          ecap[i] = (int)std::min<long long>(
+              eneed + std::max<long long>(eneed / 2, spare_slots(eneed, 16384, n)), 1LL << 30);
       }
       cudaError_t e = grow(m, vcap, ecap, m.S.W);
       if (e != cudaSuccess) {

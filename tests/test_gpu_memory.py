@@ -29,3 +29,21 @@ def test_wide_rows_are_given_up_when_memory_is_short():
     high, (xy, tri, _) = make_room()
     _, (xy1, tri1, _) = make_room(high - 160 * 2 ** 23)
     assert np.array_equal(xy1, xy) and np.array_equal(tri1, tri)
+
+
+def adapt_tiny(n):
+    """n meshes of 8 triangles, each refined to about a hundred; the most bytes in use."""
+    xy, tri = inputs.grid_mesh(3)
+    with MemPool() as pool:
+        b = pm.Batch.from_host([(xy, tri)] * n)
+        b.set_metric(np.tile(inputs.uniform_metric(xy.shape[0], 0.2), (n, 1)))
+        st = b.adapt([pm.Params(seed=1)] * n)
+        assert min(s["splits"] for s in st) > 10
+        b.close()
+        return pool.high()
+
+
+def test_very_many_tiny_meshes_take_little_more_than_they_need():
+    """The spare room of a growth does not rise with the number of meshes beyond 512: what eight times as
+    many hold above that are their own few hundred slots each (a twelfth of the spare ones)."""
+    assert adapt_tiny(4096) < 2 * adapt_tiny(512)
