@@ -199,7 +199,7 @@ pm_status create_set(const double* xy, const int32_t* nv, const int32_t* tri, co
     if (host) {
       const size_t bxy = (size_t)nvt * 2 * sizeof(double), btri = (size_t)net * 3 * sizeof(int32_t);
       const size_t bc = corner ? (size_t)nvt : 0;
-      e = cudaMallocAsync((void**)&tmp, bxy + btri + bc + 64, m.stream);
+      e = device_alloc(&tmp, bxy + btri + bc + 64, m.stream);
       if (!e) e = cudaMemcpyAsync(tmp, xy, bxy, cudaMemcpyHostToDevice, m.stream);
       if (!e) e = cudaMemcpyAsync(tmp + bxy, tri, btri, cudaMemcpyHostToDevice, m.stream);
       if (!e && corner) e = cudaMemcpyAsync(tmp + bxy + btri, corner, bc, cudaMemcpyHostToDevice,
@@ -549,7 +549,7 @@ static pm_status set_metric_impl(pm_mesh* h, const double* M, bool host) {
   const double* src = M;
   double* tmp = nullptr;
   if (host) {
-    cudaError_t e = cudaMallocAsync(&tmp, (size_t)nv * 3 * sizeof(double), m.stream);
+    cudaError_t e = device_alloc(&tmp, (size_t)nv * 3 * sizeof(double), m.stream);
     if (!e) e = cudaMemcpyAsync(tmp, M, (size_t)nv * 3 * sizeof(double), cudaMemcpyHostToDevice,
                                 m.stream);
     if (e) {
@@ -700,7 +700,7 @@ pm_status pm_get_mesh(pm_mesh* h, int32_t* nv, int32_t* ne, double* xy, int32_t*
   // bound of the live counts), then the copies of the live part
   const size_t vb = std::max(m.nv[0], 1), eb = std::max(m.ne[0], 1);
   char* buf = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&buf, vb * 5 * sizeof(double) + eb * 3 * sizeof(int32_t),
+  cudaError_t e = device_alloc(&buf, vb * 5 * sizeof(double) + eb * 3 * sizeof(int32_t),
                                   m.stream);
   pm_status s = cuda_status(e, "output buffers");
   if (s) return s;
@@ -916,7 +916,7 @@ static pm_status batch_get(pm_mesh* h, int32_t* nv, int32_t* ne, double* xy, int
     eb += m.ne[i];
   }
   char* buf = nullptr;
-  pm_status s = cuda_status(cudaMallocAsync((void**)&buf, (size_t)std::max(vb, 1LL) * 5 * 8 +
+  pm_status s = cuda_status(device_alloc(&buf, (size_t)std::max(vb, 1LL) * 5 * 8 +
                                                               (size_t)std::max(eb, 1LL) * 12,
                                             m.stream),
                             "output buffers");

@@ -130,6 +130,16 @@ struct MeshSet {
   std::vector<void*> allocs;   // device allocations owned by the set
 };
 
+// Stream-ordered allocation.  A failure is the caller's to report: it does not stay
+// behind as the thread's last error, which the next check after a launch would take for
+// that launch's.
+template <class T>
+cudaError_t device_alloc(T** p, size_t bytes, cudaStream_t s) {
+  const cudaError_t e = cudaMallocAsync((void**)p, bytes, s);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
 // ---- mesh storage (pm_mesh.cu) ----
 cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vector<int>& ecap,
                       int W);

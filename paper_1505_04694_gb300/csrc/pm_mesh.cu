@@ -79,7 +79,7 @@ struct Carver {
     size_t total = 0;
     for (auto& r : req) total += r.bytes;
     char* base = nullptr;
-    cudaError_t e = cudaMallocAsync((void**)&base, pool_size(total), m.stream);
+    cudaError_t e = device_alloc(&base, pool_size(total), m.stream);
     if (e != cudaSuccess) return e;
     m.allocs.push_back(base);
     size_t off = 0, zoff = 0, zlen = 0;  // adjacent cleared arrays share one memset
@@ -107,7 +107,7 @@ struct Carver {
 cudaError_t rows_alloc(MeshSet& m, int W) {
   const size_t n = (size_t)m.S.vslots * W;
   char* base = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&base, pool_size(std::max<size_t>(5 * n, 1) * sizeof(int)),
+  cudaError_t e = device_alloc(&base, pool_size(std::max<size_t>(5 * n, 1) * sizeof(int)),
                                   m.stream);
   if (e != cudaSuccess) return e;
   m.allocs.push_back(base);
@@ -881,7 +881,7 @@ cudaError_t set_alloc(MeshSet& m, const std::vector<int>& vcap, const std::vecto
   const size_t act_off = had_off + 2 * (size_t)n * sizeof(int);
   if (!m.st) {
     const size_t bytes = act_off + (size_t)n * sizeof(int);
-    if ((e = cudaMallocAsync((void**)&m.st, bytes, m.stream))) return e;
+    if ((e = device_alloc(&m.st, bytes, m.stream))) return e;
     if ((e = cudaMemsetAsync(m.st, 0, bytes, m.stream))) return e;
     const size_t up_off = (had_off + 63) & ~size_t(63);
     size_t need = up_off + (size_t)n * kTabUploadBytes;
@@ -1327,7 +1327,6 @@ int presize(MeshSet& m) {
   e = grow(m, vcap, ecap, W);
   if (e == cudaErrorMemoryAllocation && W > m.S.W) {
     // no room for the wider rows (320 bytes a vertex more): as they are
-    cudaGetLastError();
     e = grow(m, vcap, ecap, m.S.W);
   }
   if (e) {

@@ -298,11 +298,11 @@ int quality_mesh(MeshSet& m, double* qsum_host, double* dxy_host, double* dm_hos
   bool grad = dxy_host || dm_host;
   double *qel = nullptr, *part = nullptr, *out = nullptr, *dxy = nullptr, *dm = nullptr;
   EGrad* eg = nullptr;
-  cudaError_t e = cudaMallocAsync(&qel, std::max(ne, 1) * sizeof(double), s);
-  if (!e) e = cudaMallocAsync(&part, (RED_BLOCKS + 1) * sizeof(double), s);
-  if (!e && grad) e = cudaMallocAsync(&eg, std::max(ne, 1) * sizeof(EGrad), s);
-  if (!e && grad) e = cudaMallocAsync(&dxy, std::max(nv, 1) * 2 * sizeof(double), s);
-  if (!e && grad) e = cudaMallocAsync(&dm, std::max(nv, 1) * 3 * sizeof(double), s);
+  cudaError_t e = device_alloc(&qel, std::max(ne, 1) * sizeof(double), s);
+  if (!e) e = device_alloc(&part, (RED_BLOCKS + 1) * sizeof(double), s);
+  if (!e && grad) e = device_alloc(&eg, std::max(ne, 1) * sizeof(EGrad), s);
+  if (!e && grad) e = device_alloc(&dxy, std::max(nv, 1) * 2 * sizeof(double), s);
+  if (!e && grad) e = device_alloc(&dm, std::max(nv, 1) * 3 * sizeof(double), s);
   int status = PM_OK;
   if (e) {
     set_last_error(std::string("quality workspace: ") + cudaGetErrorString(e));
@@ -381,11 +381,10 @@ int quality_arrays(const double* xy, const double* mt, int nv, const int* tri, i
   }
   h->err = PM_ERR_CUDA;  // overwritten by the last kernel
   char* base = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&base, b_head + b_cnt + b_state + b_part + b_eg + b_off +
+  cudaError_t e = device_alloc(&base, b_head + b_cnt + b_state + b_part + b_eg + b_off +
                                                      b_col + b_pos, s);
   if (e != cudaSuccess) {
     set_last_error(std::string("quality workspace: ") + cudaGetErrorString(e));
-    cudaGetLastError();
     pinned_slot_free(h);
     return e == cudaErrorMemoryAllocation ? PM_ERR_OOM : PM_ERR_CUDA;
   }

@@ -47,3 +47,19 @@ def test_very_many_tiny_meshes_take_little_more_than_they_need():
     """The spare room of a growth does not rise with the number of meshes beyond 512: what eight times as
     many hold above that are their own few hundred slots each (a twelfth of the spare ones)."""
     assert adapt_tiny(4096) < 2 * adapt_tiny(512)
+
+
+def test_calls_work_after_one_that_ran_out_of_memory():
+    """A refused allocation is that call's error alone."""
+    xy, tri = inputs.grid_mesh(65)
+    with MemPool(1 << 28):
+        with pm.Mesh.from_host(xy, tri, device=0) as g:
+            d = 6.0e6
+            g.set_metric(np.tile([d, 0.0, d], (xy.shape[0], 1)))
+            with pytest.raises(pm.PmError, match="PM_ERR_OOM"):
+                g.adapt(pm.Params(seed=1, max_iter=0))
+            out = g.get_mesh()
+            assert np.array_equal(out[0], xy) and np.array_equal(out[1], tri)
+            with pm.Mesh.from_host(xy, tri, device=0) as h:
+                h.set_metric(inputs.uniform_metric(xy.shape[0], 0.02))
+                assert h.adapt(pm.Params(seed=1))["converged"] == 1
