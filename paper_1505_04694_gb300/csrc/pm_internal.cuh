@@ -22,7 +22,8 @@ struct ScanWork {
 };
 
 int scan_tiles(int n);
-void scan_exclusive(const int* in, int* out, int n, ScanWork& w, DevStatus* st, cudaStream_t s);
+void scan_exclusive(const int* in, int* out, int n, ScanWork& w, DevStatus* st, cudaStream_t s,
+                    const int* go = nullptr);
 void scan_alive_vertices(const Store& S, int* out, int n, ScanWork& w, DevStatus* st,
                          cudaStream_t s);
 void scan_alive_elements(const Store& S, int* out, int n, ScanWork& w, DevStatus* st,

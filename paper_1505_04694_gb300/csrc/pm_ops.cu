@@ -3126,7 +3126,9 @@ k_refine_mark(Store S, int* cnt, RowMask* mask, int tag, int pass0, int lo, cons
 
 // Per-mesh number of new vertices (edges to split), after the counters, with
 // the lists that the round's split fills cleared.
-__global__ void k_refine_newcount(Store S, const int* vscan, int* counts) {
+__global__ void k_refine_newcount(Store S, const int* vscan, int* counts, const int* before,
+                                  const DevStatus* st) {
+  if (!may_go(before, st)) return;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) counts[CN_EL] = counts[CN_CL] = 0;
   if (i >= S.nmesh) return;
@@ -4012,9 +4014,10 @@ int ops_ahead(MeshSet& m, Ahead& h) {
   select_ops(m, OS_REFINE);
   PM_LAUNCH(k_refine_mark, grid_tuned(m, m.S.vused, bs, tu.blocks_per_sm[TO_REFINE]), bs, 0,
             m.stream, m.S, w.vcnt, w.vmask, tag + 2, tag, m.lo_refine, rounds_s, rounds_c, st);
-  scan_exclusive(w.vcnt, w.vscan, m.S.vused, m.scan, m.st, m.stream);
+  // (without marks there are no counts either: the vertex slots are not read)
+  scan_exclusive(w.vcnt, w.vscan, m.S.vused, m.scan, m.st, m.stream, rounds_s + 2);
   PM_LAUNCH(k_refine_newcount, (n + 127) / 128, 128, 0, m.stream, m.S, (const int*)w.vscan,
-            w.counts);
+            w.counts, rounds_s, st);
   if (int err = sync_counts(m, kMeshWords * n + CN_NUM)) return err;
 
   const int* rc = m.hcounts + CN_RES;
@@ -4242,7 +4245,7 @@ int op_refine(MeshSet& m, int max_rounds, const Ahead& h, bool* renumber_queued)
                 (const int*)nullptr, (const int*)nullptr, (const DevStatus*)m.st);
       scan_exclusive(w.vcnt, w.vscan, m.S.vused, m.scan, m.st, m.stream);
       PM_LAUNCH(k_refine_newcount, (n + 127) / 128, 128, 0, m.stream, m.S, (const int*)w.vscan,
-                w.counts);
+                w.counts, (const int*)nullptr, (const DevStatus*)m.st);
       // (beside the marks' scan, which a split still needs; the counts are spent)
       if (ahead) renumber_queue(m, w.vcnt);
       if (int err = ahead ? sync_call(m) : sync_counts(m, kMeshWords * n)) return err;

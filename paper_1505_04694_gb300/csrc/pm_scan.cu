@@ -90,7 +90,9 @@ struct ElementAlive {
 template <class Input>
 __global__ void __launch_bounds__(SCAN_THREADS)
 k_scan(Input input, int* __restrict__ out, int n, unsigned long long* state, int* ticket,
-       unsigned epoch, DevStatus* st) {
+       unsigned epoch, DevStatus* st, const int* go) {
+  // (no ticket is taken, so none is outstanding; both words stand still meanwhile)
+  if (go && (*go == 0 || st->overflow != 0)) return;
   __shared__ int s_warp[SCAN_THREADS / 32];
   __shared__ int s_tile;
   __shared__ int s_excl;
@@ -204,7 +206,8 @@ int scan_tiles(int n) { return (n + SCAN_TILE - 1) / SCAN_TILE; }
 namespace {
 
 template <class Input>
-void scan_run(Input input, int* out, int n, ScanWork& w, DevStatus* st, cudaStream_t s) {
+void scan_run(Input input, int* out, int n, ScanWork& w, DevStatus* st, cudaStream_t s,
+              const int* go = nullptr) {
   if (n <= 0) {
     cudaMemsetAsync(out, 0, sizeof(int), s);
     return;
@@ -213,16 +216,18 @@ void scan_run(Input input, int* out, int n, ScanWork& w, DevStatus* st, cudaStre
   w.epoch = (w.epoch + 1) & 0x3FFFFFFFu;
   if (w.epoch == 0) w.epoch = 1;
   PM_LAUNCH(k_scan<Input>, tiles, SCAN_THREADS, 0, s, input, out, n, w.state, w.ticket, w.epoch,
-            st);
+            st, go);
 }
 
 }  // namespace
 
 // Exclusive scan of in[0..n) into out[0..n]; out[n] holds the total.
 // `state` needs scan_tiles(n) words and is never cleared (epochs tell runs
-// apart); `ticket` starts at zero and every scan leaves it there.
-void scan_exclusive(const int* in, int* out, int n, ScanWork& w, DevStatus* st, cudaStream_t s) {
-  scan_run(IntInput{in}, out, n, w, st, s);
+// apart); `ticket` starts at zero and every scan leaves it there.  With `go` the scan
+// does nothing when *go is zero or a row has outgrown its width.
+void scan_exclusive(const int* in, int* out, int n, ScanWork& w, DevStatus* st, cudaStream_t s,
+                    const int* go) {
+  scan_run(IntInput{in}, out, n, w, st, s, go);
 }
 
 // The same over the alive flags of the used vertex (element) slots [0, n).
