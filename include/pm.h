@@ -327,9 +327,9 @@ pm_status pm_quality_arrays_noalloc_dev(const double* xy, const double* m, int32
  *     smoothing), threads per block (64, 128 or 256) and the cap on blocks
  *     per SM (1..32) of the one-kernel-per-phase round kernels: together they
  *     set the worklist chunk each thread walks.
- *   rounds_limit[3]: per operator (collapse, flip, smoothing), the largest
- *     list (vertices) whose rounds run inside one persistent launch (0: never;
- *     at most 2^30).
+ *   rounds_limit[3]: per operator (collapse, flip, smoothing; colouring takes
+ *     the smoothing's), the largest list (vertices) whose rounds run inside one
+ *     persistent launch (0: never; at most 2^30).
  *   rounds_blocks_per_sm[3]: resident blocks per SM of those persistent
  *     launches (1 or 2; fewer when the kernel's registers allow fewer).
  *   fuse_limit[2]: flips, smoothing: inside the persistent launch, lists up

@@ -3807,10 +3807,9 @@ int after_round(MeshSet& m, const RoundIO& io) {
 // smoothing (12.88 ms at 131072 against 13.2 at 32768 on the 201 x 201 mesh), 32768
 // for collapses, whose longer lists run faster one vertex per thread on a full
 // chip (8.08 against 8.80 ms on a 317 x 317 grid coarsened to 18k triangles).
+// Colouring follows the smoothing's limit: its rounds are light too (gathers and a
+// mask), and each costs two launches and a wait outside the persistent kernel.
 constexpr int kRoundsThreads = 256;
-// Colouring rounds are light (gathers and a mask), and each costs two launches
-// and a wait outside the persistent kernel.
-constexpr int kColourLimit = 131072;
 
 // Blocks of a cooperative launch of the persistent round kernel `which`
 // (0 collapse, 1 flip, 2 smoothing, 3 colouring) on this device: the tuning's blocks per
@@ -3922,7 +3921,7 @@ int colour_set(MeshSet& m) {
   Work& w = m.w;
   const int g = grid_for(m, m.S.vused);
   const bool persist = rounds_grid(m, 3) > 0;
-  const int limit = kColourLimit;
+  const int limit = tuning().rounds_limit[2];
   bool bar_clear = true;
   zero_counts(m, 0, CN_NUM);
   PM_LAUNCH(k_colour_init, g, BLOCK, 0, m.stream, m.S, w.D[0], w.counts + CN_D0);

@@ -117,3 +117,24 @@ def test_many_small_meshes_whose_rows_overflow():
         assert_same_mesh(got, o.get_mesh(), f"mesh {i}")
         for k in ("rounds", "collapses", "splits", "flips", "moves"):
             assert sb[i][k] == so[k], (i, k, sb[i][k], so[k])
+
+
+# a colouring a kernel per phase throughout; begun so and ended in persistent rounds; persistent alone
+@pytest.mark.parametrize("limit,steps", [(0, True), (100, True), (3000, True), (ALL, False)])
+def test_colouring_takes_the_limits_route(adapted, tuned, limit, steps):
+    w, res = adapted
+    so, om = res[1]
+    tuned([ALL, ALL, limit], [ALL, ALL])
+    count = {}
+    for kernel in ("k_colour_propose", "k_colour_rounds"):
+        g = pm.Mesh.from_host(w.xy, w.tri, device=0)
+        g.set_metric(w.m)
+        pm.profile_enable(kernel)
+        sg = g.adapt(pm.Params(seed=2, select=1))
+        count[kernel] = pm.profile_read()[1]
+        pm.profile_enable(None)
+        assert_same_mesh(g.get_mesh(), om, f"{limit} {kernel}")
+        for k in STAT_KEYS:
+            assert sg[k] == so[k], (k, sg[k], so[k])
+    assert (count["k_colour_propose"] > 0) == steps
+    assert count["k_colour_rounds"] > 0  # (the first launch finds the list too long)
