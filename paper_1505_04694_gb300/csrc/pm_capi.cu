@@ -141,12 +141,14 @@ void set_mem_pool_retain(int dev) {
 cudaError_t upload_prefix(MeshSet& m, const std::vector<int>& nv, const std::vector<int>& ne) {
   const int n = m.nmesh;
   if (n == 1) return cudaSuccess;  // a single mesh's offsets are zero
-  std::vector<int> pre(2 * ((size_t)n + 1));
+  std::vector<int>& pre = m.hpre;
+  pre.assign(2 * ((size_t)n + 1), 0);
   for (int i = 0; i < n; ++i) {
     pre[i + 1] = pre[i] + nv[i];
     pre[n + 1 + i + 1] = pre[n + 1 + i] + ne[i];
   }
-  // a copy from pageable memory is staged before the call returns
+  // (the source stays as it is until the caller has waited: a device that reads
+  // pageable memory itself need not stage it)
   return cudaMemcpyAsync(m.S.tab.pre, pre.data(), pre.size() * sizeof(int),
                          cudaMemcpyHostToDevice, m.stream);
 }
@@ -303,12 +305,6 @@ pm_status adapt_set(MeshSet& m, const pm_params* P, int stride, CallStats& cs) {
   for (int i = 0; i < n; ++i) max_iter = std::max(max_iter, P[stride ? i : 0].max_iter);
   std::vector<int> active(n, 1), sent(n, 1);  // begin_call made every mesh active
   std::vector<unsigned long long> seen(3 * (size_t)n, 0);
-  // the device flags follow `active` (a copy from pageable memory is staged)
-  auto send_active = [&](const std::vector<int>& a) {
-    if (a == sent) return;
-    cudaMemcpyAsync(m.S.tab.active, a.data(), n * sizeof(int), cudaMemcpyHostToDevice, m.stream);
-    sent = a;
-  };
   const int mr = P[0].max_rounds;
   int err;
   for (int it = 0; it < max_iter; ++it) {
@@ -318,7 +314,13 @@ pm_status adapt_set(MeshSet& m, const pm_params* P, int stride, CallStats& cs) {
       any |= active[i] != 0;
     }
     if (!any) break;
-    send_active(active);
+    if (active != sent) {
+      // the device flags follow; `active` stays as it is until the iteration's
+      // read-back (a device that reads pageable memory itself need not stage it)
+      cudaMemcpyAsync(m.S.tab.active, active.data(), n * sizeof(int), cudaMemcpyHostToDevice,
+                      m.stream);
+      sent = active;
+    }
     Ahead done;
     if (mr == 0 && (err = ops_ahead(m, done))) return (pm_status)err;
     select_ops(m, OS_COARSEN);
@@ -346,7 +348,8 @@ pm_status adapt_set(MeshSet& m, const pm_params* P, int stride, CallStats& cs) {
     }
     std::copy(h, h + 3 * (size_t)n, seen.begin());
   }
-  send_active(std::vector<int>(n, 1));
+  if (sent != std::vector<int>(n, 1))  // every mesh again, as begin_call left them
+    cudaMemsetAsync(m.S.tab.active, 0xFF, n * sizeof(int), m.stream);
   int sweeps = 0, opt = 0;
   for (int i = 0; i < n; ++i) {
     sweeps = std::max(sweeps, P[stride ? i : 0].max_smooth_sweeps);

@@ -114,6 +114,7 @@ struct MeshSet {
   std::vector<long long> edead;        // dead element slots of each mesh
   std::vector<long long> seen_dead;    // those of the current call counted so far
   bool dense = false;  // no dead slot: ids are the slot offsets and the sizes are nv, ne
+  std::vector<int> hpre;               // source of upload_prefix
   char* hup = nullptr;                 // pinned: staging of the per-mesh table for upload_tab
   cudaEvent_t upev = nullptr;          // the last table upload has left the staging
   void* pinned = nullptr;      // slot of the process-wide pinned arena (hst, hcounts)
