@@ -138,3 +138,44 @@ def test_colouring_takes_the_limits_route(adapted, tuned, limit, steps):
             assert sg[k] == so[k], (k, sg[k], so[k])
     assert (count["k_colour_propose"] > 0) == steps
     assert count["k_colour_rounds"] > 0  # (the first launch finds the list too long)
+
+
+def _hub(nb, offset):
+    """A disc: a vertex off its centre joined to a ring of nb interior vertices, which a second ring of
+    nb boundary vertices surrounds; coordinates around (offset, offset)."""
+    rng = np.random.default_rng(nb)
+    t = 2 * np.pi * (np.arange(nb) + rng.uniform(-0.2, 0.2, nb)) / nb
+    u = np.stack([np.cos(t), np.sin(t)], axis=1)
+    s = 2 * np.pi * (np.arange(nb) + 0.5) / nb
+    xy = np.concatenate([[[0.2, 0.15]], 0.6 * u * rng.uniform(0.95, 1.05, (nb, 1)),
+                         np.stack([np.cos(s), np.sin(s)], axis=1)]) + offset
+    i = np.arange(nb)
+    j = (i + 1) % nb
+    tri = np.concatenate([np.stack([0 * i, 1 + i, 1 + j], axis=1),
+                          np.stack([1 + i, 1 + nb + i, 1 + j], axis=1),
+                          np.stack([1 + j, 1 + nb + i, 1 + nb + j], axis=1)]).astype(np.int32)
+    return xy, tri, inputs.uniform_metric(xy.shape[0], 2 * np.pi / nb)
+
+
+# balls of 24 to 124 elements moved in the rounds with a kernel per phase, where one of more than 32
+# takes a warp by itself, and in the persistent ones.  At offset 0 the bounds accept the moves and their
+# qualities follow; at 2^36 a coordinate's error leaves every quality to the exact pass.
+@pytest.mark.parametrize("limit", [0, ALL])
+@pytest.mark.parametrize("offset", [0.0, 2.0 ** 36])
+@pytest.mark.parametrize("nb", [24, 32, 33, 36, 64, 65, 84, 124])
+def test_moves_of_large_balls(tuned, nb, offset, limit):
+    xy, tri, m = _hub(nb, offset)
+    tuned([limit] * 3, [ALL, ALL])
+    for opname in ("smooth", "adapt"):
+        g = pm.Mesh.from_host(xy, tri, device=0)
+        g.set_metric(m)
+        o = O.OracleMesh(xy, tri).set_metric(m)
+        sg = getattr(g, opname)(pm.Params(seed=4))
+        so = getattr(o, opname)(O.make_params(seed=4))
+        for k in STAT_KEYS:
+            assert sg[k] == so[k], (opname, k, sg[k], so[k])
+        rg = g.get_raw()
+        assert_same_raw(rg, o.get_raw(), opname)
+        assert_same_adjacency(g, o, rg)
+        if opname == "smooth":
+            assert sg["moves"] > 0 and not np.array_equal(o.get_mesh()[0][0], xy[0])
