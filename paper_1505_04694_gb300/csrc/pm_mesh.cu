@@ -1318,10 +1318,14 @@ int presize(MeshSet& m) {
     et += ecap[i];
   }
   if (!need || vt >= (1LL << 31) - 4 || et >= (1LL << 31) - 4) return PM_OK;
-  // A set of many vertices nearly always meets one of more than 16 neighbours, and
-  // widening the rows later rebuilds every row in storage of its own: such sets
-  // start with 32 (20M slots: 100.2 -> 95.1 ms, 42M slots: 260 -> 255 ms; at 3M
-  // slots, where the rebuild is cheap, rows of 16 are faster, 10.93 against 11.09).
+  // A vertex of more than 16 neighbours widens every row of the set: rows in storage of
+  // their own are rebuilt and every evaluation is made again.  The larger a set, the
+  // likelier it meets one, and no count known here says so; large sets start with rows
+  // of 32.  Where a vertex needs them they save 5 to 6% (psi metric, 12M slots 52.7 ->
+  // 49.6 ms, 20M 100.2 -> 95.1) or 1 to 2% (batches, 10M 61.1 -> 60.2, 19M 104.4 ->
+  // 102.8, 42M 260 -> 255); where none does they cost 2 to 4% (psi, 8M 26.1 -> 26.8,
+  // another of 12M 33.1 -> 34.0; uniform, 12M 13.2 -> 13.7, 21M 22.7 -> 23.5).  Below the
+  // line no single mesh measured needed them (psi, 2M to 6M: 1.5 to 2% slower with them).
   constexpr long long kWideRowsFrom = 1LL << 23;
   const int W = vt >= kWideRowsFrom ? std::max(m.S.W, 32) : m.S.W;
   e = grow(m, vcap, ecap, W);
