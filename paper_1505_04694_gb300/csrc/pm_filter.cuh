@@ -31,6 +31,7 @@
 #pragma once
 
 #include <math.h>
+#include <string.h>
 
 #ifdef __CUDACC__
 #define PM_HD __host__ __device__ __forceinline__
@@ -67,6 +68,30 @@ PM_HD float f_rcp(float x) {
   return r;
 #else
   return 1.0f / x;
+#endif
+}
+
+// The power of two of a positive normal number (its exponent bits), and its reciprocal.
+PM_HD float f_pow2(float x) {
+#ifdef __CUDA_ARCH__
+  return __int_as_float(__float_as_int(x) & 0x7f800000);
+#else
+  int b;
+  memcpy(&b, &x, 4);
+  b &= 0x7f800000;
+  memcpy(&x, &b, 4);
+  return x;
+#endif
+}
+PM_HD float f_pow2_inv(float x) {
+#ifdef __CUDA_ARCH__
+  return __int_as_float(0x7f000000 - (__float_as_int(x) & 0x7f800000));
+#else
+  int b;
+  memcpy(&b, &x, 4);
+  b = 0x7f000000 - (b & 0x7f800000);
+  memcpy(&x, &b, 4);
+  return x;
 #endif
 }
 
@@ -149,18 +174,14 @@ PM_HD int f_len_cmp(const FLen& l, float lo2, float hi2) {
 // Bounds of the quality (12 sqrt 3 A / P^2) F(P / 3) of element (a, b, c) in its
 // mean metric: `up` is NaN and `lo` -1 when they would be loose, and `lo` is -1
 // unless the element is certainly counter-clockwise.  The quality grows with the
-// area and the metric's determinant, which are taken at their bounds.  The
-// determinant is k00 times its Schur complement s = k11 - k01 (k01 / k00), and each
-// factor's root is taken by itself: the product k00 k11 would leave single precision
-// at half the range (in powers of ten) that the entries have, so that a mesh in small
-// or large units would get no bound at all.  Inputs known to ku relative change the
-// determinant by at most 4 ku k00 k11 to first order (two for each product), hence s
-// by 4 ku k11; reciprocal, products and difference add 5 u k11, together 25 u k11 and
-// kx's part (with its second order, kx < 0.05, 4.2 kx k11).  As a function of
-// P the quality is h(P) = F(P / 3) / P^2 with |d ln h / d ln P| <= 5 (between -2 and 1 below the
+// area and the metric's determinant, which are taken at their bounds; as a function of
+// P it is h(P) = F(P / 3) / P^2 with |d ln h / d ln P| <= 5 (between -2 and 1 below the
 // ideal perimeter, between -5 and -2 above), so a relative error rP of P changes it by
 // at most 5 rP to first order (rP <= 0.04 is required, the rest of the series is inside
-// the factor 1.15).  `sign` receives the orientation's sign, 0 when undecided.  `kx`
+// the factor 1.15).  The determinant is taken of the metric divided by k00's power of
+// two (exact): of the entries themselves the product k00 k11 leaves single precision at
+// half the decades that a record holds, and a mesh in small or large units would get no
+// bound.  `sign` receives the orientation's sign, 0 when undecided.  `kx`
 // bounds the relative error of one vertex's metric beyond its rounding (see
 // f_metric_at): it adds to that of the mean, and four times to the determinant's.
 struct FQual {
@@ -188,22 +209,24 @@ PM_HD FQual f_quality(const VF& a, const VF& b, const VF& c, int& sign, float kx
   // sqrt(L2) - sqrt(L2 - err) <= 0.75 err / sqrt(L2) while err <= L2 / 2
   const float eP = 0.75f * ((q0.err * f_rcp(l0) + q1.err * f_rcp(l1)) + q2.err * f_rcp(l2));
   const float rP = eP * rp + 6.0f * kU;
-  // (perimeters whose powers would underflow give no bound)
+  const float two = f_pow2(k00), inv = f_pow2_inv(k00);
+  const float s00 = k00 * inv, s01 = k01 * inv, s11 = k11 * inv, kk = s00 * s11;
+  // (perimeters and metrics whose powers would underflow give no bound)
   const bool fine = rP < 0.04f && kx < 0.05f && q0.err < 0.4f * q0.L2 && q1.err < 0.4f * q1.L2 &&
-                    q2.err < 0.4f * q2.L2 && P > 1e-6f && P < 1e6f;
-  const float sc = k11 - k01 * (k01 * f_rcp(k00)), es = (30.0f * kU + 4.2f * kx) * k11;
-  const float r0 = 20.784612f * f_sqrt(k00);
+                    q2.err < 0.4f * q2.L2 && P > 1e-6f && P < 1e6f && kk > 1e-30f;
+  const float D = kk - s01 * s01, eD = (28.0f * kU + 4.2f * kx) * kk;
   const float up = 0.5f * (d.det + d.err);
   const float area = up < 0.0f ? 0.0f : up;  // a negative quality is below 0 (a NaN stays)
   const float x = P * third;
   const float s = x > 1.0f ? 3.0f * rp : x;
   const float f = s * (2.0f - s);
-  const float h = (rp * rp) * ((f * f) * f), eh = 5.75f * rP + 44.0f * kU;
-  const float q = ((area * r0) * f_sqrt(sc + es)) * h;
-  const float p = (((0.5f * (d.det - d.err)) * r0) * f_sqrt(sc - es)) * h;
+  const float h = (rp * rp) * ((f * f) * f), eh = 5.75f * rP + 40.0f * kU;
+  const float w = 20.784612f * two;
+  const float q = ((w * area) * f_sqrt(D + eD)) * h;
+  const float p = ((w * (0.5f * (d.det - d.err))) * f_sqrt(D - eD)) * h;
   FQual r;
   r.up = fine ? q + (q * eh + 1e-30f) : nanf("");
-  r.lo = fine && sign > 0 && sc > es ? p - (p * eh + 1e-30f) : -1.0f;
+  r.lo = fine && sign > 0 && D > eD ? p - (p * eh + 1e-30f) : -1.0f;
   return r;
 }
 
