@@ -3128,12 +3128,13 @@ k_refine_mark(Store S, int* cnt, RowMask* mask, int tag, int pass0, int lo, cons
 // the lists that the round's split fills cleared.
 __global__ void k_refine_newcount(Store S, const int* vscan, int* counts, const int* before,
                                   const DevStatus* st) {
-  if (!may_go(before, st)) return;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
+  // (loaded together: the launch is a chain of latencies)
+  const int go = before ? before[2] : 1, over = before ? st->overflow : 0;
+  const int vb = i < S.nmesh ? S.tab.vbase[i] : 0, nv = i < S.nmesh ? S.tab.nv[i] : 0;
+  if (go == 0 || over != 0) return;
   if (i == 0) counts[CN_EL] = counts[CN_CL] = 0;
-  if (i >= S.nmesh) return;
-  int vb = S.tab.vbase[i];
-  counts[cn_newv(S.nmesh) + i] = vscan[vb + S.tab.nv[i]] - vscan[vb];
+  if (i < S.nmesh) counts[cn_newv(S.nmesh) + i] = vscan[vb + nv] - vscan[vb];
 }
 
 __device__ __forceinline__ int mid_id(const Store& S, int vb, int nv, const int* vscan,

@@ -91,19 +91,22 @@ template <class Input>
 __global__ void __launch_bounds__(SCAN_THREADS)
 k_scan(Input input, int* __restrict__ out, int n, unsigned long long* state, int* ticket,
        unsigned epoch, DevStatus* st, const int* go) {
-  // (no ticket is taken, so none is outstanding; both words stand still meanwhile)
-  if (go && (*go == 0 || st->overflow != 0)) return;
   __shared__ int s_warp[SCAN_THREADS / 32];
   __shared__ int s_tile;
   __shared__ int s_excl;
   __shared__ int s_fail;
+  __shared__ int s_go;
   if (threadIdx.x == 0) {
+    // (read beside the ticket; every block takes one, so that the last re-arms it)
+    const int flag = go ? *go : 1, over = go ? st->overflow : 0;
     s_tile = atomicAdd(ticket, 1);
+    s_go = flag != 0 && over == 0;
     // tickets go out in order: whoever holds the last one re-arms the counter
     if (s_tile == (int)gridDim.x - 1) *ticket = 0;
     s_fail = 0;
   }
   __syncthreads();
+  if (!s_go) return;
   const int tile = s_tile;
   const long long first = (long long)tile * SCAN_TILE + (long long)threadIdx.x * SCAN_ITEMS;
   int v[SCAN_ITEMS];
