@@ -674,8 +674,8 @@ __device__ __forceinline__ int first_by_length(const Store& S, int v, int vb, co
 // equal lengths are compared exactly 39-63%; with all lengths exact it was 80%): 36
 // ms of a 512-mesh batch's collapses, 12.1 with the FP32 lengths, 11.5 held to 80
 // registers (24 warps an SM instead of 16; at 64 it spills: 12.3).  These times are
-// sums over CUDA events around each launch of one adaptation; serialised, with caches
-// flushed before each launch, the same launches take 13.
+// sums over CUDA events around each launch of one adaptation of 512 jittered grids; the
+// benchmark's, whose grids are regular, takes 13.0.
 __device__ __forceinline__ void coarsen_scan_phase(Store S, const int* D, const int* nDp,
                                                    int* target, int* cand, int* C, int* nC,
                                                    int* cmark, int tag, int pass0, int* W0,
@@ -932,7 +932,8 @@ __device__ __forceinline__ bool check_candidates(const Store& S, const CheckQueu
 // Pass 2: every listed vertex's first candidate.  Gathers bound it (L1 50-65%, DRAM
 // 31-48%, FP64 pipe below 1%, on regular grids 33%); with every test in FP64 the
 // two check passes took 47 ms of a 512-mesh batch, 26.4 with the filters, 21.3 (15.0 and
-// 6.3) with pass 3 as it is (events around each launch; serialised and cold 28).
+// 6.3) with pass 3 as it is (jittered grids; on the benchmark's regular ones, whose
+// collinear points are decided exactly, 15.2 and 12.7).
 __device__ __forceinline__ void coarsen_check_phase(Store S, const int* Win, const int* nWin,
                                                     int* Wout, int* nWout, int* target, int* cand,
                                                     int* C, int* nC, int* cmark, int tag,
@@ -1690,7 +1691,7 @@ __device__ __forceinline__ void flip_run(const Store& S, FlipQueue& Q, int cnt, 
 // Pass 2: the gains, by stages, full warps of items in each.  FP64 in full bound it
 // (57 ms of a 512-mesh batch); the FP32 bounds end most items, and the exact rest
 // runs at 64 registers, four blocks of 256 an SM (16.5 ms at three, 14.8 at four,
-// 17.9 at five, which spill; events around each launch, serialised and cold 17).
+// 17.9 at five, which spill; jittered grids, on the benchmark's regular ones 17.7).
 __device__ __forceinline__ void swap_edge_phase(Store S, const int2* items, const int* nIp,
                                                 int icap, double* gains, int tag,
                                                 unsigned long long* work, bool il = false) {
