@@ -549,10 +549,16 @@ __global__ void k_out_e(Store S, int mesh, const int* vscan, const int* escan, i
 
 // sqrt(det M) from a vertex record: the root of m00 times that of its Schur
 // complement (the product m00 m11 leaves single precision at half the range of the
-// entries), NaN unless the complement is known to about 5% (aspect ratios up to 600).
+// entries); NaN for aspect ratios beyond 600, where rounding the entries changes the
+// complement by 5% and more.
 __device__ __forceinline__ float root_det(const VF& v) {
   const float s = v.m11 - v.m01 * (v.m01 * f_rcp(v.m00));
   return s > 1e-5f * v.m11 ? f_sqrt(v.m00) * f_sqrt(s) : nanf("");
+}
+// The same with the determinant in FP64, of the metric divided by m00's power of two.
+__device__ __forceinline__ float root_det(const VF& v, double4 m) {
+  const double inv = f_pow2_inv(v.m00);
+  return f_pow2(v.m00) * f_sqrt((float)((m.x * inv) * (m.z * inv) - (m.y * inv) * (m.y * inv)));
 }
 __device__ __forceinline__ double root_det(const VD& v) {
   return sqrt(fmax(v.m00 * v.m11 - v.m01 * v.m01, 0.0));
@@ -562,14 +568,15 @@ __device__ __forceinline__ double root_det(const VD& v) {
 // the sum over live elements of area * mean sqrt(det M) of its vertices (the
 // number of unit equilateral metric triangles that tile the mesh).  Only
 // sizes storage, so single precision serves where it holds the factors (FP64 for
-// all was bound by the FP64 pipe, 2.5 ms on 19M elements, 0.45 now; units and
-// anisotropies beyond it take FP64) and the order of the atomic sums does not matter.
+// all was bound by the FP64 pipe, 2.5 ms on 19M elements, 0.47 now; units
+// beyond it take FP64) and the order of the atomic sums does not matter.
 __global__ void k_estimate(Store S, double* est) {
   const int lane = threadIdx.x & 31;
   for (int s0 = blockIdx.x * blockDim.x; s0 < S.eused; s0 += gridDim.x * blockDim.x) {
     const int s = s0 + (int)threadIdx.x;
     int mi = -1;
     float x = 0.0f;
+    double y = 0.0;
     if (s < S.eused && eslot_used(S, s, mi)) {
       int4 e = S.EN[s];
       if (e.w) {
@@ -577,24 +584,29 @@ __global__ void k_estimate(Store S, double* est) {
         const VF a = load_vf(S, vb + e.x), b = load_vf(S, vb + e.y), c = load_vf(S, vb + e.z);
         const float area =
             0.5f * fabsf(f_dx(a, b) * f_dy(a, c) - f_dy(a, b) * f_dx(a, c));
-        const float sd = (root_det(a) + root_det(b)) + root_det(c);
+        float sd = (root_det(a) + root_det(b)) + root_det(c);
+        if (!(sd == sd))
+          sd = (root_det(a, S.M[vb + e.x]) + root_det(b, S.M[vb + e.y])) +
+               root_det(c, S.M[vb + e.z]);
         x = area * (sd * (1.0f / 3.0f));
         if (!(area > 1e-34f && sd > 1e-34f && sd < 1e34f && x < 1e34f)) {
           const VD p = load_vd(S, vb + e.x), q = load_vd(S, vb + e.y), r = load_vd(S, vb + e.z);
           x = 0.0f;
-          atomicAdd(est + mi, 0.5 * fabs(orient3(p, q, r)) *
-                                  ((root_det(p) + root_det(q)) + root_det(r)) / 3.0);
+          y = 0.5 * fabs(orient3(p, q, r)) * ((root_det(p) + root_det(q)) + root_det(r)) / 3.0;
         }
       }
     }
     // a warp whose slots all belong to one mesh (meshes are contiguous runs
-    // of slots) adds its sum with one atomic
+    // of slots) adds its sums with one atomic
     const int m0 = __shfl_sync(0xffffffffu, mi, 0);
+    const bool wide = __any_sync(0xffffffffu, y != 0.0);
     if (__all_sync(0xffffffffu, mi == m0) && m0 >= 0) {
       for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-      if (lane == 0) atomicAdd(est + m0, (double)x);
+      if (wide)
+        for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+      if (lane == 0) atomicAdd(est + m0, (double)x + y);
     } else if (mi >= 0) {
-      atomicAdd(est + mi, (double)x);
+      atomicAdd(est + mi, (double)x + y);
     }
   }
 }
